@@ -108,15 +108,6 @@ __global__ void k_fill_gid(const int64_t *voff, const int32_t *gl, int32_t *gid)
     gid[v0 + u] = gl[j];
 }
 
-// Position of every vertex's graph inside the union (the bisection roots).
-__global__ void k_fill_pos(const int64_t *voff, int32_t *pos) {
-  const int j = blockIdx.y;
-  const int64_t v0 = voff[j], n = voff[j + 1] - v0;
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x)
-    pos[v0 + u] = j;
-}
-
 // First vertex of every graph of the union, indexed by batch position.
 __global__ void k_vbase(const int64_t *voff, const int32_t *gl, int64_t G, int64_t *vb) {
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < G;
@@ -503,20 +494,15 @@ void partition_union(const std::vector<const tp_graph *> &gs, const std::vector<
       }
       ULevel &X = all ? L : Xl;
       std::vector<IPRoot> roots;
-      int64_t maxlen = 0;
       for (int64_t j = 0; j < X.G(); ++j) {
         const int32_t i = X.gl[j];
         roots.push_back(IPRoot{(int32_t)boff[i], 0, k[i], lmax[i]});
-        maxlen = std::max(maxlen, X.voff[j + 1] - X.voff[j]);
       }
-      Buf<int32_t> pos(std::max<int64_t>(X.n(), 1), s);
-      launch(k_fill_pos, per_graph_grid(X.G(), maxlen), 256, 0, s, X.d_voff.get(), pos.get());
-      TP_LAUNCH_CHECK();
       if (all) {
-        initial_partition_roots(X.g.get(), roots, pos.get(), p, part.get(), s);
+        initial_partition_roots(X.g.get(), roots, X.voff, p, part.get(), s);
       } else {
         Buf<int32_t> xp(std::max<int64_t>(X.n(), 1), s);
-        initial_partition_roots(X.g.get(), roots, pos.get(), p, xp.get(), s);
+        initial_partition_roots(X.g.get(), roots, X.voff, p, xp.get(), s);
         launch(k_scatter_i32, grid_for(X.n(), 256), 256, 0, s, xp.get(), xsel.get(), X.n(),
                part.get());
         TP_LAUNCH_CHECK();

@@ -2,8 +2,7 @@
 // paper's KaMinPar uses a portfolio of greedy graph growing and 2-way FM,
 // Section "KaMinPar"). Deterministic GPU form: every node of the bisection
 // tree owns the blocks [offset, offset + kk); its vertices are bisected with
-// kk0 = ceil(kk/2) and kk1 = floor(kk/2) blocks per side by T seeded attempts,
-// one CTA each:
+// kk0 = ceil(kk/2) and kk1 = floor(kk/2) blocks per side by T seeded attempts:
 //   1. BFS from a hashed seed vertex (FIFO order, neighbours in ascending id,
 //      unreached vertices appended in ascending id), computed level by level:
 //      a vertex joins the next frontier behind the earliest frontier vertex
@@ -14,47 +13,73 @@
 //      kk0 * L_max and kk1 * L_max and the same prefix approval as k-way LP;
 //   4. the cut of the induced subgraph.
 // The attempt with the smallest cut (lowest attempt on ties) wins; the tree
-// is processed depth by depth, all nodes of a depth in one launch. Batched
+// is processed depth by depth, all nodes of a depth together. Batched
 // graphs form a forest: every graph's root carries the hash key offset and
 // L_max its graph would use alone, so each tree's result is that graph's.
+//
+// An attempt is run by one CTA whose state (BFS order, claims, connectivity,
+// sides) lives in shared memory, or, where the node is too large for that or
+// has so many edges that one SM would scan them for long, by a thread-block
+// cluster of 2 to 16 CTAs with the state in global memory; the barriers are
+// then the hardware's cluster barriers. The 2-way LP keeps every vertex's
+// connectivity difference D = (weight to side 1) - (weight to side 0) and
+// updates it along the edges of moved vertices only, so the 8 sub-rounds of a
+// round cost the edges of the movers instead of all edges, and the cut is a
+// sum over D.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <vector>
 
-#include "tp_internal.cuh"
+#include "select.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace tp {
 
 namespace {
 
-// Threads per attempt: 1024 for large nodes or few attempts in flight,
-// 512, 256 or 128 when many smaller nodes share the GPU (several CTAs per SM).
-constexpr int kIPThreads = 1024;
+constexpr int kIPMaxThreads = 1024;
 
 struct IPCtx {
   int64_t n;
-  const int64_t *xadj;
-  const int32_t *adj;
-  const int64_t *vw, *ew;  // null: unit
-  const int32_t *node_of;  // node index per vertex (-1: done)
+  const int64_t *vw;       // null: unit
   const int32_t *vlist;    // vertices sorted by (node, id)
   const int64_t *nstart;   // node start in vlist
-  const int32_t *loc;      // position of a vertex inside its node
   // the subgraph induced by every node, in local positions: vertex vlist[p]
   // has neighbours ladj[lxadj[p] .. lxadj[p + 1]) (ascending, as in the graph)
   const int64_t *lxadj;
   const int32_t *ladj;
   const int64_t *lew;  // null: unit
   const int32_t *noff, *nkk;
-  const int32_t *nkey;    // per node: the block offset its graph alone would give it (hash key)
+  const int32_t *nkey;   // per node: the block offset its graph alone would give it (hash key)
   const int64_t *nlmax;  // per node: its graph's L_max
+  const int32_t *nodes;  // nodes of this launch
   int32_t T;
   uint64_t seed;
   int32_t rounds, S;
-  // scratch, T * n entries each
-  int32_t *ord, *disc, *claimer, *cnt, *side, *mvx0, *mvx1, *ok0, *ok1;
-  int64_t *mvg0, *mvg1;
-  uint8_t *sub;  // sub-round of every vertex in the current 2-way LP round
-  int64_t *cut;  // nodes * T
+  int32_t cap;      // vertices the shared-memory state has room for
+  int32_t n_nodes;  // nodes of this depth
+  // scratch of the cluster form, T * n entries each (cnt: T * (n + n_nodes),
+  // a frontier's counts and their total)
+  int32_t *ord, *claimer, *cnt, *list;
+  void *dif;
+  uint8_t *sub;
+  uint8_t *side;  // T * n: the result of every attempt
+  int64_t *cut;   // nodes * T
+};
+
+// What the CTAs of an attempt share (in the first CTA's shared memory). The
+// movers' counters and weights rotate over three sub-rounds: the set two
+// sub-rounds ahead is cleared while nobody can still read it.
+struct IPCtl {
+  unsigned long long W, wdeg, acc;
+  unsigned long long inw[3][2], dlw[3];
+  int32_t ncnt[3][2];
+  int32_t nz, nnew, tail;
+  unsigned long long w0;
+  unsigned long long khi[2];
+  uint32_t klo[2];
 };
 
 template <int NT>
@@ -77,102 +102,32 @@ __device__ __forceinline__ int64_t bscan_excl(int64_t v, int64_t &total) {
   return off + incl - v;
 }
 
+// Exclusive scan of x[0..len) in place by one CTA, x[len] = total (int32: the
+// sums are vertex counts). Four entries a thread and step: a quarter of the
+// barriers of one entry a step.
 template <int NT>
-__device__ __forceinline__ int64_t bsum(int64_t v) {
-  int64_t t;
-  bscan_excl<NT>(v, t);
-  return t;
-}
-
-// Weighted radix select (same contract as in lp.cu): first key in ascending
-// (hi, lo) order whose inclusive weight prefix exceeds rem.
-// Called only when the keys' total weight exceeds rem, so every pass selects
-// a byte some remaining key carries: bytes on which all keys agree are taken
-// without a histogram pass.
-template <class Item>
-__device__ void ip_select(int64_t cnt, int64_t rem, Item item, uint64_t &khi, uint32_t &klo) {
-  __shared__ int64_t hist[256];
-  __shared__ uint64_t fhi, mhi;
-  __shared__ uint32_t flo, mlo;
-  __shared__ int64_t cum;
-  __shared__ unsigned long long and_hi, or_hi;
-  __shared__ unsigned and_lo, or_lo;
-  if (threadIdx.x == 0) {
-    fhi = 0, mhi = 0, flo = 0, mlo = 0, cum = 0;
-    and_hi = ~0ull, or_hi = 0, and_lo = ~0u, or_lo = 0;
+__device__ int32_t block_scan_array(int32_t *x, int32_t len) {
+  int32_t carry = 0;
+  for (int32_t q0 = 0; q0 < len; q0 += 4 * NT) {
+    const int32_t q = q0 + 4 * (int32_t)threadIdx.x;
+    int32_t v[4], sum = 0;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = q + r < len ? x[q + r] : 0, sum += v[r];
+    int64_t tot;
+    int32_t ex = carry + (int32_t)bscan_excl<NT>(sum, tot);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (q + r < len) x[q + r] = ex;
+      ex += v[r];
+    }
+    carry += (int32_t)tot;
   }
+  if (threadIdx.x == 0) x[len] = carry;
   __syncthreads();
-  {
-    unsigned long long ah = ~0ull, oh = 0;
-    unsigned al = ~0u, ol = 0;
-    for (int64_t q = threadIdx.x; q < cnt; q += blockDim.x) {
-      uint64_t hi;
-      uint32_t lo;
-      int64_t w;
-      item(q, hi, lo, w);
-      ah &= hi, oh |= hi, al &= lo, ol |= lo;
-    }
-    atomicAnd(&and_hi, ah), atomicOr(&or_hi, oh), atomicAnd(&and_lo, al), atomicOr(&or_lo, ol);
-    __syncthreads();
-  }
-  for (int pass = 0; pass < 12; ++pass) {
-    const bool in_hi = pass < 8;
-    const int shift = in_hi ? 56 - 8 * pass : 24 - 8 * (pass - 8);
-    const unsigned same = in_hi ? (unsigned)(((and_hi ^ or_hi) >> shift) & 255u)
-                                : ((and_lo ^ or_lo) >> shift) & 255u;
-    if (same == 0) {
-      if (threadIdx.x == 0) {
-        if (in_hi) fhi |= ((uint64_t)and_hi >> shift & 255u) << shift, mhi |= 255ull << shift;
-        else flo |= ((and_lo >> shift) & 255u) << shift, mlo |= 255u << shift;
-      }
-      __syncthreads();
-      continue;
-    }
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
-    __syncthreads();
-    for (int64_t q = threadIdx.x; q < cnt; q += blockDim.x) {
-      uint64_t hi;
-      uint32_t lo;
-      int64_t w;
-      item(q, hi, lo, w);
-      if ((hi & mhi) != fhi || (lo & mlo) != flo) continue;
-      uint32_t d = in_hi ? (uint32_t)(hi >> shift) & 255u : (lo >> shift) & 255u;
-      atomicAdd((unsigned long long *)&hist[d], (unsigned long long)w);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int64_t run = cum;
-      int b = 0;
-      for (; b < 255; ++b) {
-        if (run + hist[b] > rem) break;
-        run += hist[b];
-      }
-      cum = run;
-      if (in_hi) fhi |= (uint64_t)b << shift, mhi |= 255ull << shift;
-      else flo |= (uint32_t)b << shift, mlo |= 255u << shift;
-    }
-    __syncthreads();
-  }
-  khi = fhi;
-  klo = flo;
-  __syncthreads();
+  return carry;
 }
 
-// Adjacency of a node's vertex (vlist position p) in the node's induced
-// subgraph is scanned by a whole warp, lanes striding over the neighbours
-// (coalesced, and a hub does not serialise one thread); f(in, y, w) is called
-// by every lane for every 32 neighbours, y a position inside the node.
-template <class F>
-__device__ __forceinline__ void node_nbrs(const IPCtx &c, int64_t p, F &&f) {
-  const int64_t b = c.lxadj[p], e = c.lxadj[p + 1];
-  for (int64_t i0 = b; i0 < e; i0 += 32) {
-    const int64_t i = i0 + lane_id();
-    const bool in = i < e;
-    f(in, in ? c.ladj[i] : 0, in ? (c.lew ? c.lew[i] : (int64_t)1) : (int64_t)0);
-  }
-}
-
-// Induced subgraphs of all nodes of a depth: neighbour counts, then (after a
+// Neighbour counts of every listed vertex inside its node, then (after a
 // scan into lxadj) the neighbours' positions, one warp per listed vertex.
 __global__ void k_local_deg(const int64_t *xadj, const int32_t *adj, const int32_t *node_of,
                             const int32_t *vlist, int64_t m, int64_t *ldeg) {
@@ -211,255 +166,422 @@ __global__ void k_local_fill(const int64_t *xadj, const int32_t *adj, const int6
   }
 }
 
-// Exclusive scan of x[0..len) in place, block-wide; returns the total.
-template <int NT>
-__device__ int64_t block_scan_array(int32_t *x, int64_t len) {
-  int64_t carry = 0;
-  for (int64_t q0 = 0; q0 < len; q0 += blockDim.x) {
-    const int64_t q = q0 + threadIdx.x;
-    const int64_t v = q < len ? x[q] : 0;
-    int64_t tot;
-    const int64_t ex = bscan_excl<NT>(v, tot);
-    if (q < len) x[q] = (int32_t)(carry + ex);
-    carry += tot;
+// Largest weighted degree (whether connectivity differences fit 32 bits).
+__global__ void k_max_wdeg(const int64_t *xadj, const int64_t *ew, int64_t n,
+                           unsigned long long *out) {
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int64_t best = 0;
+  for (int64_t u = gw; u < n; u += nw) {
+    int64_t w = 0;
+    for (int64_t i = xadj[u] + lane_id(); i < xadj[u + 1]; i += 32) w += ew[i];
+    w = warp_sum(w);
+    best = w > best ? w : best;
   }
-  __syncthreads();
-  return carry;
+  if (lane_id() == 0) atomicMax(out, (unsigned long long)best);
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT, kIPThreads / NT) k_bisect(IPCtx c) {
-  const int32_t j = blockIdx.x / c.T, a = blockIdx.x % c.T;
-  const int64_t nb = c.nstart[j], ns = c.nstart[j + 1] - nb;
-  const int64_t R = (int64_t)a * c.n + nb;  // scratch region of this attempt
-  int32_t *ord = c.ord + R, *disc = c.disc + R, *claimer = c.claimer + R, *cnt = c.cnt + R;
-  int32_t *side = c.side + R, *mvx0 = c.mvx0 + R, *mvx1 = c.mvx1 + R, *ok0 = c.ok0 + R,
-          *ok1 = c.ok1 + R;
-  int64_t *mvg0 = c.mvg0 + R, *mvg1 = c.mvg1 + R;
-  uint8_t *sub = c.sub + R;
-  const int32_t *vs = c.vlist + nb;
+// Shared-memory state of the one-CTA form for nodes of up to cap vertices:
+// claimer / D (sizeof(V)), ord, cnt (cap + 1), list, side, sub.
+template <class V>
+__host__ __device__ constexpr size_t ip_smem_bytes(int64_t cap) {
+  return (size_t)cap * (sizeof(V) + 12 + 2) + 16;
+}
+
+__device__ __forceinline__ void dif_add(int32_t *p, int64_t w) { atomicAdd(p, (int32_t)w); }
+__device__ __forceinline__ void dif_add(int64_t *p, int64_t w) {
+  atomicAdd((unsigned long long *)p, (unsigned long long)w);
+}
+
+// One attempt of one node. SM: one CTA, state in shared memory; otherwise a
+// cluster of any size, state in global memory (L1 lines are dropped by the
+// barriers' acquire). V: type of the connectivity differences (int32_t where
+// twice every weighted degree fits). Adjacencies are scanned by groups of gs
+// lanes, gs picked from the node's average degree, so that a mesh's six
+// neighbours do not occupy a warp each.
+// Bound by latency: a mesh's BFS has about a hundred levels of four dependent
+// steps with a barrier each, a dense node is read from HBM about four times
+// (BFS claims and emission, D, the movers' rows).
+template <int NT, bool SM, class V>
+__global__ void __launch_bounds__(NT, SM && NT <= 512 ? 1024 / NT : 1) k_bisect(IPCtx c) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ IPCtl s_ctl;
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = SM ? 1 : (int)cl.num_blocks(), rank = SM ? 0 : (int)cl.block_rank();
+  IPCtl *ctl = SM ? &s_ctl : cl.map_shared_rank(&s_ctl, 0);
+  auto sync_all = [&] {
+    if (SM || cs == 1) __syncthreads();
+    else cl.sync();
+  };
+  const int32_t at = (int32_t)(blockIdx.x / (unsigned)cs);
+  const int32_t j = c.nodes[at / c.T], a = at % c.T;
+  const int64_t nb = c.nstart[j];
+  const int32_t ns = (int32_t)(c.nstart[j + 1] - nb);
   const int32_t kk = c.nkk[j], k0 = (kk + 1) / 2, k1 = kk / 2;
-  const uint64_t key = ((uint64_t)(uint32_t)c.nkey[j] << 32) | (uint32_t)kk;
-  const int lane = lane_id(), warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  auto cw = [&](int64_t x) -> int64_t { return c.vw ? c.vw[vs[x]] : 1; };
-  if (ns == 0) {
-    if (threadIdx.x == 0) c.cut[blockIdx.x] = 0;
+  if (ns == 0) {  // the whole cluster leaves
+    if (rank == 0 && threadIdx.x == 0) c.cut[(int64_t)j * c.T + a] = 0;
     return;
   }
+  const int64_t R = (int64_t)a * c.n + nb;  // scratch region of this attempt
+  int32_t *claimer, *ord, *cnt, *list;
+  uint8_t *sub, *side;
+  V *dif;
+  if constexpr (SM) {
+    dif = reinterpret_cast<V *>(smem);  // claims are done with when D begins
+    claimer = reinterpret_cast<int32_t *>(smem);
+    ord = reinterpret_cast<int32_t *>(smem + sizeof(V) * c.cap);
+    cnt = ord + c.cap;
+    list = cnt + c.cap + 1;
+    sub = reinterpret_cast<uint8_t *>(list + c.cap + 1);
+    side = sub + c.cap;
+  } else {
+    claimer = c.claimer + R;
+    ord = c.ord + R;
+    cnt = c.cnt + (int64_t)a * (c.n + c.n_nodes) + nb + j;
+    list = c.list + R;
+    dif = static_cast<V *>(c.dif) + R;
+    sub = c.sub + R;
+    side = c.side + R;
+  }
+  const int64_t *lx = c.lxadj + nb;
+  const int32_t *vs = c.vlist + nb;
+  const uint64_t key = ((uint64_t)(uint32_t)c.nkey[j] << 32) | (uint32_t)kk;
+  const int lane = lane_id();
+  const int32_t tid = rank * NT + (int32_t)threadIdx.x, nthr = cs * NT;
+  auto cw = [&](int32_t x) -> int64_t { return c.vw ? c.vw[vs[x]] : 1; };
+  // lanes per adjacency
+  const int64_t avg = (lx[ns] - lx[0]) / ns;
+  const int gs = avg > 24 ? 32 : avg > 12 ? 16 : avg > 5 ? 8 : 4;
+  const int gl = lane & (gs - 1);
+  const unsigned gmask = gs == 32 ? kFull : ((1u << gs) - 1u) << (lane & ~(gs - 1));
+  const int32_t gid = tid / gs, ngr = nthr / gs;
+
+  if (threadIdx.x == 0 && rank == 0) s_ctl = IPCtl{};
+  for (int32_t x = tid; x < ns; x += nthr) claimer[x] = INT32_MAX;
+  sync_all();
   // ---------------- BFS order
-  for (int64_t x = threadIdx.x; x < ns; x += blockDim.x) disc[x] = 0, claimer[x] = INT32_MAX;
-  __syncthreads();
-  __shared__ int64_t sh_fb, sh_fe, sh_tail;
-  if (threadIdx.x == 0) {
-    int64_t s0 = (int64_t)(round_key(c.seed, kTagIPSeed, key, (uint64_t)a) % (uint64_t)ns);
-    ord[0] = (int32_t)s0;
-    disc[s0] = 1;
-    sh_fb = 0, sh_fe = 1, sh_tail = 1;
+  const int32_t seed_v =
+      (int32_t)(round_key(c.seed, kTagIPSeed, key, (uint64_t)a) % (uint64_t)ns);
+  {
+    // vertices with neighbours (no BFS finds more) and the node's weight
+    int32_t nz = 0;
+    int64_t w = 0;
+    for (int32_t x = tid; x < ns; x += nthr) nz += lx[x + 1] > lx[x], w += cw(x);
+    nz = warp_sum(nz);
+    w = warp_sum(w);
+    if (lane == 0) {
+      if (nz) atomicAdd(&ctl->nz, nz);
+      atomicAdd(&ctl->W, (unsigned long long)w);
+    }
+    if (tid == 0) ord[0] = seed_v, claimer[seed_v] = -1;
   }
-  __syncthreads();
-  for (;;) {
-    const int64_t fb = sh_fb, fe = sh_fe, tail = sh_tail;
-    if (fb >= fe) break;
+  sync_all();
+  const int32_t nz = ctl->nz;
+  const int64_t W = (int64_t)ctl->W;
+  int32_t tail = 1;
+  for (int32_t fb = 0, fe = 1; fb < fe && tail < nz;) {
     // every undiscovered neighbour is claimed by its earliest frontier vertex
-    for (int64_t i = fb + warp; i < fe; i += nwarps)
-      node_nbrs(c, nb + ord[i], [&](bool in, int32_t y, int64_t) {
-        if (in && !disc[y]) atomicMin(&claimer[y], (int32_t)i);
-      });
-    __syncthreads();
-    for (int64_t i = fb + warp; i < fe; i += nwarps) {
-      int32_t k = 0;
-      node_nbrs(c, nb + ord[i], [&](bool in, int32_t y, int64_t) {
-        k += __popc(__ballot_sync(kFull, in && !disc[y] && claimer[y] == i));
-      });
-      if (lane == 0) cnt[i - fb] = k;
+    // (claimer: INT32_MAX unclaimed, -1 already in the order); the first
+    // claim of a vertex lists it
+    for (int32_t i = fb + gid; i < fe; i += ngr) {
+      const int32_t p = ord[i];
+      if (gl == 0) cnt[i - fb] = 0;
+      const int64_t e = lx[p + 1];
+      for (int64_t q0 = lx[p]; q0 < e; q0 += 4 * gs) {
+        int32_t y[4], cur[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) y[r] = q0 + r * gs + gl < e ? c.ladj[q0 + r * gs + gl] : -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) cur[r] = y[r] >= 0 ? claimer[y[r]] : -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          bool first = false;
+          if (cur[r] > i) first = atomicMin(&claimer[y[r]], i) == INT32_MAX;
+          const unsigned m = __ballot_sync(gmask, first);
+          if (m == 0) continue;
+          int32_t base = 0;
+          const int leader = __ffs(m) - 1;
+          if (lane == leader) base = atomicAdd(&ctl->nnew, __popc(m));
+          base = __shfl_sync(gmask, base, leader);
+          if (first) list[base + __popc(m & lanemask_lt())] = y[r];
+        }
+      }
     }
-    __syncthreads();
-    const int64_t carry = block_scan_array<NT>(cnt, fe - fb);
+    sync_all();
+    const int32_t nn = ctl->nnew;
+    if (nn == 0) break;
+    for (int32_t q = tid; q < nn; q += nthr) atomicAdd(&cnt[claimer[list[q]] - fb], 1);
+    sync_all();
+    if (rank == 0) {
+      block_scan_array<NT>(cnt, fe - fb);
+      if (threadIdx.x == 0) ctl->nnew = 0;
+    }
+    if (cs > 1) sync_all();
     // claimed neighbours in frontier order, then adjacency order
-    for (int64_t i = fb + warp; i < fe; i += nwarps) {
-      int64_t pos = tail + cnt[i - fb];
-      node_nbrs(c, nb + ord[i], [&](bool in, int32_t y, int64_t) {
-        const bool mine = in && !disc[y] && claimer[y] == i;
-        const unsigned m = __ballot_sync(kFull, mine);
-        if (mine) ord[pos + __popc(m & lanemask_lt())] = y;
-        pos += __popc(m);
-      });
+    for (int32_t i = fb + gid; i < fe; i += ngr) {
+      const int32_t c0 = cnt[i - fb], k = cnt[i - fb + 1] - c0;
+      if (k == 0) continue;
+      const int32_t p = ord[i];
+      const int64_t e = lx[p + 1];
+      int32_t done = 0;
+      for (int64_t q0 = lx[p]; done < k && q0 < e; q0 += gs) {
+        const int32_t y = q0 + gl < e ? c.ladj[q0 + gl] : -1;
+        const bool mine = y >= 0 && claimer[y] == i;
+        const unsigned m = __ballot_sync(gmask, mine);
+        if (mine) {
+          ord[tail + c0 + done + __popc(m & lanemask_lt())] = y;
+          claimer[y] = -1;
+        }
+        done += __popc(m);
+      }
     }
-    __syncthreads();
-    for (int64_t q = tail + threadIdx.x; q < tail + carry; q += blockDim.x) disc[ord[q]] = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) sh_fb = tail, sh_fe = tail + carry, sh_tail = tail + carry;
-    __syncthreads();
+    sync_all();
+    fb = fe;
+    fe = tail = tail + nn;
   }
-  {  // append unreached vertices in ascending id
-    int64_t carry = 0, tail = sh_tail;
-    for (int64_t x0 = 0; x0 < ns; x0 += blockDim.x) {
-      int64_t x = x0 + threadIdx.x;
-      int64_t f = x < ns && !disc[x];
-      int64_t tot;
-      int64_t ex = bscan_excl<NT>(f, tot);
-      if (f) ord[tail + carry + ex] = (int32_t)x;
-      carry += tot;
-    }
-    __syncthreads();
-  }
-  // ---------------- greedy growing: longest prefix within target0
-  __shared__ int64_t lw[2], inw[2], ncnt[2];
-  __shared__ int64_t sh_nact;
-  int64_t W = 0;
-  for (int64_t x = threadIdx.x; x < ns; x += blockDim.x) W += cw(x);
-  W = bsum<NT>(W);
+  // ---------------- the rest of the order, and greedy growing: the longest
+  // prefix within target0 (first CTA)
   const int64_t target0 = (int64_t)(((__int128)W * k0) / kk);
   const int64_t caps[2] = {(int64_t)k0 * c.nlmax[j], (int64_t)k1 * c.nlmax[j]};
-  {
+  if (rank == 0) {
+    int32_t end = tail;  // append unreached vertices in ascending id
+    if (tail < ns) {
+      for (int32_t x0 = 0; x0 < ns; x0 += NT) {
+        const int32_t x = x0 + (int32_t)threadIdx.x;
+        const int64_t f = x < ns && claimer[x] != -1;
+        int64_t tot;
+        const int64_t ex = bscan_excl<NT>(f, tot);
+        if (f) ord[end + ex] = x;
+        end += (int32_t)tot;
+      }
+      __syncthreads();
+    }
     int64_t carry = 0, w0 = 0;
-    for (int64_t q0 = 0; q0 < ns; q0 += blockDim.x) {
-      int64_t q = q0 + threadIdx.x;
-      int64_t w = q < ns ? cw(ord[q]) : 0;
-      int64_t tot;
-      int64_t incl = carry + bscan_excl<NT>(w, tot) + w;
-      if (q < ns) {
-        bool in0 = incl <= target0;
-        side[ord[q]] = in0 ? 0 : 1;
-        if (in0) w0 += w;
+    for (int32_t q0 = 0; q0 < ns; q0 += 4 * NT) {
+      const int32_t q = q0 + 4 * (int32_t)threadIdx.x;
+      int32_t x[4];
+      int64_t w[4], sum = 0, tot;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) x[r] = q + r < ns ? ord[q + r] : -1;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) w[r] = x[r] >= 0 ? cw(x[r]) : 0, sum += w[r];
+      int64_t incl = carry + bscan_excl<NT>(sum, tot);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        incl += w[r];
+        if (x[r] < 0) continue;
+        const bool in0 = incl <= target0;
+        side[x[r]] = in0 ? 0 : 1;
+        if (in0) w0 += w[r];
       }
       carry += tot;
     }
-    w0 = bsum<NT>(w0);
-    if (threadIdx.x == 0) lw[0] = w0, lw[1] = W - w0;
-    __syncthreads();
+    w0 = warp_sum(w0);
+    if (lane == 0) atomicAdd(&ctl->w0, (unsigned long long)w0);
   }
+  sync_all();
+  // ---------------- connectivity differences
+  {
+    int64_t wsum = 0;
+    for (int32_t x = gid; x < ns; x += ngr) {
+      int64_t d = 0;
+      const int64_t b = lx[x], e = lx[x + 1];
+#pragma unroll 4
+      for (int64_t q = b + gl; q < e; q += gs) {
+        const int64_t w = c.lew ? c.lew[q] : 1;
+        wsum += w;
+        d += side[c.ladj[q]] ? w : -w;
+      }
+      for (int o = gs >> 1; o > 0; o >>= 1) d += __shfl_xor_sync(gmask, d, o);
+      if (gl == 0) dif[x] = (V)d;
+    }
+    __syncwarp();
+    wsum = warp_sum(wsum);
+    if (lane == 0 && wsum) atomicAdd(&ctl->wdeg, (unsigned long long)wsum);
+  }
+  sync_all();
   // ---------------- 2-way label propagation
+  int64_t lw1 = W - (int64_t)ctl->w0, lw0 = (int64_t)ctl->w0;
+  const int32_t nq = (ns + 3) / 4;
+  int32_t step = 0;  // sub-rounds so far (selects the rotating counters)
   for (int32_t r = 0; r < c.rounds; ++r) {
     const uint64_t rk = round_key(c.seed, kTagIPLP, key, ((uint64_t)a << 8) + (uint64_t)r);
-    for (int64_t x = threadIdx.x; x < ns; x += blockDim.x)
-      sub[x] = (uint8_t)sub_round_of(hstep(rk, (uint64_t)x), c.S);
-    __syncthreads();
-    for (int32_t s = 0; s < c.S; ++s) {
-      // this sub-round's vertices, listed in cnt (ascending)
-      {
-        int64_t carry = 0;
-        for (int64_t x0 = 0; x0 < ns; x0 += blockDim.x) {
-          const int64_t x = x0 + threadIdx.x;
-          const int64_t f = x < ns && sub[x] == s;
-          int64_t tot;
-          const int64_t ex = bscan_excl<NT>(f, tot);
-          if (f) cnt[carry + ex] = (int32_t)x;
-          carry += tot;
-        }
-        if (threadIdx.x == 0) sh_nact = carry, inw[0] = inw[1] = 0, ncnt[0] = ncnt[1] = 0;
-        __syncthreads();
+    for (int32_t t = tid; t < nq; t += nthr)  // each thread reads only its own entries below
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (4 * t + i < ns)
+          sub[4 * t + i] = (uint8_t)sub_round_of(hstep(rk, (uint64_t)(4 * t + i)), c.S);
+    bool moved = false;
+    for (int32_t s = 0; s < c.S && s < 256; ++s, ++step) {
+      const int cur = step % 3, nxt = (step + 1) % 3;
+      if (tid == 0) {
+        ctl->inw[nxt][0] = ctl->inw[nxt][1] = ctl->dlw[nxt] = 0;
+        ctl->ncnt[nxt][0] = ctl->ncnt[nxt][1] = 0;
       }
-      const int64_t nact = sh_nact;
-      for (int64_t q = warp; q < nact; q += nwarps) {
-        const int32_t x = cnt[q];
-        int64_t r0 = 0, r1 = 0;
-        node_nbrs(c, nb + x, [&](bool in, int32_t y, int64_t w) {
-          if (in) (side[y] ? r1 : r0) += w;
-        });
-        r0 = warp_sum(r0);
-        r1 = warp_sum(r1);
-        if (lane != 0) continue;
-        const int32_t own = side[x], oth = 1 - own;
-        const int64_t Rown = own ? r1 : r0, Roth = own ? r0 : r1;
-        const int64_t w = cw(x);
-        if (Roth > Rown && lw[oth] + w <= caps[oth]) {
-          const int64_t g = Roth - Rown;
-          unsigned long long p = atomicAdd((unsigned long long *)&ncnt[oth], 1ull);
-          atomicAdd((unsigned long long *)&inw[oth], (unsigned long long)w);
-          if (oth == 0) mvx0[p] = x, mvg0[p] = g, ok0[p] = 0;
-          else mvx1[p] = x, mvg1[p] = g, ok1[p] = 0;
-        }
-      }
-      __syncthreads();
-      for (int t = 0; t < 2; ++t) {
-        int32_t *mx = t == 0 ? mvx0 : mvx1, *ok = t == 0 ? ok0 : ok1;
-        int64_t *mg = t == 0 ? mvg0 : mvg1;
-        int64_t m = ncnt[t];
-        if (lw[t] + inw[t] <= caps[t]) {
-          for (int64_t q = threadIdx.x; q < m; q += blockDim.x) ok[q] = 1;
-        } else if (caps[t] - lw[t] >= 0) {
-          auto item = [&](int64_t q, uint64_t &hi, uint32_t &lo, int64_t &w) {
-            hi = ~(uint64_t)mg[q];
-            lo = (uint32_t)mx[q];
-            w = cw(mx[q]);
-          };
-          uint64_t khi;
-          uint32_t klo;
-          ip_select(m, caps[t] - lw[t], item, khi, klo);
-          for (int64_t q = threadIdx.x; q < m; q += blockDim.x) {
-            uint64_t hi = ~(uint64_t)mg[q];
-            uint32_t lo = (uint32_t)mx[q];
-            ok[q] = hi < khi || (hi == khi && lo < klo);
+      // movers into side 0 are listed from the front, into side 1 from the back
+      for (int32_t t0 = tid - lane; t0 < nq; t0 += nthr) {
+        const int32_t t = t0 + lane;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int32_t x = 4 * t + i;
+          int to = -1;
+          int64_t w = 0;
+          if (t < nq && x < ns && sub[x] == s) {
+            const int own = side[x];
+            const int64_t d = own ? -(int64_t)dif[x] : (int64_t)dif[x];
+            if (d > 0) {
+              w = cw(x);
+              if ((own ? lw0 : lw1) + w <= caps[1 - own]) to = 1 - own;
+            }
+          }
+          const unsigned m0 = __ballot_sync(kFull, to == 0), m1 = __ballot_sync(kFull, to == 1);
+          if (!(m0 | m1)) continue;
+          const unsigned mine = to == 0 ? m0 : m1;
+          int32_t base = 0;
+          if (to >= 0) {
+            atomicAdd(&ctl->inw[cur][to], (unsigned long long)w);
+            if (lane == __ffs(mine) - 1) base = atomicAdd(&ctl->ncnt[cur][to], __popc(mine));
+          }
+          const int32_t b0 = m0 ? __shfl_sync(kFull, base, __ffs(m0) - 1) : 0;
+          const int32_t b1 = m1 ? __shfl_sync(kFull, base, __ffs(m1) - 1) : 0;
+          if (to >= 0) {
+            const int32_t pos = (to ? b1 : b0) + __popc(mine & lanemask_lt());
+            list[to ? ns - 1 - pos : pos] = x;
           }
         }
-        __syncthreads();
       }
-      for (int t = 0; t < 2; ++t) {
-        int32_t *mx = t == 0 ? mvx0 : mvx1, *ok = t == 0 ? ok0 : ok1;
-        for (int64_t q = threadIdx.x; q < ncnt[t]; q += blockDim.x) {
-          if (!ok[q]) continue;
-          int64_t w = cw(mx[q]);
-          side[mx[q]] = t;
-          atomicAdd((unsigned long long *)&lw[t], (unsigned long long)w);
-          atomicAdd((unsigned long long *)&lw[1 - t], (unsigned long long)(-w));
+      sync_all();
+      const int32_t m0 = ctl->ncnt[cur][0], m1 = ctl->ncnt[cur][1];
+      if (m0 + m1 == 0) continue;
+      moved = true;
+      // a side whose movers do not all fit takes the longest fitting prefix in
+      // (gain desc, vertex asc) order
+      const bool sel0 = m0 && lw0 + (int64_t)ctl->inw[cur][0] > caps[0];
+      const bool sel1 = m1 && lw1 + (int64_t)ctl->inw[cur][1] > caps[1];
+      uint64_t khi[2] = {~0ull, ~0ull};
+      uint32_t klo[2] = {~0u, ~0u};
+      if (sel0 || sel1) {
+        for (int t = 0; t < 2; ++t) {
+          if (!(t ? sel1 : sel0) || rank != (t && cs > 1 ? 1 : 0)) continue;
+          auto item = [&](int64_t q, uint64_t &hi, uint32_t &lo, int64_t &w) {
+            const int32_t x = list[t ? ns - 1 - q : q];
+            const int64_t d = (int64_t)dif[x];
+            hi = ~(uint64_t)(t ? d : -d);
+            lo = (uint32_t)x;
+            w = cw(x);
+          };
+          uint64_t h;
+          uint32_t l;
+          block_select(t ? m1 : m0, caps[t] - (t ? lw1 : lw0), item, h, l);
+          if (threadIdx.x == 0) ctl->khi[t] = h, ctl->klo[t] = l;
+        }
+        sync_all();
+        if (sel0) khi[0] = ctl->khi[0], klo[0] = ctl->klo[0];
+        if (sel1) khi[1] = ctl->khi[1], klo[1] = ctl->klo[1];
+      }
+      // approved moves, and their neighbours' differences. A mover's own
+      // difference may change under its neighbours' moves meanwhile, so with
+      // a threshold the decisions are taken before any update.
+      if (sel0 || sel1) {
+        for (int32_t q = tid; q < m0 + m1; q += nthr) {
+          const int t = q >= m0;
+          const int32_t lq = t ? ns - 1 - (q - m0) : q;
+          const int32_t x = list[lq];
+          const int64_t d = (int64_t)dif[x];
+          const uint64_t hi = ~(uint64_t)(t ? d : -d);
+          if (hi > khi[t] || (hi == khi[t] && (uint32_t)x >= klo[t]))
+            if (t ? sel1 : sel0) list[lq] = ~x;  // refused
+        }
+        sync_all();
+      }
+      for (int32_t q = gid; q < m0 + m1; q += ngr) {
+        const int t = q >= m0;
+        const int32_t x = list[t ? ns - 1 - (q - m0) : q];
+        if (x < 0) continue;
+        if (gl == 0) {
+          side[x] = (uint8_t)t;
+          const int64_t w = cw(x);
+          atomicAdd(&ctl->dlw[cur], (unsigned long long)(t ? w : -w));
+        }
+        const int64_t b = lx[x], e = lx[x + 1];
+#pragma unroll 4
+        for (int64_t i = b + gl; i < e; i += gs) {
+          const int64_t w = 2 * (c.lew ? c.lew[i] : (int64_t)1);
+          dif_add(&dif[c.ladj[i]], t ? w : -w);
         }
       }
-      __syncthreads();
+      sync_all();
+      const int64_t dl = (int64_t)ctl->dlw[cur];
+      lw1 += dl;
+      lw0 -= dl;
     }
+    // nothing moved in a whole round: every later round would find the same
+    if (!moved) break;
   }
-  // ---------------- cut of the induced subgraph
-  int64_t cutv = 0;
-  for (int64_t x = warp; x < ns; x += nwarps) {
-    const int32_t sx = side[x];
-    node_nbrs(c, nb + x, [&](bool in, int32_t y, int64_t w) {
-      if (in && side[y] != sx) cutv += w;
-    });
+  // ---------------- cut of the induced subgraph: a vertex's outside weight
+  // is (weighted degree +- D) / 2, the cut half of their sum
+  {
+    int64_t acc = 0;
+    for (int32_t x = tid; x < ns; x += nthr) {
+      const int64_t d = (int64_t)dif[x];
+      acc += side[x] ? -d : d;
+      if (SM) c.side[R + x] = side[x];
+    }
+    acc = warp_sum(acc);
+    if (lane == 0 && acc) atomicAdd(&ctl->acc, (unsigned long long)acc);
   }
-  cutv = bsum<NT>(cutv);
-  if (threadIdx.x == 0) c.cut[blockIdx.x] = cutv / 2;
+  sync_all();
+  if (tid == 0)
+    c.cut[(int64_t)j * c.T + a] = ((int64_t)ctl->wdeg + (int64_t)ctl->acc) / 4;
 }
 
-// Pick the winning attempt of every node and move its vertices on.
-__global__ void k_pick(IPCtx c, const int32_t *child0, const int32_t *child1, int32_t *next_node,
+// The winning attempt of every node (smallest cut, lowest attempt on ties);
+// blockIdx.y slices a node. flag[p] = 1 where position p lies on its side 0;
+// vertices of finished children get their block.
+__global__ void k_pick(IPCtx c, const int32_t *child0, const int32_t *child1, int32_t *flag,
                        int32_t *part) {
   const int32_t j = blockIdx.x;
-  __shared__ int32_t best;
-  if (threadIdx.x == 0) {
-    int32_t b = 0;
-    for (int32_t a = 1; a < c.T; ++a)
-      if (c.cut[j * c.T + a] < c.cut[j * c.T + b]) b = a;
-    best = b;
-  }
-  __syncthreads();
   const int64_t nb = c.nstart[j], ns = c.nstart[j + 1] - nb;
-  const int32_t kk = c.nkk[j], k0 = (kk + 1) / 2;
-  for (int64_t x = threadIdx.x; x < ns; x += blockDim.x) {
-    int32_t u = c.vlist[nb + x];
-    int32_t sd = c.side[(int64_t)best * c.n + nb + x];
-    int32_t ch = sd == 0 ? child0[j] : child1[j];
-    next_node[u] = ch;
-    if (ch < 0) part[u] = sd == 0 ? c.noff[j] : c.noff[j] + k0;
+  const int64_t x0 = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
+  if (x0 - threadIdx.x >= ns) return;
+  int32_t best = 0;
+  for (int32_t a = 1; a < c.T; ++a)
+    if (c.cut[(int64_t)j * c.T + a] < c.cut[(int64_t)j * c.T + best]) best = a;
+  const int32_t k0 = (c.nkk[j] + 1) / 2;
+  const int32_t c0 = child0[j], c1 = child1[j];
+  for (int64_t x = x0; x < ns; x += (int64_t)gridDim.y * blockDim.x) {
+    const int sd = c.side[(int64_t)best * c.n + nb + x];
+    flag[nb + x] = sd == 0;
+    if ((sd ? c1 : c0) < 0) part[c.vlist[nb + x]] = sd == 0 ? c.noff[j] : c.noff[j] + k0;
   }
 }
 
-__global__ void k_node_keys(const int32_t *node_of, int64_t n, uint64_t *keys, int64_t *count) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    int32_t nd = node_of[u];
-    keys[u] = nd < 0 ? ~0ull : ((uint64_t)nd << 32) | (uint64_t)u;
-    if (nd >= 0) atomicAdd((unsigned long long *)&count[nd], 1ull);
-  }
+// Side-0 vertices of every node: prefix of the flags at the node starts.
+__global__ void k_side_prefix(const int64_t *pre, const int64_t *nstart, int32_t nodes,
+                              int64_t *out) {
+  for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= nodes; j += gridDim.x * blockDim.x)
+    out[j] = pre[nstart[j]];
 }
 
-__global__ void k_node_lists(const uint64_t *keys, const int64_t *nstart, int64_t m, int32_t *vlist,
-                             int32_t *loc) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t k = keys[i];
-    int32_t u = (int32_t)(k & 0xffffffffu), nd = (int32_t)(k >> 32);
-    vlist[i] = u;
-    loc[u] = (int32_t)(i - nstart[nd]);
+// The next depth's vertex list: every node's list split stably into its
+// children's (a stable partition replaces a sort by (node, id): the list is
+// in that order already).
+__global__ void k_split(const int64_t *nstart, const int32_t *child0, const int32_t *child1,
+                        const int64_t *next_start, const int64_t *pre, const int32_t *flag,
+                        const int32_t *vlist, int64_t m, int32_t *node_of, int32_t *loc,
+                        int32_t *next_vlist) {
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < m;
+       p += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = vlist[p], j = node_of[u];
+    const int64_t r0 = pre[p] - pre[nstart[j]];
+    const bool s0 = flag[p] != 0;
+    const int32_t ch = s0 ? child0[j] : child1[j];
+    if (ch >= 0) {
+      const int64_t r = s0 ? r0 : p - nstart[j] - r0;
+      next_vlist[next_start[ch] + r] = u;
+      loc[u] = (int32_t)r;
+    }
+    node_of[u] = ch;
   }
 }
 
@@ -467,6 +589,288 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     p[i] = v;
+}
+
+// First depth: the vertices in order, each in its root (rs: the roots' starts).
+__global__ void k_first_lists(const int64_t *rs, int32_t roots, int64_t n, int32_t *vlist,
+                              int32_t *node_of, int32_t *loc) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    int32_t lo = 0, hi = roots - 1;
+    while (lo < hi) {
+      const int32_t mid = (lo + hi + 1) / 2;
+      if (rs[mid] <= u) lo = mid;
+      else hi = mid - 1;
+    }
+    vlist[u] = (int32_t)u;
+    node_of[u] = lo;
+    loc[u] = (int32_t)(u - rs[lo]);
+  }
+}
+
+// Node table of one depth on the host.
+struct Depth {
+  std::vector<int32_t> off, kk, key, c0, c1;
+  std::vector<int64_t> lmax, start, entries;  // entries: estimate of the adjacency entries
+  int32_t nodes() const { return (int32_t)off.size(); }
+  void add(int32_t o, int32_t k, int32_t h, int64_t l, int64_t ent) {
+    off.push_back(o), kk.push_back(k), key.push_back(h), lmax.push_back(l), entries.push_back(ent);
+  }
+};
+
+// Its device copy, one upload: start (nodes + 1) and lmax, then off, kk, key,
+// c0, c1 and the launch classes' node lists.
+struct DepthDev {
+  Buf<int64_t> buf;
+  const int64_t *start = nullptr, *lmax = nullptr;
+  const int32_t *off = nullptr, *kk = nullptr, *key = nullptr, *c0 = nullptr, *c1 = nullptr,
+                *order = nullptr;
+  void upload(const Depth &d, const std::vector<int32_t> &ord, std::vector<int64_t> &host,
+              cudaStream_t s) {
+    const size_t N = (size_t)d.nodes();
+    host.assign(2 * N + 1 + (6 * N + 1) / 2, 0);
+    std::copy(d.start.begin(), d.start.end(), host.begin());
+    std::copy(d.lmax.begin(), d.lmax.end(), host.begin() + N + 1);
+    int32_t *h = reinterpret_cast<int32_t *>(host.data() + 2 * N + 1);
+    std::copy(d.off.begin(), d.off.end(), h);
+    std::copy(d.kk.begin(), d.kk.end(), h + N);
+    std::copy(d.key.begin(), d.key.end(), h + 2 * N);
+    std::copy(d.c0.begin(), d.c0.end(), h + 3 * N);
+    std::copy(d.c1.begin(), d.c1.end(), h + 4 * N);
+    std::copy(ord.begin(), ord.end(), h + 5 * N);
+    buf.alloc(host.size(), s);
+    TP_CUDA(cudaMemcpyAsync(buf.get(), host.data(), host.size() * 8, cudaMemcpyHostToDevice, s));
+    start = buf.get();
+    lmax = start + N + 1;
+    off = reinterpret_cast<const int32_t *>(lmax + N);
+    kk = off + N, key = kk + N, c0 = key + N, c1 = c0 + N, order = c1 + N;
+  }
+};
+
+// How a node's attempts are run: one CTA of `threads` with its state in
+// shared memory (cluster = 0), or a cluster of CTAs.
+struct Shape {
+  int threads, cluster;
+  bool operator==(const Shape &o) const { return threads == o.threads && cluster == o.cluster; }
+};
+
+// Shared memory of the one-CTA form: what a block may have beside the static
+// part (select and scan buffers).
+constexpr size_t kIPSmem = 220 * 1024;
+// A node of more adjacency entries than this is scanned by a cluster while
+// SMs are idle: one SM reads about 0.1 TB/s, so a million 12-byte entries
+// take it over 100 us a pass.
+constexpr int64_t kIPClusterEntries = (int64_t)1 << 19;
+
+template <class V>
+int64_t ip_smem_cap() {
+  return (int64_t)((kIPSmem - 16) / (sizeof(V) + 14));
+}
+
+template <class V>
+Shape ip_shape(int64_t ns, int64_t entries, int64_t attempts) {
+  const bool fits = ns <= ip_smem_cap<V>();
+  int64_t cl = 1;
+  while (cl < 16 && 2 * cl * attempts <= num_sms()) cl <<= 1;
+  if (!fits || (entries > kIPClusterEntries && cl > 1)) return Shape{kIPMaxThreads, (int)cl};
+  // smaller CTAs, several per SM, where many attempts are in flight
+  const bool many = attempts >= 2LL * num_sms();
+  const int threads = many ? (ns <= 512 ? 128 : ns <= 2048 ? 256 : ns <= 6144 ? 512 : 1024)
+                           : (ns <= 256 ? 256 : ns <= 1024 ? 512 : 1024);
+  return Shape{threads, 0};
+}
+
+template <int NT, bool SM, class V>
+void launch_bisect(const IPCtx &c, int64_t attempts, int cluster, cudaStream_t s) {
+  const size_t smem = SM ? ip_smem_bytes<V>(c.cap) : 0;
+  auto kern = k_bisect<NT, SM, V>;
+  if (SM)
+    TP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIPSmem));
+  else
+    TP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg{};
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  // smaller clusters where the device cannot hold all attempts' at once
+  for (; !SM && cluster > 1; cluster >>= 1) {
+    attr[0].val.clusterDim.x = (unsigned)cluster;
+    cfg.gridDim = dim3((unsigned)(attempts * cluster));
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) == cudaSuccess && fit >= attempts) break;
+    (void)cudaGetLastError();
+  }
+  attr[0].val.clusterDim.x = (unsigned)(SM ? 1 : cluster);
+  cfg.gridDim = dim3((unsigned)(attempts * (SM ? 1 : cluster)));
+  TP_CUDA(cudaLaunchKernelEx(&cfg, kern, c));
+  count_launch();
+}
+
+template <class V>
+void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
+                   const std::vector<int64_t> &root_start, const tp_params &p, int32_t *d_part,
+                   cudaStream_t s) {
+  const int64_t n = g->n;
+  const int32_t T = std::max(1, p.ip_attempts);
+  const bool weighted = !g->unit_ew;
+  Depth d;
+  for (size_t r = 0; r < roots.size(); ++r) {
+    TP_REQUIRE(roots[r].k >= 2, TP_ERR_INVALID);
+    const int64_t nr = root_start[r + 1] - root_start[r];
+    d.add(roots[r].off, roots[r].k, roots[r].key, roots[r].l_max,
+          (int64_t)((double)g->m2 * (double)nr / (double)n));
+  }
+  d.start = root_start;
+  Buf<int32_t> node_of(n, s), vlist(n, s), next_vlist(n, s), loc(n, s), flag(n, s);
+  Buf<int64_t> pre(n + 1, s), lxadj;
+  Buf<int32_t> ladj;
+  Buf<int64_t> lew;
+  Buf<uint8_t> side(T * n, s);
+  Buf<int32_t> ord, claimer, cnt, list;  // cluster form only
+  Buf<V> dif;
+  Buf<uint8_t> sub;
+  DepthDev dev, next_dev;
+  std::vector<int64_t> host, next_host;
+  for (int depth = 0; d.nodes() > 0; ++depth) {
+    const int32_t nodes = d.nodes();
+    const int64_t m = d.start[nodes];
+    // children of every node at the next depth (-1: leaf, assign the block)
+    Depth nx;
+    d.c0.assign(nodes, -1), d.c1.assign(nodes, -1);
+    for (int32_t j = 0; j < nodes; ++j) {
+      const int32_t k0 = (d.kk[j] + 1) / 2, k1 = d.kk[j] / 2;
+      if (k0 >= 2) d.c0[j] = nx.nodes(), nx.add(d.off[j], k0, d.key[j], d.lmax[j], d.entries[j] / 2);
+      if (k1 >= 2)
+        d.c1[j] = nx.nodes(),
+        nx.add(d.off[j] + k0, k1, d.key[j] + k0, d.lmax[j], d.entries[j] / 2);
+    }
+    // launch classes: nodes of the same shape, the largest first
+    std::vector<int32_t> order(nodes);
+    std::vector<Shape> shape(nodes);
+    for (int32_t j = 0; j < nodes; ++j) {
+      order[j] = j;
+      shape[j] = ip_shape<V>(d.start[j + 1] - d.start[j], d.entries[j], (int64_t)nodes * T);
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+      if (shape[x].cluster != shape[y].cluster) return shape[x].cluster > shape[y].cluster;
+      return shape[x].threads > shape[y].threads;
+    });
+    DepthDev &cur = depth % 2 ? next_dev : dev;
+    cur.upload(d, order, depth % 2 ? next_host : host, s);
+    if (depth == 0) {
+      launch(k_first_lists, grid_for(n, 256), 256, 0, s, cur.start, nodes, n, vlist.get(),
+             node_of.get(), loc.get());
+      TP_LAUNCH_CHECK();
+    }
+    IPCtx c{};
+    // a single root's induced subgraph is the graph itself
+    const bool whole = depth == 0 && nodes == 1;
+    if (whole) {
+      c.lxadj = g->xadj.get();
+      c.ladj = g->adj.get();
+      c.lew = weighted ? g->ew.get() : nullptr;
+    } else if (m) {
+      if (!ladj.get()) {
+        lxadj.alloc(n + 1, s);
+        ladj.alloc(std::max<int64_t>(g->m2, 1), s);
+        if (weighted) lew.alloc(std::max<int64_t>(g->m2, 1), s);
+      }
+      const unsigned wg = grid_for(m * 32, 256);
+      launch(k_local_deg, wg, 256, 0, s, g->xadj.get(), g->adj.get(), node_of.get(), vlist.get(), m,
+             lxadj.get());
+      TP_LAUNCH_CHECK();
+      exclusive_scan_i64(lxadj.get(), lxadj.get(), m, s);
+      launch(k_local_fill, wg, 256, 0, s, g->xadj.get(), g->adj.get(),
+             weighted ? g->ew.get() : nullptr, node_of.get(), loc.get(), vlist.get(), m, lxadj.get(),
+             ladj.get(), weighted ? lew.get() : nullptr);
+      TP_LAUNCH_CHECK();
+      c.lxadj = lxadj.get();
+      c.ladj = ladj.get();
+      c.lew = weighted ? lew.get() : nullptr;
+    }
+    Buf<int64_t> cut((int64_t)nodes * T, s);
+    c.n = n;
+    c.n_nodes = nodes;
+    c.vw = g->unit_vw ? nullptr : g->vw.get();
+    c.vlist = vlist.get();
+    c.nstart = cur.start;
+    c.noff = cur.off;
+    c.nkk = cur.kk;
+    c.nkey = cur.key;
+    c.nlmax = cur.lmax;
+    c.T = T;
+    c.seed = p.seed;
+    c.rounds = p.refine_rounds;
+    c.S = p.sub_rounds;
+    c.side = side.get();
+    c.cut = cut.get();
+    if (shape[order[0]].cluster) {
+      const size_t counts = (size_t)T * (size_t)(n + nodes);
+      if (!ord.get()) {
+        ord.alloc(T * n, s), claimer.alloc(T * n, s), list.alloc(T * n, s);
+        dif.alloc(T * n, s), sub.alloc(T * n, s);
+      }
+      if (cnt.n < counts) cnt.alloc(counts, s);
+      c.ord = ord.get(), c.claimer = claimer.get(), c.cnt = cnt.get(), c.list = list.get();
+      c.dif = dif.get(), c.sub = sub.get();
+    }
+    for (int32_t b = 0; b < nodes;) {
+      const Shape sh = shape[order[b]];
+      int32_t e = b;
+      int64_t largest = 1;
+      for (; e < nodes && shape[order[e]] == sh; ++e)
+        largest = std::max(largest, d.start[order[e] + 1] - d.start[order[e]]);
+      c.nodes = cur.order + b;
+      c.cap = (int32_t)((largest + 15) & ~(int64_t)15);
+      const int64_t att = (int64_t)(e - b) * T;
+      if (sh.cluster) launch_bisect<kIPMaxThreads, false, V>(c, att, sh.cluster, s);
+      else if (sh.threads == 128) launch_bisect<128, true, V>(c, att, 1, s);
+      else if (sh.threads == 256) launch_bisect<256, true, V>(c, att, 1, s);
+      else if (sh.threads == 512) launch_bisect<512, true, V>(c, att, 1, s);
+      else launch_bisect<1024, true, V>(c, att, 1, s);
+      b = e;
+    }
+    int64_t widest = 1;
+    for (int32_t j = 0; j < nodes; ++j) widest = std::max(widest, d.start[j + 1] - d.start[j]);
+    const dim3 pg((unsigned)nodes, (unsigned)std::min<int64_t>((widest + 255) / 256, 256));
+    launch(k_pick, pg, 256, 0, s, c, cur.c0, cur.c1, flag.get(), d_part);
+    TP_LAUNCH_CHECK();
+    if (nx.nodes()) {
+      // the children's sizes, from the prefix of the side flags
+      exclusive_scan_i32_to_i64(flag.get(), pre.get(), m, s);
+      Buf<int64_t> sp(nodes + 1, s);
+      launch(k_side_prefix, grid_for(nodes + 1, 256), 256, 0, s, pre.get(), cur.start, nodes,
+             sp.get());
+      TP_LAUNCH_CHECK();
+      std::vector<int64_t> hp((size_t)nodes + 1);
+      TP_CUDA(cudaMemcpyAsync(hp.data(), sp.get(), (nodes + 1) * sizeof(int64_t),
+                              cudaMemcpyDeviceToHost, s));
+      TP_CUDA(cudaStreamSynchronize(s));
+      nx.start.assign(1, 0);
+      for (int32_t j = 0; j < nodes; ++j) {
+        const int64_t n0 = hp[j + 1] - hp[j], n1 = d.start[j + 1] - d.start[j] - n0;
+        if (d.c0[j] >= 0) nx.start.push_back(nx.start.back() + n0);
+        if (d.c1[j] >= 0) nx.start.push_back(nx.start.back() + n1);
+      }
+      Buf<int64_t> ns(nx.start.size(), s);
+      TP_CUDA(cudaMemcpyAsync(ns.get(), nx.start.data(), nx.start.size() * 8,
+                              cudaMemcpyHostToDevice, s));
+      if (m) {
+        launch(k_split, grid_for(m, 256), 256, 0, s, cur.start, cur.c0, cur.c1, ns.get(), pre.get(),
+               flag.get(), vlist.get(), m, node_of.get(), loc.get(), next_vlist.get());
+        TP_LAUNCH_CHECK();
+      }
+      TP_CUDA(cudaStreamSynchronize(s));  // nx.start moves on below
+      std::swap(vlist, next_vlist);
+    }
+    d = std::move(nx);
+  }
+  TP_CUDA(cudaStreamSynchronize(s));  // host tables outlive their copies
 }
 
 }  // namespace
@@ -481,147 +885,29 @@ void initial_partition(const tp_graph *g, int32_t k, int64_t l_max, const tp_par
     TP_LAUNCH_CHECK();
     return;
   }
-  initial_partition_roots(g, {IPRoot{0, 0, k, l_max}}, nullptr, p, d_part, s);
+  initial_partition_roots(g, {IPRoot{0, 0, k, l_max}}, {0, n}, p, d_part, s);
 }
 
 void initial_partition_roots(const tp_graph *g, const std::vector<IPRoot> &roots,
-                             const int32_t *d_node_of, const tp_params &p, int32_t *d_part,
-                             cudaStream_t s) {
+                             const std::vector<int64_t> &root_start, const tp_params &p,
+                             int32_t *d_part, cudaStream_t s) {
   TP_REQUIRE(!g->compressed, TP_ERR_INVALID);
   const int64_t n = g->n;
   if (n == 0 || roots.empty()) return;
-  launch(k_fill_i32, grid_for(n, 256), 256, 0, s, d_part, n, 0);
-  TP_LAUNCH_CHECK();
-  const int32_t T = std::max(1, p.ip_attempts);
-  Buf<int32_t> node_of(n, s), next_node(n, s), vlist(n, s), loc(n, s);
-  if (d_node_of)
-    TP_CUDA(cudaMemcpyAsync(node_of.get(), d_node_of, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-  else
-    launch(k_fill_i32, grid_for(n, 256), 256, 0, s, node_of.get(), n, 0);
-  Buf<int32_t> ord(T * n, s), disc(T * n, s), claimer(T * n, s), cnt(T * n, s), side(T * n, s),
-      mvx0(T * n, s), mvx1(T * n, s), ok0(T * n, s), ok1(T * n, s);
-  Buf<int64_t> mvg0(T * n, s), mvg1(T * n, s);
-  Buf<uint8_t> sub(T * n, s);
-  Buf<uint64_t> keys(n, s);
-  std::vector<int32_t> off, kks, hkey;
-  std::vector<int64_t> lmx;
-  for (const IPRoot &r : roots) {
-    TP_REQUIRE(r.k >= 2, TP_ERR_INVALID);
-    off.push_back(r.off), kks.push_back(r.k), hkey.push_back(r.key), lmx.push_back(r.l_max);
+  // connectivity differences in 32 bits where they and their steps (twice an
+  // edge weight) fit; a bound from sizes first, the largest weighted degree
+  // only where that does not settle it
+  constexpr int64_t kFit = (int64_t)1 << 29;
+  bool small = g->unit_ew ? n < kFit : (double)g->m2 * (double)g->max_ew < (double)kFit;
+  if (!small && !g->unit_ew) {
+    Buf<unsigned long long> mx(1, s);
+    TP_CUDA(cudaMemsetAsync(mx.get(), 0, sizeof(unsigned long long), s));
+    launch(k_max_wdeg, grid_for(n * 32, 256), 256, 0, s, g->xadj.get(), g->ew.get(), n, mx.get());
+    TP_LAUNCH_CHECK();
+    small = read_scalar(mx.get(), s) < (unsigned long long)kFit;
   }
-  while (!off.empty()) {
-    const int32_t nodes = (int32_t)off.size();
-    // vertex lists per node
-    Buf<int64_t> nstart(nodes + 1, s);
-    TP_CUDA(cudaMemsetAsync(nstart.get(), 0, (nodes + 1) * sizeof(int64_t), s));
-    launch(k_node_keys, grid_for(n, 256), 256, 0, s, node_of.get(), n, keys.get(), nstart.get());
-    TP_LAUNCH_CHECK();
-    radix_sort_pairs(keys.get(), nullptr, n, 64, s);
-    exclusive_scan_i64(nstart.get(), nstart.get(), nodes, s);
-    std::vector<int64_t> hstart((size_t)nodes + 1);
-    TP_CUDA(cudaMemcpyAsync(hstart.data(), nstart.get(), (nodes + 1) * sizeof(int64_t),
-                            cudaMemcpyDeviceToHost, s));
-    TP_CUDA(cudaStreamSynchronize(s));
-    const int64_t m = hstart[(size_t)nodes];
-    int64_t max_ns = 0;
-    for (int32_t jn = 0; jn < nodes; ++jn) max_ns = std::max(max_ns, hstart[jn + 1] - hstart[jn]);
-    if (m) {
-      launch(k_node_lists, grid_for(m, 256), 256, 0, s, keys.get(), nstart.get(), m, vlist.get(), loc.get());
-      TP_LAUNCH_CHECK();
-    }
-    // induced subgraph of every node in local positions
-    const bool weighted = !g->unit_ew;
-    Buf<int64_t> lxadj(m + 1, s);
-    Buf<int32_t> ladj;
-    Buf<int64_t> lew;
-    if (m) {
-      const unsigned wg = grid_for(m * 32, 256);
-      launch(k_local_deg, wg, 256, 0, s, g->xadj.get(), g->adj.get(), node_of.get(), vlist.get(), m,
-             lxadj.get());
-      TP_LAUNCH_CHECK();
-      exclusive_scan_i64(lxadj.get(), lxadj.get(), m, s);
-      const int64_t lm = read_scalar(lxadj.get() + m, s);
-      ladj.alloc(std::max<int64_t>(lm, 1), s);
-      if (weighted) lew.alloc(std::max<int64_t>(lm, 1), s);
-      launch(k_local_fill, wg, 256, 0, s, g->xadj.get(), g->adj.get(),
-             weighted ? g->ew.get() : nullptr, node_of.get(), loc.get(), vlist.get(), m, lxadj.get(),
-             ladj.get(), weighted ? lew.get() : nullptr);
-      TP_LAUNCH_CHECK();
-    }
-    // children of every node at the next depth (-1: leaf, assign the block)
-    std::vector<int32_t> c0(nodes), c1(nodes), noff, nkk, nkey;
-    std::vector<int64_t> nlmx;
-    for (int32_t jn = 0; jn < nodes; ++jn) {
-      int32_t k0 = (kks[jn] + 1) / 2, k1 = kks[jn] / 2;
-      c0[jn] = -1, c1[jn] = -1;
-      if (k0 >= 2) {
-        c0[jn] = (int32_t)noff.size();
-        noff.push_back(off[jn]), nkk.push_back(k0), nkey.push_back(hkey[jn]), nlmx.push_back(lmx[jn]);
-      }
-      if (k1 >= 2) {
-        c1[jn] = (int32_t)noff.size();
-        noff.push_back(off[jn] + k0), nkk.push_back(k1), nkey.push_back(hkey[jn] + k0);
-        nlmx.push_back(lmx[jn]);
-      }
-    }
-    // one upload of the node table: off, kk, key, child0, child1 (int32), l_max
-    std::vector<int32_t> tbl32((size_t)5 * nodes);
-    for (int32_t jn = 0; jn < nodes; ++jn) {
-      tbl32[jn] = off[jn], tbl32[nodes + jn] = kks[jn], tbl32[2 * nodes + jn] = hkey[jn];
-      tbl32[3 * nodes + jn] = c0[jn], tbl32[4 * nodes + jn] = c1[jn];
-    }
-    Buf<int32_t> d_tbl(5 * nodes, s);
-    Buf<int64_t> d_lmax(nodes, s);
-    TP_CUDA(cudaMemcpyAsync(d_tbl.get(), tbl32.data(), tbl32.size() * 4, cudaMemcpyHostToDevice, s));
-    TP_CUDA(cudaMemcpyAsync(d_lmax.get(), lmx.data(), nodes * 8, cudaMemcpyHostToDevice, s));
-    const int32_t *d_off = d_tbl.get(), *d_kk = d_tbl.get() + nodes, *d_key = d_tbl.get() + 2 * nodes;
-    const int32_t *d_c0 = d_tbl.get() + 3 * nodes, *d_c1 = d_tbl.get() + 4 * nodes;
-    Buf<int64_t> cut((int64_t)nodes * T, s);
-    IPCtx c;
-    c.n = n;
-    c.xadj = g->xadj.get();
-    c.adj = g->adj.get();
-    c.vw = g->unit_vw ? nullptr : g->vw.get();
-    c.ew = g->unit_ew ? nullptr : g->ew.get();
-    c.node_of = node_of.get();
-    c.vlist = vlist.get();
-    c.nstart = nstart.get();
-    c.loc = loc.get();
-    c.lxadj = lxadj.get();
-    c.ladj = ladj.get();
-    c.lew = weighted ? lew.get() : nullptr;
-    c.noff = d_off;
-    c.nkk = d_kk;
-    c.nkey = d_key;
-    c.nlmax = d_lmax.get();
-    c.T = T;
-    c.seed = p.seed;
-    c.rounds = p.refine_rounds;
-    c.S = p.sub_rounds;
-    c.ord = ord.get(), c.disc = disc.get(), c.claimer = claimer.get(), c.cnt = cnt.get();
-    c.side = side.get(), c.mvx0 = mvx0.get(), c.mvx1 = mvx1.get(), c.ok0 = ok0.get(),
-    c.ok1 = ok1.get();
-    c.mvg0 = mvg0.get(), c.mvg1 = mvg1.get();
-    c.sub = sub.get();
-    c.cut = cut.get();
-    // small nodes with enough attempts in flight: smaller CTAs, several per SM
-    const int64_t ctas = (int64_t)nodes * T;
-    const bool many = ctas >= 4LL * num_sms();
-    if (many && max_ns <= 512) launch(k_bisect<128>, (unsigned)ctas, 128, 0, s, c);
-    else if (many && max_ns <= 4096) launch(k_bisect<256>, (unsigned)ctas, 256, 0, s, c);
-    else if (many && max_ns <= 16384) launch(k_bisect<512>, (unsigned)ctas, 512, 0, s, c);
-    else launch(k_bisect<kIPThreads>, (unsigned)ctas, kIPThreads, 0, s, c);
-    TP_LAUNCH_CHECK();
-    launch(k_fill_i32, grid_for(n, 256), 256, 0, s, next_node.get(), n, -1);
-    launch(k_pick, (unsigned)nodes, 256, 0, s, c, d_c0, d_c1, next_node.get(), d_part);
-    TP_LAUNCH_CHECK();
-    std::swap(node_of, next_node);
-    TP_CUDA(cudaStreamSynchronize(s));  // host vectors above outlive their copies
-    off.swap(noff);
-    kks.swap(nkk);
-    hkey.swap(nkey);
-    lmx.swap(nlmx);
-  }
+  if (small) bisect_forest<int32_t>(g, roots, root_start, p, d_part, s);
+  else bisect_forest<int64_t>(g, roots, root_start, p, d_part, s);
 }
 
 }  // namespace tp

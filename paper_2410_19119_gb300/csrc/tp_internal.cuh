@@ -475,16 +475,16 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
 tp_graph *decompress(const tp_graph *z, cudaStream_t s);
 void initial_partition(const tp_graph *g, int32_t k, int64_t l_max, const tp_params &p,
                        int32_t *d_part, cudaStream_t s);
-// Roots of a bisection forest (batched graphs): root j owns the vertices with
-// node_of[u] == j and assigns blocks off .. off + k - 1; key is the block
+// Roots of a bisection forest (batched graphs): root j owns the vertices
+// root_start[j] .. root_start[j + 1] - 1 and assigns blocks off .. off + k - 1; key is the block
 // offset its graph alone would use (it seeds the hashes), l_max its graph's.
 struct IPRoot {
   int32_t off, key, k;
   int64_t l_max;
 };
 void initial_partition_roots(const tp_graph *g, const std::vector<IPRoot> &roots,
-                             const int32_t *d_node_of, const tp_params &p, int32_t *d_part,
-                             cudaStream_t s);
+                             const std::vector<int64_t> &root_start, const tp_params &p,
+                             int32_t *d_part, cudaStream_t s);
 void block_weights(const tp_graph *g, const int32_t *part, int32_t k, int64_t *d_B,
                    cudaStream_t s);
 int64_t edge_cut(const tp_graph *g, const int32_t *part, cudaStream_t s);
