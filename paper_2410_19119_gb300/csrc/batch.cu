@@ -263,6 +263,7 @@ void extract(const ULevel &L, const std::vector<int32_t> &sel, int64_t nb, const
   }
   const tp_graph *og = L.g.get();
   X.g.reset(alloc_union(X.voff[G], X.eoff[G], og->unit_vw, og->unit_ew, W, og->max_ew, s));
+  X.g->sum_ew = og->sum_ew;
   upload_tables(X, nb, s);
   X.gid.alloc(std::max<int64_t>(X.voff[G], 1), s);
   Buf<int32_t> d_sel(G, s);
@@ -317,7 +318,9 @@ void partition_union(const std::vector<const tp_graph *> &gs, const std::vector<
   std::vector<int64_t> W(nb, 0), U(nb, 1), lmax(nb, 0), boff(nb, 0);
   std::vector<int32_t> kk(nb, 1);
   int64_t K = 0;
+  int32_t kmax = 0;
   for (int32_t i : idx) {
+    kmax = std::max(kmax, k[i]);
     W[i] = gs[i]->total_vw;
     kk[i] = k[i];
     U[i] = cluster_cap(W[i], k[i], eps_ppm);
@@ -351,6 +354,7 @@ void partition_union(const std::vector<const tp_graph *> &gs, const std::vector<
     L->eoff.assign(G0 + 1, 0);
     bool unit_vw = true, unit_ew = true;
     int64_t Wt = 0, max_ew = 1, maxlen = 0;
+    __int128 sum_ew = 0;
     std::vector<SrcGraph> src(G0);
     for (int64_t j = 0; j < G0; ++j) {
       const tp_graph *g = gs[idx[j]];
@@ -360,12 +364,14 @@ void partition_union(const std::vector<const tp_graph *> &gs, const std::vector<
       unit_ew &= g->unit_ew != 0;
       Wt += g->total_vw;
       max_ew = std::max(max_ew, g->max_ew);
+      sum_ew += ew_sum_bound(g);
       maxlen = std::max(maxlen, std::max(g->n, g->m2));
       src[j] = SrcGraph{g->xadj.get(), g->adj.get(), g->unit_vw ? nullptr : g->vw.get(),
                         g->unit_ew ? nullptr : g->ew.get()};
     }
     TP_REQUIRE(L->voff[G0] + nb < INT32_MAX, TP_ERR_INVALID);
     L->g.reset(alloc_union(L->voff[G0], L->eoff[G0], unit_vw, unit_ew, Wt, max_ew, s));
+    L->g->sum_ew = sum_ew > INT64_MAX ? INT64_MAX : (int64_t)sum_ew;
     upload_tables(*L, nb, s);
     L->gid.alloc(std::max<int64_t>(L->n(), 1), s);
     Buf<SrcGraph> d_src(G0, s);
@@ -525,6 +531,7 @@ void partition_union(const std::vector<const tp_graph *> &gs, const std::vector<
     seg.lb = d_boff.get();
     seg.cap = d_lmax.get();
     seg.k = d_k.get();
+    seg.kmax = kmax;
     seg.ngraphs = nb;
     rebalance_moves_seg(L.g.get(), seg, L.d_gl.get(), L.G(), cur.get(), B.get(), p, s);
     lp_refine(L.g.get(), (int32_t)K, 0, p, l, cur.get(), B.get(), s, &seg);

@@ -288,6 +288,7 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
                                              map, cg->vw.get());
     TP_LAUNCH_CHECK();
     cg->total_vw = g->total_vw;
+    cg->sum_ew = ew_sum_bound(g);
 
     // inter-cluster entries: counts, offsets, emission
     tp_params dp;

@@ -668,11 +668,19 @@ int64_t ip_smem_cap() {
 }
 
 template <class V>
-Shape ip_shape(int64_t ns, int64_t entries, int64_t attempts) {
-  const bool fits = ns <= ip_smem_cap<V>();
-  int64_t cl = 1;
-  while (cl < 16 && 2 * cl * attempts <= num_sms()) cl <<= 1;
-  if (!fits || (entries > kIPClusterEntries && cl > 1)) return Shape{kIPMaxThreads, (int)cl};
+bool ip_large(int64_t ns, int64_t entries) {
+  return ns > ip_smem_cap<V>() || entries > kIPClusterEntries;
+}
+
+// attempts: of all nodes of the depth; large_attempts: of those that a
+// cluster would run (they share the SMs among themselves).
+template <class V>
+Shape ip_shape(int64_t ns, int64_t entries, int64_t attempts, int64_t large_attempts) {
+  if (ip_large<V>(ns, entries)) {
+    int64_t cl = 1;
+    while (cl < 16 && 2 * cl * large_attempts <= num_sms()) cl <<= 1;
+    if (cl > 1 || ns > ip_smem_cap<V>()) return Shape{kIPMaxThreads, (int)cl};
+  }
   // smaller CTAs, several per SM, where many attempts are in flight
   const bool many = attempts >= 2LL * num_sms();
   const int threads = many ? (ns <= 512 ? 128 : ns <= 2048 ? 256 : ns <= 6144 ? 512 : 1024)
@@ -752,9 +760,13 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
     // launch classes: nodes of the same shape, the largest first
     std::vector<int32_t> order(nodes);
     std::vector<Shape> shape(nodes);
+    int64_t large = 0;
+    for (int32_t j = 0; j < nodes; ++j)
+      large += ip_large<V>(d.start[j + 1] - d.start[j], d.entries[j]);
     for (int32_t j = 0; j < nodes; ++j) {
       order[j] = j;
-      shape[j] = ip_shape<V>(d.start[j + 1] - d.start[j], d.entries[j], (int64_t)nodes * T);
+      shape[j] = ip_shape<V>(d.start[j + 1] - d.start[j], d.entries[j], (int64_t)nodes * T,
+                             large * T);
     }
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
       if (shape[x].cluster != shape[y].cluster) return shape[x].cluster > shape[y].cluster;
@@ -898,7 +910,7 @@ void initial_partition_roots(const tp_graph *g, const std::vector<IPRoot> &roots
   // edge weight) fit; a bound from sizes first, the largest weighted degree
   // only where that does not settle it
   constexpr int64_t kFit = (int64_t)1 << 29;
-  bool small = g->unit_ew ? n < kFit : (double)g->m2 * (double)g->max_ew < (double)kFit;
+  bool small = g->unit_ew ? n < kFit : ew_sum_bound(g) < kFit;
   if (!small && !g->unit_ew) {
     Buf<unsigned long long> mx(1, s);
     TP_CUDA(cudaMemsetAsync(mx.get(), 0, sizeof(unsigned long long), s));

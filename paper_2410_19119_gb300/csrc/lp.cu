@@ -64,11 +64,14 @@ struct RateCtx {
   // M_FAV output
   int32_t *fav;
   // M_REBAL (batched graphs: rb_best and blk_of hold one entry per graph)
-  int32_t blk, k;
+  int32_t blk;
   int64_t *rb_loss;
   int32_t *rb_t;
   long long *rb_best;
   const int32_t *blk_of;
+  // labels are blocks: how many (one graph; batched graphs have seg.k), and
+  // the most of any graph (0: labels are clusters)
+  int32_t k, kmax;
   // batched graphs (seg.gid == null: one graph)
   SegLp seg;
   // lists and global tables
@@ -129,6 +132,17 @@ __device__ __forceinline__ int64_t cap_of(const RateCtx &c, int64_t u) {
 }
 __device__ __forceinline__ int32_t no_fav(const RateCtx &c, int64_t u) {
   return (int32_t)(c.g.n + (c.seg.gid ? c.seg.gid[u] : 0));
+}
+
+// Blocks of u's graph: labels lb .. lb + k - 1 (direct tables, rebalancing).
+__device__ __forceinline__ int32_t block_range(const RateCtx &c, int64_t u, int32_t &lb) {
+  if (!c.seg.gid) {
+    lb = 0;
+    return c.k;
+  }
+  const int32_t g = c.seg.gid[u];
+  lb = (int32_t)c.seg.lb[g];
+  return c.seg.k[g];
 }
 
 template <int MODE>
@@ -260,12 +274,13 @@ __device__ __forceinline__ void finalize_warp(const RateCtx &c, const Best &b, i
   } else if (MODE == M_FAV) {
     if (lane == 0) c.fav[u] = b.r > 0 ? b.x : no_fav(c, u);
   } else {
-    // the graph's blocks are lb .. lb + k - 1 (one graph: 0 .. k - 1)
-    int32_t blk = c.blk, k = c.k, lb = 0;
+    int32_t lb;
+    const int32_t k = block_range(c, u, lb);
+    int32_t blk = c.blk;
     long long *best = c.rb_best;
     if (c.seg.gid) {
       const int32_t g = c.seg.gid[u];
-      blk = c.blk_of[g], k = c.seg.k[g], lb = (int32_t)c.seg.lb[g];
+      blk = c.blk_of[g];
       best += g;
     }
     const int64_t cap = cap_of(c, u);
@@ -290,31 +305,54 @@ __device__ __forceinline__ void finalize_warp(const RateCtx &c, const Best &b, i
   }
 }
 
-// Rates vertex u with one warp; the table must be empty on entry and is
-// empty again on exit. The scan takes two passes: the top rating among the
-// other labels (and the own rating), then the tie order among the labels at
-// that rating only, so tie hashes are formed for tied candidates alone; in
-// LP mode a vertex whose top rating does not beat its own cannot move and
-// skips the second pass.
-template <bool COMP, int MODE, class V>
-__device__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *vals, int logcap,
-                                 MoverBuf *mb) {
+// Adds the labels of u's neighbours to a warp's table: add(label, weight).
+// CSR rows are read 128 entries a step, all loads of a kind issued before the
+// first is used, so a row costs two round trips (entries, then labels) per
+// 128 neighbours.
+template <bool COMP, class F>
+__device__ __forceinline__ void warp_labels(const RateCtx &c, int64_t u, F &&add) {
+  if constexpr (COMP) {
+    warp_neighbours<true>(c.g, u, -1, [&](bool has, int32_t v, int64_t w, int64_t) {
+      if (has) add(c.label[v], w);
+    });
+  } else {
+    const int64_t e = c.g.xadj[u + 1];
+    for (int64_t i = c.g.xadj[u] + lane_id(); i - lane_id() < e; i += 128) {
+      int32_t v[4], x[4];
+      int64_t w[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const bool in = i + 32 * r < e;
+        v[r] = in ? __ldcs(c.g.adj + i + 32 * r) : -1;
+        w[r] = in && c.g.ew ? __ldcs(c.g.ew + i + 32 * r) : 1;
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) x[r] = v[r] >= 0 ? c.label[v[r]] : -1;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (x[r] >= 0) add(x[r], w[r]);
+    }
+  }
+}
+
+// Picks u's label from a warp's filled table: slot(i, x, R) gives the label
+// (negative: none) and rating of slot i < cap. The scan takes two passes: the
+// top rating among the other labels (and the own rating), then the tie order
+// among the labels at that rating only, so tie hashes are formed for tied
+// candidates alone; in LP mode a vertex whose top rating does not beat its
+// own cannot move and skips the second pass.
+template <int MODE, class Slot>
+__device__ __forceinline__ Best pick_warp(const RateCtx &c, int64_t u, int64_t cu, int cap,
+                                          Slot &&slot) {
   const int lane = lane_id();
   const int32_t own = c.label[u];
-  const int64_t cu = node_w(c.g, u), capu = cap_of(c, u);
-  // every lane adds its neighbour's label to the table (shared-memory
-  // atomics are far cheaper than grouping equal labels across lanes first)
-  warp_neighbours<COMP>(c.g, u, -1, [&](bool has, int32_t v, int64_t w, int64_t) {
-    if (has) tbl_add<V>(keys, vals, logcap, c.label[v], w, c.g.err);
-  });
-  __syncwarp();
-  __threadfence_block();
-  const int cap = 1 << logcap;
+  const int64_t capu = cap_of(c, u);
   int64_t rmax = -1, rown = 0;
   for (int i = lane; i < cap; i += 32) {
-    const int32_t x = keys[i];
+    int32_t x;
+    int64_t R;
+    slot(i, x, R);
     if (x < 0) continue;
-    const int64_t R = (int64_t)vals[i];
     if (x == own) rown = R;
     else rmax = R > rmax ? R : rmax;
   }
@@ -327,8 +365,10 @@ __device__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *
     const TieKey hv = tie_key<MODE>(c, u);
     // the best label ignoring the cap: the top-rated one first in tie order
     for (int i = lane; i < cap; i += 32) {
-      const int32_t x = keys[i];
-      if (x < 0 || x == own || (int64_t)vals[i] != rmax) continue;
+      int32_t x;
+      int64_t R;
+      slot(i, x, R);
+      if (x < 0 || x == own || R != rmax) continue;
       const uint32_t t = MODE == M_REBAL ? 0u : tie_of(hv, x);
       if (better(rmax, t, x, b.r, b.t, b.x)) b.r = rmax, b.t = t, b.x = x;
     }
@@ -338,9 +378,10 @@ __device__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *
     if (MODE != M_FAV && b.x != INT32_MAX && c.lw[b.x] + cu > capu) {
       b.init();
       for (int i = lane; i < cap; i += 32) {
-        const int32_t x = keys[i];
+        int32_t x;
+        int64_t R;
+        slot(i, x, R);
         if (x < 0 || x == own) continue;
-        const int64_t R = (int64_t)vals[i];
         if (MODE == M_LP && R <= rown) continue;
         const uint32_t t = MODE == M_REBAL ? 0u : tie_of(hv, x);
         if (better(R, t, x, b.r, b.t, b.x) && c.lw[x] + cu <= capu) b.r = R, b.t = t, b.x = x;
@@ -349,7 +390,28 @@ __device__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *
       b.rown = rown;
     }
   }
-  for (int i = lane; i < cap; i += 32) keys[i] = -1, vals[i] = 0;
+  return b;
+}
+
+// Rates vertex u with one warp; the hash table must be empty on entry and is
+// empty again on exit.
+template <bool COMP, int MODE, class V>
+__device__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *vals, int logcap,
+                                 MoverBuf *mb) {
+  // every lane adds its neighbour's label to the table (shared-memory
+  // atomics are far cheaper than grouping equal labels across lanes first)
+  warp_labels<COMP>(c, u, [&](int32_t x, int64_t w) {
+    tbl_add<V>(keys, vals, logcap, x, w, c.g.err);
+  });
+  __syncwarp();
+  __threadfence_block();
+  const int cap = 1 << logcap;
+  const int64_t cu = node_w(c.g, u);
+  const Best b = pick_warp<MODE>(c, u, cu, cap, [&](int i, int32_t &x, int64_t &R) {
+    x = keys[i];
+    R = (int64_t)vals[i];
+  });
+  for (int i = lane_id(); i < cap; i += 32) keys[i] = -1, vals[i] = 0;
   __syncwarp();
   finalize_warp<MODE>(c, b, u, cu, mb);
 }
@@ -381,10 +443,11 @@ __device__ __forceinline__ void init_table(WarpSmem<LOG, V> &w) {
 // Small tier: one warp per listed vertex (c.list), or, in rebalancing mode
 // (c.list == nullptr), every vertex of the small and lane tiers, filtered in
 // 32-vertex slabs.
-template <bool COMP, int MODE>
+template <bool COMP, int MODE, class V>
 __global__ void k_rate_small(RateCtx c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  WarpSmem<kSmallLog> &ws = reinterpret_cast<WarpSmem<kSmallLog> *>(smem_raw)[threadIdx.x >> 5];
+  WarpSmem<kSmallLog, V> &ws =
+      reinterpret_cast<WarpSmem<kSmallLog, V> *>(smem_raw)[threadIdx.x >> 5];
   init_table(ws);
   MoverBuf mb{ws.mu, ws.mt, ws.mo, ws.mg, 0};
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -396,7 +459,7 @@ __global__ void k_rate_small(RateCtx c) {
       int64_t i, u;
       if (tier_entry<MODE>(c, k, i, u)) {
         const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
-        rate_vertex_warp<COMP, MODE>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
+        rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
       }
     }
   } else {
@@ -410,7 +473,7 @@ __global__ void k_rate_small(RateCtx c) {
         am &= am - 1;
         const int64_t v = base + j;
         const int64_t d = COMP ? zip_nbr(c.g, v).deg : c.g.xadj[v + 1] - c.g.xadj[v];
-        rate_vertex_warp<COMP, MODE>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
+        rate_vertex_warp<COMP, MODE, V>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
       }
     }
   }
@@ -988,6 +1051,50 @@ __global__ void k_rate_list(RateCtx c) {
   if (MODE == M_LP) flush_movers(c, mb);
 }
 
+// Few labels (refinement and rebalancing: the k blocks of the vertex's graph,
+// at most kDirectMax): a rating is one counter per block, indexed by the
+// label, so there is nothing to hash, and a vertex clears and scans k
+// counters instead of up to 16384 slots. One warp per listed vertex of degree
+// <= kBigTinySplit; the block and hub kernels take the same tables (DIR).
+constexpr int kDirectMax = 1024;
+constexpr int kDirectWarps = 4;
+
+template <bool COMP, int MODE, class V>
+__global__ void __launch_bounds__(32 * kDirectWarps) k_rate_direct(RateCtx c, int kmax) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int32_t mu[kDirectWarps][32], mt[kDirectWarps][32], mo[kDirectWarps][32];
+  __shared__ int64_t mg[kDirectWarps][32];
+  const int w = threadIdx.x >> 5, lane = lane_id();
+  V *vals = reinterpret_cast<V *>(smem_raw) + (size_t)w * kmax;
+  for (int i = lane; i < kmax; i += 32) vals[i] = 0;
+  __syncwarp();
+  MoverBuf mb{mu[w], mt[w], mo[w], mg[w], 0};
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int64_t kb, ke;
+  tier_range(c, kb, ke);
+  for (int64_t q = kb + gw; q < ke; q += nw) {
+    int64_t pos, u;
+    if (!tier_entry<MODE>(c, q, pos, u)) continue;
+    int32_t lb;
+    const int32_t k = block_range(c, u, lb);
+    warp_labels<COMP>(c, u, [&](int32_t x, int64_t wt) {
+      const uint32_t i = (uint32_t)(x - lb);
+      if (i < (uint32_t)k) atomicAdd(&vals[i], (V)wt);
+    });
+    __syncwarp();
+    const int64_t cu = node_w(c.g, u);
+    const Best b = pick_warp<MODE>(c, u, cu, k, [&](int i, int32_t &x, int64_t &R) {
+      R = (int64_t)vals[i];
+      x = R ? lb + i : -1;  // weights are positive: a block with a neighbour has a rating
+    });
+    for (int i = lane; i < k; i += 32) vals[i] = 0;
+    __syncwarp();
+    finalize_warp<MODE>(c, b, u, cu, &mb);
+  }
+  if (MODE == M_LP) flush_movers(c, mb);
+}
+
 // ---------------------------------------------------------------- big tier
 // One block per listed vertex: its ratings are summed in a shared-memory
 // hash table of 2^logc >= 1.5 deg slots (keys, then 32-bit counts for unit
@@ -1169,15 +1276,19 @@ __device__ __forceinline__ void block_reduce_best(Best &b, Best *wb) {
   __syncthreads();
 }
 
-template <bool COMP, int MODE, bool WT>
-__global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int maxlog) {
-  using V = typename std::conditional<WT, unsigned long long, uint32_t>::type;
+// V: uint32_t where all edge weights together fit, else 64 bits (32-bit shared
+// atomics are native, and the smaller tables leave room for more blocks).
+// DIR: a counter per block of the vertex's graph (kmax: most of any graph)
+// instead of the hash table.
+template <bool COMP, int MODE, class V, bool DIR>
+__global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int maxlog, int kmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const size_t slots = DIR ? (size_t)((kmax + 3) & ~3) : (size_t)1 << maxlog;
   int32_t *keys = reinterpret_cast<int32_t *>(smem_raw);
-  V *vals = reinterpret_cast<V *>(smem_raw + sizeof(int32_t) * ((size_t)1 << maxlog));
+  V *vals = reinterpret_cast<V *>(smem_raw + (DIR ? 0 : sizeof(int32_t) * slots));
   // compressed: the record's bytes (at most 5 per neighbour, + alignment),
   // then its decoded values
-  uint8_t *stage = reinterpret_cast<uint8_t *>(vals + ((size_t)1 << maxlog));
+  uint8_t *stage = reinterpret_cast<uint8_t *>(vals + slots);
   uint32_t *vbuf = reinterpret_cast<uint32_t *>(stage + block_stage_bytes(block_max_deg(maxlog)));
   __shared__ int64_t red[kBlockThreads / 32 + 1];
   __shared__ Best wb[kBlockThreads / 32];
@@ -1192,21 +1303,46 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
     const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
     int logc = 5;
     while (logc < maxlog && ((int64_t)1 << logc) < d + d / 2) ++logc;
-    const int cap = 1 << logc;
-    for (int k = tid; k < cap; k += kBlockThreads) keys[k] = -1, vals[k] = 0;
+    int32_t lb = 0;
+    const int cap = DIR ? block_range(c, u, lb) : 1 << logc;
+    for (int k = tid; k < cap; k += kBlockThreads) {
+      if (!DIR) keys[k] = -1;
+      vals[k] = 0;
+    }
     __syncthreads();
+    auto add = [&](int32_t x, V w) {
+      if constexpr (DIR) {
+        if ((uint32_t)(x - lb) < (uint32_t)cap) atomicAdd(&vals[x - lb], w);
+      } else {
+        blk_add<V>(keys, vals, logc, x, w, c.g.err);
+      }
+    };
+    auto slot_label = [&](int k) -> int32_t {
+      if constexpr (DIR) return vals[k] ? lb + k : -1;
+      else return keys[k];
+    };
     if (COMP) {
       const ZipNbr z = zip_nbr(c.g, u);  // one chunk: the big tier is below the chunking threshold
       block_decode_range(c.g, u, z.data, z.end, z.deg, stage, vbuf, red, [&](int cnt) {
-        for (int e = tid; e < cnt; e += kBlockThreads)
-          blk_add<V>(keys, vals, logc, c.label[vbuf[e]], (V)1, c.g.err);
+        for (int e = tid; e < cnt; e += kBlockThreads) add(c.label[vbuf[e]], (V)1);
       });
     } else {
+      // four entries a thread and step, their loads together
       const int64_t b = c.g.xadj[u];
-      for (int64_t e = tid; e < d; e += kBlockThreads) {
-        const int32_t v = __ldcs(c.g.adj + b + e);
-        blk_add<V>(keys, vals, logc, c.label[v], (V)(c.g.ew ? __ldcs(c.g.ew + b + e) : 1),
-                   c.g.err);
+      for (int64_t e0 = tid; e0 < d; e0 += 4 * kBlockThreads) {
+        int32_t v[4], x[4];
+        V w[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int64_t e = e0 + r * kBlockThreads;
+          v[r] = e < d ? __ldcs(c.g.adj + b + e) : -1;
+          w[r] = e < d && c.g.ew ? (V)__ldcs(c.g.ew + b + e) : (V)1;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = v[r] >= 0 ? c.label[v[r]] : -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (x[r] >= 0) add(x[r], w[r]);
       }
     }
     __syncthreads();
@@ -1216,7 +1352,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
     const int64_t cu = node_w(c.g, u), capu = cap_of(c, u);
     int64_t rmax = -1, rown = 0;
     for (int k = tid; k < cap; k += kBlockThreads) {
-      const int32_t x = keys[k];
+      const int32_t x = slot_label(k);
       if (x < 0) continue;
       const int64_t R = (int64_t)vals[k];
       if (x == own) rown = R;
@@ -1230,7 +1366,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
     const TieKey hv = rate ? tie_key<MODE>(c, u) : TieKey{0, 0};
     if (rate) {
       for (int k = tid; k < cap; k += kBlockThreads) {
-        const int32_t x = keys[k];
+        const int32_t x = slot_label(k);
         if (x < 0 || x == own || (int64_t)vals[k] != rmax) continue;
         const uint32_t t = MODE == M_REBAL ? 0u : tie_of(hv, x);
         if (better(rmax, t, x, b.r, b.t, b.x)) b.r = rmax, b.t = t, b.x = x;
@@ -1243,7 +1379,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
       const int64_t rown = b.rown;
       b.init();
       for (int k = tid; k < cap; k += kBlockThreads) {
-        const int32_t x = keys[k];
+        const int32_t x = slot_label(k);
         if (x < 0 || x == own) continue;
         const int64_t R = (int64_t)vals[k];
         if (MODE == M_LP && R <= rown) continue;
@@ -1267,10 +1403,11 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
 // ratings in a shared-memory table and adds them into the vertex's global
 // table (the paper's rating maps as flush buffers against contention).
 constexpr int kHugeStage = (5 * kChunkSize + 64 + 15) & ~15;  // one chunk's bytes + alignment
-template <bool COMP, int MODE>
+template <bool COMP, int MODE, class V, bool DIR>
 __global__ void __launch_bounds__(kBlockThreads) k_rate_huge_chunks(RateCtx c) {
-  __shared__ int32_t keys[1 << kHugeLog];
-  __shared__ unsigned long long vals[1 << kHugeLog];
+  static_assert(kDirectMax <= 1 << kHugeLog, "a counter per block fits the chunk's table");
+  __shared__ int32_t keys[DIR ? 1 : 1 << kHugeLog];
+  __shared__ V vals[1 << kHugeLog];
   __shared__ __align__(16) uint8_t stage[COMP ? kHugeStage : 16];
   __shared__ uint32_t vbuf[COMP ? kChunkSize : 1];
   __shared__ int64_t red[kBlockThreads / 32 + 1];
@@ -1278,7 +1415,10 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_huge_chunks(RateCtx c) {
   __shared__ int32_t claimed[1 << kHugeLog];
   __shared__ int32_t s_nclaim, s_base;
   const int tid = threadIdx.x;
-  for (int k = tid; k < (1 << kHugeLog); k += kBlockThreads) keys[k] = -1, vals[k] = 0;
+  for (int k = tid; k < (1 << kHugeLog); k += kBlockThreads) {
+    if (!DIR) keys[k] = -1;
+    vals[k] = 0;
+  }
   __syncthreads();
   // bucket mode: this sub-round's chunk items; else every chunk, skipping
   // inactive hubs (the hub of an item found by binary search)
@@ -1307,23 +1447,41 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_huge_chunks(RateCtx c) {
     }
     const int64_t u = c.list[i];
     if (!c.bpos && !active<MODE>(c, u)) continue;  // uniform over the block
+    int32_t lb = 0;
+    const int32_t nblk = DIR ? block_range(c, u, lb) : 0;
+    auto add = [&](int32_t x, V w) {
+      if constexpr (DIR) {
+        if ((uint32_t)(x - lb) < (uint32_t)nblk) atomicAdd(&vals[x - lb], w);
+      } else {
+        blk_add<V>(keys, vals, kHugeLog, x, w, c.g.err);
+      }
+    };
     if (COMP) {
       const ZipNbr z = zip_nbr(c.g, u);
       uint64_t cb, ce;
       int64_t cnt;
       zip_chunk(c.g, z, j, cb, ce, cnt);
       block_decode_range(c.g, u, cb, ce, cnt, stage, vbuf, red, [&](int n) {
-        for (int e = tid; e < n; e += kBlockThreads)
-          blk_add<unsigned long long>(keys, vals, kHugeLog, c.label[vbuf[e]], 1ull, c.g.err);
+        for (int e = tid; e < n; e += kBlockThreads) add(c.label[vbuf[e]], (V)1);
       });
     } else {
+      // the chunk's entries (at most four a thread), their loads together
+      static_assert(kChunkSize <= 4 * kBlockThreads, "one step per chunk");
       const int64_t b = c.g.xadj[u] + j * kChunkSize;
       const int64_t e = min(b + kChunkSize, c.g.xadj[u + 1]);
-      for (int64_t q = b + tid; q < e; q += kBlockThreads) {
-        const int32_t v = __ldcs(c.g.adj + q);
-        blk_add<unsigned long long>(keys, vals, kHugeLog, c.label[v],
-                                    (unsigned long long)(c.g.ew ? __ldcs(c.g.ew + q) : 1), c.g.err);
+      int32_t v[4], x[4];
+      V w[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int64_t q = b + tid + r * kBlockThreads;
+        v[r] = q < e ? __ldcs(c.g.adj + q) : -1;
+        w[r] = q < e && c.g.ew ? (V)__ldcs(c.g.ew + q) : (V)1;
       }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) x[r] = v[r] >= 0 ? c.label[v[r]] : -1;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (x[r] >= 0) add(x[r], w[r]);
     }
     __syncthreads();
     int32_t *tk = c.tkeys + c.tbase + c.toff[i];
@@ -1345,9 +1503,13 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_huge_chunks(RateCtx c) {
 #pragma unroll
       for (int q = 0; q < kFlush; ++q) {
         const int k = tid + q * kBlockThreads;
-        lab[q] = keys[k];
         w[q] = (int64_t)vals[k];
-        keys[k] = -1;
+        if constexpr (DIR) {
+          lab[q] = w[q] ? lb + k : -1;
+        } else {
+          lab[q] = keys[k];
+          keys[k] = -1;
+        }
         vals[k] = 0;
         pend[q] = lab[q] >= 0;
         h[q] = pend[q] ? slot_of(lab[q], lc) : 0;
@@ -1714,34 +1876,58 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
     TP_LAUNCH_CHECK();
     if (prof) prof_end(PF_RATE_LANE, s, per_launch * tier_round_bytes(g, n_lane, T.edges[TIER_LANE]));
   }
+  // sums in 32 bits wherever all edge weights of the graph together fit
+  // (compressed levels have unit weights)
+  const bool narrow = g->unit_ew || ew_sum_bound(g) < ((int64_t)1 << 31);
+  // few labels: direct tables for every tier above the small one, and for the
+  // small one where k counters are no more than its largest hash table
+  const bool direct = MODE != M_FAV && c.kmax > 0 && c.kmax <= kDirectMax;
+  auto run_direct = [&](const int32_t *list, int64_t cnt, int t) {
+    RateCtx m = c;
+    m.list = list;
+    m.list_n = cnt;
+    bucketed(m, t);
+    constexpr int DM = MODE == M_FAV ? M_LP : MODE;
+    const unsigned blocks =
+        (unsigned)std::min<int64_t>((cnt + kDirectWarps - 1) / kDirectWarps, (int64_t)sms * 16);
+    const size_t sm = (size_t)c.kmax * kDirectWarps * (narrow ? 4 : 8);
+    if (comp) launch(k_rate_direct<true, DM, uint32_t>, blocks, 32 * kDirectWarps, sm, s, m, c.kmax);
+    else if (narrow) launch(k_rate_direct<false, DM, uint32_t>, blocks, 32 * kDirectWarps, sm, s, m, c.kmax);
+    else launch(k_rate_direct<false, DM, unsigned long long>, blocks, 32 * kDirectWarps, sm, s, m, c.kmax);
+    TP_LAUNCH_CHECK();
+  };
   if (n_small > 0) {
     if (prof) prof_begin(PF_RATE_SMALL, s);
-    int wpb = p.warps_per_block >= 1 && p.warps_per_block <= 16 ? p.warps_per_block : 8;
-    size_t sm = sizeof(WarpSmem<kSmallLog>) * wpb;
-    RateCtx m = c;
-    int64_t items = g->n;
-    if (MODE != M_REBAL) {
-      m.list = T.small.get();
-      m.list_n = T.n_small;
-      items = T.n_small;
-      bucketed(m, 0);
+    if (MODE != M_REBAL && direct && c.kmax <= 1 << kSmallLog) {
+      run_direct(T.small.get(), T.n_small, 0);
     } else {
-      m.list = nullptr;
+      int wpb = p.warps_per_block >= 1 && p.warps_per_block <= 16 ? p.warps_per_block : 8;
+      size_t sm = (narrow ? sizeof(WarpSmem<kSmallLog, uint32_t>) : sizeof(WarpSmem<kSmallLog>)) * wpb;
+      RateCtx m = c;
+      int64_t items = g->n;
+      if (MODE != M_REBAL) {
+        m.list = T.small.get();
+        m.list_n = T.n_small;
+        items = T.n_small;
+        bucketed(m, 0);
+      } else {
+        m.list = nullptr;
+      }
+      const int64_t per_warp = MODE != M_REBAL ? 1 : 32;  // list entries / vertices per warp step
+      unsigned blocks = (unsigned)std::min<int64_t>((items + per_warp * wpb - 1) / (per_warp * wpb),
+                                                    (int64_t)sms * 16);
+      if (comp) launch(k_rate_small<true, MODE, uint32_t>, blocks, 32 * wpb, sm, s, m);
+      else if (narrow) launch(k_rate_small<false, MODE, uint32_t>, blocks, 32 * wpb, sm, s, m);
+      else launch(k_rate_small<false, MODE, int64_t>, blocks, 32 * wpb, sm, s, m);
+      TP_LAUNCH_CHECK();
     }
-    const int64_t per_warp = MODE != M_REBAL ? 1 : 32;  // list entries / vertices per warp step
-    unsigned blocks = (unsigned)std::min<int64_t>((items + per_warp * wpb - 1) / (per_warp * wpb),
-                                                  (int64_t)sms * 16);
-    if (comp) launch(k_rate_small<true, MODE>, blocks, 32 * wpb, sm, s, m);
-    else launch(k_rate_small<false, MODE>, blocks, 32 * wpb, sm, s, m);
-    TP_LAUNCH_CHECK();
     if (prof) prof_end(PF_RATE_SMALL, s, per_launch * tier_round_bytes(g, T.count[TIER_SMALL], T.edges[TIER_SMALL]));
   }
   if (T.n_mid + T.n_mid2 > 0) {
     if (prof) prof_begin(PF_RATE_MID, s);
-    // counts in 32 bits at unit weights (compressed levels have unit weights)
-    const bool unit = g->unit_ew != 0;
     auto run = [&](const int32_t *list, int64_t cnt, int t, bool big_tables) {
       if (!cnt) return;
+      if (direct) return run_direct(list, cnt, t);
       RateCtx m = c;
       m.list = list;
       m.list_n = cnt;
@@ -1755,10 +1941,10 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
     else launch(k_rate_list<false, MODE, LG, V>, blocks, 32 * kMidWarps, sm, s, m);          \
   } while (0)
       if (big_tables) {
-        if (unit) TP_MID(kMidLog, uint32_t);
+        if (narrow) TP_MID(kMidLog, uint32_t);
         else TP_MID(kMidLog, int64_t);
       } else {
-        if (unit) TP_MID(kMidSmallLog, uint32_t);
+        if (narrow) TP_MID(kMidSmallLog, uint32_t);
         else TP_MID(kMidSmallLog, int64_t);
       }
 #undef TP_MID
@@ -1770,27 +1956,33 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   }
   if (T.n_big0 + T.n_big1 + T.n_big + T.n_big2 > 0) {
     if (prof) prof_begin(PF_RATE_BIG, s);
-    const bool wt = !g->unit_ew;
     auto run = [&](const int32_t *list, int64_t cnt, int maxlog, int t) {
       if (!cnt) return;
       RateCtx m = c;
       m.list = list;
       m.list_n = cnt;
       bucketed(m, t);
-      const size_t sm = ((size_t)1 << maxlog) * (sizeof(int32_t) + (wt ? 8 : 4)) +
-                        (comp ? block_stage_bytes(block_max_deg(maxlog)) +
-                                    block_vbuf_bytes(block_max_deg(maxlog))
-                              : 0);
-      const int per_sm = std::max(1, (int)((size_t)(228 * 1024) / (sm + 2048)));
+      const size_t table = direct ? (size_t)((c.kmax + 3) & ~3) * (narrow ? 4 : 8)
+                                  : ((size_t)1 << maxlog) * (sizeof(int32_t) + (narrow ? 4 : 8));
+      const size_t sm = table + (comp ? block_stage_bytes(block_max_deg(maxlog)) +
+                                            block_vbuf_bytes(block_max_deg(maxlog))
+                                      : 0);
+      const int per_sm = std::max(1, std::min(8, (int)((size_t)(228 * 1024) / (sm + 2048))));
       const unsigned blocks = (unsigned)std::min<int64_t>(cnt, (int64_t)sms * per_sm);
-#define TP_BLK(CM, WW) launch(k_rate_block<CM, MODE, WW>, blocks, kBlockThreads, sm, s, m, maxlog)
-      if (comp) TP_BLK(true, false);
-      else if (wt) TP_BLK(false, true);
-      else TP_BLK(false, false);
+      constexpr int DM = MODE == M_FAV ? M_LP : MODE;
+#define TP_BLK(CM, V)                                                                            \
+  do {                                                                                           \
+    if (direct) launch(k_rate_block<CM, DM, V, true>, blocks, kBlockThreads, sm, s, m, maxlog, c.kmax); \
+    else launch(k_rate_block<CM, MODE, V, false>, blocks, kBlockThreads, sm, s, m, maxlog, 0);   \
+  } while (0)
+      if (comp) TP_BLK(true, uint32_t);
+      else if (narrow) TP_BLK(false, uint32_t);
+      else TP_BLK(false, unsigned long long);
 #undef TP_BLK
       TP_LAUNCH_CHECK();
     };
-    run(T.big0.get(), T.n_big0, kBlockTinyLog, 3);
+    if (T.n_big0 && direct) run_direct(T.big0.get(), T.n_big0, 3);
+    else run(T.big0.get(), T.n_big0, kBlockTinyLog, 3);
     run(T.big1.get(), T.n_big1, kBlockMidLog, 4);
     run(T.big.get(), T.n_big, kBlockSmallLog, 5);
     run(T.big2.get(), T.n_big2, kBlockBigLog, 6);
@@ -1809,8 +2001,16 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
     m.n_chunks = T.n_huge_chunks;
     const unsigned blocks = (unsigned)std::max<int64_t>(
         1, std::min<int64_t>(T.n_huge_chunks, (int64_t)sms * 6));
-    if (comp) launch(k_rate_huge_chunks<true, MODE>, blocks, kBlockThreads, 0, s, m);
-    else launch(k_rate_huge_chunks<false, MODE>, blocks, kBlockThreads, 0, s, m);
+    constexpr int DM = MODE == M_FAV ? M_LP : MODE;
+#define TP_HUGE(CM, V)                                                                           \
+  do {                                                                                           \
+    if (direct) launch(k_rate_huge_chunks<CM, DM, V, true>, blocks, kBlockThreads, 0, s, m);     \
+    else launch(k_rate_huge_chunks<CM, MODE, V, false>, blocks, kBlockThreads, 0, s, m);         \
+  } while (0)
+    if (comp) TP_HUGE(true, uint32_t);
+    else if (narrow) TP_HUGE(false, uint32_t);
+    else TP_HUGE(false, unsigned long long);
+#undef TP_HUGE
     TP_LAUNCH_CHECK();
     m.seg_start = T.huge_seg_start.get();
     m.n_segs = T.n_huge_segs;
@@ -1835,8 +2035,9 @@ void configure_kernels_once() {
   set_smem_limits(k_rate_list<true, M, LG, V>, sizeof(WarpSmem<LG, V>) * kMidWarps); \
   set_smem_limits(k_rate_list<false, M, LG, V>, sizeof(WarpSmem<LG, V>) * kMidWarps);
 #define TP_CFG_MODE(M)                                              \
-  set_smem_limits(k_rate_small<true, M>, small16);                  \
-  set_smem_limits(k_rate_small<false, M>, small16);                 \
+  set_smem_limits(k_rate_small<true, M, uint32_t>, small16);        \
+  set_smem_limits(k_rate_small<false, M, uint32_t>, small16);       \
+  set_smem_limits(k_rate_small<false, M, int64_t>, small16);        \
   TP_CFG_MID(M, kMidSmallLog, uint32_t)                             \
   TP_CFG_MID(M, kMidSmallLog, int64_t)                              \
   TP_CFG_MID(M, kMidLog, uint32_t)                                  \
@@ -1854,13 +2055,18 @@ void configure_kernels_once() {
                                   block_stage_bytes(kChunkThreshold) +
                                   block_vbuf_bytes(kChunkThreshold));
 #define TP_CFG_BLOCK(M)                                   \
-  set_smem_limits(k_rate_block<true, M, false>, blk);     \
-  set_smem_limits(k_rate_block<false, M, false>, blk);    \
-  set_smem_limits(k_rate_block<false, M, true>, blk);
+  set_smem_limits(k_rate_block<true, M, uint32_t, false>, blk);            \
+  set_smem_limits(k_rate_block<false, M, uint32_t, false>, blk);           \
+  set_smem_limits(k_rate_block<false, M, unsigned long long, false>, blk);
   TP_CFG_BLOCK(M_LP)
   TP_CFG_BLOCK(M_FAV)
   TP_CFG_BLOCK(M_REBAL)
 #undef TP_CFG_BLOCK
+  // direct tables: the record staging of compressed graphs dominates
+  const size_t dir = (size_t)kDirectMax * 4 + block_stage_bytes(kChunkThreshold) +
+                     block_vbuf_bytes(kChunkThreshold);
+  set_smem_limits(k_rate_block<true, M_LP, uint32_t, true>, dir);
+  set_smem_limits(k_rate_block<true, M_REBAL, uint32_t, true>, dir);
 }
 
 void configure_kernels() {
@@ -2232,6 +2438,8 @@ void lp_subround(tp_graph *g, const LpState &st, LpWork &w, uint64_t rk, int32_t
   c.lw = st.lw;
   c.cap = st.cap;
   c.seg = st.seg;
+  c.k = st.k;
+  c.kmax = st.kmax;
   c.rk = rk;
   c.rk_dev = rk_dev;
   c.S = S;
@@ -2516,6 +2724,8 @@ void lp_refine(tp_graph *g, int32_t k, int64_t l_max, const tp_params &p, int32_
   LpWork w;
   w.init(g->n, k, s);
   LpState st{d_part, d_B, k, l_max};
+  st.k = k;
+  st.kmax = seg ? seg->kmax : k;
   if (seg) st.seg = *seg;
   lp_rounds(g, st, w, p.seed, kTagRefine, (uint64_t)level, 0, p.refine_rounds, p.sub_rounds, p, s);
   release_hub_tables(g, s);
@@ -2577,7 +2787,7 @@ void rebalance_moves(tp_graph *g, int32_t k, int64_t l_max, int32_t *d_part, int
     c.lw = d_B;
     c.cap = l_max;
     c.blk = blk;
-    c.k = k;
+    c.k = c.kmax = k;
     c.rb_loss = rb_loss.get();
     c.rb_t = rb_t.get();
     c.rb_best = best.get();
@@ -2680,6 +2890,7 @@ void rebalance_moves_seg(tp_graph *g, const SegLp &seg, const int32_t *d_graphs,
     c.label = d_part;
     c.lw = d_B;
     c.seg = seg;
+    c.kmax = seg.kmax;
     c.blk_of = blk_of.get();
     c.rb_loss = rb_loss.get();
     c.rb_t = rb_t.get();

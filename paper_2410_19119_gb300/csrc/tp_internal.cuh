@@ -166,6 +166,9 @@ struct tp_graph {
   int64_t total_vw = 0;
   int64_t max_deg = 0;
   int64_t max_ew = 1;  // largest edge weight (1 for unit weights)
+  // weighted: no less than the sum of all edge weights (-1: not known; a
+  // contraction's weights sum to no more than its input's)
+  int64_t sum_ew = -1;
   // CSR
   tp::Buf<int64_t> xadj;
   tp::Buf<int32_t> adj;
@@ -208,6 +211,15 @@ struct GView {
   int32_t *err;
 };
 GView view(const tp_graph *g);
+
+// No less than the sum of all edge weights (INT64_MAX where nothing smaller
+// is known).
+inline int64_t ew_sum_bound(const tp_graph *g) {
+  if (g->unit_ew) return g->m2;
+  if (g->sum_ew >= 0) return g->sum_ew;
+  const __int128 b = (__int128)g->m2 * g->max_ew;
+  return b > INT64_MAX ? INT64_MAX : (int64_t)b;
+}
 
 // ---------------------------------------------------------------- hashing
 // Counter-based hashing of the deterministic LP (library's own statement of
@@ -384,6 +396,7 @@ struct SegLp {
   const int64_t *lb = nullptr;    // per graph: its first label
   const int64_t *cap = nullptr;   // per graph: the label-weight cap
   const int32_t *k = nullptr;     // per graph: its blocks (refinement, rebalancing)
+  int32_t kmax = 0;               // most blocks of any graph (0: labels are clusters)
   int64_t ngraphs = 0;            // table entries
 };
 struct LpState {
@@ -391,6 +404,7 @@ struct LpState {
   int64_t *lw;
   int64_t nlabels;
   int64_t cap;  // uniform cap for every label (one graph)
+  int32_t k = 0, kmax = 0;  // labels are blocks: how many, the most of any graph (0: clusters)
   SegLp seg{};
 };
 // Workspace for sub-rounds on one graph (per-label counters + mover lists).
