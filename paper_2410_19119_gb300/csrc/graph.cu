@@ -199,8 +199,12 @@ tp_graph *new_graph() { return new tp_graph(); }
 // ---------------------------------------------------------------- reductions
 namespace {
 
-__global__ void k_sum_max(const int64_t *vw, const int64_t *xadj, int64_t n, int64_t *out) {
-  // out[0] += sum vw (or n if vw null); out[1] = max degree
+// out[0] += sum vw (or n if vw null); out[1] = max degree. One atomic pair
+// per block: one per warp queued 2 x 39 000 atomics on two words (57 us for
+// 3 M vertices, several times the 24 MB it reads).
+__global__ void __launch_bounds__(256) k_sum_max(const int64_t *vw, const int64_t *xadj, int64_t n,
+                                                 int64_t *out) {
+  __shared__ int64_t ss[8], sm[8];
   int64_t s = 0, m = 0;
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
        u += (int64_t)gridDim.x * blockDim.x) {
@@ -212,46 +216,180 @@ __global__ void k_sum_max(const int64_t *vw, const int64_t *xadj, int64_t n, int
   }
   s = warp_sum(s);
   m = warp_max(m);
-  if (lane_id() == 0) {
+  if (lane_id() == 0) ss[threadIdx.x >> 5] = s, sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += ss[w], m = sm[w] > m ? sm[w] : m;
     atomicAdd((unsigned long long *)&out[0], (unsigned long long)s);
     atomicMax((long long *)&out[1], (long long)m);
   }
 }
 
-// Structural validation of a CSR graph, one warp per vertex.
-__global__ void k_validate(GView g, int32_t *bad) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int lane = lane_id();
-  if (warp == 0 && lane == 0 && (g.xadj[0] != 0 || g.xadj[g.n] != g.m2)) atomicCAS(bad, 0, 1);
-  for (int64_t u = warp; u < g.n; u += nw) {
-    int64_t b = g.xadj[u], e = g.xadj[u + 1];
+// ---- adjacency entries in tiles
+// Work per adjacency entry (validation, encoding) is cut into tiles of kTile
+// consecutive entries, one block each, so hubs and low-degree vertices load
+// the GPU alike (a warp per vertex left most lanes idle at degree 16 and a
+// hub of 1e5 neighbours to a single warp). tile_first[t] is the first vertex
+// whose row starts at or behind entry t * kTile (tiles 0 .. m2 / kTile, one
+// sentinel more: n + 1); vertex n stands for the end of the last row.
+constexpr int kTileThreads = 256;
+constexpr int kTileItems = 8;
+constexpr int kTile = kTileThreads * kTileItems;
+
+// Row-wise checks of a CSR graph (offsets, vertex weights) and the tiles'
+// first vertices. bad[0] is set where a row is malformed; tile_first is
+// complete only where it is not. empties (nullable): set if any row is empty.
+__global__ void k_rows(const int64_t *xadj, const int64_t *vw, int64_t n, int64_t m2,
+                       int32_t *tile_first, int32_t *bad, int32_t *empties) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u <= n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = xadj[u], pb = u ? xadj[u - 1] : -1;
+    const bool ok = b >= 0 && b <= m2 && b >= pb && (u != 0 || b == 0) && (u != n || b == m2) &&
+                    (u == n || !vw || vw[u] > 0);
+    if (!ok) {
+      atomicCAS(bad, 0, 1);
+      continue;
+    }
+    if (empties && b == pb) *empties = 1;  // (every writer writes the same)
+    // tiles t with pb < t * kTile <= b (for u = 0 that is tile 0)
+    for (int64_t t = pb < 0 ? 0 : pb / kTile + 1; t * kTile <= b; ++t) tile_first[t] = (int32_t)u;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) tile_first[m2 / kTile + 1] = (int32_t)(n + 1);
+}
+
+__device__ __forceinline__ int tpad(int i) { return i + (i >> 5); }
+
+// Row of every entry of tile t, relative to base = tile_first[t] - 1 (the row
+// that contains the tile's first entry unless a row starts there): the rows
+// that start inside the tile mark their first entry and a block-wide maximum
+// scan carries the marks on (of several rows with one start, the last is the
+// one with entries). row holds kTile + kTile / 32 words, indexed by tpad.
+__device__ __forceinline__ void tile_rows(const int64_t *xadj, const int32_t *tile_first, int64_t t,
+                                          int64_t n, int32_t *row) {
+  __shared__ int32_t wmax[kTileThreads / 32];
+  const int64_t e0 = t * kTile;
+  const int32_t base = tile_first[t] - 1;
+  for (int i = threadIdx.x; i < kTile; i += kTileThreads) row[tpad(i)] = 0;
+  __syncthreads();
+  const int64_t rend = min((int64_t)tile_first[t + 1], n);
+  for (int64_t r = (int64_t)base + 1 + threadIdx.x; r < rend; r += kTileThreads)
+    atomicMax(&row[tpad((int)(xadj[r] - e0))], (int32_t)(r - base));
+  __syncthreads();
+  const int i0 = threadIdx.x * kTileItems;
+  int32_t v[kTileItems], m = 0;
+#pragma unroll
+  for (int j = 0; j < kTileItems; ++j) v[j] = m = max(m, row[tpad(i0 + j)]);
+  int32_t x = m;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane_id() >= o) x = max(x, y);
+  }
+  if (lane_id() == 31) wmax[threadIdx.x >> 5] = x;
+  __syncthreads();
+  int32_t before = __shfl_up_sync(kFull, x, 1);
+  if (lane_id() == 0) before = 0;
+  for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before = max(before, wmax[w]);
+#pragma unroll
+  for (int j = 0; j < kTileItems; ++j) row[tpad(i0 + j)] = max(before, v[j]);
+  __syncthreads();
+}
+
+// Entry-wise checks of a CSR graph whose rows are well-formed: ids in range,
+// no loops, strictly ascending rows, positive weights, and symmetry. A row is
+// a set once it ascends, so symmetry needs one search per edge, not two: every
+// entry (u, v) with v > u must have its mirror in row v, and as many entries
+// lie above the diagonal as below (balance sums to zero), so the mirrors are
+// all of the lower ones. The upper entries of a tile are listed first, so the
+// searches run with full warps, kSearch of them in step per thread: bound by
+// the searches' dependent loads.
+constexpr int kSearch = 4;
+__global__ void __launch_bounds__(kTileThreads) k_validate(GView g, const int32_t *tile_first,
+                                                           int64_t ntiles,
+                                                           const int32_t *bad_rows, int32_t *bad,
+                                                           unsigned long long *balance) {
+  __shared__ int32_t row[kTile + kTile / 32];
+  __shared__ uint16_t upper[kTile];
+  __shared__ int32_t n_upper;
+  if (*bad_rows) return;  // set by k_rows: the rows cannot be followed
+  int64_t diff = 0;  // (thread 0)
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    if (threadIdx.x == 0) n_upper = 0;
+    tile_rows(g.xadj, tile_first, t, g.n, row);  // (with barriers)
+    const int64_t e0 = t * kTile;
+    const int32_t base = tile_first[t] - 1;
+    const int len = (int)min((int64_t)kTile, g.m2 - e0);
+    const int32_t *adj = g.adj + e0;
     int code = 0;
-    if (e < b || b < 0 || e > g.m2) code = 2;
-    if (!code && g.vw && lane == 0 && g.vw[u] <= 0) code = 3;
-    for (int64_t i = b + lane; !code && i < e; i += 32) {
-      int64_t v = g.adj[i];
-      if (v < 0 || v >= g.n) {
-        code = 4;
-        break;
-      }
-      if (v == u) code = 5;
-      else if (i > b && g.adj[i - 1] >= v) code = 6;
-      else if (g.ew && g.ew[i] <= 0) code = 7;
-      else {
-        // u must appear in N(v) with the same weight
-        int64_t lo = g.xadj[v], hi = g.xadj[v + 1];
-        while (lo < hi) {
-          int64_t mid = lo + (hi - lo) / 2;
-          if (g.adj[mid] < u) lo = mid + 1;
-          else hi = mid;
+    int32_t vv[kTileItems], pv[kTileItems];
+#pragma unroll
+    for (int j = 0; j < kTileItems; ++j) {
+      const int i = threadIdx.x + j * kTileThreads;
+      vv[j] = i < len ? adj[i] : 0;
+      pv[j] = i < len && e0 + i > 0 ? adj[i - 1] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < kTileItems; ++j) {
+      const int i = threadIdx.x + j * kTileThreads;
+      bool up = false;
+      if (i < len) {
+        const int32_t r = row[tpad(i)], u = base + r, v = vv[j];
+        if ((uint32_t)v >= (uint32_t)g.n || v == u) {
+          code = 4;
+        } else {
+          const bool inside = i ? row[tpad(i - 1)] == r : g.xadj[u] < e0;
+          if (inside && pv[j] >= v) code = 6;
+          if (g.ew && g.ew[e0 + i] <= 0) code = 7;
+          up = v > u;
         }
-        if (lo >= g.xadj[v + 1] || g.adj[lo] != u) code = 8;
-        else if (g.ew && g.ew[lo] != g.ew[i]) code = 8;
+      }
+      const unsigned m = __ballot_sync(kFull, up);
+      if (m) {
+        int32_t at = 0;
+        if (lane_id() == 0) at = atomicAdd(&n_upper, __popc(m));
+        at = __shfl_sync(kFull, at, 0);
+        if (up) upper[at + __popc(m & lanemask_lt())] = (uint16_t)i;
+      }
+    }
+    __syncthreads();
+    const int nu = n_upper;
+    if (threadIdx.x == 0) diff += 2 * nu - len;
+    for (int q0 = threadIdx.x; q0 < nu; q0 += kSearch * kTileThreads) {
+      int32_t u[kSearch], left[kSearch];
+      const int32_t *p[kSearch];
+      int most = 0;
+#pragma unroll
+      for (int k = 0; k < kSearch; ++k) {
+        const int q = q0 + k * kTileThreads;
+        const int i = q < nu ? upper[q] : -1;
+        u[k] = i >= 0 ? base + row[tpad(i)] : 0;
+        const int32_t v = i >= 0 ? adj[i] : 0;
+        const int64_t b = i >= 0 ? g.xadj[v] : 0;
+        left[k] = i >= 0 ? (int32_t)(g.xadj[v + 1] - b) : -1;
+        p[k] = g.adj + b;
+        most = max(most, left[k]);
+      }
+      // the last entry <= u of each row: halves until one entry is left
+      while (most > 1) {
+#pragma unroll
+        for (int k = 0; k < kSearch; ++k) {
+          const int32_t h = left[k] > 1 ? left[k] >> 1 : 0;
+          if (h && p[k][h] <= u[k]) p[k] += h;
+          left[k] -= h;
+        }
+        most -= most >> 1;
+      }
+#pragma unroll
+      for (int k = 0; k < kSearch; ++k) {
+        if (left[k] < 0) continue;
+        if (left[k] == 0 || *p[k] != u[k]) code = 8;
+        else if (g.ew && g.ew[p[k] - g.adj] != g.ew[e0 + upper[q0 + k * kTileThreads]]) code = 8;
       }
     }
     if (code) atomicCAS(bad, 0, code);
+    __syncthreads();  // row, upper and n_upper are rebuilt by the next tile
   }
+  if (threadIdx.x == 0 && diff) atomicAdd(balance, (unsigned long long)diff);
 }
 
 __global__ void k_zip_degrees(GView g, int64_t *deg) {
@@ -514,118 +652,252 @@ void release_hub_tables(tp_graph *g, cudaStream_t s) {
 namespace {
 
 __device__ __forceinline__ int vlen(uint64_t x) {
-  int l = 1;
-  while (x >= 128) x >>= 7, ++l;
-  return l;
+  const int bits = 64 - __clzll((long long)(x | 1));
+  return (bits + 6) / 7;
+}
+__device__ __forceinline__ int vlen32(uint32_t x) { return (38 - __clz(x | 1)) / 7; }
+
+__device__ __forceinline__ uint32_t first_code(int32_t v, int32_t u) {
+  return v >= u ? 2u * (uint32_t)(v - u) : 2u * (uint32_t)(u - v) + 1u;
 }
 
-__device__ __forceinline__ uint64_t first_code(int64_t v0, int64_t u) {
-  return v0 >= u ? 2ull * (uint64_t)(v0 - u) : 2ull * (uint64_t)(u - v0) + 1ull;
-}
-
-constexpr int64_t kZipLaneMax = 256;  // thread per vertex up to this degree
-
-// Encoded size of every neighbourhood of degree <= kZipLaneMax, one thread
-// per vertex (the warp kernel below takes the rest).
-__global__ void k_zip_size_lane(GView g, int64_t *size) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = g.xadj[u], d = g.xadj[u + 1] - b;
-    if (d > kZipLaneMax) continue;
-    int64_t acc = vlen((uint64_t)b);
-    int32_t prev = 0;
-    for (int64_t i = 0; i < d; ++i) {
-      const int32_t v = g.adj[b + i];
-      acc += i == 0 ? vlen(first_code(v, u)) : vlen((uint64_t)(v - prev));
-      prev = v;
-    }
-    size[u] = acc;
+// Stores the n-byte VarInt of x (n = vlen32(x)) at p.
+__device__ __forceinline__ void put_varint(uint8_t *p, uint32_t x, int n) {
+  p[0] = (uint8_t)(n > 1 ? x | 0x80u : x);
+  if (n > 1) p[1] = (uint8_t)(n > 2 ? x >> 7 | 0x80u : x >> 7);
+  if (n > 2) {
+    p[2] = (uint8_t)(n > 3 ? x >> 14 | 0x80u : x >> 14);
+    if (n > 3) p[3] = (uint8_t)(n > 4 ? x >> 21 | 0x80u : x >> 21);
+    if (n > 4) p[4] = (uint8_t)(x >> 28);
   }
 }
+__device__ __forceinline__ void put_varint64(uint8_t *p, uint64_t x) {
+  for (; x >= 128; x >>= 7) *p++ = (uint8_t)(0x80u | (x & 0x7fu));
+  *p = (uint8_t)x;
+}
 
-// Writes every neighbourhood of degree <= kZipLaneMax, one thread per vertex.
-__global__ void k_zip_write_lane(GView g, const int64_t *off, uint8_t *out) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = g.xadj[u], d = g.xadj[u + 1] - b;
-    if (d > kZipLaneMax) continue;
-    uint64_t p = (uint64_t)off[u];
-    auto put = [&](uint64_t x) {
-      while (x >= 128) {
-        out[p++] = (uint8_t)(0x80u | (x & 0x7fu));
-        x >>= 7;
+// Encoding in tiles of adjacency entries. The bytes of a tile are those of its
+// entries and of the headers (and chunk tables) of the rows that start in it,
+// an unbroken piece of the stream, so their number per tile, summed over the
+// tiles, gives every tile its place. A row's first edge id is the number of
+// the entry it starts at, so headers need nothing but the mark of the start:
+// start[i] is the row with entries that starts at entry i of the tile
+// (relative to base, 0: none), empty[i] the number of empty rows just before
+// it, whose headers hold the same number (k_zip_empty writes them). Pass 2
+// puts a tile together in shared memory, eight entries a thread, and writes it
+// in 16-byte pieces. Bound by instruction issue; the adjacency is read twice
+// and the stream written once.
+// Pass 1 (WRITE = false): bytes per tile. Pass 2: bytes, offsets, and the
+// position of every chunk start (cpos[e / kChunkSize]: they lie at least
+// kChunkSize apart). HUBS: some rows are chunked.
+// First row of [0, hi] that starts at entry b (row hi does).
+__device__ __forceinline__ int64_t first_row_at(const int64_t *xadj, int64_t hi, int64_t b) {
+  int64_t lo = 0;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) / 2;
+    if (xadj[mid] < b) lo = mid + 1;
+    else hi = mid;
+  }
+  return hi;
+}
+
+constexpr int kZipStage = 12 * 1024;
+template <bool WRITE, bool HUBS>
+__global__ void __launch_bounds__(kTileThreads)
+    k_zip_tiles(GView g, const int32_t *tile_first, int64_t ntiles, int64_t *tsize, uint8_t *out,
+                uint32_t *o32, uint64_t *o64, int64_t *cpos) {
+  __shared__ int32_t start[kTile + kTile / 32], empty[kTile];
+  __shared__ int32_t val[kTile + kTile / 32];
+  __shared__ int64_t wsum[kTileThreads / 32];
+  __shared__ int32_t wrow[kTileThreads / 32];
+  __shared__ int32_t s_empties;
+  __shared__ __align__(16) uint8_t stage[WRITE ? kZipStage : 16];
+  const int lane = lane_id(), w = threadIdx.x >> 5;
+  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int64_t e0 = t * kTile;
+    const int len = (int)min((int64_t)kTile, g.m2 - e0);
+    for (int i = threadIdx.x; i < kTile; i += kTileThreads) {
+      if (i < len) val[tpad(i)] = g.adj[e0 + i];
+      start[tpad(i)] = 0;
+    }
+    if (threadIdx.x == 0) s_empties = 0;
+    __syncthreads();
+    const int32_t base = tile_first[t] - 1;
+    const int64_t rend = min((int64_t)tile_first[t + 1], g.n);
+    for (int64_t r = (int64_t)base + 1 + threadIdx.x; r < rend; r += kTileThreads) {
+      const int64_t b = g.xadj[r];
+      if (g.xadj[r + 1] == b) continue;
+      const int i = (int)(b - e0);
+      start[tpad(i)] = (int32_t)(r - base);
+      const bool after = r > 0 && g.xadj[r - 1] == b;
+      empty[i] = after ? (int32_t)(r - first_row_at(g.xadj, r, b)) : 0;
+      if (after) s_empties = 1;
+    }
+    __syncthreads();
+    const bool empties = s_empties != 0;
+    // codes of eight consecutive entries, and the bytes before each
+    const int i0 = threadIdx.x * kTileItems;
+    uint32_t code[kTileItems];
+    int64_t bytes = 0;
+    int32_t chunks = 0;  // HUBS: bit j: entry j begins a later chunk of its row
+    int32_t prev = i0 && i0 < len ? val[tpad(i0 - 1)] : (i0 == 0 && e0 ? g.adj[e0 - 1] : 0);
+    int32_t u = base;  // HUBS: row of the current entry
+    int64_t ub = 0, ud = 0;
+    if constexpr (HUBS) {  // the last row that starts before this thread's entries
+      int32_t m = 0;
+#pragma unroll
+      for (int j = 0; j < kTileItems; ++j) m = max(m, start[tpad(i0 + j)]);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, m, o);
+        if (lane >= o) m = max(m, y);
       }
-      out[p++] = (uint8_t)x;
+      if (lane == 31) wrow[w] = m;
+      __syncthreads();
+      m = __shfl_up_sync(kFull, m, 1);
+      if (lane == 0) m = 0;
+      for (int q = 0; q < w; ++q) m = max(m, wrow[q]);
+      u = base + m;
+      if (i0 < len && u >= 0) ub = g.xadj[u], ud = g.xadj[u + 1] - ub;
+    }
+#pragma unroll
+    for (int j = 0; j < kTileItems; ++j) {
+      const int i = i0 + j;
+      code[j] = 0;
+      if (i >= len) continue;
+      const int32_t v = val[tpad(i)], st = start[tpad(i)];
+      bool first = st != 0;
+      if (first) bytes += (int64_t)(1 + (empties ? empty[i] : 0)) * vlen((uint64_t)(e0 + i));
+      if constexpr (HUBS) {
+        if (first) u = base + st, ub = e0 + i, ud = g.xadj[u + 1] - ub;
+        if (ud > kChunkThreshold) {
+          const int64_t rel = e0 + i - ub;
+          if (rel == 0) bytes += 4 * ((ud + kChunkSize - 1) / kChunkSize - 1);
+          else if (rel % kChunkSize == 0) first = true, chunks |= 1 << j;
+        }
+        code[j] = first ? first_code(v, u) : (uint32_t)(v - prev);
+      } else {
+        code[j] = first ? first_code(v, base + st) : (uint32_t)(v - prev);
+      }
+      prev = v;
+      bytes += vlen32(code[j]);
+    }
+    const int64_t incl = warp_incl_scan(bytes);
+    if (lane == 31) wsum[w] = incl;
+    __syncthreads();
+    int64_t before = 0, total = 0;
+    for (int q = 0; q < kTileThreads / 32; ++q) {
+      before += q < w ? wsum[q] : 0;
+      total += wsum[q];
+    }
+    if (!WRITE) {
+      if (threadIdx.x == 0) {
+        // the last tile also holds the headers of the empty rows at the end
+        const int64_t tail = t == ntiles - 1 ? g.n - first_row_at(g.xadj, g.n, g.m2) : 0;
+        tsize[t] = total + tail * vlen((uint64_t)g.m2);
+      }
+      __syncthreads();
+      continue;
+    }
+    const int64_t begin = tsize[t];
+    const int shift = (int)(begin & 15);
+    const bool staged = total + shift <= kZipStage;
+    auto write = [&](uint8_t *buf) {  // buf: where the tile's first byte goes
+      int64_t at = before + incl - bytes;
+#pragma unroll
+      for (int j = 0; j < kTileItems; ++j) {
+        const int i = i0 + j;
+        if (i >= len) continue;
+        const int64_t e = e0 + i;
+        const int32_t st = start[tpad(i)];
+        if (st) {  // room for the empty rows' headers, then the row's own
+          const int hl = vlen((uint64_t)e);
+          if (empties) at += (int64_t)empty[i] * hl;
+          if (o32) o32[base + st] = (uint32_t)(begin + at);
+          else o64[base + st] = (uint64_t)(begin + at);
+          put_varint64(buf + at, (uint64_t)e);
+          at += hl;
+          if constexpr (HUBS) {  // and for the chunk table (k_zip_tables)
+            const int64_t d = g.xadj[base + st + 1] - e;
+            if (d > kChunkThreshold) at += 4 * ((d + kChunkSize - 1) / kChunkSize - 1);
+          }
+        }
+        const int n = vlen32(code[j]);
+        if (HUBS && (chunks >> j & 1)) cpos[e / kChunkSize] = begin + at;
+        put_varint(buf + at, code[j], n);
+        at += n;
+      }
     };
-    put((uint64_t)b);
-    int32_t prev = 0;
-    for (int64_t i = 0; i < d; ++i) {
-      const int32_t v = g.adj[b + i];
-      put(i == 0 ? first_code(v, u) : (uint64_t)(v - prev));
-      prev = v;
-    }
-  }
-}
-
-// Encoded size of every neighbourhood above kZipLaneMax (warp per vertex).
-__global__ void k_zip_size(GView g, int64_t *size) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int lane = lane_id();
-  for (int64_t u = warp; u < g.n; u += nw) {
-    int64_t b = g.xadj[u], d = g.xadj[u + 1] - b;
-    if (d <= kZipLaneMax) continue;
-    int64_t nch = d > kChunkThreshold ? (d + kChunkSize - 1) / kChunkSize : 1;
-    int64_t csz = nch > 1 ? kChunkSize : d;
-    int64_t acc = 0;
-    for (int64_t i = lane; i < d; i += 32) {
-      int64_t v = g.adj[b + i];
-      acc += (i % csz == 0) ? vlen(first_code(v, u)) : vlen((uint64_t)(v - g.adj[b + i - 1]));
-    }
-    acc = warp_sum(acc);
-    if (lane == 0) size[u] = acc + vlen((uint64_t)b) + (d ? 4 * (nch - 1) : 0);
-  }
-}
-
-// Writes every neighbourhood above kZipLaneMax at its offset (warp per vertex).
-__global__ void k_zip_write(GView g, const int64_t *off, uint8_t *out) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int lane = lane_id();
-  for (int64_t u = warp; u < g.n; u += nw) {
-    int64_t b = g.xadj[u], d = g.xadj[u + 1] - b;
-    if (d <= kZipLaneMax) continue;
-    uint64_t pos = (uint64_t)off[u];
-    int hl = vlen((uint64_t)b);
-    if (lane == 0) {
-      uint64_t x = (uint64_t)b;
-      for (int i = 0; i < hl; ++i, x >>= 7) out[pos + i] = (uint8_t)((x & 0x7f) | (i + 1 < hl ? 0x80 : 0));
-    }
-    if (d == 0) continue;
-    int64_t nch = d > kChunkThreshold ? (d + kChunkSize - 1) / kChunkSize : 1;
-    int64_t csz = nch > 1 ? kChunkSize : d;
-    uint64_t p = pos + hl + 4 * (nch - 1);
-    for (int64_t i0 = 0; i0 < d; i0 += 32) {
-      int64_t i = i0 + lane;
-      uint64_t x = 0;
-      int len = 0;
-      if (i < d) {
-        int64_t v = g.adj[b + i];
-        x = (i % csz == 0) ? first_code(v, u) : (uint64_t)(v - g.adj[b + i - 1]);
-        len = vlen(x);
-      }
-      int incl = warp_incl_scan(len);
-      uint64_t at = p + (uint64_t)(incl - len);
-      if (i < d) {
-        for (int q = 0; q < len; ++q, x >>= 7)
-          out[at + q] = (uint8_t)((x & 0x7f) | (q + 1 < len ? 0x80 : 0));
-        if (i % csz == 0 && i > 0) {
-          uint32_t rel = (uint32_t)(at - pos);
-          uint64_t t = pos + hl + 4 * (i / csz - 1);
-          for (int q = 0; q < 4; ++q) out[t + q] = (uint8_t)(rel >> (8 * q));
+    if (staged) write(stage + shift);
+    else write(out + begin);
+    __syncthreads();
+    if (staged) {  // whole 16-byte pieces, the ragged ends byte by byte
+      uint8_t *dst = out + (begin - shift);
+      const uint8_t *src = stage;
+      const int n = (int)total + shift;
+      for (int p = 16 * threadIdx.x; p < n; p += 16 * kTileThreads) {
+        if (p >= shift && p + 16 <= n) {
+          *reinterpret_cast<uint4 *>(dst + p) = *reinterpret_cast<const uint4 *>(src + p);
+        } else {
+          for (int q = max(p, shift); q < min(p + 16, n); ++q) dst[q] = src[q];
         }
       }
-      p += (uint64_t)__shfl_sync(kFull, incl, 31);
+    }
+    __syncthreads();
+  }
+}
+
+// Headers and offsets of the empty rows, and the offset of the end (row n). An
+// empty row's header lies (w - u) headers before that of the next row w with
+// entries, or before the end of the stream, and holds the same number.
+__global__ void k_zip_empty(const int64_t *xadj, int64_t n, int64_t body, bool empties,
+                            uint8_t *out, uint32_t *o32, uint64_t *o64) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (o32) o32[n] = (uint32_t)body;
+    else o64[n] = (uint64_t)body;
+  }
+  if (!empties) return;
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t b = xadj[u];
+    if (xadj[u + 1] != b) continue;
+    int64_t lo = u + 1, hi = n;  // the last row that starts at entry b
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) / 2;
+      if (xadj[mid] > b) hi = mid - 1;
+      else lo = mid;
+    }
+    const int hl = vlen((uint64_t)b);
+    const int64_t end = lo == n ? body : (o32 ? (int64_t)o32[lo] : (int64_t)o64[lo]);
+    const int64_t off = end - (lo - u) * hl;
+    if (o32) o32[u] = (uint32_t)off;
+    else o64[u] = (uint64_t)off;
+    uint64_t x = (uint64_t)b;
+    for (int i = 0; i < hl; ++i, x >>= 7)
+      out[off + i] = (uint8_t)((x & 0x7f) | (i + 1 < hl ? 0x80 : 0));
+  }
+}
+
+// Chunk tables of the rows above kChunkThreshold: a warp per 32 rows, all of
+// it on each chunked one.
+__global__ void k_zip_tables(const int64_t *xadj, int64_t n, const uint32_t *o32,
+                             const uint64_t *o64, const int64_t *cpos, uint8_t *out) {
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int lane = lane_id();
+  for (int64_t base = gw * 32; base < n; base += nw * 32) {
+    const int64_t u = base + lane;
+    unsigned hubs = __ballot_sync(kFull, u < n && xadj[u + 1] - xadj[u] > kChunkThreshold);
+    while (hubs) {
+      const int64_t h = base + __ffs(hubs) - 1;
+      hubs &= hubs - 1;
+      const int64_t b = xadj[h], nch = (xadj[h + 1] - b + kChunkSize - 1) / kChunkSize;
+      const int64_t off = o32 ? (int64_t)o32[h] : (int64_t)o64[h];
+      for (int64_t k = 1 + lane; k < nch; k += 32) {
+        const uint32_t rel = (uint32_t)(cpos[(b + k * kChunkSize) / kChunkSize] - off);
+        uint8_t *t = out + off + vlen((uint64_t)b) + 4 * (k - 1);
+        for (int q = 0; q < 4; ++q) t[q] = (uint8_t)(rel >> (8 * q));
+      }
     }
   }
 }
@@ -636,52 +908,164 @@ __global__ void k_zip_terminal(uint64_t pos, int64_t m2, uint8_t *out) {
   for (int i = 0; i < l; ++i, x >>= 7) out[pos + i] = (uint8_t)((x & 0x7f) | (i + 1 < l ? 0x80 : 0));
 }
 
-__global__ void k_off_narrow(const int64_t *off, int64_t cnt, uint32_t *o32) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
-       i += (int64_t)gridDim.x * blockDim.x)
-    o32[i] = (uint32_t)off[i];
-}
-
 __global__ void k_off_narrow_u64(const uint64_t *off, int64_t cnt, uint32_t *o32) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
        i += (int64_t)gridDim.x * blockDim.x)
     o32[i] = (uint32_t)off[i];
 }
 
-__global__ void k_off_copy(const int64_t *off, int64_t cnt, uint64_t *o64) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
-       i += (int64_t)gridDim.x * blockDim.x)
-    o64[i] = (uint64_t)off[i];
-}
-
-// Decode every neighbourhood into CSR (round trip), warp per vertex.
-__global__ void k_unzip(GView g, const int64_t *xadj, int32_t *adj) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t u = warp; u < g.n; u += nw) {
-    const int64_t pos = xadj[u];
-    const int64_t deg = xadj[u + 1] - pos;
-    int64_t seen = 0;
-    warp_neighbours<true>(g, u, -1, [&](bool has, int32_t v, int64_t, int64_t idx) {
-      if (has && idx < deg) adj[pos + idx] = v;
-      seen += __popc(__ballot_sync(kFull, has));
-    });
-    if (lane_id() == 0 && seen != deg) latch_error(g.err, TP_ERR_CORRUPT);
+// First edge ids of all rows: the headers (entry n: the terminal header).
+__global__ void k_zip_first(GView g, int64_t *xadj) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u <= g.n;
+       u += (int64_t)gridDim.x * blockDim.x) {
+    uint64_t a;
+    read_varint(g.bytes + off_at(g, u), a);
+    xadj[u] = (int64_t)a;
   }
 }
 
-__global__ void k_zip_header_check(GView g, int32_t *bad) {
+__global__ void k_zip_header_check(GView g, const int64_t *xadj, int32_t *bad) {
   for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t a, b;
-    if (off_at(g, u + 1) < off_at(g, u)) {
+       u += (int64_t)gridDim.x * blockDim.x)
+    if (off_at(g, u + 1) < off_at(g, u) || (uint64_t)xadj[u + 1] < (uint64_t)xadj[u] ||
+        (u == 0 && xadj[0] != 0))
       atomicCAS(bad, 0, 1);
+}
+
+// Decoding into CSR. A warp takes 32 consecutive records; every lane decodes
+// its own, a word of the stream at a time, into a piece of shared memory where
+// the warp's neighbours lie as they will in the adjacency, and the warp copies
+// the piece out coalesced. (A warp per record used 30 of the 128 bytes of its
+// window and left most lanes idle: 3.15 ms for a mesh of 3 M vertices, where
+// this takes 0.15.) Records of more than kUnzipLane neighbours are listed, a
+// chunk per item, for k_unzip_items. Every rule of the format is checked:
+// VarInts of at most five bytes, gaps of at least one, ids inside the graph,
+// the record's bytes used up exactly.
+constexpr int kUnzipLane = 128;    // most neighbours of a lane's record
+constexpr int kUnzipWarps = 8;
+constexpr int kUnzipPiece = 1024;  // neighbours of a warp's piece
+
+__global__ void __launch_bounds__(32 * kUnzipWarps)
+    k_unzip_lane(GView g, const int64_t *xadj, int32_t *adj, uint64_t *items,
+                 unsigned long long *n_items) {
+  __shared__ int32_t piece_all[kUnzipWarps][kUnzipPiece];
+  int32_t *piece = piece_all[threadIdx.x >> 5];
+  const int lane = lane_id();
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t base = gw * 32; base < g.n; base += nw * 32) {
+    const int64_t u = base + lane;
+    const bool in = u < g.n;
+    const int64_t pos = in ? xadj[u] : 0;
+    const int64_t deg = in ? xadj[u + 1] - pos : 0;
+    const bool mine = deg > 0 && deg <= kUnzipLane;
+    if (deg > kUnzipLane) {
+      const int64_t nch = deg > kChunkThreshold ? (deg + kChunkSize - 1) / kChunkSize : 1;
+      const unsigned long long at = atomicAdd(n_items, (unsigned long long)nch);
+      for (int64_t j = 0; j < nch; ++j) items[at + j] = (uint64_t)u << 32 | (uint64_t)j;
+    }
+    // the lanes' neighbours side by side in the piece; a warp whose records
+    // do not fit writes straight to the adjacency
+    const int32_t cnt = mine ? (int32_t)deg : 0;
+    const int32_t incl = warp_incl_scan(cnt);
+    const int32_t total = __shfl_sync(kFull, incl, 31);
+    const bool staged = total <= kUnzipPiece;
+    bool bad = false;
+    if (mine) {
+      int32_t *dst = staged ? piece + (incl - cnt) : adj + pos;
+      const uint64_t b = off_at(g, u), e = off_at(g, u + 1);
+      uint64_t skip;
+      const int hl = read_varint(g.bytes + b, skip);
+      int64_t left = (int64_t)(e - b) - hl;  // bytes of the codes
+      const uint64_t p = b + (uint64_t)hl;
+      const uint32_t *wp = reinterpret_cast<const uint32_t *>(g.bytes + (p & ~(uint64_t)3));
+      uint32_t word = 0;
+      int have = 0;     // bytes of word not yet taken
+      bad = left < 0;   // the header runs over the record's end
+      if (left > 0) {
+        word = __ldg(wp) >> (8 * (p & 3));
+        have = 4 - (int)(p & 3);
+      }
+      int64_t id = u;
+      int32_t k = 0;
+      while (k < cnt && !bad) {
+        uint32_t v = 0;
+        int n = 0;
+        for (;;) {  // one VarInt
+          if (left == 0 || n == 5) {
+            bad = true;
+            break;
+          }
+          if (have == 0) word = __ldg(++wp), have = 4;
+          const uint32_t by = word & 255u;
+          word >>= 8;
+          --have, --left;
+          v |= (by & 0x7fu) << (7 * n++);
+          if (!(by & 0x80u)) break;
+        }
+        if (k == 0) id = (v & 1u) ? id - (int64_t)(v >> 1) : id + (int64_t)(v >> 1);
+        else id += v, bad |= v == 0;
+        bad |= id < 0 || id >= g.n;
+        dst[k++] = (int32_t)id;
+      }
+      bad |= left != 0;
+    }
+    if (__any_sync(kFull, bad) && lane == 0) latch_error(g.err, TP_ERR_CORRUPT);
+    __syncwarp();
+    if (staged) {
+      // rows of the piece are contiguous in the adjacency except across the
+      // listed ones, so each entry finds its row by its lane's range
+      const int64_t shift = pos - (incl - cnt);  // adjacency position minus piece position
+      const unsigned gaps = __ballot_sync(kFull, deg > kUnzipLane);
+      if (!gaps) {
+        const int64_t s0 = __shfl_sync(kFull, shift, 0);
+        for (int i = lane; i < total; i += 32) adj[s0 + i] = piece[i];
+      } else {
+        for (int l = 0; l < 32; ++l) {
+          const int32_t c = __shfl_sync(kFull, cnt, l), x = __shfl_sync(kFull, incl, l) - c;
+          const int64_t sl = __shfl_sync(kFull, shift, l);
+          for (int i = x + lane; i < x + c; i += 32) adj[sl + i] = piece[i];
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// The listed records, a warp per chunk.
+__global__ void k_unzip_items(GView g, const int64_t *xadj, int32_t *adj, const uint64_t *items,
+                              const unsigned long long *n_items) {
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t n = (int64_t)*n_items;
+  for (int64_t k = gw; k < n; k += nw) {
+    const int64_t u = (int64_t)(items[k] >> 32), j = (int64_t)(items[k] & 0xffffffffu);
+    const ZipNbr z = zip_nbr(g, u);
+    uint64_t cb = 0, ce = 0;
+    int64_t cnt = 0;
+    bool ok = z.data <= z.end;  // the chunk table lies inside the record
+    if (ok) {
+      zip_chunk(g, z, j, cb, ce, cnt);
+      ok = cb >= z.data && cb <= ce && ce <= z.end && (j > 0 || cb == z.data) &&
+           (j + 1 < z.nchunks || ce == z.end);
+    }
+    if (!ok) {
+      if (lane_id() == 0) latch_error(g.err, TP_ERR_CORRUPT);
       continue;
     }
-    read_varint(g.bytes + off_at(g, u), a);
-    read_varint(g.bytes + off_at(g, u + 1), b);
-    if (b < a || (u == 0 && a != 0)) atomicCAS(bad, 0, 1);
+    const int64_t at = xadj[u] + j * kChunkSize;
+    warp_decode_chunk(g, u, cb, ce, cnt, [&](bool has, int32_t v, int64_t i) {
+      if (has && i < cnt) adj[at + i] = v;
+    });
   }
+}
+
+// Offsets inside the stream and in order; then the entries from the terminal
+// header (-1 where the offsets are bad).
+__global__ void k_off_check(const uint64_t *off, int64_t n, uint64_t nbytes, int32_t *bad) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u <= n;
+       u += (int64_t)gridDim.x * blockDim.x)
+    if (off[u] >= nbytes || (u && off[u] < off[u - 1])) atomicCAS(bad, 0, 1);
 }
 
 __global__ void k_widen(const uint32_t *a, uint64_t *b, int64_t n) {
@@ -698,21 +1082,43 @@ __global__ void k_ones(int64_t *p, int64_t n) {
 
 }  // namespace
 
-static void finish_graph_stats(tp_graph *g, cudaStream_t s) {
-  Buf<int64_t> acc(2, s);
-  TP_CUDA(cudaMemsetAsync(acc.get(), 0, 2 * sizeof(int64_t), s));
-  if (g->n) {
-    launch(k_sum_max, grid_for(g->n, 256), 256, 0, s, g->unit_vw ? nullptr : g->vw.get(),
-                                                    g->compressed ? nullptr : g->xadj.get(), g->n,
-                                                    acc.get());
-    TP_LAUNCH_CHECK();
-  }
-  int64_t h[2];
-  TP_CUDA(cudaMemcpyAsync(h, acc.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
-  TP_CUDA(cudaStreamSynchronize(s));
+// Total vertex weight, largest degree and largest edge weight. acc holds two
+// zeroed words.
+static void launch_stats(const tp_graph *g, int64_t *acc, cudaStream_t s) {
+  if (!g->n) return;
+  launch(k_sum_max, grid_for(g->n, 256, (int64_t)num_sms() * 4), 256, 0, s,
+         g->unit_vw ? nullptr : g->vw.get(), g->compressed ? nullptr : g->xadj.get(), g->n, acc);
+  TP_LAUNCH_CHECK();
+}
+
+static void set_stats(tp_graph *g, const int64_t *h, cudaStream_t s) {
   g->total_vw = h[0];
   if (!g->compressed) g->max_deg = h[1];
   g->max_ew = g->unit_ew ? 1 : max_i64(g->ew.get(), g->m2, s);
+}
+
+// Validates CSR arrays on the device and fills the graph's statistics.
+// Returns whether they make a valid graph. Synchronises.
+static bool validate_csr(tp_graph *g, cudaStream_t s) {
+  const int64_t ntiles = g->m2 / kTile + 1;
+  Buf<int32_t> tile_first(ntiles + 1, s);
+  // [0] weight [1] degree [2] upper minus lower entries [3] bad rows, bad entries (32 bits each)
+  Buf<int64_t> acc(4, s);
+  TP_CUDA(cudaMemsetAsync(acc.get(), 0, 4 * sizeof(int64_t), s));
+  int32_t *bad = reinterpret_cast<int32_t *>(acc.get() + 3);
+  launch(k_rows, grid_for(g->n + 1, 256), 256, 0, s, g->xadj.get(), g->unit_vw ? nullptr : g->vw.get(),
+         g->n, g->m2, tile_first.get(), bad, nullptr);
+  if (g->m2)
+    launch(k_validate, grid_for(ntiles, 1, (int64_t)num_sms() * 16), kTileThreads, 0, s, view(g),
+           tile_first.get(), ntiles, bad, bad + 1, (unsigned long long *)(acc.get() + 2));
+  TP_LAUNCH_CHECK();
+  launch_stats(g, acc.get(), s);
+  int64_t h[4];
+  TP_CUDA(cudaMemcpyAsync(h, acc.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
+  TP_CUDA(cudaStreamSynchronize(s));
+  if (h[2] != 0 || h[3] != 0) return false;
+  set_stats(g, h, s);
+  return true;
 }
 
 // Offsets are u32 while the byte stream is below 4 GiB, else u64. Setting
@@ -736,35 +1142,41 @@ tp_graph *compress(const tp_graph *c, cudaStream_t s) {
     TP_CUDA(cudaMemsetAsync(z->err.get(), 0, sizeof(int32_t), s));
     GView v = view(c);
     int64_t n = c->n;
-    Buf<int64_t> off(n + 1, s);
-    if (n) {
-      launch(k_zip_size_lane, grid_for(n, 256), 256, 0, s, v, off.get());
-      if (c->max_deg > kZipLaneMax || c->max_deg == 0) launch(k_zip_size, grid_for(n * 32, 256), 256, 0, s, v, off.get());
-      TP_LAUNCH_CHECK();
-    }
-    exclusive_scan_i64(off.get(), off.get(), n, s);
-    int64_t body = read_scalar(off.get() + n, s);
+    const int64_t ntiles = c->m2 / kTile + 1;
+    Buf<int32_t> tile_first(ntiles + 1, s), flags(2, s);  // [0] (unused) [1] empty rows
+    TP_CUDA(cudaMemsetAsync(flags.get(), 0, 2 * sizeof(int32_t), s));
+    Buf<int64_t> tsize(ntiles + 1, s), cpos;
+    const bool hubs = c->max_deg > kChunkThreshold;
+    if (hubs) cpos.alloc(c->m2 / kChunkSize + 1, s);
+    launch(k_rows, grid_for(n + 1, 256), 256, 0, s, c->xadj.get(), nullptr, n, c->m2,
+           tile_first.get(), flags.get(), flags.get() + 1);
+    const unsigned tb = grid_for(ntiles, 1, (int64_t)num_sms() * 16);
+    launch(hubs ? k_zip_tiles<false, true> : k_zip_tiles<false, false>, tb, kTileThreads, 0, s, v,
+           tile_first.get(), ntiles, tsize.get(), nullptr, nullptr, nullptr, nullptr);
+    TP_LAUNCH_CHECK();
+    exclusive_scan_i64(tsize.get(), tsize.get(), ntiles, s);
+    int64_t body = 0;
+    int32_t empties = 0;
+    TP_CUDA(cudaMemcpyAsync(&empties, flags.get() + 1, 4, cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaMemcpyAsync(&body, tsize.get() + ntiles, 8, cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
     int tl = 1;
     for (uint64_t x = (uint64_t)c->m2; x >= 128; x >>= 7) ++tl;
     z->nbytes = (uint64_t)body + tl;
     z->bytes.alloc(z->nbytes + kBytePad, s);
-    TP_CUDA(cudaMemsetAsync(z->bytes.get(), 0, z->nbytes + kBytePad, s));
-    if (n) {
-      launch(k_zip_write_lane, grid_for(n, 256), 256, 0, s, v, off.get(), z->bytes.get());
-      if (c->max_deg > kZipLaneMax || c->max_deg == 0)
-        launch(k_zip_write, grid_for(n * 32, 256), 256, 0, s, v, off.get(), z->bytes.get());
-      TP_LAUNCH_CHECK();
-    }
-    launch(k_zip_terminal, 1, 1, 0, s, (uint64_t)body, c->m2, z->bytes.get());
-    TP_LAUNCH_CHECK();
+    TP_CUDA(cudaMemsetAsync(z->bytes.get() + z->nbytes, 0, kBytePad, s));
     z->off_is64 = wide_offsets(z->nbytes);
-    if (z->off_is64) {
-      z->off64.alloc(n + 1, s);
-      launch(k_off_copy, grid_for(n + 1, 256), 256, 0, s, off.get(), n + 1, z->off64.get());
-    } else {
-      z->off32.alloc(n + 1, s);
-      launch(k_off_narrow, grid_for(n + 1, 256), 256, 0, s, off.get(), n + 1, z->off32.get());
-    }
+    if (z->off_is64) z->off64.alloc(n + 1, s);
+    else z->off32.alloc(n + 1, s);
+    launch(hubs ? k_zip_tiles<true, true> : k_zip_tiles<true, false>, tb, kTileThreads, 0, s, v,
+           tile_first.get(), ntiles, tsize.get(), z->bytes.get(), z->off32.get(), z->off64.get(),
+           cpos.get());
+    launch(k_zip_empty, empties ? grid_for(n, 256) : 1, 256, 0, s, c->xadj.get(), n, body,
+           empties != 0, z->bytes.get(), z->off32.get(), z->off64.get());
+    if (hubs)
+      launch(k_zip_tables, grid_for(n, 256), 256, 0, s, c->xadj.get(), n, z->off32.get(),
+             z->off64.get(), cpos.get(), z->bytes.get());
+    launch(k_zip_terminal, 1, 1, 0, s, (uint64_t)body, c->m2, z->bytes.get());
     TP_LAUNCH_CHECK();
     z->total_vw = c->total_vw;
     TP_CUDA(cudaStreamSynchronize(s));
@@ -787,28 +1199,46 @@ tp_graph *decompress(const tp_graph *z, cudaStream_t s) {
     int64_t n = z->n;
     Buf<int32_t> bad(1, s);
     TP_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(int32_t), s));
-    if (n) {
-      launch(k_zip_header_check, grid_for(n, 256), 256, 0, s, v, bad.get());
-      TP_LAUNCH_CHECK();
-    }
-    TP_REQUIRE(read_scalar(bad.get(), s) == 0, TP_ERR_CORRUPT);
     c->xadj.alloc(n + 1, s);
-    compute_degrees(z, c->xadj.get(), s);
-    exclusive_scan_i64(c->xadj.get(), c->xadj.get(), n, s);
-    int64_t m2 = read_scalar(c->xadj.get() + n, s);
-    TP_REQUIRE(m2 == z->m2, TP_ERR_CORRUPT);
+    launch(k_zip_first, grid_for(n + 1, 256), 256, 0, s, v, c->xadj.get());
+    if (n) launch(k_zip_header_check, grid_for(n, 256), 256, 0, s, v, c->xadj.get(), bad.get());
+    TP_LAUNCH_CHECK();
+    int32_t hbad = 0;
+    int64_t m2 = 0;
+    TP_CUDA(cudaMemcpyAsync(&hbad, bad.get(), sizeof(hbad), cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaMemcpyAsync(&m2, c->xadj.get() + n, 8, cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
+    // (without vertices nothing else looks at the terminal header)
+    TP_REQUIRE(hbad == 0 && (n == 0 ? z->m2 == 0 : m2 == z->m2), TP_ERR_CORRUPT);
+    if (n == 0) {
+      m2 = 0;
+      TP_CUDA(cudaMemsetAsync(c->xadj.get(), 0, 8, s));
+    }
     c->adj.alloc(m2 + kAdjPad, s);
     TP_CUDA(cudaMemsetAsync(c->adj.get() + m2, 0, kAdjPad * sizeof(int32_t), s));
+    Buf<int64_t> acc(3, s);  // [0] weight [1] degree [2] listed items
+    TP_CUDA(cudaMemsetAsync(acc.get(), 0, 3 * sizeof(int64_t), s));
+    // items: a chunk each of the rows above kUnzipLane neighbours
+    Buf<uint64_t> items((size_t)(m2 / kUnzipLane + 1), s);
+    unsigned long long *n_items = (unsigned long long *)(acc.get() + 2);
     if (n) {
-      launch(k_unzip, grid_for(n * 32, 256), 256, 0, s, v, c->xadj.get(), c->adj.get());
+      launch(k_unzip_lane, grid_for(n, 32 * kUnzipWarps), 32 * kUnzipWarps, 0, s, v, c->xadj.get(),
+             c->adj.get(), items.get(), n_items);
+      launch(k_unzip_items, grid_for((m2 / kUnzipLane + 1) * 32, 256), 256, 0, s, v, c->xadj.get(),
+             c->adj.get(), items.get(), n_items);
       TP_LAUNCH_CHECK();
     }
-    int32_t e = read_scalar(z->err.get(), s);
+    launch_stats(c, acc.get(), s);
+    int32_t e = 0;
+    int64_t h[2];
+    TP_CUDA(cudaMemcpyAsync(&e, z->err.get(), sizeof(e), cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaMemcpyAsync(h, acc.get(), sizeof(h), cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
     if (e) {
       TP_CUDA(cudaMemsetAsync(z->err.get(), 0, sizeof(int32_t), s));
       throw Error{(tp_status)e};
     }
-    finish_graph_stats(c, s);
+    set_stats(c, h, s);
   } catch (...) {
     delete c;
     throw;
@@ -816,8 +1246,11 @@ tp_graph *decompress(const tp_graph *z, cudaStream_t s) {
   return c;
 }
 
-__global__ void k_terminal_m2(const uint8_t *bytes, const uint64_t *off, int64_t n, int64_t *m2) {
+__global__ void k_terminal_m2(const uint8_t *bytes, const uint64_t *off, int64_t n,
+                              const int32_t *bad, int64_t *m2) {
   uint64_t x;
+  *m2 = -1;
+  if (*bad) return;
   read_varint(bytes + off[n], x);
   *m2 = (int64_t)x;
 }
@@ -834,16 +1267,19 @@ tp_graph *from_compressed(int64_t n, uint64_t nbytes, const uint8_t *bytes, cons
     z->err.alloc(1, s);
     TP_CUDA(cudaMemsetAsync(z->err.get(), 0, sizeof(int32_t), s));
     z->bytes.alloc(nbytes + kBytePad, s);
-    TP_CUDA(cudaMemsetAsync(z->bytes.get(), 0, nbytes + kBytePad, s));
+    TP_CUDA(cudaMemsetAsync(z->bytes.get() + nbytes, 0, kBytePad, s));
     TP_CUDA(cudaMemcpyAsync(z->bytes.get(), bytes, nbytes, kind, s));
     Buf<uint64_t> o(n + 1, s);
     TP_CUDA(cudaMemcpyAsync(o.get(), off, (n + 1) * sizeof(uint64_t), kind, s));
     // offsets must lie inside the stream before anything dereferences them
-    std::vector<uint64_t> ho(n + 1);
-    TP_CUDA(cudaMemcpyAsync(ho.data(), o.get(), (n + 1) * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    TP_CUDA(cudaStreamSynchronize(s));
-    for (int64_t u = 0; u <= n; ++u)
-      TP_REQUIRE(ho[u] < nbytes && (u == 0 || ho[u] >= ho[u - 1]), TP_ERR_CORRUPT);
+    Buf<int64_t> m2(1, s);
+    Buf<int32_t> bad(1, s);
+    TP_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(int32_t), s));
+    launch(k_off_check, grid_for(n + 1, 256), 256, 0, s, o.get(), n, nbytes, bad.get());
+    launch(k_terminal_m2, 1, 1, 0, s, z->bytes.get(), o.get(), n, bad.get(), m2.get());
+    TP_LAUNCH_CHECK();
+    z->m2 = read_scalar(m2.get(), s);
+    TP_REQUIRE(z->m2 >= 0, TP_ERR_CORRUPT);
     z->off_is64 = wide_offsets(nbytes);
     if (z->off_is64) {
       z->off64 = std::move(o);
@@ -852,21 +1288,18 @@ tp_graph *from_compressed(int64_t n, uint64_t nbytes, const uint8_t *bytes, cons
       launch(k_off_narrow_u64, grid_for(n + 1, 256), 256, 0, s, o.get(), n + 1, z->off32.get());
       TP_LAUNCH_CHECK();
     }
-    Buf<int64_t> m2(1, s);
-    launch(k_terminal_m2, 1, 1, 0, s, z->bytes.get(), z->off_is64 ? z->off64.get() : o.get(), n, m2.get());
-    TP_LAUNCH_CHECK();
-    z->m2 = read_scalar(m2.get(), s);
-    TP_REQUIRE(z->m2 >= 0, TP_ERR_CORRUPT);
     tp_graph *c = decompress(z, s);  // throws TP_ERR_CORRUPT on a malformed stream
-    Buf<int32_t> bad(1, s);
-    TP_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(int32_t), s));
-    launch(k_validate, grid_for(std::max<int64_t>(n, 1) * 32, 256), 256, 0, s, view(c), bad.get());
-    TP_LAUNCH_CHECK();
-    int32_t b = read_scalar(bad.get(), s);
     z->total_vw = n;
     z->max_deg = c->max_deg;
+    bool valid = false;
+    try {
+      valid = validate_csr(c, s);
+    } catch (...) {
+      delete c;
+      throw;
+    }
     delete c;
-    TP_REQUIRE(b == 0, TP_ERR_CORRUPT);
+    TP_REQUIRE(valid, TP_ERR_CORRUPT);
   } catch (...) {
     delete z;
     throw;
@@ -902,12 +1335,7 @@ tp_graph *from_csr(int64_t n, const int64_t *xadj, const int32_t *adj, const int
       g->ew.alloc(m2, s);
       if (m2) TP_CUDA(cudaMemcpyAsync(g->ew.get(), ewgt, m2 * sizeof(int64_t), kind, s));
     }
-    Buf<int32_t> bad(1, s);
-    TP_CUDA(cudaMemsetAsync(bad.get(), 0, sizeof(int32_t), s));
-    launch(k_validate, grid_for(std::max<int64_t>(n, 1) * 32, 256), 256, 0, s, view(g), bad.get());
-    TP_LAUNCH_CHECK();
-    TP_REQUIRE(read_scalar(bad.get(), s) == 0, TP_ERR_INVALID);
-    finish_graph_stats(g, s);
+    TP_REQUIRE(validate_csr(g, s), TP_ERR_INVALID);
   } catch (...) {
     delete g;
     throw;
