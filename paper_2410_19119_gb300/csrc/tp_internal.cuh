@@ -454,6 +454,10 @@ void lp_bucket(tp_graph *g, LpWork &w, uint64_t rk, int32_t S, const tp_params &
                const SegLp *seg = nullptr);
 void lp_rounds(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, uint64_t tag, uint64_t a,
                uint64_t b0, int32_t rounds, int32_t S, const tp_params &p, cudaStream_t stream);
+// All rounds of a small level in one launch (lp_small.cu); false: not such a level.
+bool lp_rounds_small(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, uint64_t tag,
+                     uint64_t a, uint64_t b0, int32_t rounds, int32_t S, const tp_params &p,
+                     cudaStream_t stream);
 // ev_begin / ev_end (nullable) are recorded around the LP rounds alone.
 // seg (batched graphs): vb, cap (U of every graph) and gid; lgid and lb are
 // taken equal to gid and vb (labels are vertices).
