@@ -79,8 +79,9 @@ __global__ void k_rate_small(RateCtx c) {
 template <bool W>
 __host__ __device__ constexpr int lane_warps() { return W ? 4 : kLaneWarps; }
 
-// LONG: some compressed records exceed the 80-byte window (skewed graphs);
-// a separate instantiation keeps the common kernel free of that path.
+// LONG: some compressed records exceed the 80-byte window (skewed graphs), or
+// (weighted) labels beyond kLaneKeyLabels; separate instantiations keep the
+// common kernels free of those paths.
 template <bool COMP, int MODE, bool W, bool LONG = false, bool SEG = false>
 __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM)
     k_rate_lane(RateCtx c) {
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
   const int32_t nw = (int32_t)((gridDim.x * blockDim.x) >> 5);
   // bucket mode: this sub-round's lane-tier vertices come as a list
   const bool list_mode = MODE == M_LP && c.bucket != nullptr;
-  int32_t bcount = 0, bnext = gw * kLaneWin;
+  int32_t bcount = 0, bnext = gw * c.lane_win;
   const int32_t *blist = c.bucket;
   const uint64_t *brec = COMP ? c.bucket_rec : nullptr;
   int64_t base = (int64_t)gw * 256;
@@ -120,9 +121,9 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
     if (list_mode) {
       if (bnext >= bcount) break;
       wstart = bnext;
-      take = bcount - bnext < kLaneWin ? bcount - bnext : kLaneWin;
+      take = bcount - bnext < c.lane_win ? bcount - bnext : c.lane_win;
       // never step past the end (keeps bnext below 2^31)
-      bnext = bcount - bnext > nw * kLaneWin ? bnext + nw * kLaneWin : bcount;
+      bnext = bcount - bnext > nw * c.lane_win ? bnext + nw * c.lane_win : bcount;
     } else {
       // fill the queue, 32 vertices of the current 256-vertex slab at a time
       while (pending < kLaneWin && base < c.g.n) {
@@ -163,8 +164,13 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
         }
       }
       const unsigned maxdeg = __reduce_max_sync(kFull, (unsigned)deg);
-      if (maxdeg <= 16) lane_batch<COMP, MODE, W, 16, SEG>(c, has, u, deg, col, wcol, cnt, mb, nmv);
-      else lane_batch<COMP, MODE, W, kLaneMaxDeg, SEG>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+      constexpr bool WIDE = W && LONG;
+      if (W && maxdeg <= 8)  // coarse levels of meshes
+        lane_batch<COMP, MODE, W, 8, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+      else if (maxdeg <= 16)
+        lane_batch<COMP, MODE, W, 16, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+      else
+        lane_batch<COMP, MODE, W, kLaneMaxDeg, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
     }
     __syncwarp();
     if (nmv) {  // the window's movers, coalesced
@@ -974,9 +980,19 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   if (n_lane > 0) {
     if (prof) prof_begin(PF_RATE_LANE, s);
     constexpr int LM = MODE == M_REBAL ? M_LP : MODE;
+    // windows of this launch's list: full where every warp gets one, shorter
+    // ones spread a small list over the warps (a coarse level of 4e4 lane
+    // vertices: four batches in series on 40 warps took 65 us, one each on 156
+    // warps 27). From the host: a value in a register of the compressed kernel
+    // costs it a tenth of its speed.
+    auto lane_window = [&](int64_t warps) {
+      const int64_t list = (n_lane + std::max(c.S, 1) - 1) / std::max(c.S, 1);
+      c.lane_win = (int32_t)std::min<int64_t>(kLaneWin, ((list + warps - 1) / warps + 31) & ~31ll);
+    };
     if (g->unit_ew) {
       unsigned blocks = (unsigned)std::min<int64_t>(
           (g->n + 256 * kLaneWarps - 1) / (256 * kLaneWarps), (int64_t)sms * kLaneBlocksPerSM);
+      lane_window((int64_t)blocks * kLaneWarps);
       // batched graphs are CSR unions
       if (comp && T.lane_long) launch(k_rate_lane<true, LM, false, true>, blocks, 32 * kLaneWarps, 0, s, c);
       else if (comp) launch(k_rate_lane<true, LM, false>, blocks, 32 * kLaneWarps, 0, s, c);
@@ -986,7 +1002,12 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
       constexpr int WW = lane_warps<true>();
       unsigned blocks =
           (unsigned)std::min<int64_t>((g->n + 256 * WW - 1) / (256 * WW), (int64_t)sms * 16);
-      if (c.seg.gid) launch(k_rate_lane<false, LM, true, false, true>, blocks, 32 * WW, 0, s, c);
+      lane_window((int64_t)blocks * WW);
+      // labels are vertices or, in refinement, block numbers
+      const bool wide = g->n > kLaneKeyLabels || c.nlabels > kLaneKeyLabels;
+      if (c.seg.gid && wide) launch(k_rate_lane<false, LM, true, true, true>, blocks, 32 * WW, 0, s, c);
+      else if (c.seg.gid) launch(k_rate_lane<false, LM, true, false, true>, blocks, 32 * WW, 0, s, c);
+      else if (wide) launch(k_rate_lane<false, LM, true, true>, blocks, 32 * WW, 0, s, c);
       else launch(k_rate_lane<false, LM, true>, blocks, 32 * WW, 0, s, c);
     }
     TP_LAUNCH_CHECK();
@@ -1530,6 +1551,7 @@ void lp_subround(tp_graph *g, const LpState &st, LpWork &w, uint64_t rk, int32_t
   c.label = st.label;
   c.lw = st.lw;
   c.cap = st.cap;
+  c.nlabels = st.nlabels;
   c.seg = st.seg;
   c.k = st.k;
   c.kmax = st.kmax;

@@ -25,6 +25,7 @@ struct RateCtx {
   const int32_t *label;
   const int64_t *lw;
   int64_t cap;
+  int64_t nlabels;
   uint64_t rk;
   const uint64_t *rk_dev;  // if set, the round key is read here (replayed round graphs)
   int32_t S, s;
@@ -65,6 +66,7 @@ struct RateCtx {
   const int32_t *bucket;
   const int64_t *bucket_off;
   int64_t bucket_nb;
+  int32_t lane_win;  // vertices of a warp's window (32 .. kLaneWin)
   // per listed vertex: record start << 8 | record length (compressed graphs)
   const uint64_t *bucket_rec;
   // this round's sub-round + 1 of every vertex (null: hash on the fly)
@@ -622,7 +624,13 @@ __device__ __forceinline__ int32_t load_label(const int32_t *p) {
   return LIVE ? *p : __ldg(p);
 }
 
-template <bool COMP, int MODE, bool W, int N, bool SEG, bool LIVE = false, class Movers>
+// Labels below this fit a 32-bit sort key with the slot (weighted lane tier).
+constexpr int64_t kLaneKeyLabels = ((int64_t)1 << 27) - 1;
+
+// WIDE (weighted): labels beyond kLaneKeyLabels, sorted with the weights in
+// 64-bit keys.
+template <bool COMP, int MODE, bool W, int N, bool SEG, bool LIVE = false, bool WIDE = false,
+          class Movers>
 __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u, int deg,
                                            uint32_t *col, uint32_t *wcol, uint8_t *cnt,
                                            Movers &mb, int &nmv) {
@@ -630,23 +638,15 @@ __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u
   int32_t rown = 0, rmax = 0;
   int32_t *ccol = reinterpret_cast<int32_t *>(col);
   if constexpr (W) {  // weighted levels are CSR; candidates listed in the column
-    // label << 32 | weight; padding: label INT32_MAX, weight 0
-    constexpr uint64_t kPad = (uint64_t)INT32_MAX << 32;
     const int64_t b = has ? c.g.xadj[u] : 0;
-    uint64_t a[kLaneMaxDeg];
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      a[i] = i < deg ? ((uint64_t)(uint32_t)load_label<LIVE>(c.label + __ldcs(c.g.adj + b + i)) << 32) |
-                           (uint32_t)__ldcs(c.g.ew + b + i)
-                     : kPad;
-    oem_sort<N>(a);
+    const int32_t *adj = c.g.adj + b;
+    const int64_t *ew = c.g.ew + b;
     int ncand = 0;
     uint32_t run = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const int32_t x = (int32_t)(a[i] >> 32);
-      run += (uint32_t)a[i];
-      const bool end = i + 1 == N || (int32_t)(a[i + 1] >> 32) != x;
+    // one sorted entry: label x (INT32_MAX: padding), its weight, and whether
+    // it is the last of its label
+    auto step = [&](int32_t x, uint32_t wt, bool end) {
+      run += wt;
       const bool real = end && x != INT32_MAX;
       const bool cand = real && x != own;
       ccol[ncand * 32] = x;
@@ -655,6 +655,36 @@ __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u
       rmax = cand ? max(rmax, (int32_t)run) : rmax;
       ncand += cand;
       run = end ? 0u : run;
+    };
+    if constexpr (WIDE) {  // label << 32 | weight; padding: label INT32_MAX, weight 0
+      uint64_t a[kLaneMaxDeg];
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        a[i] = i < deg ? ((uint64_t)(uint32_t)load_label<LIVE>(c.label + __ldcs(adj + i)) << 32) |
+                             (uint32_t)__ldcs(ew + i)
+                       : (uint64_t)INT32_MAX << 32;
+      oem_sort<N>(a);
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        step((int32_t)(a[i] >> 32), (uint32_t)a[i],
+             i + 1 == N || (int32_t)(a[i + 1] >> 32) != (int32_t)(a[i] >> 32));
+    } else {
+      // label << 5 | slot, the weights apart in the lane's column: a comparator
+      // of the sort is two instructions instead of six on 64-bit pairs
+      uint32_t a[kLaneMaxDeg], wt[kLaneMaxDeg];
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        a[i] = i < deg ? (uint32_t)load_label<LIVE>(c.label + __ldcs(adj + i)) << 5 | (uint32_t)i
+                       : 0xffffffffu;
+        wcol[i * 32] = i < deg ? (uint32_t)__ldcs(ew + i) : 0u;
+      }
+      oem_sort<N>(a);
+#pragma unroll
+      for (int i = 0; i < N; ++i) wt[i] = a[i] == 0xffffffffu ? 0u : wcol[(a[i] & 31u) * 32];
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        step(a[i] == 0xffffffffu ? INT32_MAX : (int32_t)(a[i] >> 5), wt[i],
+             i + 1 == N || a[i + 1] >> 5 != a[i] >> 5);
     }
     const int64_t cu = has ? node_w(c.g, u) : 1;
     LaneCand best{-1, 0xffffffffu, INT32_MAX};

@@ -25,6 +25,7 @@ namespace {
 constexpr int kLpSmallWarps = 16;
 constexpr int kLpSmallThreads = 32 * kLpSmallWarps;
 constexpr int kLpSmallCluster = 16;
+constexpr int kLpSmallItems = 4;
 constexpr int64_t kLpSmallVertices = 16384;  // most vertices of a CTA (its bucket list)
 constexpr int64_t kLpSmallEntries = (int64_t)1 << 17;  // most adjacency entries of a CTA's share
 
@@ -198,7 +199,10 @@ __global__ void __launch_bounds__(kLpSmallThreads)
 // graph, no vertex above the mid tier, 32-bit ratings, at most 32 sub-rounds,
 // and so few vertices and entries that 16 CTAs rate an eighth of them in about
 // the time that the kernels of a sub-round take to launch. The smallest
-// cluster that gives every warp at most one batch or vertex per sub-round.
+// cluster that gives a CTA at most kLpSmallItems batches or vertices per
+// sub-round: the lanes of a batch read different rows and labels, and an SM's
+// L1 looks up one line a cycle (a batch of degree 16 takes about 700), so 16
+// batches on one SM cost more than four on each of four and their barriers.
 int lp_small_cluster(const tp_graph *g, const LpState &st, int32_t S) {
   const TierCache &T = g->tiers;
   if (st.seg.gid || S > 32 || T.lane_long ||
@@ -209,7 +213,7 @@ int lp_small_cluster(const tp_graph *g, const LpState &st, int32_t S) {
     return 0;
   const int64_t items = (T.count[TIER_LANE] / 32 + T.count[TIER_SMALL] + T.count[TIER_MID]) / S;
   int cs = 1;
-  while (cs < kLpSmallCluster && (cs * kLpSmallWarps < items || g->n > kLpSmallVertices * cs)) cs <<= 1;
+  while (cs < kLpSmallCluster && (cs * kLpSmallItems < items || g->n > kLpSmallVertices * cs)) cs <<= 1;
   return cs;
 }
 
