@@ -3,16 +3,21 @@
 // clusters a and b, intra-cluster edges vanish.
 //
 // GPU form: coarse ids are ranks of the non-empty labels (mark + exclusive
-// scan, so ids are deterministic where the paper's atomic counters are not);
-// every inter-cluster adjacency entry is emitted as the key a*n' + b at a
-// position fixed by a scan of per-vertex (per-chunk for hubs) counts, sorted
-// with the library's LSD radix sort, and duplicate keys are reduced into the
-// canonical coarse CSR (neighbours ascending, int64 weights). Memory (the
-// paper's third peak): a fine edge weight rides in the low bits of its key
-// when both fit 64 bits, so weighted levels sort no separate values, and the
-// reduction numbers the runs tile by tile (a count per 4096 entries) instead
-// of through per-entry head flags and prefix sums.
+// scan, so ids are deterministic where the paper's atomic counters are not).
+// The fine vertices are listed by coarse vertex, and a warp (or a block) per
+// coarse vertex walks its members' rows once and sums the weights per
+// neighbouring cluster in a shared-memory hash table; the distinct neighbours
+// are sorted there and written out. Tables come in four sizes (256 and 1024
+// slots a warp, 4096 and 16384 a block): a coarse vertex starts with the size
+// that its members' entries suggest and moves to the next if its distinct
+// neighbours overflow it, so nothing depends on the guess. The few beyond the
+// largest table (coarse vertices of hubs) emit every inter-cluster entry as
+// the key a*n' + b, which the library's LSD radix sort and a run-length
+// reduction turn into their rows. (Sorting all entries took five passes over
+// them; a mesh merges about 17 entries into one.) Weights are summed in 32
+// bits where all edge weights together fit.
 #include <algorithm>
+#include <memory>
 
 #include "decode.cuh"
 
@@ -26,13 +31,20 @@ __global__ void k_mark(const int32_t *C, int64_t n, int32_t *flag) {
     flag[C[u]] = 1;
 }
 
-__global__ void k_map(const int32_t *C, const int64_t *rank, const int64_t *vw, int64_t n,
-                      int32_t *map, int64_t *cvw) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+// Coarse id of every vertex, its place among the cluster's members, the
+// cluster's weight, members and entries (compressed graphs: bytes of the
+// records, no fewer than entries; it only picks the first table size).
+__global__ void k_map(GView g, const int32_t *C, const int64_t *rank, int32_t *map, int64_t *cvw,
+                      int32_t *place, int32_t *mcnt, unsigned long long *ent) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
        u += (int64_t)gridDim.x * blockDim.x) {
-    int32_t a = (int32_t)rank[C[u]];
+    const int32_t a = (int32_t)rank[C[u]];
     map[u] = a;
-    atomicAdd((unsigned long long *)&cvw[a], (unsigned long long)(vw ? vw[u] : 1));
+    place[u] = atomicAdd(&mcnt[a], 1);
+    if (g.vw) atomicAdd((unsigned long long *)&cvw[a], (unsigned long long)g.vw[u]);
+    const int64_t e = g.compressed ? (int64_t)(off_at(g, u + 1) - off_at(g, u))
+                                   : g.xadj[u + 1] - g.xadj[u];
+    atomicAdd(&ent[a], (unsigned long long)e);
   }
 }
 
@@ -43,64 +55,556 @@ __global__ void k_seg_rank(const int64_t *rank, const int64_t *voff, int64_t nse
     coff[i] = rank[voff[i]];
 }
 
-__device__ __forceinline__ bool thread_tier(uint8_t t) { return t == TIER_LANE || t == TIER_SMALL; }
+__global__ void k_members(const int32_t *map, const int32_t *place, const int64_t *mstart,
+                          int64_t n, int32_t *members) {
+  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
+       u += (int64_t)gridDim.x * blockDim.x)
+    members[mstart[map[u]] + place[u]] = (int32_t)u;
+}
 
-// Per-vertex count of inter-cluster entries, one thread per low-degree vertex.
+// ---------------------------------------------------------------- table sizes
+// Size 0 and 1: a warp's table of 256 / 1024 slots; 2 and 3: a block's of 4096
+// / 16384; 4: keys and the radix sort. A table takes up to kAggFill distinct
+// neighbours; a coarse vertex starts with a size whose fill is no less than a
+// fifth of its entries (meshes merge far more than that into one, skewed
+// graphs less and move up).
+constexpr int kAggSizes = 4;
+__host__ __device__ constexpr int agg_log(int size) { return size == 0 ? 8 : size == 1 ? 10 : size == 2 ? 12 : 14; }
+__host__ __device__ constexpr int agg_fill(int size) { return size == 0 ? 192 : size == 1 ? 768 : size == 2 ? 2816 : 10240; }
+__host__ __device__ constexpr int64_t agg_start(int size) {
+  return size == 0 ? 1024 : size == 1 ? 4096 : size == 2 ? 14336 : 40960;
+}
+
+// Lists every coarse vertex under its first size, its weight where members
+// weigh one each. lists: kAggSizes + 1 lists of nc entries, cnt: their lengths.
+__global__ void k_agg_classes(const unsigned long long *ent, const int32_t *mcnt, int64_t nc,
+                              int64_t *cvw, int32_t *lists, int32_t *cnt) {
+  for (int64_t a0 = (int64_t)blockIdx.x * blockDim.x; a0 < nc;
+       a0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t a = a0 + threadIdx.x;
+    int cl = -1;
+    if (a < nc) {
+      const int64_t e = (int64_t)ent[a];
+      cl = 0;
+      while (cl < kAggSizes && e > agg_start(cl)) ++cl;
+      if (cvw) cvw[a] = mcnt[a];
+    }
+    const unsigned peers = __match_any_sync(kFull, cl);
+    if (cl >= 0) {
+      const int leader = __ffs(peers) - 1;
+      int32_t base = 0;
+      if (lane_id() == leader) base = atomicAdd(&cnt[cl], __popc(peers));
+      base = __shfl_sync(peers, base, leader);
+      lists[(int64_t)cl * nc + base + __popc(peers & lanemask_lt())] = (int32_t)a;
+    }
+  }
+}
+
+struct AggCtx {
+  GView g;
+  const int32_t *map, *members;
+  const int64_t *mstart;
+  int64_t nc;
+  int32_t *lists, *cnt;        // per size: coarse vertices still to do, how many
+  unsigned long long *cursor;  // entries written so far
+  int32_t *out_key;            // neighbours of every coarse vertex, sorted, at toff
+  void *out_val;
+  int64_t *toff, *deg;
+  unsigned long long *max_w;
+};
+
+// Adds w to label x's slot. Returns 0: added, 1: added in a slot it claimed,
+// 2: no slot left.
+template <class V>
+__device__ __forceinline__ int agg_add(int32_t *keys, V *vals, int logc, int32_t x, V w) {
+  const uint32_t mask = (1u << logc) - 1u;
+  uint32_t h = ((uint32_t)x * 0x9E3779B1u) >> (32 - logc);
+  for (uint32_t probe = 0; probe <= mask; ++probe, h = (h + 1) & mask) {
+    int32_t k = *(volatile int32_t *)&keys[h];
+    int claimed = 0;
+    if (k == -1) {
+      const int32_t prev = atomicCAS(&keys[h], -1, x);
+      claimed = prev == -1;
+      k = claimed ? x : prev;
+    }
+    if (k == x) {
+      atomicAdd(&vals[h], w);
+      return claimed;
+    }
+  }
+  return 2;
+}
+
+// A compressed record of more bytes than this has more than kLaneMaxDeg
+// neighbours (header and VarInts of at most ten and five bytes).
+constexpr uint64_t kLaneRecordMost = 10 + 5 * kLaneMaxDeg;
+constexpr uint64_t kLaneRecordShort = 65;  // fits lane_decode's first window
+
+// This lane's member of those from m on, and where its row lies (entries, or
+// bytes of the record).
+struct AggMember {
+  int32_t u;
+  uint64_t b, e;
+};
 template <bool COMP>
-__global__ void k_count_thread(GView g, const uint8_t *tier, const int32_t *map, int64_t *cnt) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    if (!thread_tier(tier[u])) continue;
+__device__ __forceinline__ AggMember agg_member(const AggCtx &c, int64_t m, int64_t mend) {
+  AggMember r{0, 0, 0};
+  if (m + lane_id() < mend) {
+    r.u = c.members[m + lane_id()];
+    r.b = COMP ? off_at(c.g, r.u) : (uint64_t)c.g.xadj[r.u];
+    r.e = COMP ? off_at(c.g, r.u + 1) : (uint64_t)c.g.xadj[r.u + 1];
+  }
+  return r;
+}
+
+// One warp sums the rows of members m, m + step, ... (32 at a time) of coarse
+// vertex a into the table; fill() tells the distinct neighbours so far (of the
+// warp or the block), add_fill(k) counts k more. Rows of up to 32 entries are
+// walked a lane each (compressed: decoded into the lane's column), several
+// entries in flight; row(u, entries) takes the longer ones and says whether
+// the table held. Returns whether it held throughout.
+template <bool COMP, class V, class Fill, class AddFill, class Row>
+__device__ __forceinline__ bool agg_rows(const AggCtx &c, int32_t a, int64_t m, int64_t mend,
+                                         int64_t step, int32_t *keys, V *vals, int logc,
+                                         uint32_t *col, int limit, AggMember first, Fill fill,
+                                         AddFill add_fill, Row row) {
+  constexpr int U = COMP ? 8 : 4;
+  const int lane = lane_id();
+  for (AggMember mem = first; m < mend; m += step, mem = agg_member<COMP>(c, m, mend)) {
+    const bool in = m + lane < mend;
+    const int32_t u = mem.u;
+    int deg = 0;
+    int64_t b = 0;
+    bool wide = false;
+    if (in) {
+      if (COMP) {
+        const uint64_t rb = mem.b, re = mem.e;
+        if (re - rb <= kLaneRecordShort) deg = lane_decode<false, true>(c.g, rb, re, col);
+        else if (re - rb <= kLaneRecordMost) deg = lane_decode<true, true>(c.g, rb, re, col);
+        else deg = kLaneMaxDeg + 1;
+      } else {
+        b = (int64_t)mem.b;
+        deg = (int)min((int64_t)(mem.e - mem.b), (int64_t)kLaneMaxDeg + 1);
+      }
+      wide = deg > kLaneMaxDeg;
+      if (wide) deg = 0;
+    }
+    const unsigned wides = __ballot_sync(kFull, wide);
+    const int most = (int)__reduce_max_sync(kFull, (unsigned)deg);
+    int32_t prev = u;
+    for (int i0 = 0; i0 < most; i0 += U) {
+      int32_t x[U];
+      V w[U];
+#pragma unroll
+      for (int r = 0; r < U; ++r) {
+        const int i = i0 + r;
+        x[r] = -1;
+        w[r] = 1;
+        if (i < deg) {
+          if (COMP) {
+            const uint32_t v = col[i * 32];
+            prev = i == 0 ? ((v & 1u) ? u - (int32_t)(v >> 1) : u + (int32_t)(v >> 1))
+                          : prev + (int32_t)v;
+            prev = (int32_t)min((uint32_t)prev, (uint32_t)(c.g.n - 1));
+            x[r] = prev;
+          } else {
+            x[r] = c.g.adj[b + i];
+            if (c.g.ew) w[r] = (V)c.g.ew[b + i];
+          }
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < U; ++r) x[r] = x[r] >= 0 ? c.map[x[r]] : a;
+      unsigned claimed = 0;
+      bool full = false;
+#pragma unroll
+      for (int r = 0; r < U; ++r)
+        if (x[r] != a) {
+          const int res = agg_add<V>(keys, vals, logc, x[r], w[r]);
+          claimed += res == 1;
+          full |= res == 2;
+        }
+      claimed = __reduce_add_sync(kFull, claimed);
+      if (claimed) add_fill((int)claimed);
+      if (__any_sync(kFull, full) || fill() > limit) return false;
+    }
+    for (unsigned q = wides; q; q &= q - 1)
+      if (!row(__shfl_sync(kFull, u, __ffs(q) - 1))) return false;
+  }
+  return true;
+}
+
+// A long row, or of a CSR row the pieces of 128 entries number first, first +
+// step, ..., by a warp, 128 entries in flight (compressed: a decoder's step).
+template <bool COMP, class V, class Fill, class AddFill>
+__device__ __forceinline__ bool agg_long_row(const AggCtx &c, int32_t a, int32_t u, int first,
+                                             int step, int32_t *keys, V *vals, int logc, int limit,
+                                             Fill fill, AddFill add_fill) {
+  const int lane = lane_id();
+  bool bad = false;
+  auto settle = [&](unsigned claimed, bool full) {
+    claimed = __reduce_add_sync(kFull, claimed);
+    if (claimed) add_fill((int)claimed);
+    bad = __any_sync(kFull, full) || fill() > limit;
+  };
+  if constexpr (COMP) {
+    warp_neighbours<true>(c.g, u, -1, [&](bool has, int32_t v, int64_t, int64_t) {
+      if (bad) return;
+      const int32_t x = has ? c.map[v] : a;
+      const int res = x != a ? agg_add<V>(keys, vals, logc, x, (V)1) : 0;
+      settle(res == 1, res == 2);
+    });
+  } else {
+    const int64_t e = c.g.xadj[u + 1];
+    for (int64_t i0 = c.g.xadj[u] + 128 * first; i0 < e && !bad; i0 += 128 * (int64_t)step) {
+      int32_t x[4];
+      V w[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int64_t i = i0 + 32 * r + lane;
+        x[r] = i < e ? c.g.adj[i] : -1;
+        w[r] = i < e && c.g.ew ? (V)c.g.ew[i] : (V)1;
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) x[r] = x[r] >= 0 ? c.map[x[r]] : a;
+      unsigned claimed = 0;
+      bool full = false;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (x[r] != a) {
+          const int res = agg_add<V>(keys, vals, logc, x[r], w[r]);
+          claimed += res == 1;
+          full |= res == 2;
+        }
+      settle(claimed, full);
+    }
+  }
+  return !bad;
+}
+
+// Ascending bitonic sort of a[0 .. n2) (a power of two) by nt threads, t this
+// one's number; sync separates the steps.
+template <class Sync>
+__device__ __forceinline__ void bitonic(uint64_t *a, int n2, int t, int nt, Sync sync) {
+  for (int k = 2; k <= n2; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int i = t; i < n2 / 2; i += nt) {
+        const int lo = 2 * i - (i & (j - 1)), hi = lo + j;
+        const uint64_t x = a[lo], y = a[hi];
+        if ((x > y) == ((lo & k) == 0)) a[lo] = y, a[hi] = x;
+      }
+      sync();
+    }
+}
+
+// Sizes 0 and 1: a warp per coarse vertex.
+template <bool COMP, int SIZE, class V>
+struct AggWarp {
+  union {
+    uint64_t items[SIZE == 0 ? 256 : 1024];        // neighbour << 32 | slot, once the rows are done
+    uint32_t col[COMP ? kLaneMaxDeg * 32 : 1];     // decoded records
+  };
+  int32_t keys[1 << agg_log(SIZE)];
+  V vals[1 << agg_log(SIZE)];
+};
+__host__ __device__ constexpr int agg_warps(int size) { return size == 0 ? 8 : 4; }
+
+template <bool COMP, int SIZE, class V>
+__global__ void __launch_bounds__(32 * agg_warps(SIZE)) k_agg_warp(AggCtx c) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int L = agg_log(SIZE), SLOTS = 1 << L;
+  using Warp = AggWarp<COMP, SIZE, V>;
+  Warp &s = reinterpret_cast<Warp *>(smem)[threadIdx.x >> 5];
+  const int lane = lane_id();
+  V *out_val = static_cast<V *>(c.out_val);
+  for (int i = lane; i < SLOTS; i += 32) s.keys[i] = -1, s.vals[i] = 0;
+  __syncwarp();
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int64_t cnt = c.cnt[SIZE];
+  unsigned long long most = 0;
+  // the next coarse vertex's list entry, members and their rows are loaded
+  // while this one is summed, sorted and written: its own chain of dependent
+  // loads (entry, range, member, offset, record) would leave the warp waiting
+  const int32_t *list = c.lists + (int64_t)SIZE * c.nc;
+  int32_t a_next = gw < cnt ? list[gw] : 0;
+  int64_t m0_next = 0, m1_next = 0;
+  if (gw < cnt) m0_next = c.mstart[a_next], m1_next = c.mstart[a_next + 1];
+  AggMember mem_next = agg_member<COMP>(c, m0_next, m1_next);
+  for (int64_t q = gw; q < cnt; q += nw) {
+    const int32_t a = a_next;
+    const int64_t m0 = m0_next, m1 = m1_next;
+    const AggMember mem = mem_next;
+    const bool more = q + nw < cnt;
+    if (more) a_next = list[q + nw];
+    int n_fill = 0;
+    auto fill = [&] { return n_fill; };
+    auto add_fill = [&](int k) { n_fill += k; };
+    const bool ok = agg_rows<COMP, V>(
+        c, a, m0, m1, 32, s.keys, s.vals, L, s.col + lane, agg_fill(SIZE), mem, fill, add_fill,
+        [&](int32_t u) {
+          return agg_long_row<COMP, V>(c, a, u, 0, 1, s.keys, s.vals, L, agg_fill(SIZE), fill, add_fill);
+        });
+    __syncwarp();
+    m0_next = more ? c.mstart[a_next] : 0;
+    m1_next = more ? c.mstart[a_next + 1] : 0;
+    if (!ok) {  // to the next size
+      mem_next = agg_member<COMP>(c, m0_next, m1_next);
+      if (lane == 0)
+        c.lists[(int64_t)(SIZE + 1) * c.nc + atomicAdd(&c.cnt[SIZE + 1], 1)] = a;
+      for (int i = lane; i < SLOTS; i += 32) s.keys[i] = -1, s.vals[i] = 0;
+      __syncwarp();
+      continue;
+    }
+    // the occupied slots, sorted by neighbour
+    int d = 0;
+    for (int i = lane; i < SLOTS; i += 32) {
+      const int32_t k = s.keys[i];
+      const unsigned m = __ballot_sync(kFull, k >= 0);
+      if (k >= 0) s.items[d + __popc(m & lanemask_lt())] = (uint64_t)(uint32_t)k << 32 | (uint32_t)i;
+      d += __popc(m);
+    }
+    __syncwarp();
+    unsigned long long base = 0;
+    if (lane == 0) {
+      base = d ? atomicAdd(c.cursor, (unsigned long long)d) : 0ull;  // (used after the sort)
+      c.deg[a] = d;
+    }
+    mem_next = agg_member<COMP>(c, m0_next, m1_next);
+    if (d <= 32) {  // in registers
+      uint64_t x = lane < d ? s.items[lane] : ~0ull;
+#pragma unroll
+      for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+          const uint64_t y = __shfl_xor_sync(kFull, x, j);
+          const bool up = ((lane & k) == 0) == ((lane & j) == 0);
+          x = up ? (x < y ? x : y) : (x < y ? y : x);
+        }
+      base = __shfl_sync(kFull, base, 0);
+      if (lane < d) {
+        const V w = s.vals[(uint32_t)x];
+        c.out_key[base + lane] = (int32_t)(x >> 32);
+        out_val[base + lane] = w;
+        most = w > most ? w : most;
+      }
+    } else {
+      int n2 = 64;
+      while (n2 < d) n2 <<= 1;
+      for (int i = d + lane; i < n2; i += 32) s.items[i] = ~0ull;
+      __syncwarp();
+      bitonic(s.items, n2, lane, 32, [] { __syncwarp(); });
+      base = __shfl_sync(kFull, base, 0);
+      for (int i = lane; i < d; i += 32) {
+        const uint64_t x = s.items[i];
+        const V w = s.vals[(uint32_t)x];
+        c.out_key[base + i] = (int32_t)(x >> 32);
+        out_val[base + i] = w;
+        most = w > most ? w : most;
+      }
+    }
+    if (lane == 0) c.toff[a] = (int64_t)base;
+    if (COMP && mem_next.e > mem_next.b) prefetch_l2(c.g.bytes + mem_next.b);
+    __syncwarp();
+    for (int i = lane; i < SLOTS; i += 32) s.keys[i] = -1, s.vals[i] = 0;
+    __syncwarp();
+  }
+  most = warp_max(most);
+  if (lane == 0 && most) atomicMax(c.max_w, most);
+}
+
+// Sizes 2 and 3: a block per coarse vertex, its warps taking 32 members each
+// in turn.
+constexpr int64_t kAggDecodeDeg = 1024;  // compressed graphs beyond this degree are decoded first
+constexpr int kAggThreads = 256;
+constexpr int kAggWide = 256;
+template <class V>
+__host__ __device__ constexpr int agg_block_fill(int size) {
+  // the largest table with 64-bit sums: items of half the size beside it
+  return size == 3 && sizeof(V) == 8 ? 4096 : agg_fill(size);
+}
+template <class V>
+__host__ __device__ constexpr int agg_block_items(int size) {
+  return size == 2 ? 4096 : sizeof(V) == 8 ? 4096 : 10240;
+}
+template <bool COMP, class V>
+__host__ __device__ constexpr size_t agg_block_smem(int size) {
+  return ((size_t)1 << agg_log(size)) * (4 + sizeof(V)) + 8 * (size_t)agg_block_items<V>(size) +
+         (COMP && size == 2 ? (size_t)4 * kLaneMaxDeg * kAggThreads : 0);
+}
+
+template <bool COMP, int SIZE, class V>
+__global__ void __launch_bounds__(kAggThreads) k_agg_block(AggCtx c) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int L = agg_log(SIZE), SLOTS = 1 << L, FILL = agg_block_fill<V>(SIZE);
+  constexpr int ITEMS = agg_block_items<V>(SIZE);
+  uint64_t *items = reinterpret_cast<uint64_t *>(smem);
+  V *vals = reinterpret_cast<V *>(items + ITEMS);
+  int32_t *keys = reinterpret_cast<int32_t *>(vals + SLOTS);
+  // columns of decoded records: their own, or where the items will be (the
+  // largest table leaves no room beside it; items are listed after the rows)
+  uint32_t *cols = SIZE == 2 ? reinterpret_cast<uint32_t *>(keys + SLOTS)
+                             : reinterpret_cast<uint32_t *>(items);
+  static_assert(8 * ITEMS >= 4 * kLaneMaxDeg * kAggThreads, "columns fit where the items go");
+  __shared__ int32_t s_fill, s_fail, s_d, s_wide, s_next;
+  __shared__ int32_t wide[kAggWide];  // long rows, shared out over the warps after the others
+  __shared__ unsigned long long s_base;
+  const int tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
+  V *out_val = static_cast<V *>(c.out_val);
+  const int64_t cnt = c.cnt[SIZE];
+  unsigned long long most = 0;
+  for (int64_t q = blockIdx.x; q < cnt; q += gridDim.x) {
+    const int32_t a = c.lists[(int64_t)SIZE * c.nc + q];
+    const int64_t m0 = c.mstart[a] + 32 * w, m1 = c.mstart[a + 1];
+    for (int i = tid; i < SLOTS; i += kAggThreads) keys[i] = -1, vals[i] = 0;
+    if (tid == 0) s_fill = 0, s_fail = 0, s_d = 0, s_wide = 0, s_next = 0;
+    __syncthreads();
+    auto fill = [&] { return __shfl_sync(kFull, *(volatile int32_t *)&s_fill, 0); };
+    auto add_fill = [&](int k) {
+      if (lane == 0) atomicAdd(&s_fill, k);
+      __syncwarp();
+    };
+    bool ok = agg_rows<COMP, V>(
+        c, a, m0, m1, kAggThreads, keys, vals, L, cols + (size_t)w * kLaneMaxDeg * 32 + lane, FILL,
+        agg_member<COMP>(c, m0, m1), fill, add_fill, [&](int32_t u) {
+          int at = 0;
+          if (lane == 0) {
+            at = atomicAdd(&s_wide, 1);
+            if (at < kAggWide) wide[at] = u;
+          }
+          at = __shfl_sync(kFull, at, 0);
+          return at < kAggWide ||
+                 agg_long_row<COMP, V>(c, a, u, 0, 1, keys, vals, L, FILL, fill, add_fill);
+        });
+    __syncthreads();
+    const int nwide = min(s_wide, kAggWide);
+    if (COMP) {  // a record is decoded by one warp
+      while (ok) {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(&s_next, 1);
+        i = __shfl_sync(kFull, i, 0);
+        if (i >= nwide) break;
+        ok = agg_long_row<COMP, V>(c, a, wide[i], 0, 1, keys, vals, L, FILL, fill, add_fill);
+      }
+    } else {  // every warp takes its pieces of each row
+      for (int i = 0; i < nwide && ok; ++i)
+        ok = agg_long_row<COMP, V>(c, a, wide[i], (w + i) % (kAggThreads / 32), kAggThreads / 32, keys,
+                                   vals, L, FILL, fill, add_fill);
+    }
+    if (!ok && lane == 0) s_fail = 1;
+    __syncthreads();
+    if (s_fail || s_fill > FILL) {  // uniform: to the next size
+      if (tid == 0)
+        c.lists[(int64_t)(SIZE + 1) * c.nc + atomicAdd(&c.cnt[SIZE + 1], 1)] = a;
+      __syncthreads();
+      continue;
+    }
+    for (int i = tid; i < SLOTS; i += kAggThreads) {
+      const int32_t k = keys[i];
+      const unsigned m = __ballot_sync(kFull, k >= 0);
+      int32_t base = 0;
+      if (lane == 0 && m) base = atomicAdd(&s_d, __popc(m));
+      base = __shfl_sync(kFull, base, 0);
+      if (k >= 0) items[base + __popc(m & lanemask_lt())] = (uint64_t)(uint32_t)k << 32 | (uint32_t)i;
+    }
+    __syncthreads();
+    const int d = s_d;
+    int n2 = 64;
+    while (n2 < d) n2 <<= 1;
+    if (n2 <= ITEMS) {
+      for (int i = d + tid; i < n2; i += kAggThreads) items[i] = ~0ull;
+      __syncthreads();
+      bitonic(items, n2, tid, kAggThreads, [] { __syncthreads(); });
+    } else {
+      // more than 8192: the first 8192 and the rest (below 2048) sorted apart,
+      // then each item goes to its rank in both
+      constexpr int H = 8192;
+      int r2 = 64;
+      while (r2 < d - H) r2 <<= 1;
+      for (int i = d + tid; i < H + r2; i += kAggThreads) items[i] = ~0ull;
+      __syncthreads();
+      bitonic(items, H, tid, kAggThreads, [] { __syncthreads(); });
+      bitonic(items + H, r2, tid, kAggThreads, [] { __syncthreads(); });
+    }
+    if (tid == 0) {
+      s_base = d ? atomicAdd(c.cursor, (unsigned long long)d) : 0ull;
+      c.toff[a] = (int64_t)s_base;
+      c.deg[a] = d;
+    }
+    __syncthreads();
+    const bool two = n2 > ITEMS;
+    for (int i = tid; i < d; i += kAggThreads) {
+      const uint64_t x = items[i];
+      int pos = i;
+      if (two) {  // rank in the other run
+        constexpr int H = 8192;
+        int lo = i < H ? H : 0, hi = i < H ? d : H;
+        const int first = lo;
+        while (lo < hi) {
+          const int mid = (lo + hi) / 2;
+          if (items[mid] < x) lo = mid + 1;
+          else hi = mid;
+        }
+        pos = (i < H ? i : i - H) + lo - first;
+      }
+      const V wt = vals[(uint32_t)x];
+      c.out_key[s_base + pos] = (int32_t)(x >> 32);
+      out_val[s_base + pos] = wt;
+      most = wt > most ? wt : most;
+    }
+    __syncthreads();  // the next coarse vertex reuses the shared memory
+  }
+  most = warp_max(most);
+  if (lane == 0 && most) atomicMax(c.max_w, most);
+}
+
+// ---------------------------------------------------------------- hubs' coarse vertices
+// The rows of their members in items of up to kChunkSize entries (compressed
+// records below the chunking threshold whole), a warp each.
+__global__ void k_mark_sorted(const int32_t *list, int64_t cnt, uint8_t *sorted) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
+       i += (int64_t)gridDim.x * blockDim.x)
+    sorted[list[i]] = 1;
+}
+
+template <bool COMP>
+__global__ void k_row_items(GView g, const int32_t *map, const uint8_t *sorted, uint64_t *items,
+                            unsigned long long *n_items) {
+  for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x; u0 < g.n;
+       u0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t u = u0 + threadIdx.x;
+    int64_t k = 0;
+    if (u < g.n && sorted[map[u]]) {
+      if (COMP) {
+        const ZipNbr z = zip_nbr(g, u);
+        k = z.deg ? z.nchunks : 0;
+      } else {
+        k = (g.xadj[u + 1] - g.xadj[u] + kChunkSize - 1) / kChunkSize;
+      }
+    }
+    const int64_t incl = warp_incl_scan(k);
+    const int64_t total = __shfl_sync(kFull, incl, 31);
+    if (total == 0) continue;  // uniform over the warp
+    unsigned long long base = 0;
+    if (lane_id() == 0) base = atomicAdd(n_items, (unsigned long long)total);
+    base = __shfl_sync(kFull, base, 0) + (unsigned long long)(incl - k);
+    for (int64_t j = 0; j < k; ++j) items[base + j] = (uint64_t)u << 32 | (uint64_t)j;
+  }
+}
+
+template <bool COMP>
+__global__ void k_item_count(GView g, const int32_t *map, const uint64_t *items, int64_t n,
+                             int64_t *cnt) {
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t it = gw; it < n; it += nw) {
+    const int64_t u = (int64_t)(items[it] >> 32), j = (int64_t)(items[it] & 0xffffffffu);
     const int32_t a = map[u];
     int64_t c = 0;
-    thread_neighbours<COMP>(g, u, [&](int32_t v, int64_t) { c += map[v] != a; });
-    cnt[u] = c;
-  }
-}
-
-// Per-vertex count of inter-cluster entries, one warp per medium vertex
-// (hubs are counted per chunk below).
-template <bool COMP>
-__global__ void k_count(GView g, const uint8_t *tier, const int32_t *map, int64_t *cnt) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t u = warp; u < g.n; u += nw) {
-    if (thread_tier(tier[u])) continue;
-    int64_t c = 0;
-    if (tier[u] != TIER_HUGE) {
-      int32_t a = map[u];
-      warp_neighbours<COMP>(g, u, -1, [&](bool has, int32_t v, int64_t, int64_t) {
-        c += __popc(__ballot_sync(kFull, has && map[v] != a));
-      });
-    }
-    if (lane_id() == 0) cnt[u] = c;
-  }
-}
-
-__device__ __forceinline__ int64_t find_item(const int64_t *start, int64_t cnt, int64_t item) {
-  int64_t lo = 0, hi = cnt - 1;
-  while (lo < hi) {
-    int64_t mid = (lo + hi + 1) / 2;
-    if (start[mid] <= item) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
-template <bool COMP>
-__global__ void k_count_chunks(GView g, const int32_t *huge, int64_t n_huge,
-                               const int64_t *chunk_start, int64_t n_items, const int32_t *map,
-                               int64_t *cnt) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t it = warp; it < n_items; it += nw) {
-    int64_t i = find_item(chunk_start, n_huge, it);
-    int64_t u = huge[i];
-    int32_t a = map[u];
-    int64_t c = 0;
-    warp_neighbours<COMP>(g, u, it - chunk_start[i], [&](bool has, int32_t v, int64_t, int64_t) {
-      c += __popc(__ballot_sync(kFull, has && map[v] != a));
+    warp_neighbours<COMP>(g, u, j, [&](bool has, int32_t v, int64_t, int64_t) {
+      c += has && map[v] != a;
     });
+    c = warp_sum(c);
     if (lane_id() == 0) cnt[it] = c;
   }
 }
@@ -114,61 +618,26 @@ __device__ __forceinline__ uint64_t entry_key(int32_t a, int32_t b, int64_t nc, 
 }
 
 template <bool COMP>
-__device__ __forceinline__ void emit(const GView &g, int64_t u, int64_t chunk, const int32_t *map,
-                                     int64_t nc, int wbits, int64_t pos, uint64_t *keys,
-                                     uint64_t *vals) {
-  int32_t a = map[u];
-  warp_neighbours<COMP>(g, u, chunk, [&](bool has, int32_t v, int64_t w, int64_t) {
-    int32_t b = has ? map[v] : a;
-    bool keep = has && b != a;
-    unsigned m = __ballot_sync(kFull, keep);
-    if (keep) {
-      int64_t at = pos + __popc(m & lanemask_lt());
-      keys[at] = entry_key(a, b, nc, w, wbits);
-      if (vals) vals[at] = (uint64_t)w;
-    }
-    pos += __popc(m);
-  });
-}
-
-template <bool COMP>
-__global__ void k_emit_thread(GView g, const uint8_t *tier, const int32_t *map, int64_t nc,
-                              int wbits, const int64_t *off, uint64_t *keys, uint64_t *vals) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    if (!thread_tier(tier[u])) continue;
+__global__ void k_item_emit(GView g, const int32_t *map, const uint64_t *items, int64_t n,
+                            int64_t nc, int wbits, const int64_t *off, uint64_t *keys,
+                            uint64_t *vals) {
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t it = gw; it < n; it += nw) {
+    const int64_t u = (int64_t)(items[it] >> 32), j = (int64_t)(items[it] & 0xffffffffu);
     const int32_t a = map[u];
-    int64_t pos = off[u];
-    thread_neighbours<COMP>(g, u, [&](int32_t v, int64_t w) {
-      const int32_t b = map[v];
-      if (b == a) return;
-      keys[pos] = entry_key(a, b, nc, w, wbits);
-      if (vals) vals[pos] = (uint64_t)w;
-      ++pos;
+    int64_t pos = off[it];
+    warp_neighbours<COMP>(g, u, j, [&](bool has, int32_t v, int64_t w, int64_t) {
+      const int32_t b = has ? map[v] : a;
+      const bool keep = has && b != a;
+      const unsigned m = __ballot_sync(kFull, keep);
+      if (keep) {
+        const int64_t at = pos + __popc(m & lanemask_lt());
+        keys[at] = entry_key(a, b, nc, w, wbits);
+        if (vals) vals[at] = (uint64_t)w;
+      }
+      pos += __popc(m);
     });
-  }
-}
-
-template <bool COMP>
-__global__ void k_emit(GView g, const uint8_t *tier, const int32_t *map, int64_t nc, int wbits,
-                       const int64_t *off, uint64_t *keys, uint64_t *vals) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t u = warp; u < g.n; u += nw)
-    if (!thread_tier(tier[u]) && tier[u] != TIER_HUGE)
-      emit<COMP>(g, u, -1, map, nc, wbits, off[u], keys, vals);
-}
-
-template <bool COMP>
-__global__ void k_emit_chunks(GView g, const int32_t *huge, int64_t n_huge,
-                              const int64_t *chunk_start, int64_t n_items, const int32_t *map,
-                              int64_t nc, int wbits, int64_t base, const int64_t *off,
-                              uint64_t *keys, uint64_t *vals) {
-  int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t it = warp; it < n_items; it += nw) {
-    int64_t i = find_item(chunk_start, n_huge, it);
-    emit<COMP>(g, huge[i], it - chunk_start[i], map, nc, wbits, base + off[it], keys, vals);
   }
 }
 
@@ -203,12 +672,13 @@ __global__ void __launch_bounds__(kRleThreads) k_rle_count(const uint64_t *keys,
 
 // Pass 2: every entry adds its weight to its run's slot (the runs before it,
 // from the tile's offset plus a block scan); a run's first entry also writes
-// the neighbour and counts the coarse vertex's degree.
+// the neighbour and the coarse vertex, and counts its degree.
 __global__ void __launch_bounds__(kRleThreads) k_rle_write(const uint64_t *keys,
                                                            const uint64_t *vals, int64_t m,
                                                            int64_t nc, int wbits, int64_t ntiles,
                                                            const int64_t *toff, int32_t *adj,
-                                                           int64_t *ew, int64_t *deg) {
+                                                           int64_t *ew, int32_t *row,
+                                                           int64_t *deg) {
   __shared__ int32_t ws[kRleThreads / 32];
   const uint64_t wmask = wbits ? ((uint64_t)1 << wbits) - 1 : 0;
   const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -237,6 +707,7 @@ __global__ void __launch_bounds__(kRleThreads) k_rle_write(const uint64_t *keys,
         const uint64_t wt = wbits ? (k & wmask) : (vals ? vals[i] : 1ull);
         if (h) {
           adj[slot] = (int32_t)(key % (uint64_t)nc);
+          row[slot] = (int32_t)(key / (uint64_t)nc);
           atomicAdd((unsigned long long *)&deg[key / (uint64_t)nc], 1ull);
         }
         atomicAdd((unsigned long long *)&ew[slot], (unsigned long long)wt);
@@ -247,11 +718,77 @@ __global__ void __launch_bounds__(kRleThreads) k_rle_write(const uint64_t *keys,
   }
 }
 
+// The rows from the tables into the coarse CSR (sorted = those of hubs' coarse
+// vertices, which come from the runs below).
+template <class V>
+__global__ void k_copy_rows(const int64_t *toff, const int64_t *xadj, const uint8_t *sorted,
+                            int64_t nc, int lanes, const int32_t *key, const V *val, int32_t *adj,
+                            int64_t *ew) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t ng = (int64_t)gridDim.x * blockDim.x / lanes;
+  for (int64_t a = t / lanes; a < nc; a += ng) {
+    if (sorted && sorted[a]) continue;
+    const int64_t b = xadj[a], d = xadj[a + 1] - b, src = toff[a];
+#pragma unroll 4
+    for (int64_t i = t % lanes; i < d; i += lanes) {
+      adj[b + i] = key[src + i];
+      ew[b + i] = (int64_t)val[src + i];
+    }
+  }
+}
+
+// The runs of the sorted entries into the coarse CSR (start: first run of
+// every coarse vertex), and the largest weight among them.
+__global__ void k_copy_runs(const int64_t *start, const int64_t *xadj, int64_t runs,
+                            const int32_t *row, const int32_t *key, const int64_t *val,
+                            int32_t *adj, int64_t *ew) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < runs;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t a = row[i];
+    const int64_t to = xadj[a] + i - start[a];
+    adj[to] = key[i];
+    ew[to] = val[i];
+  }
+}
+
+__global__ void k_add_i64(const int64_t *a, int64_t n, int64_t *b) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    b[i] += a[i];
+}
+
+// The block of k_agg_block / k_agg_warp grids: as many as fit the SMs, no more
+// than the longest the list can become.
+template <bool COMP, class V>
+void launch_agg(const AggCtx &c, const int64_t (&most)[kAggSizes], cudaStream_t s) {
+  const int sms = num_sms();
+  auto run = [&](auto kern, int64_t blocks, int threads, size_t smem) {
+    TP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int per_sm = std::max(1, std::min(2048 / threads, (int)((size_t)(228 * 1024) / (smem + 1024))));
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sms * per_sm));
+    launch(kern, grid, threads, smem, s, c);
+    TP_LAUNCH_CHECK();
+  };
+  constexpr int W0 = agg_warps(0), W1 = agg_warps(1);
+  if (most[0]) run(k_agg_warp<COMP, 0, V>, (most[0] + W0 - 1) / W0, 32 * W0, sizeof(AggWarp<COMP, 0, V>) * W0);
+  if (most[1]) run(k_agg_warp<COMP, 1, V>, (most[1] + W1 - 1) / W1, 32 * W1, sizeof(AggWarp<COMP, 1, V>) * W1);
+  if (most[2]) run(k_agg_block<COMP, 2, V>, most[2], kAggThreads, agg_block_smem<COMP, V>(2));
+  if (most[3]) run(k_agg_block<COMP, 3, V>, most[3], kAggThreads, agg_block_smem<COMP, V>(3));
+}
+
 }  // namespace
 
 tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStream_t s,
                    const int64_t *seg_voff, int64_t nseg, int64_t *seg_coff) {
   int64_t n = g->n;
+  // a compressed graph with long records is decoded first (each chunk once, by
+  // a warp): in the tables' kernels such a record is one warp's, and R-MAT
+  // 2^22 spent 39 ms in them where decoding and the CSR kernels take 8
+  std::unique_ptr<tp_graph> csr;
+  if (g->compressed && g->max_deg > kAggDecodeDeg) {
+    csr.reset(decompress(g, s));
+    g = csr.get();
+  }
   tp_graph *cg = new_graph();
   try {
     cg->err.alloc(1, s);
@@ -264,17 +801,19 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
       TP_CUDA(cudaStreamSynchronize(s));
       return cg;
     }
-    Buf<int32_t> flag(n, s);
-    TP_CUDA(cudaMemsetAsync(flag.get(), 0, n * sizeof(int32_t), s));
-    launch(k_mark, grid_for(n, 256), 256, 0, s, C, n, flag.get());
-    TP_LAUNCH_CHECK();
     Buf<int64_t> rank(n + 1, s);
-    exclusive_scan_i32_to_i64(flag.get(), rank.get(), n, s);
+    {
+      Buf<int32_t> flag(n, s);
+      TP_CUDA(cudaMemsetAsync(flag.get(), 0, n * sizeof(int32_t), s));
+      launch(k_mark, grid_for(n, 256), 256, 0, s, C, n, flag.get());
+      TP_LAUNCH_CHECK();
+      exclusive_scan_i32_to_i64(flag.get(), rank.get(), n, s);
+    }
     if (seg_voff) {
       launch(k_seg_rank, grid_for(nseg + 1, 256), 256, 0, s, rank.get(), seg_voff, nseg, seg_coff);
       TP_LAUNCH_CHECK();
     }
-    int64_t nc = read_scalar(rank.get() + n, s);
+    const int64_t nc = read_scalar(rank.get() + n, s);
     cg->n = nc;
     Buf<int32_t> own_map;
     int32_t *map = d_map;
@@ -282,108 +821,167 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
       own_map.alloc(n, s);
       map = own_map.get();
     }
-    cg->vw.alloc(nc, s);
-    TP_CUDA(cudaMemsetAsync(cg->vw.get(), 0, nc * sizeof(int64_t), s));
-    launch(k_map, grid_for(n, 256), 256, 0, s, C, rank.get(), g->unit_vw ? nullptr : g->vw.get(), n,
-                                             map, cg->vw.get());
-    TP_LAUNCH_CHECK();
     cg->total_vw = g->total_vw;
     cg->sum_ew = ew_sum_bound(g);
-
-    // inter-cluster entries: counts, offsets, emission
-    tp_params dp;
-    tp_params_default(&dp);
-    if (!g->tiers.built) build_tiers(const_cast<tp_graph *>(g), dp, s);
-    const TierCache &T = g->tiers;
-    GView v = view(g);
+    cg->vw.alloc(nc, s);
+    if (!g->unit_vw) TP_CUDA(cudaMemsetAsync(cg->vw.get(), 0, nc * sizeof(int64_t), s));
+    const GView v = view(g);
     const bool comp = g->compressed;
-    Buf<int64_t> off(n + 1, s);
-    unsigned wb = grid_for(n * 32, 256);
-    unsigned tb = grid_for(n, 256);
-    const bool warp_work = T.n_mid + T.n_mid2 + T.n_big0 + T.n_big1 + T.n_big + T.n_big2 > 0;
-    if (comp) launch(k_count_thread<true>, tb, 256, 0, s, v, T.tier.get(), map, off.get());
-    else launch(k_count_thread<false>, tb, 256, 0, s, v, T.tier.get(), map, off.get());
-    if (warp_work || T.n_huge) {  // the warp kernel also zeroes the hub entries
-      if (comp) launch(k_count<true>, wb, 256, 0, s, v, T.tier.get(), map, off.get());
-      else launch(k_count<false>, wb, 256, 0, s, v, T.tier.get(), map, off.get());
-    }
-    TP_LAUNCH_CHECK();
-    exclusive_scan_i64(off.get(), off.get(), n, s);
-    int64_t m_small = read_scalar(off.get() + n, s);
-    int64_t m_huge = 0;
-    Buf<int64_t> hoff;
-    if (T.n_huge) {
-      hoff.alloc(T.n_huge_chunks + 1, s);
-      unsigned hb = grid_for(T.n_huge_chunks * 32, 256);
-      if (comp)
-        launch(k_count_chunks<true>, hb, 256, 0, s, v, T.huge.get(), T.n_huge, T.huge_chunk_start.get(),
-                                                T.n_huge_chunks, map, hoff.get());
-      else
-        launch(k_count_chunks<false>, hb, 256, 0, s, v, T.huge.get(), T.n_huge, T.huge_chunk_start.get(),
-                                                 T.n_huge_chunks, map, hoff.get());
-      TP_LAUNCH_CHECK();
-      exclusive_scan_i64(hoff.get(), hoff.get(), T.n_huge_chunks, s);
-      m_huge = read_scalar(hoff.get() + T.n_huge_chunks, s);
-    }
-    int64_t m = m_small + m_huge;
-    const bool weighted = !g->unit_ew;
-    // weights ride in the keys' low bits when the pair fits 64 bits
-    const int kbits = bits_for((uint64_t)nc * (uint64_t)nc - 1);
-    const int wbits = weighted && kbits + bits_for((uint64_t)g->max_ew) <= 64
-                          ? bits_for((uint64_t)g->max_ew)
-                          : 0;
-    Buf<uint64_t> keys(std::max<int64_t>(m, 1), s), vals;
-    if (weighted && !wbits) vals.alloc(std::max<int64_t>(m, 1), s);
-    if (comp)
-      launch(k_emit_thread<true>, tb, 256, 0, s, v, T.tier.get(), map, nc, wbits, off.get(), keys.get(), vals.get());
-    else
-      launch(k_emit_thread<false>, tb, 256, 0, s, v, T.tier.get(), map, nc, wbits, off.get(), keys.get(), vals.get());
-    if (warp_work) {
-      if (comp) launch(k_emit<true>, wb, 256, 0, s, v, T.tier.get(), map, nc, wbits, off.get(), keys.get(), vals.get());
-      else launch(k_emit<false>, wb, 256, 0, s, v, T.tier.get(), map, nc, wbits, off.get(), keys.get(), vals.get());
-    }
-    TP_LAUNCH_CHECK();
-    if (T.n_huge) {
-      unsigned hb = grid_for(T.n_huge_chunks * 32, 256);
-      if (comp)
-        launch(k_emit_chunks<true>, hb, 256, 0, s, v, T.huge.get(), T.n_huge, T.huge_chunk_start.get(),
-                                               T.n_huge_chunks, map, nc, wbits, m_small, hoff.get(),
-                                               keys.get(), vals.get());
-      else
-        launch(k_emit_chunks<false>, hb, 256, 0, s, v, T.huge.get(), T.n_huge, T.huge_chunk_start.get(),
-                                                T.n_huge_chunks, map, nc, wbits, m_small, hoff.get(),
-                                                keys.get(), vals.get());
+    const bool narrow = ew_sum_bound(g) < ((int64_t)1 << 31);
+
+    // members by coarse vertex, and the first table size of each
+    Buf<int32_t> members(n, s), lists((kAggSizes + 1) * nc, s);
+    Buf<int64_t> mstart(nc + 1, s);
+    // [0] cursor [1] largest weight [2] items; then the lists' lengths (int32)
+    Buf<int64_t> acc(3 + (kAggSizes + 2) / 2, s);
+    TP_CUDA(cudaMemsetAsync(acc.get(), 0, acc.n * sizeof(int64_t), s));
+    int32_t *cnt = reinterpret_cast<int32_t *>(acc.get() + 3);
+    {
+      Buf<int32_t> place(n, s), mcnt(nc, s);
+      Buf<unsigned long long> ent(nc, s);
+      TP_CUDA(cudaMemsetAsync(mcnt.get(), 0, nc * sizeof(int32_t), s));
+      TP_CUDA(cudaMemsetAsync(ent.get(), 0, nc * sizeof(unsigned long long), s));
+      launch(k_map, grid_for(n, 256), 256, 0, s, v, C, rank.get(), map, cg->vw.get(), place.get(),
+             mcnt.get(), ent.get());
+      exclusive_scan_i32_to_i64(mcnt.get(), mstart.get(), nc, s);
+      launch(k_members, grid_for(n, 256), 256, 0, s, map, place.get(), mstart.get(), n, members.get());
+      launch(k_agg_classes, grid_for(nc, 256), 256, 0, s, ent.get(), mcnt.get(), nc,
+             g->unit_vw ? cg->vw.get() : nullptr, lists.get(), cnt);
       TP_LAUNCH_CHECK();
     }
-    off.release();
-    hoff.release();
-    radix_sort_pairs(keys.get(), vals.get(), m, kbits, s, wbits);
-    // runs per tile, their offsets, then the coarse CSR
-    const int64_t ntiles = (m + kRleTile - 1) / kRleTile;
-    Buf<int64_t> toff(ntiles + 1, s);
-    const unsigned rb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)num_sms() * 16));
-    if (ntiles) {
-      launch(k_rle_count, rb, kRleThreads, 0, s, keys.get(), m, wbits, ntiles, toff.get());
+    rank.release();
+    int32_t hc[kAggSizes + 1];
+    TP_CUDA(cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
+    // lists can grow by those that move up from the smaller sizes
+    int64_t most[kAggSizes], sofar = 0;
+    for (int i = 0; i < kAggSizes; ++i) most[i] = sofar += hc[i];
+
+    // the tables' rows: no more entries than the graph has
+    Buf<int32_t> tkey(std::max<int64_t>(g->m2, 1), s);
+    Buf<uint32_t> tval32;
+    Buf<unsigned long long> tval64;
+    if (narrow) tval32.alloc(std::max<int64_t>(g->m2, 1), s);
+    else tval64.alloc(std::max<int64_t>(g->m2, 1), s);
+    Buf<int64_t> toff(nc, s);
+    cg->xadj.alloc(nc + 1, s);
+    TP_CUDA(cudaMemsetAsync(cg->xadj.get(), 0, (nc + 1) * sizeof(int64_t), s));
+    AggCtx c{};
+    c.g = v;
+    c.map = map;
+    c.members = members.get();
+    c.mstart = mstart.get();
+    c.nc = nc;
+    c.lists = lists.get();
+    c.cnt = cnt;
+    c.cursor = (unsigned long long *)acc.get();
+    c.max_w = (unsigned long long *)(acc.get() + 1);
+    c.out_key = tkey.get();
+    c.out_val = narrow ? (void *)tval32.get() : (void *)tval64.get();
+    c.toff = toff.get();
+    c.deg = cg->xadj.get();
+    if (comp) launch_agg<true, uint32_t>(c, most, s);
+    else if (narrow) launch_agg<false, uint32_t>(c, most, s);
+    else launch_agg<false, unsigned long long>(c, most, s);
+    int64_t ha[3 + (kAggSizes + 2) / 2];
+    TP_CUDA(cudaMemcpyAsync(ha, acc.get(), sizeof(ha), cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
+    const int64_t n_sorted = reinterpret_cast<const int32_t *>(ha + 3)[kAggSizes];
+    int64_t max_w = ha[1], m2 = ha[0], runs = 0;
+
+    // coarse vertices beyond the tables: keys, sort, run lengths
+    Buf<uint8_t> sorted;
+    Buf<int32_t> rkey, rrow;
+    Buf<int64_t> rval, rstart;
+    if (n_sorted) {
+      sorted.alloc(nc, s);
+      TP_CUDA(cudaMemsetAsync(sorted.get(), 0, nc, s));
+      launch(k_mark_sorted, grid_for(n_sorted, 256), 256, 0, s, lists.get() + kAggSizes * nc, n_sorted,
+             sorted.get());
+      Buf<uint64_t> items((size_t)(n + g->m2 / kChunkSize + 1), s);
+      unsigned long long *n_items = (unsigned long long *)(acc.get() + 2);
+      if (comp) launch(k_row_items<true>, grid_for(n, 256), 256, 0, s, v, map, sorted.get(), items.get(), n_items);
+      else launch(k_row_items<false>, grid_for(n, 256), 256, 0, s, v, map, sorted.get(), items.get(), n_items);
       TP_LAUNCH_CHECK();
+      const int64_t ni = (int64_t)read_scalar(n_items, s);
+      Buf<int64_t> off(ni + 1, s);
+      const unsigned ib = grid_for(ni * 32, 256);
+      if (ni) {
+        if (comp) launch(k_item_count<true>, ib, 256, 0, s, v, map, items.get(), ni, off.get());
+        else launch(k_item_count<false>, ib, 256, 0, s, v, map, items.get(), ni, off.get());
+        TP_LAUNCH_CHECK();
+      }
+      exclusive_scan_i64(off.get(), off.get(), ni, s);
+      const int64_t m = read_scalar(off.get() + ni, s);
+      // weights ride in the keys' low bits when the pair fits 64 bits
+      const bool weighted = !g->unit_ew;
+      const int kbits = bits_for((uint64_t)nc * (uint64_t)nc - 1);
+      const int wbits = weighted && kbits + bits_for((uint64_t)g->max_ew) <= 64
+                            ? bits_for((uint64_t)g->max_ew)
+                            : 0;
+      Buf<uint64_t> keys(std::max<int64_t>(m, 1), s), vals;
+      if (weighted && !wbits) vals.alloc(std::max<int64_t>(m, 1), s);
+      if (ni) {
+        if (comp)
+          launch(k_item_emit<true>, ib, 256, 0, s, v, map, items.get(), ni, nc, wbits, off.get(),
+                 keys.get(), vals.get());
+        else
+          launch(k_item_emit<false>, ib, 256, 0, s, v, map, items.get(), ni, nc, wbits, off.get(),
+                 keys.get(), vals.get());
+        TP_LAUNCH_CHECK();
+      }
+      items.release();
+      off.release();
+      radix_sort_pairs(keys.get(), vals.get(), m, kbits, s, wbits);
+      const int64_t ntiles = (m + kRleTile - 1) / kRleTile;
+      Buf<int64_t> rtile(ntiles + 1, s);
+      const unsigned rb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)num_sms() * 16));
+      if (ntiles) {
+        launch(k_rle_count, rb, kRleThreads, 0, s, keys.get(), m, wbits, ntiles, rtile.get());
+        TP_LAUNCH_CHECK();
+      }
+      exclusive_scan_i64(rtile.get(), rtile.get(), ntiles, s);
+      runs = read_scalar(rtile.get() + ntiles, s);
+      rkey.alloc(std::max<int64_t>(runs, 1), s);
+      rrow.alloc(std::max<int64_t>(runs, 1), s);
+      rval.alloc(std::max<int64_t>(runs, 1), s);
+      rstart.alloc(nc + 1, s);
+      TP_CUDA(cudaMemsetAsync(rval.get(), 0, rval.n * sizeof(int64_t), s));
+      TP_CUDA(cudaMemsetAsync(rstart.get(), 0, (nc + 1) * sizeof(int64_t), s));
+      if (ntiles) {
+        launch(k_rle_write, rb, kRleThreads, 0, s, keys.get(), vals.get(), m, nc, wbits, ntiles,
+               rtile.get(), rkey.get(), rval.get(), rrow.get(), rstart.get());
+        TP_LAUNCH_CHECK();
+      }
+      keys.release();
+      vals.release();
+      launch(k_add_i64, grid_for(nc, 256), 256, 0, s, rstart.get(), nc, cg->xadj.get());
+      TP_LAUNCH_CHECK();
+      exclusive_scan_i64(rstart.get(), rstart.get(), nc, s);
+      max_w = std::max(max_w, max_i64(rval.get(), runs, s));
+      m2 += runs;
     }
-    exclusive_scan_i64(toff.get(), toff.get(), ntiles, s);
-    int64_t m2 = read_scalar(toff.get() + ntiles, s);
+    exclusive_scan_i64(cg->xadj.get(), cg->xadj.get(), nc, s);
     cg->m2 = m2;
+    cg->max_ew = max_w;
     cg->adj.alloc(m2 + kAdjPad, s);
     TP_CUDA(cudaMemsetAsync(cg->adj.get() + m2, 0, kAdjPad * sizeof(int32_t), s));
     cg->ew.alloc(m2, s);
-    cg->xadj.alloc(nc + 1, s);
-    if (m2) TP_CUDA(cudaMemsetAsync(cg->ew.get(), 0, m2 * sizeof(int64_t), s));
-    TP_CUDA(cudaMemsetAsync(cg->xadj.get(), 0, (nc + 1) * sizeof(int64_t), s));
-    if (ntiles) {
-      launch(k_rle_write, rb, kRleThreads, 0, s, keys.get(), vals.get(), m, nc, wbits, ntiles,
-             toff.get(), cg->adj.get(), cg->ew.get(), cg->xadj.get());
+    if (m2) {
+      const int lanes = m2 / nc > 24 ? 32 : 8;
+      const unsigned gr = grid_for(nc * lanes, 256);
+      if (narrow)
+        launch(k_copy_rows<uint32_t>, gr, 256, 0, s, toff.get(), cg->xadj.get(), sorted.get(), nc,
+               lanes, tkey.get(), tval32.get(), cg->adj.get(), cg->ew.get());
+      else
+        launch(k_copy_rows<unsigned long long>, gr, 256, 0, s, toff.get(), cg->xadj.get(), sorted.get(),
+               nc, lanes, tkey.get(), tval64.get(), cg->adj.get(), cg->ew.get());
+      if (runs)
+        launch(k_copy_runs, grid_for(runs, 256), 256, 0, s, rstart.get(), cg->xadj.get(), runs,
+               rrow.get(), rkey.get(), rval.get(), cg->adj.get(), cg->ew.get());
       TP_LAUNCH_CHECK();
     }
-    keys.release();
-    vals.release();
-    exclusive_scan_i64(cg->xadj.get(), cg->xadj.get(), nc, s);
-    cg->max_ew = max_i64(cg->ew.get(), m2, s);  // synchronises
+    TP_CUDA(cudaStreamSynchronize(s));
   } catch (...) {
     delete cg;
     throw;

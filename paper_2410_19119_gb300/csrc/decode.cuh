@@ -12,6 +12,10 @@
 
 namespace tp {
 
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // Single-thread VarInt read (up to 10 bytes). Returns bytes consumed. The
 // stream is padded with zero bytes, so all ten bytes a VarInt may span are
 // loaded at once (one memory round trip instead of one per byte).
@@ -312,6 +316,71 @@ __device__ __forceinline__ int64_t thread_neighbours(const GView &g, int64_t u, 
     shift = 0;
   }
   return cnt;
+}
+
+// Decodes u's compressed record into its shared-memory column: the raw
+// values (first the signed first neighbour, then the gaps) go to
+// col[i * 32]; returns the degree. The record's first 80 bytes are
+// loaded at once as five 16-byte groups from its 16-byte aligned start, so
+// no load waits on another (a longer record, up to 165 bytes at degree 32
+// with five-byte gaps, loads its further groups as the decoder reaches
+// them), and consumed a 32-bit word at a time. Bytes
+// before the record are turned into value ends and, like the header, are
+// written to slot 0, which the first neighbour then overwrites; bytes after
+// it are turned into continuation bytes, so they end no value.
+// COUNT: the degree is not known to be at most kLaneMaxDeg; the first
+// kLaneMaxDeg values are kept and the record's degree is returned (for records
+// without a chunk table).
+template <bool LONG, bool COUNT = false>
+__device__ __forceinline__ int lane_decode(const GView &g, uint64_t b, uint64_t e, uint32_t *col) {
+  constexpr int G = 5;  // 80-byte window
+  const uint64_t ws = b & ~(uint64_t)15;
+  const int p0 = (int)(b - ws), endp = (int)(e - ws);
+  const uint4 *src = reinterpret_cast<const uint4 *>(g.bytes + ws);
+  uint4 q[G];
+#pragma unroll
+  for (int j = 0; j < G; ++j) q[j] = 16 * j < endp ? __ldcs(src + j) : make_uint4(0, 0, 0, 0);
+  int fi = 0;         // words of q[0] already taken
+  int nextg = G;      // next 16-byte group to load (records longer than the window)
+  auto pop = [&]() -> uint32_t {
+    const uint32_t w = fi == 0 ? q[0].x : fi == 1 ? q[0].y : fi == 2 ? q[0].z : q[0].w;
+    if (++fi == 4) {
+#pragma unroll
+      for (int j = 0; j + 1 < G; ++j) q[j] = q[j + 1];
+      if (LONG) {
+        q[G - 1] = 16 * nextg < endp ? __ldcs(src + nextg) : make_uint4(0, 0, 0, 0);
+        ++nextg;
+      }
+      fi = 0;
+    }
+    return w;
+  };
+  int wi = p0 >> 2;
+  for (int j = 0; j < wi; ++j) pop();
+  // leading bytes of the first word: forced value ends
+  uint32_t lead = 0x80808080u & ((1u << (8 * (p0 & 3))) - 1u);
+  int idx = -1 - (p0 & 3);  // value index; < 0 for the leading bytes and the header
+  uint32_t acc = 0;
+  int accb = 0;
+  for (; 4 * wi < endp; ++wi) {
+    uint32_t w = pop() & ~lead;
+    lead = 0;
+    const int vhi = endp - 4 * wi;  // bytes of this word inside the record
+    if (vhi < 4) w |= 0x80808080u & ~((1u << (8 * vhi)) - 1u);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t by = (w >> (8 * j)) & 0xffu;
+      acc |= (by & 0x7fu) << accb;
+      accb += 7;
+      if (!(by & 0x80u)) {
+        col[(COUNT ? min(max(idx, 0), kLaneMaxDeg - 1) : max(idx, 0)) * 32] = acc;
+        ++idx;
+        acc = 0;
+        accb = 0;
+      }
+    }
+  }
+  return COUNT ? max(idx, 0) : min(max(idx, 0), kLaneMaxDeg);
 }
 
 }  // namespace tp

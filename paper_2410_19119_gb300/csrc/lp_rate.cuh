@@ -450,72 +450,6 @@ __device__ __forceinline__ bool lane_better(const LaneCand &a, const LaneCand &b
   return better(a.r, a.t, a.x, b.r, b.t, b.x);
 }
 
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-// Decodes u's compressed record into its shared-memory column: the raw
-// values (first the signed first neighbour, then the gaps) go to
-// col[i * 32]; returns the degree. The record's first 80 bytes are
-// loaded at once as five 16-byte groups from its 16-byte aligned start, so
-// no load waits on another (a longer record, up to 165 bytes at degree 32
-// with five-byte gaps, loads its further groups as the decoder reaches
-// them), and consumed a 32-bit word at a time. Bytes
-// before the record are turned into value ends and, like the header, are
-// written to slot 0, which the first neighbour then overwrites; bytes after
-// it are turned into continuation bytes, so they end no value.
-template <bool LONG>
-__device__ __forceinline__ int lane_decode(const GView &g, uint64_t b, uint64_t e, uint32_t *col) {
-  constexpr int G = 5;  // 80-byte window
-  const uint64_t ws = b & ~(uint64_t)15;
-  const int p0 = (int)(b - ws), endp = (int)(e - ws);
-  const uint4 *src = reinterpret_cast<const uint4 *>(g.bytes + ws);
-  uint4 q[G];
-#pragma unroll
-  for (int j = 0; j < G; ++j) q[j] = 16 * j < endp ? __ldcs(src + j) : make_uint4(0, 0, 0, 0);
-  int fi = 0;         // words of q[0] already taken
-  int nextg = G;      // next 16-byte group to load (records longer than the window)
-  auto pop = [&]() -> uint32_t {
-    const uint32_t w = fi == 0 ? q[0].x : fi == 1 ? q[0].y : fi == 2 ? q[0].z : q[0].w;
-    if (++fi == 4) {
-#pragma unroll
-      for (int j = 0; j + 1 < G; ++j) q[j] = q[j + 1];
-      if (LONG) {
-        q[G - 1] = 16 * nextg < endp ? __ldcs(src + nextg) : make_uint4(0, 0, 0, 0);
-        ++nextg;
-      }
-      fi = 0;
-    }
-    return w;
-  };
-  int wi = p0 >> 2;
-  for (int j = 0; j < wi; ++j) pop();
-  // leading bytes of the first word: forced value ends
-  uint32_t lead = 0x80808080u & ((1u << (8 * (p0 & 3))) - 1u);
-  int idx = -1 - (p0 & 3);  // value index; < 0 for the leading bytes and the header
-  uint32_t acc = 0;
-  int accb = 0;
-  for (; 4 * wi < endp; ++wi) {
-    uint32_t w = pop() & ~lead;
-    lead = 0;
-    const int vhi = endp - 4 * wi;  // bytes of this word inside the record
-    if (vhi < 4) w |= 0x80808080u & ~((1u << (8 * vhi)) - 1u);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t by = (w >> (8 * j)) & 0xffu;
-      acc |= (by & 0x7fu) << accb;
-      accb += 7;
-      if (!(by & 0x80u)) {
-        col[max(idx, 0) * 32] = acc;
-        ++idx;
-        acc = 0;
-        accb = 0;
-      }
-    }
-  }
-  return min(max(idx, 0), kLaneMaxDeg);
-}
-
 // Record range of a compressed lane-tier vertex: from the bucket list when
 // it carries the ranges (coalesced with the vertex ids), else the offsets.
 __device__ __forceinline__ void lane_record(const GView &g, const uint64_t *rec, int64_t pos,
