@@ -157,6 +157,21 @@ __device__ __forceinline__ AggMember agg_member(const AggCtx &c, int64_t m, int6
   return r;
 }
 
+// A warp's inter-cluster entries on their way to the table (compressed graphs,
+// which are meshes here: skewed ones are decoded first). Most entries of a mesh
+// lie inside the cluster (about two in three), so those that do not are queued
+// and added 32 at a time with every lane busy: adding them where they were
+// found ran the probing code for a third of the lanes, 16 times a row batch,
+// unrolled beyond the instruction cache (mesh of 4.2 M vertices: 0.70 -> 0.60
+// ms). CSR levels, with more entries between clusters, fewer instructions per
+// entry and more warps, are faster adding directly (R-MAT 2^22: 1.7 against 2.0 ms).
+constexpr int kAggStep = 4;  // entries a lane has in flight
+template <class V>
+struct AggQueue {
+  int32_t x[32 + 32 * kAggStep];
+  V w[32 + 32 * kAggStep];
+};
+
 // One warp sums the rows of members m, m + step, ... (32 at a time) of coarse
 // vertex a into the table; fill() tells the distinct neighbours so far (of the
 // warp or the block), add_fill(k) counts k more. Rows of up to 32 entries are
@@ -166,10 +181,32 @@ __device__ __forceinline__ AggMember agg_member(const AggCtx &c, int64_t m, int6
 template <bool COMP, class V, class Fill, class AddFill, class Row>
 __device__ __forceinline__ bool agg_rows(const AggCtx &c, int32_t a, int64_t m, int64_t mend,
                                          int64_t step, int32_t *keys, V *vals, int logc,
-                                         uint32_t *col, int limit, AggMember first, Fill fill,
-                                         AddFill add_fill, Row row) {
-  constexpr int U = COMP ? 8 : 4;
+                                         uint32_t *col, AggQueue<V> *qu, int limit,
+                                         AggMember first, Fill fill, AddFill add_fill, Row row) {
+  constexpr int U = kAggStep;
   const int lane = lane_id();
+  int nq = 0;  // queued entries
+  // adds queued entries 32 at a time, down to fewer than `keep`; whether the table holds
+  auto drain = [&](int keep) -> bool {
+    __syncwarp();
+    int at = 0;
+    for (; nq - at >= keep; at += 32) {
+      const int i = at + lane;
+      const int res = i < nq ? agg_add<V>(keys, vals, logc, qu->x[i], qu->w[i]) : 0;
+      const unsigned claimed = __ballot_sync(kFull, res == 1);
+      if (claimed) add_fill(__popc(claimed));
+      if (__any_sync(kFull, res == 2) || fill() > limit) return false;
+    }
+    if (at) {  // the rest to the front
+      const bool mine = at + lane < nq;
+      const int32_t mx = mine ? qu->x[at + lane] : 0;
+      const V mw = mine ? qu->w[at + lane] : V(0);
+      __syncwarp();
+      if (mine) qu->x[lane] = mx, qu->w[lane] = mw;
+      nq = max(nq - at, 0);
+    }
+    return true;
+  };
   for (AggMember mem = first; m < mend; m += step, mem = agg_member<COMP>(c, m, mend)) {
     const bool in = m + lane < mend;
     const int32_t u = mem.u;
@@ -215,23 +252,38 @@ __device__ __forceinline__ bool agg_rows(const AggCtx &c, int32_t a, int64_t m, 
       }
 #pragma unroll
       for (int r = 0; r < U; ++r) x[r] = x[r] >= 0 ? c.map[x[r]] : a;
-      unsigned claimed = 0;
-      bool full = false;
+      if constexpr (COMP) {
 #pragma unroll
-      for (int r = 0; r < U; ++r)
-        if (x[r] != a) {
-          const int res = agg_add<V>(keys, vals, logc, x[r], w[r]);
-          claimed += res == 1;
-          full |= res == 2;
+        for (int r = 0; r < U; ++r) {
+          const unsigned m = __ballot_sync(kFull, x[r] != a);
+          if (m == 0) continue;
+          if (x[r] != a) {
+            const int at = nq + __popc(m & lanemask_lt());
+            qu->x[at] = x[r];
+            qu->w[at] = w[r];
+          }
+          nq += __popc(m);
         }
-      claimed = __reduce_add_sync(kFull, claimed);
-      if (claimed) add_fill((int)claimed);
-      if (__any_sync(kFull, full) || fill() > limit) return false;
+        if (nq >= 32 && !drain(32)) return false;
+      } else {
+        unsigned claimed = 0;
+        bool full = false;
+#pragma unroll
+        for (int r = 0; r < U; ++r)
+          if (x[r] != a) {
+            const int res = agg_add<V>(keys, vals, logc, x[r], w[r]);
+            claimed += res == 1;
+            full |= res == 2;
+          }
+        claimed = __reduce_add_sync(kFull, claimed);
+        if (claimed) add_fill((int)claimed);
+        if (__any_sync(kFull, full) || fill() > limit) return false;
+      }
     }
     for (unsigned q = wides; q; q &= q - 1)
       if (!row(__shfl_sync(kFull, u, __ffs(q) - 1))) return false;
   }
-  return true;
+  return !COMP || nq == 0 || drain(1);
 }
 
 // A long row, or of a CSR row the pieces of 128 entries number first, first +
@@ -306,11 +358,13 @@ struct AggWarp {
   };
   int32_t keys[1 << agg_log(SIZE)];
   V vals[1 << agg_log(SIZE)];
+  AggQueue<V> queue[COMP ? 1 : 0];
 };
 __host__ __device__ constexpr int agg_warps(int size) { return size == 0 ? 8 : 4; }
 
 template <bool COMP, int SIZE, class V>
-__global__ void __launch_bounds__(32 * agg_warps(SIZE)) k_agg_warp(AggCtx c) {
+__global__ void __launch_bounds__(32 * agg_warps(SIZE), SIZE == 0 && !COMP ? 6 : 3)
+    k_agg_warp(AggCtx c) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int L = agg_log(SIZE), SLOTS = 1 << L;
   using Warp = AggWarp<COMP, SIZE, V>;
@@ -341,7 +395,7 @@ __global__ void __launch_bounds__(32 * agg_warps(SIZE)) k_agg_warp(AggCtx c) {
     auto fill = [&] { return n_fill; };
     auto add_fill = [&](int k) { n_fill += k; };
     const bool ok = agg_rows<COMP, V>(
-        c, a, m0, m1, 32, s.keys, s.vals, L, s.col + lane, agg_fill(SIZE), mem, fill, add_fill,
+        c, a, m0, m1, 32, s.keys, s.vals, L, s.col + lane, s.queue, agg_fill(SIZE), mem, fill, add_fill,
         [&](int32_t u) {
           return agg_long_row<COMP, V>(c, a, u, 0, 1, s.keys, s.vals, L, agg_fill(SIZE), fill, add_fill);
         });
@@ -418,9 +472,13 @@ __global__ void __launch_bounds__(32 * agg_warps(SIZE)) k_agg_warp(AggCtx c) {
 constexpr int64_t kAggDecodeDeg = 1024;  // compressed graphs beyond this degree are decoded first
 constexpr int kAggThreads = 256;
 constexpr int kAggWide = 256;
+// The largest table with 64-bit sums has half the slots.
+template <class V>
+__host__ __device__ constexpr int agg_block_log(int size) {
+  return size == 3 && sizeof(V) == 8 ? 13 : agg_log(size);
+}
 template <class V>
 __host__ __device__ constexpr int agg_block_fill(int size) {
-  // the largest table with 64-bit sums: items of half the size beside it
   return size == 3 && sizeof(V) == 8 ? 4096 : agg_fill(size);
 }
 template <class V>
@@ -429,14 +487,14 @@ __host__ __device__ constexpr int agg_block_items(int size) {
 }
 template <bool COMP, class V>
 __host__ __device__ constexpr size_t agg_block_smem(int size) {
-  return ((size_t)1 << agg_log(size)) * (4 + sizeof(V)) + 8 * (size_t)agg_block_items<V>(size) +
+  return ((size_t)1 << agg_block_log<V>(size)) * (4 + sizeof(V)) + 8 * (size_t)agg_block_items<V>(size) +
          (COMP && size == 2 ? (size_t)4 * kLaneMaxDeg * kAggThreads : 0);
 }
 
 template <bool COMP, int SIZE, class V>
-__global__ void __launch_bounds__(kAggThreads) k_agg_block(AggCtx c) {
+__global__ void __launch_bounds__(kAggThreads, SIZE == 2 ? 3 : 1) k_agg_block(AggCtx c) {
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int L = agg_log(SIZE), SLOTS = 1 << L, FILL = agg_block_fill<V>(SIZE);
+  constexpr int L = agg_block_log<V>(SIZE), SLOTS = 1 << L, FILL = agg_block_fill<V>(SIZE);
   constexpr int ITEMS = agg_block_items<V>(SIZE);
   uint64_t *items = reinterpret_cast<uint64_t *>(smem);
   V *vals = reinterpret_cast<V *>(items + ITEMS);
@@ -447,6 +505,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_block(AggCtx c) {
                              : reinterpret_cast<uint32_t *>(items);
   static_assert(8 * ITEMS >= 4 * kLaneMaxDeg * kAggThreads, "columns fit where the items go");
   __shared__ int32_t s_fill, s_fail, s_d, s_wide, s_next;
+  __shared__ AggQueue<V> queue[COMP ? kAggThreads / 32 : 1];
   __shared__ int32_t wide[kAggWide];  // long rows, shared out over the warps after the others
   __shared__ unsigned long long s_base;
   const int tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
@@ -465,8 +524,8 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_block(AggCtx c) {
       __syncwarp();
     };
     bool ok = agg_rows<COMP, V>(
-        c, a, m0, m1, kAggThreads, keys, vals, L, cols + (size_t)w * kLaneMaxDeg * 32 + lane, FILL,
-        agg_member<COMP>(c, m0, m1), fill, add_fill, [&](int32_t u) {
+        c, a, m0, m1, kAggThreads, keys, vals, L, cols + (size_t)w * kLaneMaxDeg * 32 + lane,
+        queue + (COMP ? w : 0), FILL, agg_member<COMP>(c, m0, m1), fill, add_fill, [&](int32_t u) {
           int at = 0;
           if (lane == 0) {
             at = atomicAdd(&s_wide, 1);
