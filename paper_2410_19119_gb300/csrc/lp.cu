@@ -944,8 +944,13 @@ double tier_round_bytes(const tp_graph *g, int64_t n_t, int64_t e_t) {
   return adj + 4.0 * (double)e_t + 12.0 * (double)n_t;
 }
 
+// Entries in the tiers above the small one from which their kernels go side by
+// side: a fork and join cost about 10 us of launches per sub-round.
+constexpr int64_t kForkEntries = (int64_t)1 << 22;
+
 template <int MODE>
-void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
+void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s,
+                TierStreams *side = nullptr) {
   build_tiers(g, p, s);
   ensure_hub_tables(g, s);
   TierCache &T = g->tiers;
@@ -977,6 +982,12 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   const double per_launch = MODE == M_LP && c.S > 0 ? 1.0 / c.S : 0.0;
   const int64_t n_lane = MODE == M_REBAL ? 0 : T.count[TIER_LANE];
   const int64_t n_small = T.count[TIER_SMALL] + (MODE == M_REBAL ? T.count[TIER_LANE] : 0);
+  const bool fork = side && !prof &&
+                    T.edges[TIER_MID] + T.edges[TIER_BIG] + T.edges[TIER_HUGE] >= kForkEntries &&
+                    side->make();
+  cudaStream_t s_mid = fork ? side->st[0] : s, s_big = fork ? side->st[1] : s,
+               s_big2 = fork ? side->st[2] : s, s_huge = fork ? side->st[3] : s;
+  if (fork) side->begin(s);
   if (n_lane > 0) {
     if (prof) prof_begin(PF_RATE_LANE, s);
     constexpr int LM = MODE == M_REBAL ? M_LP : MODE;
@@ -1019,7 +1030,7 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   // few labels: direct tables for every tier above the small one, and for the
   // small one where k counters are no more than its largest hash table
   const bool direct = MODE != M_FAV && c.kmax > 0 && c.kmax <= kDirectMax;
-  auto run_direct = [&](const int32_t *list, int64_t cnt, int t) {
+  auto run_direct = [&](const int32_t *list, int64_t cnt, int t, cudaStream_t s) {
     RateCtx m = c;
     m.list = list;
     m.list_n = cnt;
@@ -1036,7 +1047,7 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   if (n_small > 0) {
     if (prof) prof_begin(PF_RATE_SMALL, s);
     if (MODE != M_REBAL && direct && c.kmax <= 1 << kSmallLog) {
-      run_direct(T.small.get(), T.n_small, 0);
+      run_direct(T.small.get(), T.n_small, 0, s);
     } else {
       int wpb = p.warps_per_block >= 1 && p.warps_per_block <= 16 ? p.warps_per_block : 8;
       size_t sm = (narrow ? sizeof(WarpSmem<kSmallLog, uint32_t>) : sizeof(WarpSmem<kSmallLog>)) * wpb;
@@ -1061,10 +1072,11 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
     if (prof) prof_end(PF_RATE_SMALL, s, per_launch * tier_round_bytes(g, T.count[TIER_SMALL], T.edges[TIER_SMALL]));
   }
   if (T.n_mid + T.n_mid2 > 0) {
+    cudaStream_t s = s_mid;
     if (prof) prof_begin(PF_RATE_MID, s);
     auto run = [&](const int32_t *list, int64_t cnt, int t, bool big_tables) {
       if (!cnt) return;
-      if (direct) return run_direct(list, cnt, t);
+      if (direct) return run_direct(list, cnt, t, s);
       RateCtx m = c;
       m.list = list;
       m.list_n = cnt;
@@ -1093,7 +1105,7 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
   }
   if (T.n_big0 + T.n_big1 + T.n_big + T.n_big2 > 0) {
     if (prof) prof_begin(PF_RATE_BIG, s);
-    auto run = [&](const int32_t *list, int64_t cnt, int maxlog, int t) {
+    auto run = [&](const int32_t *list, int64_t cnt, int maxlog, int t, cudaStream_t s) {
       if (!cnt) return;
       RateCtx m = c;
       m.list = list;
@@ -1118,14 +1130,15 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
 #undef TP_BLK
       TP_LAUNCH_CHECK();
     };
-    if (T.n_big0 && direct) run_direct(T.big0.get(), T.n_big0, 3);
-    else run(T.big0.get(), T.n_big0, kBlockTinyLog, 3);
-    run(T.big1.get(), T.n_big1, kBlockMidLog, 4);
-    run(T.big.get(), T.n_big, kBlockSmallLog, 5);
-    run(T.big2.get(), T.n_big2, kBlockBigLog, 6);
+    if (T.n_big0 && direct) run_direct(T.big0.get(), T.n_big0, 3, s_big);
+    else run(T.big0.get(), T.n_big0, kBlockTinyLog, 3, s_big);
+    run(T.big1.get(), T.n_big1, kBlockMidLog, 4, s_big);
+    run(T.big.get(), T.n_big, kBlockSmallLog, 5, s_big2);
+    run(T.big2.get(), T.n_big2, kBlockBigLog, 6, s_big2);
     if (prof) prof_end(PF_RATE_BIG, s, per_launch * tier_round_bytes(g, T.n_big0 + T.n_big1 + T.n_big + T.n_big2, T.edges[TIER_BIG]));
   }
   if (T.n_huge > 0) {
+    cudaStream_t s = s_huge;
     if (prof) prof_begin(PF_RATE_HUGE, s);
     RateCtx m = c;
     m.list = T.huge.get();
@@ -1159,6 +1172,7 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s) {
     TP_LAUNCH_CHECK();
     if (prof) prof_end(PF_RATE_HUGE, s, per_launch * tier_round_bytes(g, T.n_huge, T.edges[TIER_HUGE]));
   }
+  if (fork) side->end(s);
 }
 
 template <class K>
@@ -1463,6 +1477,46 @@ void lp_bucket(tp_graph *g, LpWork &w, uint64_t rk, int32_t S, const tp_params &
   if (tiers) tier_buckets(g, w, S, stream);
 }
 
+bool TierStreams::make() {
+  if (made) return st[0] != nullptr;
+  made = true;
+  bool ok = cudaEventCreateWithFlags(&forked, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < kN && ok; ++i)
+    ok = cudaStreamCreateWithFlags(&st[i], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&joined[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    (void)cudaGetLastError();
+    for (int i = 0; i < kN; ++i) {
+      if (st[i]) cudaStreamDestroy(st[i]);
+      st[i] = nullptr;
+    }
+  }
+  return ok;
+}
+
+void TierStreams::begin(cudaStream_t s) {
+  TP_CUDA(cudaEventRecord(forked, s));
+  open = true;
+  for (int i = 0; i < kN; ++i) TP_CUDA(cudaStreamWaitEvent(st[i], forked, 0));
+}
+
+void TierStreams::end(cudaStream_t s) {
+  for (int i = 0; i < kN; ++i) {
+    TP_CUDA(cudaEventRecord(joined[i], st[i]));
+    TP_CUDA(cudaStreamWaitEvent(s, joined[i], 0));
+  }
+  open = false;
+}
+
+TierStreams::~TierStreams() {
+  for (int i = 0; i < kN; ++i) {
+    if (open && st[i]) cudaStreamSynchronize(st[i]);
+    if (joined[i]) cudaEventDestroy(joined[i]);
+    if (st[i]) cudaStreamDestroy(st[i]);
+  }
+  if (forked) cudaEventDestroy(forked);
+}
+
 void LpWork::init(int64_t n_vertices, int64_t n_labels, cudaStream_t s) {
   if (n_vertices <= n && n_labels <= nlabels) return;
   n = std::max(n, n_vertices);
@@ -1581,7 +1635,7 @@ void lp_subround(tp_graph *g, const LpState &st, LpWork &w, uint64_t rk, int32_t
       c.hs_item = w.hs_item.get();
     }
   }
-  rate_tiers<M_LP>(g, c, p, stream);
+  rate_tiers<M_LP>(g, c, p, stream, &w.streams);
   prof_begin(PF_APPROVE, stream);
   if (approval) {
     TP_CUDA(cudaGraphLaunch(approval, stream));

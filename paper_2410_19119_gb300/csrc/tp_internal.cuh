@@ -407,6 +407,24 @@ struct LpState {
   int32_t k = 0, kmax = 0;  // labels are blocks: how many, the most of any graph (0: clusters)
   SegLp seg{};
 };
+// Side streams on which the degree tiers of one sub-round are rated next to
+// each other: they only read the labels and append movers, and each alone
+// leaves most of the GPU waiting on its loads. begin() makes them wait for the
+// main stream, end() the main stream for them; a fork left open (an error in
+// between) is waited for before the workspace goes.
+struct TierStreams {
+  static constexpr int kN = 4;
+  cudaStream_t st[kN] = {};
+  cudaEvent_t forked = nullptr, joined[kN] = {};
+  bool made = false, open = false;
+  bool make();  // false: could not (everything then runs on the main stream)
+  void begin(cudaStream_t s);
+  void end(cudaStream_t s);
+  TierStreams() = default;
+  TierStreams(const TierStreams &) = delete;
+  TierStreams &operator=(const TierStreams &) = delete;
+  ~TierStreams();
+};
 // Workspace for sub-rounds on one graph (per-label counters + mover lists).
 struct LpWork {
   int64_t nlabels = 0, n = 0;
@@ -440,6 +458,7 @@ struct LpWork {
   // huge tier, in bucket order of its hubs: prefix of chunk and segment
   // counts (n_huge + 1) and the items themselves (hub position << 32 | index)
   Buf<int64_t> hc_pre, hs_pre, hc_item, hs_item;
+  TierStreams streams;  // last: gone before the buffers
   void init(int64_t n_vertices, int64_t n_labels, cudaStream_t s);
 };
 // approval (nullable): a CUDA graph of this level's approval kernels to
