@@ -946,7 +946,7 @@ double tier_round_bytes(const tp_graph *g, int64_t n_t, int64_t e_t) {
 
 // Entries in the tiers above the small one from which their kernels go side by
 // side: a fork and join cost about 10 us of launches per sub-round.
-constexpr int64_t kForkEntries = (int64_t)1 << 22;
+constexpr int64_t kForkEntries = (int64_t)1 << 19;
 
 template <int MODE>
 void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s,
