@@ -392,33 +392,7 @@ __global__ void __launch_bounds__(kTileThreads) k_validate(GView g, const int32_
   if (threadIdx.x == 0 && diff) atomicAdd(balance, (unsigned long long)diff);
 }
 
-__global__ void k_zip_degrees(GView g, int64_t *deg) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < g.n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    uint64_t a, b;
-    read_varint(g.bytes + off_at(g, u), a);
-    read_varint(g.bytes + off_at(g, u + 1), b);
-    deg[u] = (int64_t)(b - a);
-  }
-}
-
-__global__ void k_csr_degrees(const int64_t *xadj, int64_t n, int64_t *deg) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x)
-    deg[u] = xadj[u + 1] - xadj[u];
-}
-
 }  // namespace
-
-void compute_degrees(const tp_graph *g, int64_t *d_deg, cudaStream_t s) {
-  if (g->n == 0) return;
-  GView v = view(g);
-  if (g->compressed)
-    launch(k_zip_degrees, grid_for(g->n, 256), 256, 0, s, v, d_deg);
-  else
-    launch(k_csr_degrees, grid_for(g->n, 256), 256, 0, s, g->xadj.get(), g->n, d_deg);
-  TP_LAUNCH_CHECK();
-}
 
 // ---------------------------------------------------------------- tiers
 namespace {
@@ -428,80 +402,144 @@ namespace {
 // common (skewed graphs: long gaps), else the warp tier rates them.
 constexpr uint64_t kLaneShortRecord = 65;
 
-// Lane-tier candidates (degree <= lane_max) and how many have long records.
-__global__ void k_lane_records(const int64_t *deg, int64_t n, int32_t lane_max,
-                               const uint32_t *off32, const uint64_t *off64,
-                               unsigned long long *cnt) {
-  unsigned long long a = 0, l = 0;
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    if (deg[u] > lane_max) continue;
-    const uint64_t len = off32 ? (uint64_t)(off32[u + 1] - off32[u]) : off64[u + 1] - off64[u];
-    ++a;
-    l += len > kLaneShortRecord;
+// Degrees of a compressed graph from its headers (a lane reads its own, the
+// next one's comes from the next lane), the number of lane-tier candidates
+// (degree <= lane_max) and how many of them have long records.
+__global__ void __launch_bounds__(256) k_zip_degrees(GView g, int32_t lane_max, int64_t *deg,
+                                                     unsigned long long *cnt) {
+  __shared__ uint32_t sa[8], sl[8];
+  const int lane = lane_id();
+  uint32_t a = 0, l = 0;
+  for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x; u0 < g.n;
+       u0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t u = u0 + threadIdx.x;
+    const bool in = u < g.n;
+    uint64_t first = 0, rb = 0;
+    if (u <= g.n) {
+      rb = off_at(g, u);
+      read_varint(g.bytes + rb, first);
+    }
+    uint64_t next = __shfl_down_sync(kFull, first, 1), re = __shfl_down_sync(kFull, rb, 1);
+    if (!in) continue;  // (a whole warp, or lanes behind every shuffle source)
+    if (lane == 31) {
+      re = off_at(g, u + 1);
+      read_varint(g.bytes + re, next);
+    }
+    const int64_t d = (int64_t)(next - first);
+    deg[u] = d;
+    if (d <= lane_max) ++a, l += re - rb > kLaneShortRecord;
   }
-  a = warp_sum(a);
-  l = warp_sum(l);
-  if (lane_id() == 0 && a) atomicAdd(&cnt[0], a);
-  if (lane_id() == 0 && l) atomicAdd(&cnt[1], l);
+  a = __reduce_add_sync(kFull, a);
+  l = __reduce_add_sync(kFull, l);
+  if (lane == 0) sa[threadIdx.x >> 5] = a, sl[threadIdx.x >> 5] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) a += sa[w], l += sl[w];
+    if (a) atomicAdd(&cnt[0], (unsigned long long)a);
+    if (l) atomicAdd(&cnt[1], (unsigned long long)l);
+  }
 }
 
-__global__ void k_classify(const int64_t *deg, int64_t n, int32_t lane_max, int32_t small_max,
-                           int32_t mid_max, const uint32_t *off32, const uint64_t *off64,
-                           bool long_records, uint8_t *tier, int32_t *flag_small,
-                           int32_t *flag_mid, int32_t *flag_mid2, int32_t *flag_big0,
-                           int32_t *flag_big1, int32_t *flag_big,
-                           int32_t *flag_big2, int32_t *flag_huge, unsigned long long *stats) {
-  int64_t e[5] = {0, 0, 0, 0, 0}, c[5] = {0, 0, 0, 0, 0};
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x) {
-    int64_t d = deg[u];
+// Tier lists: class 0 is the lane tier (no list), 1..8 the lists of TierCache
+// in its order. Block b owns kTierSpan vertices and counts its vertices per
+// class (cnt[class * nblocks + b]; an exclusive scan of the counts of classes
+// 1..8 gives every block its place in one array of all lists) and adds up
+// entries and vertices per tier. One pass and one scan for all lists; a flag
+// array, a scan, a readback and a compaction per list took 30 launches and ten
+// synchronisations.
+constexpr int kTierSpan = 2048;
+constexpr int kTierLists = 8;
+
+__device__ __forceinline__ int64_t deg_of(const int64_t *xadj, const int64_t *deg, int64_t u) {
+  return deg ? deg[u] : xadj[u + 1] - xadj[u];
+}
+
+__global__ void __launch_bounds__(256)
+    k_classify(const int64_t *xadj, const int64_t *deg, int64_t n, int32_t lane_max,
+               int32_t small_max, int32_t mid_max, const uint32_t *off32, const uint64_t *off64,
+               bool long_records, uint8_t *tier, uint8_t *cls, int64_t *cnt,
+               unsigned long long *stats) {
+  __shared__ int32_t count[kTierLists + 1];
+  __shared__ unsigned long long st[10];
+  if (threadIdx.x <= kTierLists) count[threadIdx.x] = 0;
+  if (threadIdx.x < 10) st[threadIdx.x] = 0;
+  __syncthreads();
+  int64_t e[5] = {0, 0, 0, 0, 0};
+  int32_t c[5] = {0, 0, 0, 0, 0};
+  const int64_t lo = (int64_t)blockIdx.x * kTierSpan;
+  for (int64_t u = lo + threadIdx.x; u < min(lo + kTierSpan, n); u += 256) {
+    const int64_t d = deg_of(xadj, deg, u);
     bool lane = lane_max > 0 && d <= lane_max;
     if (lane && !long_records && (off32 || off64)) {
       const uint64_t len = off32 ? (uint64_t)(off32[u + 1] - off32[u]) : off64[u + 1] - off64[u];
       lane = len <= kLaneShortRecord;
     }
-    uint8_t t = lane ? TIER_LANE
-                : d <= small_max ? TIER_SMALL
-                : d <= mid_max ? TIER_MID
-                : d <= kChunkThreshold ? TIER_BIG
-                               : TIER_HUGE;
+    const uint8_t t = lane ? TIER_LANE
+                      : d <= small_max ? TIER_SMALL
+                      : d <= mid_max ? TIER_MID
+                      : d <= kChunkThreshold ? TIER_BIG
+                                     : TIER_HUGE;
+    const uint8_t k = t == TIER_LANE    ? 0
+                      : t == TIER_SMALL ? 1
+                      : t == TIER_MID   ? (d <= kMidSplit ? 2 : 3)
+                      : t == TIER_HUGE  ? 8
+                      : d <= kBigTinySplit ? 4
+                      : d <= kBigMidSplit  ? 5
+                      : d <= kBigSplit     ? 6
+                                           : 7;
     tier[u] = t;
-    flag_small[u] = t == TIER_SMALL;
-    flag_mid[u] = t == TIER_MID && d <= kMidSplit;
-    flag_mid2[u] = t == TIER_MID && d > kMidSplit;
-    flag_big0[u] = t == TIER_BIG && d <= kBigTinySplit;
-    flag_big1[u] = t == TIER_BIG && d > kBigTinySplit && d <= kBigMidSplit;
-    flag_big[u] = t == TIER_BIG && d > kBigMidSplit && d <= kBigSplit;
-    flag_big2[u] = t == TIER_BIG && d > kBigSplit;
-    flag_huge[u] = t == TIER_HUGE;
-    e[t] += d;
-    c[t] += 1;
+    cls[u] = k;
+    if (k) atomicAdd(&count[k], 1);
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      if (i == t) e[i] += d, ++c[i];
   }
-  for (int t = 0; t < 5; ++t) {
-    int64_t v = warp_sum(e[t]), w = warp_sum(c[t]);
-    if (lane_id() == 0 && v) atomicAdd(&stats[t], (unsigned long long)v);
-    if (lane_id() == 0 && w) atomicAdd(&stats[5 + t], (unsigned long long)w);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int32_t w = warp_sum(c[i]);
+    if (w == 0) continue;
+    const int64_t v = warp_sum(e[i]);
+    if (lane_id() == 0) atomicAdd(&st[i], (unsigned long long)v), atomicAdd(&st[5 + i], (unsigned long long)w);
   }
+  __syncthreads();
+  if (threadIdx.x < kTierLists)
+    cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = count[threadIdx.x + 1];
+  if (threadIdx.x < 10 && st[threadIdx.x]) atomicAdd(&stats[threadIdx.x], st[threadIdx.x]);
 }
 
-__global__ void k_compact(const int32_t *flag, const int64_t *pos, int64_t n, int32_t *out) {
-  for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n;
-       u += (int64_t)gridDim.x * blockDim.x)
-    if (flag[u]) out[pos[u]] = (int32_t)u;
+// The lists' lengths behind the per-tier figures: off holds the scanned counts.
+__global__ void k_tier_sizes(const int64_t *off, int64_t nblocks, unsigned long long *out) {
+  const int k = threadIdx.x;
+  if (k < kTierLists) out[k] = (unsigned long long)(off[(k + 1) * nblocks] - off[k * nblocks]);
+}
+
+__global__ void __launch_bounds__(256) k_tier_lists(const uint8_t *cls, int64_t n,
+                                                    const int64_t *off, int32_t *lists) {
+  __shared__ int64_t place[kTierLists];
+  __shared__ int32_t used[kTierLists];
+  if (threadIdx.x < kTierLists) {
+    place[threadIdx.x] = off[(int64_t)threadIdx.x * gridDim.x + blockIdx.x];
+    used[threadIdx.x] = 0;
+  }
+  __syncthreads();
+  const int64_t lo = (int64_t)blockIdx.x * kTierSpan;
+  for (int64_t u = lo + threadIdx.x; u < min(lo + kTierSpan, n); u += 256) {
+    const int k = cls[u];
+    if (k) lists[place[k - 1] + atomicAdd(&used[k - 1], 1)] = (int32_t)u;
+  }
 }
 
 // Table capacity per listed vertex: the smallest power of two >= 2*deg.
-__global__ void k_table_caps(const int32_t *list, int64_t cnt, const int64_t *deg, int64_t *slots,
-                             int32_t *logcap, int64_t *chunks) {
+__global__ void k_table_caps(const int32_t *list, int64_t cnt, const int64_t *xadj,
+                             const int64_t *deg, int64_t *slots, int32_t *logcap, int64_t *chunks) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
        i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t d = deg[list[i]];
+    int64_t d = deg_of(xadj, deg, list[i]);
     int lc = 1;
     while (((int64_t)1 << lc) < 2 * d) ++lc;
     logcap[i] = lc;
     slots[i] = (int64_t)1 << lc;
-    if (chunks) chunks[i] = (d + kChunkSize - 1) / kChunkSize;
+    chunks[i] = (d + kChunkSize - 1) / kChunkSize;
   }
 }
 
@@ -543,73 +581,71 @@ void build_tiers(tp_graph *g, const tp_params &p, cudaStream_t s) {
     T.built = true;
     return;
   }
-  Buf<int64_t> deg(n, s);
-  compute_degrees(g, deg.get(), s);
-  Buf<int32_t> fs(n, s), fm(n, s), fm2(n, s), fb0(n, s), fb1(n, s), fb(n, s), fb2(n, s), fh(n, s);
-  Buf<unsigned long long> te(10, s);
-  TP_CUDA(cudaMemsetAsync(te.get(), 0, 10 * sizeof(unsigned long long), s));
+  Buf<int64_t> deg;
+  const int64_t *xadj = g->compressed ? nullptr : g->xadj.get();
+  Buf<unsigned long long> te(10 + kTierLists, s);
+  TP_CUDA(cudaMemsetAsync(te.get(), 0, te.n * sizeof(unsigned long long), s));
   const uint32_t *o32 = g->compressed && !g->off_is64 ? g->off32.get() : nullptr;
   const uint64_t *o64 = g->compressed && g->off_is64 ? g->off64.get() : nullptr;
   bool long_records = false;
-  if ((o32 || o64) && lane_max > 0) {  // long lane records where more than 5% are long
-    launch(k_lane_records, grid_for(n, 256), 256, 0, s, deg.get(), n, lane_max, o32, o64, te.get());
-    unsigned long long lc[2];
-    TP_CUDA(cudaMemcpyAsync(lc, te.get(), sizeof(lc), cudaMemcpyDeviceToHost, s));
-    TP_CUDA(cudaStreamSynchronize(s));
-    long_records = lc[1] * 20 > lc[0];
-    T.lane_long = long_records;
+  if (g->compressed) {  // long lane records where more than 5% are long
+    deg.alloc(n, s);
+    launch(k_zip_degrees, grid_for(n, 256, (int64_t)num_sms() * 8), 256, 0, s, view(g), lane_max,
+           deg.get(), te.get());
+    TP_LAUNCH_CHECK();
+    if (lane_max > 0) {
+      unsigned long long lc[2];
+      TP_CUDA(cudaMemcpyAsync(lc, te.get(), sizeof(lc), cudaMemcpyDeviceToHost, s));
+      TP_CUDA(cudaStreamSynchronize(s));
+      long_records = lc[1] * 20 > lc[0];
+      T.lane_long = long_records;
+    }
     TP_CUDA(cudaMemsetAsync(te.get(), 0, 2 * sizeof(unsigned long long), s));
   }
-  launch(k_classify, grid_for(n, 256), 256, 0, s, deg.get(), n, lane_max, small_max, mid_max,
-         o32, o64, long_records, T.tier.get(), fs.get(), fm.get(), fm2.get(), fb0.get(), fb1.get(),
-         fb.get(), fb2.get(), fh.get(), te.get());
+  const int64_t nblocks = (n + kTierSpan - 1) / kTierSpan;
+  Buf<int64_t> off(kTierLists * nblocks + 1, s);
+  Buf<uint8_t> cls(n, s);
+  launch(k_classify, (unsigned)nblocks, 256, 0, s, xadj, deg.get(), n, lane_max, small_max, mid_max, o32,
+         o64, long_records, T.tier.get(), cls.get(), off.get(), te.get());
   TP_LAUNCH_CHECK();
-  unsigned long long hte[10];
+  exclusive_scan_i64(off.get(), off.get(), kTierLists * nblocks, s);
+  launch(k_tier_sizes, 1, 32, 0, s, off.get(), nblocks, te.get() + 10);
+  TP_LAUNCH_CHECK();
+  unsigned long long hte[10 + kTierLists];
   TP_CUDA(cudaMemcpyAsync(hte, te.get(), sizeof(hte), cudaMemcpyDeviceToHost, s));
   TP_CUDA(cudaStreamSynchronize(s));
   for (int t = 0; t < 5; ++t) T.edges[t] = (int64_t)hte[t], T.count[t] = (int64_t)hte[5 + t];
-  Buf<int64_t> pos(n + 1, s);
-  auto make_list = [&](Buf<int32_t> &flag, Buf<int32_t> &list, int64_t &cnt) {
-    exclusive_scan_i32_to_i64(flag.get(), pos.get(), n, s);
-    cnt = read_scalar(pos.get() + n, s);
-    list.alloc(cnt, s);
-    if (cnt) {
-      launch(k_compact, grid_for(n, 256), 256, 0, s, flag.get(), pos.get(), n, list.get());
+  {
+    int64_t *const len[kTierLists] = {&T.n_small, &T.n_mid, &T.n_mid2, &T.n_big0,
+                                      &T.n_big1,  &T.n_big, &T.n_big2, &T.n_huge};
+    TierList *const list[kTierLists] = {&T.small, &T.mid, &T.mid2, &T.big0,
+                                        &T.big1,  &T.big, &T.big2, &T.huge};
+    int64_t total = 0;
+    for (int k = 0; k < kTierLists; ++k) total += *len[k] = (int64_t)hte[10 + k];
+    T.lists.alloc(total, s);
+    if (total) {
+      launch(k_tier_lists, (unsigned)nblocks, 256, 0, s, cls.get(), n, off.get(), T.lists.get());
       TP_LAUNCH_CHECK();
     }
-  };
-  make_list(fs, T.small, T.n_small);
-  make_list(fm, T.mid, T.n_mid);
-  make_list(fm2, T.mid2, T.n_mid2);
-  make_list(fb0, T.big0, T.n_big0);
-  make_list(fb1, T.big1, T.n_big1);
-  make_list(fb, T.big, T.n_big);
-  make_list(fb2, T.big2, T.n_big2);
-  make_list(fh, T.huge, T.n_huge);
+    int32_t *at = T.lists.get();
+    for (int k = 0; k < kTierLists; ++k) list[k]->p = at, at += *len[k];
+  }
   // global rating tables for the huge tier (the big tier rates in shared memory)
-  auto tables = [&](Buf<int32_t> &list, int64_t cnt, Buf<int64_t> &toff, Buf<int32_t> &tcap,
-                    int64_t &slots, Buf<int64_t> *chunk_start, int64_t *nchunks) {
-    toff.alloc(cnt + 1, s);
-    tcap.alloc(std::max<int64_t>(cnt, 1), s);
-    slots = 0;
-    if (!cnt) return;
-    Buf<int64_t> ch;
-    if (chunk_start) {
-      chunk_start->alloc(cnt + 1, s);
-      ch.alloc(cnt, s);
-    }
-    launch(k_table_caps, grid_for(cnt, 256), 256, 0, s, list.get(), cnt, deg.get(), toff.get(),
-                                                      tcap.get(), chunk_start ? ch.get() : nullptr);
+  T.huge_toff.alloc(T.n_huge + 1, s);
+  T.huge_tcap.alloc(std::max<int64_t>(T.n_huge, 1), s);
+  if (T.n_huge) {
+    T.huge_chunk_start.alloc(T.n_huge + 1, s);
+    Buf<int64_t> ch(T.n_huge, s);
+    launch(k_table_caps, grid_for(T.n_huge, 256), 256, 0, s, T.huge.get(), T.n_huge, xadj, deg.get(),
+           T.huge_toff.get(), T.huge_tcap.get(), ch.get());
     TP_LAUNCH_CHECK();
-    exclusive_scan_i64(toff.get(), toff.get(), cnt, s);
-    slots = read_scalar(toff.get() + cnt, s);
-    if (chunk_start) {
-      exclusive_scan_i64(ch.get(), chunk_start->get(), cnt, s);
-      *nchunks = read_scalar(chunk_start->get() + cnt, s);
-    }
-  };
-  tables(T.huge, T.n_huge, T.huge_toff, T.huge_tcap, T.huge_slots, &T.huge_chunk_start,
-         &T.n_huge_chunks);
+    exclusive_scan_i64(T.huge_toff.get(), T.huge_toff.get(), T.n_huge, s);
+    exclusive_scan_i64(ch.get(), T.huge_chunk_start.get(), T.n_huge, s);
+    TP_CUDA(cudaMemcpyAsync(&T.huge_slots, T.huge_toff.get() + T.n_huge, 8, cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaMemcpyAsync(&T.n_huge_chunks, T.huge_chunk_start.get() + T.n_huge, 8,
+                            cudaMemcpyDeviceToHost, s));
+    TP_CUDA(cudaStreamSynchronize(s));
+  }
   if (T.n_huge) {
     T.huge_seg_start.alloc(T.n_huge + 1, s);
     launch(k_table_segs, grid_for(T.n_huge, 256), 256, 0, s, T.huge_tcap.get(), T.n_huge,

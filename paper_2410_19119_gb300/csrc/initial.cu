@@ -743,6 +743,7 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
   Buf<V> dif;
   Buf<uint8_t> sub;
   DepthDev dev, next_dev;
+  TierStreams streams;  // (after the buffers: gone before them)
   std::vector<int64_t> host, next_host;
   for (int depth = 0; d.nodes() > 0; ++depth) {
     const int32_t nodes = d.nodes();
@@ -831,8 +832,12 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
       c.ord = ord.get(), c.claimer = claimer.get(), c.cnt = cnt.get(), c.list = list.get();
       c.dif = dif.get(), c.sub = sub.get();
     }
-    for (int32_t b = 0; b < nodes;) {
+    // classes side by side: each is as long as its longest attempt
+    const bool fork = !(shape[order[0]] == shape[order[nodes - 1]]) && streams.make();
+    if (fork) streams.begin(s);
+    for (int32_t b = 0, number = 0; b < nodes; ++number) {
       const Shape sh = shape[order[b]];
+      const cudaStream_t cls = fork && number ? streams.st[(number - 1) % TierStreams::kN] : s;
       int32_t e = b;
       int64_t largest = 1;
       for (; e < nodes && shape[order[e]] == sh; ++e)
@@ -840,13 +845,14 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
       c.nodes = cur.order + b;
       c.cap = (int32_t)((largest + 15) & ~(int64_t)15);
       const int64_t att = (int64_t)(e - b) * T;
-      if (sh.cluster) launch_bisect<kIPMaxThreads, false, V>(c, att, sh.cluster, s);
-      else if (sh.threads == 128) launch_bisect<128, true, V>(c, att, 1, s);
-      else if (sh.threads == 256) launch_bisect<256, true, V>(c, att, 1, s);
-      else if (sh.threads == 512) launch_bisect<512, true, V>(c, att, 1, s);
-      else launch_bisect<1024, true, V>(c, att, 1, s);
+      if (sh.cluster) launch_bisect<kIPMaxThreads, false, V>(c, att, sh.cluster, cls);
+      else if (sh.threads == 128) launch_bisect<128, true, V>(c, att, 1, cls);
+      else if (sh.threads == 256) launch_bisect<256, true, V>(c, att, 1, cls);
+      else if (sh.threads == 512) launch_bisect<512, true, V>(c, att, 1, cls);
+      else launch_bisect<1024, true, V>(c, att, 1, cls);
       b = e;
     }
+    if (fork) streams.end(s);
     int64_t widest = 1;
     for (int32_t j = 0; j < nodes; ++j) widest = std::max(widest, d.start[j + 1] - d.start[j]);
     const dim3 pg((unsigned)nodes, (unsigned)std::min<int64_t>((widest + 255) / 256, 256));

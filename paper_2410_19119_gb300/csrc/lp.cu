@@ -169,6 +169,10 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
         lane_batch<COMP, MODE, W, 8, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
       else if (maxdeg <= 16)
         lane_batch<COMP, MODE, W, 16, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+      else if (!W && !COMP && maxdeg <= 24)
+        // half of the batches of a mesh of average degree 16 (the compressed
+        // kernel, with the decoder beside them, lost a fifth to a third size)
+        lane_batch<COMP, MODE, W, 24, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
       else
         lane_batch<COMP, MODE, W, kLaneMaxDeg, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
     }

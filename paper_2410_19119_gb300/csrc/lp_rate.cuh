@@ -481,8 +481,8 @@ __device__ __forceinline__ void lane_prefetch(const GView &g, const uint64_t *re
   }
 }
 
-// Batcher's odd-even merge sort of a[0..N), ascending (N a power of two;
-// 63 comparators for 16 elements, 191 for 32), registers only. The network
+// Batcher's odd-even merge sort of a[0..N), ascending (63 comparators for 16
+// elements, 191 for 32), registers only. The network
 // is generated by template recursion so every index is a constant.
 template <class T>
 __device__ __forceinline__ void cmp_swap(T &x, T &y) {
@@ -491,32 +491,35 @@ __device__ __forceinline__ void cmp_swap(T &x, T &y) {
   y = hi;
 }
 
-// Merges the two sorted halves of the subsequence a[LO], a[LO + R], ...
-template <int LO, int N, int R, class T>
+// Merges the two sorted halves of the subsequence a[LO], a[LO + R], ...; only
+// the first LIM elements exist (those beyond would be larger than any, and
+// every comparator leaves the larger of its pair at the higher index).
+template <int LO, int N, int R, int LIM, class T>
 __device__ __forceinline__ void oem_merge(T (&a)[kLaneMaxDeg]) {
   constexpr int M = 2 * R;
   if constexpr (M < N) {
-    oem_merge<LO, N, M>(a);
-    oem_merge<LO + R, N, M>(a);
+    oem_merge<LO, N, M, LIM>(a);
+    oem_merge<LO + R, N, M, LIM>(a);
 #pragma unroll
-    for (int i = LO + R; i + R < LO + N; i += M) cmp_swap(a[i], a[i + R]);
-  } else {
+    for (int i = LO + R; i + R < LO + N && i + R < LIM; i += M) cmp_swap(a[i], a[i + R]);
+  } else if constexpr (LO + R < LIM) {
     cmp_swap(a[LO], a[LO + R]);
   }
 }
 
-template <int LO, int N, class T>
+template <int LO, int N, int LIM, class T>
 __device__ __forceinline__ void oem_sort_range(T (&a)[kLaneMaxDeg]) {
-  if constexpr (N > 1) {
-    oem_sort_range<LO, N / 2>(a);
-    oem_sort_range<LO + N / 2, N / 2>(a);
-    oem_merge<LO, N, 1>(a);
+  if constexpr (N > 1 && LO < LIM) {
+    oem_sort_range<LO, N / 2, LIM>(a);
+    oem_sort_range<LO + N / 2, N / 2, LIM>(a);
+    oem_merge<LO, N, 1, LIM>(a);
   }
 }
 
+// N: 8, 16, 24 (the network of 32 without its last quarter) or 32.
 template <int N, class T>
 __device__ __forceinline__ void oem_sort(T (&a)[kLaneMaxDeg]) {
-  oem_sort_range<0, N>(a);
+  oem_sort_range<0, (N <= 8 ? 8 : N <= 16 ? 16 : 32), N>(a);
 }
 
 // Mover records of one warp's window, written out with one atomic per window.

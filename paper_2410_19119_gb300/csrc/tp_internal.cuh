@@ -117,18 +117,25 @@ constexpr int64_t kBigTinySplit = 1024;     // big tier: degrees up to here use 
 constexpr int64_t kBigMidSplit = 2048;      // big tier: degrees up to here use 4096-slot tables
 constexpr int64_t kBigSplit = 4096;         // big tier: degrees up to here use 8192-slot tables
 
+struct TierList {  // a range of TierCache::lists
+  int32_t *p = nullptr;
+  int32_t *get() const { return p; }
+};
+
 struct TierCache {
   bool built = false;
   int32_t small_max = 0, mid_max = 0, lane_max = 0;
   bool lane_long = false;  // compressed lane records may exceed 80 bytes (skewed graphs)
   int64_t count[5] = {0, 0, 0, 0, 0};  // vertices per tier
   Buf<uint8_t> tier;         // n
-  // vertex lists per tier (ascending); the mid tier is listed in two parts,
+  // vertex lists per tier, side by side in one array (ascending by blocks of
+  // 2048 vertices); the mid tier is listed in two parts,
   // degree <= kMidSplit (warp tables of 512 slots) and above (1024), the big
   // tier in four, degree <= kBigTinySplit (block tables of 2048 slots, many
   // blocks per SM), <= kBigMidSplit (4096), <= kBigSplit (8192) and above
   // (16384)
-  Buf<int32_t> small, mid, mid2, big0, big1, big, big2, huge;
+  Buf<int32_t> lists;
+  TierList small, mid, mid2, big0, big1, big, big2, huge;
   int64_t n_small = 0, n_mid = 0, n_mid2 = 0, n_big0 = 0, n_big1 = 0, n_big = 0, n_big2 = 0,
           n_huge = 0;
   Buf<int64_t> huge_toff;  // global table offsets (slots), size n_huge + 1
@@ -150,7 +157,7 @@ struct TierCache {
   // Later frees go to stream s (the cache may have been built on a stream
   // that no longer exists; see tp_graph::rehome).
   void rehome(cudaStream_t s) {
-    tier.s = small.s = mid.s = mid2.s = big0.s = big1.s = big.s = big2.s = huge.s = s;
+    tier.s = lists.s = s;
     huge_toff.s = huge_tcap.s = s;
     huge_chunk_start.s = tkeys.s = tvals.s = tlist.s = tcount.s = s;
     huge_seg_start.s = huge_seg_best.s = s;
@@ -377,7 +384,6 @@ int64_t max_i64(const int64_t *d, int64_t n, cudaStream_t s);  // 0 for n == 0; 
 
 // ---------------------------------------------------------------- graph helpers (graph.cu)
 tp_graph *new_graph();
-void compute_degrees(const tp_graph *g, int64_t *d_deg, cudaStream_t s);  // n entries
 void build_tiers(tp_graph *g, const tp_params &p, cudaStream_t s);
 // Hub rating tables: allocated (empty) for a rating call, released after it.
 void ensure_hub_tables(tp_graph *g, cudaStream_t s);
