@@ -28,6 +28,7 @@
 // per target runs a weighted radix select over the key (gain desc, vertex
 // asc) and approves exactly the longest fitting prefix.
 #include <algorithm>
+#include <memory>
 #include <mutex>
 
 #include "lp_rate.cuh"
@@ -197,6 +198,116 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
       __syncwarp();
       pending = left;
     }
+  }
+}
+
+// Lane tier with quiet vertices left out. A vertex whose rating found no label
+// better than its own moves in no later sub-round, whatever the tie order and
+// the label weights, until a neighbour moves; k_wake forgets the marks of the
+// neighbours of every moved vertex. In refinement the interior of every block
+// is quiet after the first round, which leaves a tenth of a mesh to rate. A
+// warp's window of the list is filtered into a queue of list positions, so the
+// batches stay full.
+template <bool COMP, bool W>
+__global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM)
+    k_rate_lane_quiet(RateCtx c) {
+  constexpr int WARPS = lane_warps<W>();
+  __shared__ uint32_t lab_all[WARPS][kLaneMaxDeg][32];
+  __shared__ uint32_t aux_all[WARPS][W ? kLaneMaxDeg : 1][32];
+  __shared__ uint8_t cnt_all[WARPS][COMP && !W ? kLaneMaxDeg : 1][32];
+  __shared__ int32_t queue_all[WARPS][64];
+  __shared__ BatchMovers movers_all[WARPS];
+  const int lane = lane_id(), w = threadIdx.x >> 5;
+  uint32_t *col = &lab_all[w][0][lane];
+  uint32_t *wcol = &aux_all[w][0][lane];
+  uint8_t *cnt = &cnt_all[w][0][lane];
+  int32_t *queue = queue_all[w];
+  BatchMovers &mb = movers_all[w];
+  const int64_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = (gridDim.x * blockDim.x) >> 5;
+  const int64_t bstart = c.bucket_off[(int64_t)c.s * c.bucket_nb];
+  const int64_t bcount = c.bucket_off[(int64_t)(c.s + 1) * c.bucket_nb] - bstart;
+  const int32_t *blist = c.bucket + bstart;
+  const uint64_t *brec = COMP ? c.bucket_rec + bstart : nullptr;
+  const int epoch = *c.epoch;
+  int64_t win = gw * c.lane_win;  // this window's start; at: next position in it
+  int at = 0, pending = 0;
+  for (;;) {
+    while (pending < 32 && win < bcount) {
+      const int64_t p = win + at + lane;
+      const bool act = at + lane < c.lane_win && p < bcount && c.quiet[blist[p]] != epoch;
+      const unsigned m = __ballot_sync(kFull, act);
+      if (act) queue[pending + __popc(m & lanemask_lt())] = (int32_t)p;
+      pending += __popc(m);
+      at += 32;
+      if (at >= c.lane_win) at = 0, win += nw * c.lane_win;
+    }
+    if (pending == 0) break;
+    __syncwarp();
+    const int take = min(pending, 32);
+    const bool has = lane < take;
+    const int32_t p = has ? queue[lane] : 0;
+    const int32_t rest = take + lane < pending ? queue[take + lane] : 0;
+    __syncwarp();
+    if (take + lane < pending) queue[lane] = rest;
+    pending -= take;
+    const int32_t u = has ? blist[p] : 0;
+    int deg = 0, nmv = 0;
+    if (has) {
+      if (COMP) {
+        uint64_t rb, re;
+        lane_record(c.g, brec, p, u, rb, re);
+        deg = lane_decode<false>(c.g, rb, re, col);
+      } else {
+        deg = min((int)(c.g.xadj[u + 1] - c.g.xadj[u]), kLaneMaxDeg);
+      }
+    }
+    const unsigned maxdeg = __reduce_max_sync(kFull, (unsigned)deg);
+    if (maxdeg <= 16)
+      lane_batch<COMP, M_LP, W, 16, false, false, false, true>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+    else
+      lane_batch<COMP, M_LP, W, kLaneMaxDeg, false, false, false, true>(c, has, u, deg, col, wcol, cnt, mb, nmv);
+    __syncwarp();
+    if (nmv) {
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(c.counters, (unsigned long long)nmv);
+      base = __shfl_sync(kFull, base, 0);
+      if (lane < nmv) {
+        c.mv_u[base + lane] = mb.u[lane];
+        c.mv_t[base + lane] = mb.t[lane];
+        c.mv_o[base + lane] = mb.o[lane];
+        c.mv_g[base + lane] = mb.g[lane];
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// The neighbours of every moved vertex are quiet no longer: low-degree movers
+// by a thread each, the others by a warp. Where a sub-round moved so many that
+// little would stay quiet, the epoch advances instead, which ends all marks.
+template <bool COMP>
+__global__ void k_wake(GView g, const uint8_t *tier, const unsigned long long *counters,
+                       const int32_t *mv_u, const int8_t *mv_ok, int64_t limit, uint8_t *quiet,
+                       int32_t *epoch) {
+  const int64_t nm = (int64_t)counters[0];
+  if (nm > limit) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;
+    return;
+  }
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < nm;
+       i0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = i0 + threadIdx.x;
+    const bool in = i < nm && mv_ok[i];
+    const int32_t u = in ? mv_u[i] : 0;
+    const bool low = in && (tier[u] == TIER_LANE || tier[u] == TIER_SMALL);
+    if (low) thread_neighbours<COMP>(g, u, [&](int32_t v, int64_t) { quiet[v] = 0; });
+    __syncwarp();
+    for (unsigned q = __ballot_sync(kFull, in && !low); q; q &= q - 1)
+      warp_neighbours<COMP>(g, __shfl_sync(kFull, u, __ffs(q) - 1), -1,
+                            [&](bool has, int32_t v, int64_t, int64_t) {
+                              if (has) quiet[v] = 0;
+                            });
   }
 }
 
@@ -1009,7 +1120,9 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s,
           (g->n + 256 * kLaneWarps - 1) / (256 * kLaneWarps), (int64_t)sms * kLaneBlocksPerSM);
       lane_window((int64_t)blocks * kLaneWarps);
       // batched graphs are CSR unions
-      if (comp && T.lane_long) launch(k_rate_lane<true, LM, false, true>, blocks, 32 * kLaneWarps, 0, s, c);
+      if (MODE == M_LP && c.quiet && comp) launch(k_rate_lane_quiet<true, false>, blocks, 32 * kLaneWarps, 0, s, c);
+      else if (MODE == M_LP && c.quiet) launch(k_rate_lane_quiet<false, false>, blocks, 32 * kLaneWarps, 0, s, c);
+      else if (comp && T.lane_long) launch(k_rate_lane<true, LM, false, true>, blocks, 32 * kLaneWarps, 0, s, c);
       else if (comp) launch(k_rate_lane<true, LM, false>, blocks, 32 * kLaneWarps, 0, s, c);
       else if (c.seg.gid) launch(k_rate_lane<false, LM, false, false, true>, blocks, 32 * kLaneWarps, 0, s, c);
       else launch(k_rate_lane<false, LM, false>, blocks, 32 * kLaneWarps, 0, s, c);
@@ -1020,7 +1133,8 @@ void rate_tiers(tp_graph *g, RateCtx c, const tp_params &p, cudaStream_t s,
       lane_window((int64_t)blocks * WW);
       // labels are vertices or, in refinement, block numbers
       const bool wide = g->n > kLaneKeyLabels || c.nlabels > kLaneKeyLabels;
-      if (c.seg.gid && wide) launch(k_rate_lane<false, LM, true, true, true>, blocks, 32 * WW, 0, s, c);
+      if (MODE == M_LP && c.quiet) launch(k_rate_lane_quiet<false, true>, blocks, 32 * WW, 0, s, c);
+      else if (c.seg.gid && wide) launch(k_rate_lane<false, LM, true, true, true>, blocks, 32 * WW, 0, s, c);
       else if (c.seg.gid) launch(k_rate_lane<false, LM, true, false, true>, blocks, 32 * WW, 0, s, c);
       else if (wide) launch(k_rate_lane<false, LM, true, true>, blocks, 32 * WW, 0, s, c);
       else launch(k_rate_lane<false, LM, true>, blocks, 32 * WW, 0, s, c);
@@ -1547,7 +1661,12 @@ void LpWork::init(int64_t n_vertices, int64_t n_labels, cudaStream_t s) {
 // The approval of one sub-round: the same five kernels and counter reset on
 // every sub-round of a level (only the data differs).
 constexpr int kApproveKernels = 5;
-void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStream_t stream) {
+// wake (nullable): the graph whose quiet vertices the moves wake, S its
+// sub-rounds. Marks pay while a round moves few vertices: beyond an eighth
+// of the vertices (a mesh vertex wakes 16, movers side by side the same ones)
+// hardly any would last.
+void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStream_t stream,
+                     const tp_graph *wake = nullptr, LpWork *w = nullptr, int32_t S = 1) {
   const unsigned blocks = (unsigned)num_sms() * 4;
   const unsigned wide = grid_for(std::max<int64_t>(wn, 1), 256, (int64_t)num_sms() * 64);
   launch(k_approve_fit, wide, 256, 0, stream, a);
@@ -1555,6 +1674,18 @@ void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStr
   launch(k_approve_scatter, blocks, 256, 0, stream, a);
   launch(k_approve_contested, (unsigned)num_sms() * 2, 256, 0, stream, a);
   launch(k_apply, wide, 256, 0, stream, a);
+  if (wake) {
+    const int64_t limit = wake->n / (8 * (int64_t)S);
+    const unsigned wb = grid_for(std::max<int64_t>(limit, 1), 256);
+    const uint8_t *tier = wake->tiers.tier.get();
+    const unsigned long long *cnt = (const unsigned long long *)counters;
+    if (wake->compressed)
+      launch(k_wake<true>, wb, 256, 0, stream, view(wake), tier, cnt, a.mv_u, a.mv_ok, limit,
+             w->quiet.get(), w->epoch.get());
+    else
+      launch(k_wake<false>, wb, 256, 0, stream, view(wake), tier, cnt, a.mv_u, a.mv_ok, limit,
+             w->quiet.get(), w->epoch.get());
+  }
   TP_LAUNCH_CHECK();
   TP_CUDA(cudaMemsetAsync(counters, 0, 4 * sizeof(int64_t), stream));
 }
@@ -1565,7 +1696,8 @@ void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStr
 struct ApprovalGraph {
   cudaStream_t cs = nullptr;
   cudaGraphExec_t exec = nullptr;
-  ApprovalGraph(const ApproveCtx &a, int64_t wn, int64_t *counters) {
+  ApprovalGraph(const ApproveCtx &a, int64_t wn, int64_t *counters, const tp_graph *wake,
+                LpWork *w, int32_t S) {
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
       (void)cudaGetLastError();
       cs = nullptr;
@@ -1578,7 +1710,7 @@ struct ApprovalGraph {
     capture_counting(true);
     bool ok = true;
     try {
-      launch_approval(a, wn, counters, cs);
+      launch_approval(a, wn, counters, cs, wake, w, S);
     } catch (...) {
       ok = false;
     }
@@ -1624,6 +1756,7 @@ void lp_subround(tp_graph *g, const LpState &st, LpWork &w, uint64_t rk, int32_t
   c.in_w = w.in_w.get();
   c.counters = (unsigned long long *)w.counters.get();
   if (w.bucket_S == S) {
+    if (w.quiet_on) c.quiet = w.quiet.get(), c.epoch = w.epoch.get();
     c.bucket = w.bucket.get();
     c.bucket_off = w.bucket_off.get();
     c.bucket_nb = w.bucket_nblocks;
@@ -1643,9 +1776,10 @@ void lp_subround(tp_graph *g, const LpState &st, LpWork &w, uint64_t rk, int32_t
   prof_begin(PF_APPROVE, stream);
   if (approval) {
     TP_CUDA(cudaGraphLaunch(approval, stream));
-    count_launches(kApproveKernels);
+    count_launches(kApproveKernels + (w.quiet_on ? 1 : 0));
   } else {
-    launch_approval(approve_ctx(g, st, w), w.n, w.counters.get(), stream);
+    launch_approval(approve_ctx(g, st, w), w.n, w.counters.get(), stream, w.quiet_on ? g : nullptr, &w,
+                    S);
   }
   prof_end(PF_APPROVE, stream, 0.0);
 }
@@ -1657,6 +1791,8 @@ __global__ void k_round_key(uint64_t seed, uint64_t tag, uint64_t a, uint64_t b0
   *rk = round_key(seed, tag, a, b0 + (uint64_t)*r);
   *r += 1;
 }
+
+__global__ void k_set_i32(int32_t *p, int32_t v) { *p = v; }
 
 // Small levels: a whole LP round (round key, bucketing, every sub-round's
 // rating and approval) is recorded once as a CUDA graph on a private stream
@@ -1738,14 +1874,36 @@ void lp_rounds(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, uint64_
   if (p.use_graphs && g->n <= std::min<int64_t>(p.graph_n, kRoundGraphMaxN) && !prof_active() &&
       lp_rounds_graph(g, st, w, seed, tag, a, b0, rounds, S, p, stream))
     return;
-  ApprovalGraph ag(approve_ctx(g, st, w), w.n, w.counters.get());
+  build_tiers(g, p, stream);
+  const TierCache &T = g->tiers;
+  // quiet vertices: one graph, most entries in the lane tier, and so few
+  // sub-rounds that the epoch (one step each at most) fits its byte. In
+  // clustering nearly every vertex moves in the first two rounds, which go
+  // without (labels are vertices then: kmax is 0).
+  const int32_t quiet_from = st.kmax ? 0 : 2;
+  const bool quiet_ok = !st.seg.gid && S <= 32 && (int64_t)rounds * S < 250 && rounds > quiet_from &&
+                        !T.lane_long && !prof_active() && 5 * T.edges[TIER_LANE] >= 4 * g->m2 &&
+                        g->n <= kLaneKeyLabels && st.nlabels <= kLaneKeyLabels;
+  std::unique_ptr<ApprovalGraph> ag;
   for (int32_t r = 0; r < rounds; ++r) {
+    const bool quiet = quiet_ok && r >= quiet_from;
+    if (quiet && !w.quiet_on) {
+      if ((int64_t)w.quiet.n < g->n) w.quiet.alloc(g->n, stream);
+      if (!w.epoch.get()) w.epoch.alloc(1, stream);
+      TP_CUDA(cudaMemsetAsync(w.quiet.get(), 0, g->n, stream));
+      launch(k_set_i32, 1, 1, 0, stream, w.epoch.get(), 1);
+    }
+    if (!ag || quiet != w.quiet_on) {
+      w.quiet_on = quiet;
+      ag.reset(new ApprovalGraph(approve_ctx(g, st, w), w.n, w.counters.get(), quiet ? g : nullptr, &w, S));
+    }
     uint64_t rk = round_key(seed, tag, a, b0 + (uint64_t)r);
     lp_bucket(g, w, rk, S, p, stream, nullptr, true, &st.seg);
-    for (int32_t s = 0; s < S; ++s) lp_subround(g, st, w, rk, S, s, p, stream, ag.exec);
+    for (int32_t s = 0; s < S; ++s) lp_subround(g, st, w, rk, S, s, p, stream, ag->exec);
     w.bucket_S = 0;
     w.tb_valid = false;
   }
+  w.quiet_on = false;
 }
 
 // ---------------------------------------------------------------- two-hop packing

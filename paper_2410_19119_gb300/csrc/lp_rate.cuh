@@ -69,6 +69,10 @@ struct RateCtx {
   int32_t lane_win;  // vertices of a warp's window (32 .. kLaneWin)
   // per listed vertex: record start << 8 | record length (compressed graphs)
   const uint64_t *bucket_rec;
+  // quiet[u] == *epoch: u's last rating found no label better than its own and
+  // no neighbour has moved since, so it need not be rated (k_rate_lane_quiet)
+  uint8_t *quiet;
+  const int32_t *epoch;
   // this round's sub-round + 1 of every vertex (null: hash on the fly)
   const uint8_t *sub_byte;
   // bucket mode of the warp/block tiers: this tier's list positions grouped
@@ -522,6 +526,11 @@ __device__ __forceinline__ void oem_sort(T (&a)[kLaneMaxDeg]) {
   oem_sort_range<0, (N <= 8 ? 8 : N <= 16 ? 16 : 32), N>(a);
 }
 
+// Mover records of one batch.
+struct BatchMovers {
+  int32_t u[32], t[32], o[32], g[32];
+};
+
 // Mover records of one warp's window, written out with one atomic per window.
 struct LaneMovers {
   int32_t u[kLaneWin], t[kLaneWin], o[kLaneWin], g[kLaneWin];
@@ -566,8 +575,9 @@ constexpr int64_t kLaneKeyLabels = ((int64_t)1 << 27) - 1;
 
 // WIDE (weighted): labels beyond kLaneKeyLabels, sorted with the weights in
 // 64-bit keys.
+// QUIET: vertices without a better label are marked quiet.
 template <bool COMP, int MODE, bool W, int N, bool SEG, bool LIVE = false, bool WIDE = false,
-          class Movers>
+          bool QUIET = false, class Movers>
 __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u, int deg,
                                            uint32_t *col, uint32_t *wcol, uint8_t *cnt,
                                            Movers &mb, int &nmv) {
@@ -649,6 +659,7 @@ __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u
         }
       }
     }
+    if (QUIET && has && rmax <= rown) c.quiet[u] = (uint8_t)*c.epoch;
     emit_lane<MODE>(c, has, u, own, rown, cu, best, mb, nmv);
   } else if constexpr (COMP) {
     // compressed, unit weights: the sorted runs become a list of (label,
@@ -715,6 +726,7 @@ __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u
         }
       }
     }
+    if (QUIET && has && rmax <= rown) c.quiet[u] = (uint8_t)*c.epoch;
     emit_lane<MODE>(c, has, u, own, rown, cu, best, mb, nmv);
   } else {
     // CSR, unit weights: the labels are sorted with the own label as padding (its
@@ -814,6 +826,7 @@ __device__ __forceinline__ void lane_batch(const RateCtx &c, bool has, int32_t u
     }
     LaneCand best{-1, 0xffffffffu, INT32_MAX};
     if (go) best = b1;
+    if (QUIET && has && rmax <= rown) c.quiet[u] = (uint8_t)*c.epoch;
     emit_lane<MODE>(c, has, u, own, rown, cu, best, mb, nmv);
     return;
   }

@@ -29,10 +29,6 @@ constexpr int kLpSmallItems = 4;
 constexpr int64_t kLpSmallVertices = 16384;  // most vertices of a CTA (its bucket list)
 constexpr int64_t kLpSmallEntries = (int64_t)1 << 17;  // most adjacency entries of a CTA's share
 
-struct BatchMovers {
-  int32_t u[32], t[32], o[32], g[32];
-};
-
 // A warp's part of the shared memory: the lane tier's columns or a hash table.
 struct LpSmallWarp {
   uint32_t lab[kLaneMaxDeg][32];  // or 1024 keys

@@ -464,6 +464,10 @@ struct LpWork {
   // huge tier, in bucket order of its hubs: prefix of chunk and segment
   // counts (n_huge + 1) and the items themselves (hub position << 32 | index)
   Buf<int64_t> hc_pre, hs_pre, hc_item, hs_item;
+  // quiet vertices (see k_rate_lane_quiet): marks, their epoch, whether in use
+  Buf<uint8_t> quiet;    // n
+  Buf<int32_t> epoch;    // 1
+  bool quiet_on = false;
   TierStreams streams;  // last: gone before the buffers
   void init(int64_t n_vertices, int64_t n_labels, cudaStream_t s);
 };
