@@ -16,23 +16,38 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// Single-thread VarInt read (up to 10 bytes). Returns bytes consumed. The
-// stream is padded with zero bytes, so all ten bytes a VarInt may span are
-// loaded at once (one memory round trip instead of one per byte).
+// The 7-bit payloads of four bytes, the first lowest.
+__device__ __forceinline__ uint32_t payload28(uint32_t w) {
+  return (w & 0x7fu) | (w >> 1 & 0x3f80u) | (w >> 2 & 0x1fc000u) | (w >> 3 & 0xfe00000u);
+}
+
+// Single-thread VarInt read (up to 10 bytes). Returns bytes consumed. Three
+// aligned words hold the first eight bytes wherever p lies (the stream is
+// padded behind its end, and begins aligned); the value is taken from them
+// without a loop. (Ten byte loads and a select chain cost three times the
+// instructions, twice per record in every kernel that needs a degree.)
 __device__ __forceinline__ int read_varint(const uint8_t *p, uint64_t &x) {
-  uint32_t b[10];
-#pragma unroll
-  for (int i = 0; i < 10; ++i) b[i] = p[i];
-  uint64_t v = 0;
-  int len = 10;
-  bool open = true;
-#pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    if (open) v |= (uint64_t)(b[i] & 0x7fu) << (7 * i);
-    if (open && !(b[i] & 0x80u)) len = i + 1, open = false;
+  const uint32_t *wp =
+      reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3);
+  const unsigned sh = 8u * (unsigned)(reinterpret_cast<uintptr_t>(p) & 3);
+  const uint32_t w0 = wp[0], w1 = wp[1], w2 = wp[2];
+  const uint32_t lo = __funnelshift_r(w0, w1, sh), hi = __funnelshift_r(w1, w2, sh);
+  const uint32_t stop = ~lo & 0x80808080u;
+  if (stop) {  // up to four bytes: everything below the stop bit
+    x = payload28(lo & (stop ^ (stop - 1)));
+    return __ffs(stop) >> 3;
   }
-  x = v;
-  return len;
+  const uint32_t stop2 = ~hi & 0x80808080u;
+  const uint64_t low = payload28(lo);
+  if (stop2) {
+    x = low | (uint64_t)payload28(hi & (stop2 ^ (stop2 - 1))) << 28;
+    return 4 + (__ffs(stop2) >> 3);
+  }
+  const uint32_t b8 = p[8], b9 = p[9];
+  x = low | (uint64_t)payload28(hi) << 28 | (uint64_t)(b8 & 0x7fu) << 56;
+  if (!(b8 & 0x80u)) return 9;
+  x |= (uint64_t)(b9 & 0x7fu) << 63;
+  return 10;
 }
 
 __device__ __forceinline__ uint64_t off_at(const GView &g, int64_t u) {
@@ -225,6 +240,78 @@ __device__ __forceinline__ bool warp_decode_chunk(const GView &g, int64_t u, uin
   return true;
 }
 
+// The same for streams that were checked when their graph was made (every
+// graph's are), with half the instructions: the payloads of a lane's word and
+// the one before it are packed into 56 bits once, so each value is a shift and
+// a mask; ids are 32-bit sums, clamped into [0, n) to keep later accesses in
+// bounds. A step that cannot advance still latches TP_ERR_CORRUPT and ends.
+template <class F>
+__device__ __forceinline__ bool warp_decode_trusted(const GView &g, int64_t u, uint64_t p,
+                                                    uint64_t end, int64_t count, F &&f) {
+  const int lane = lane_id();
+  const uint32_t nmax = (uint32_t)(g.n - 1);
+  uint32_t done = 0;
+  const uint32_t total_count = (uint32_t)count;
+  uint32_t prev = (uint32_t)u;  // id of the last value of the previous step
+  while (done < total_count) {
+    const uint64_t base = p & ~(uint64_t)3;
+    const uint64_t q = base + 4 * (uint64_t)lane;
+    uint32_t w = q < end ? *reinterpret_cast<const uint32_t *>(g.bytes + q) : 0x80808080u;
+    uint32_t skip = 0;  // lane 0: bytes of its word before p
+    if (lane == 0) {
+      skip = (uint32_t)(p - base);
+      w &= 0xffffffffu << (8 * skip);  // they end values, which are discarded
+    }
+    if (q < end && q + 4 > end) w |= 0x80808080u << (8 * (uint32_t)(end - q));
+    const uint32_t up = __shfl_up_sync(kFull, w, 1);
+    const uint32_t pw = lane ? up : 0u;
+    const uint64_t pay = (uint64_t)payload28(w) << 28 | payload28(pw);
+    // continuation bits of the eight bytes, the lane's own four in bits 4..7
+    const uint32_t own4 = ((w & 0x80808080u) >> 7) * 0x10204080u >> 28;
+    const uint32_t cont = ((pw & 0x80808080u) >> 7) * 0x10204080u >> 28 | own4 << 4;
+    const uint32_t ends = ~own4 & (0xfu << skip) & 0xfu;
+    const uint32_t nl = __popc(ends);
+    const uint32_t incl = warp_incl_scan(nl);
+    const uint32_t total = __shfl_sync(kFull, incl, 31);
+    if (total == 0 || done + total > total_count) {
+      if (lane == 0) latch_error(g.err, TP_ERR_CORRUPT);
+      return false;
+    }
+    uint32_t idx = incl - nl;
+    const bool head = done == 0 && idx == 0 && nl > 0;  // this lane holds the chunk's first value
+    uint32_t val[4], sum = 0;
+    bool first = head;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int k = __clz(~(cont << (28 - j)));  // continuation bytes just before byte j
+      const uint64_t m = ((uint64_t)1 << (7 * (k + 1))) - 1;
+      uint32_t v = (uint32_t)(pay >> (7 * (4 + j - k)) & m);
+      const bool is = ends >> j & 1u;
+      if (is && first) v = (v & 1u) ? 0u - (v >> 1) : v >> 1, first = false;  // signed offset from u
+      sum += is ? v : 0u;
+      val[j] = sum;
+    }
+    const uint32_t before = prev + warp_incl_scan(sum) - sum;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const bool is = ends >> j & 1u;
+      f(is, (int32_t)min(before + val[j], nmax), (int64_t)(done + idx));
+      idx += is;
+    }
+    prev = __shfl_sync(kFull, before + sum, 31);
+    done += total;
+    // behind the last value's last byte
+    const uint32_t lastlane = 31 - __clz(__ballot_sync(kFull, nl > 0));
+    const int hb = 31 - __clz(__shfl_sync(kFull, ends, lastlane));
+    p = base + 4 * (uint64_t)lastlane + (uint64_t)hb + 1;
+  }
+  if (p != end) {
+    if (lane == 0) latch_error(g.err, TP_ERR_CORRUPT);
+    return false;
+  }
+  return true;
+}
+
 // Visits the neighbours of u in warp-wide batches: f(bool has, int32_t v,
 // int64_t w, int64_t idx), idx = position of v in u's neighbourhood (the
 // batches are not in neighbourhood order for the compressed format). For
@@ -232,8 +319,10 @@ __device__ __forceinline__ bool warp_decode_chunk(const GView &g, int64_t u, uin
 // decoder step calls f four times. chunk < 0 visits the whole
 // neighbourhood; otherwise only chunk `chunk` (chunks of kChunkSize
 // entries, for CSR as well).
+// zp (compressed, nullable): u's layout where the caller has it.
 template <bool COMP, class F>
-__device__ __forceinline__ void warp_neighbours(const GView &g, int64_t u, int64_t chunk, F &&f) {
+__device__ __forceinline__ void warp_neighbours(const GView &g, int64_t u, int64_t chunk, F &&f,
+                                                const ZipNbr *zp = nullptr) {
   const int lane = lane_id();
   if (!COMP) {
     const int64_t b0 = g.xadj[u];
@@ -250,7 +339,7 @@ __device__ __forceinline__ void warp_neighbours(const GView &g, int64_t u, int64
       f(has, v, w, k - b0);
     }
   } else {
-    ZipNbr z = zip_nbr(g, u);
+    const ZipNbr z = zp ? *zp : zip_nbr(g, u);
     if (z.deg == 0) return;
     int64_t j0 = chunk >= 0 ? chunk : 0, j1 = chunk >= 0 ? chunk + 1 : z.nchunks;
     for (int64_t j = j0; j < j1; ++j) {
@@ -258,8 +347,8 @@ __device__ __forceinline__ void warp_neighbours(const GView &g, int64_t u, int64
       int64_t cnt;
       zip_chunk(g, z, j, cb, ce, cnt);
       const int64_t at = j * kChunkSize;
-      if (!warp_decode_chunk(g, u, cb, ce, cnt,
-                             [&](bool has, int32_t v, int64_t i) { f(has, v, (int64_t)1, at + i); }))
+      if (!warp_decode_trusted(g, u, cb, ce, cnt,
+                               [&](bool has, int32_t v, int64_t i) { f(has, v, (int64_t)1, at + i); }))
         return;
     }
   }

@@ -55,8 +55,9 @@ __global__ void k_rate_small(RateCtx c) {
     for (int64_t k = kb + gw; k < ke; k += nw) {
       int64_t i, u;
       if (tier_entry<MODE>(c, k, i, u)) {
-        const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
-        rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
+        ZipNbr z;
+        const int64_t d = row_degree<COMP>(c.g, u, z);
+        rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
       }
     }
   } else {
@@ -69,8 +70,9 @@ __global__ void k_rate_small(RateCtx c) {
         int j = __ffs(am) - 1;
         am &= am - 1;
         const int64_t v = base + j;
-        const int64_t d = COMP ? zip_nbr(c.g, v).deg : c.g.xadj[v + 1] - c.g.xadj[v];
-        rate_vertex_warp<COMP, MODE, V>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb);
+        ZipNbr z;
+        const int64_t d = row_degree<COMP>(c.g, v, z);
+        rate_vertex_warp<COMP, MODE, V>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
       }
     }
   }
@@ -330,8 +332,9 @@ __global__ void k_rate_list(RateCtx c) {
   for (int64_t k = kb + gw; k < ke; k += nw) {
     int64_t i, u;
     if (!tier_entry<MODE>(c, k, i, u)) continue;
-    const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
-    rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, LOG), &mb);
+    ZipNbr z;
+    const int64_t d = row_degree<COMP>(c.g, u, z);
+    rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, LOG), &mb, &z);
   }
   if (MODE == M_LP) flush_movers(c, mb);
 }
@@ -585,7 +588,8 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
   for (int64_t k = kb + blockIdx.x; k < ke; k += gridDim.x) {
     int64_t i, u;
     if (!tier_entry<MODE>(c, k, i, u)) continue;  // uniform over the block
-    const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
+    ZipNbr z;
+    const int64_t d = row_degree<COMP>(c.g, u, z);  // one chunk: below the chunking threshold
     int logc = 5;
     while (logc < maxlog && ((int64_t)1 << logc) < d + d / 2) ++logc;
     int32_t lb = 0;
@@ -607,7 +611,6 @@ __global__ void __launch_bounds__(kBlockThreads) k_rate_block(RateCtx c, int max
       else return keys[k];
     };
     if (COMP) {
-      const ZipNbr z = zip_nbr(c.g, u);  // one chunk: the big tier is below the chunking threshold
       block_decode_range(c.g, u, z.data, z.end, z.deg, stage, vbuf, red, [&](int cnt) {
         for (int e = tid; e < cnt; e += kBlockThreads) add(c.label[vbuf[e]], (V)1);
       });

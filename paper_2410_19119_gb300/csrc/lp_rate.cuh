@@ -289,11 +289,15 @@ __device__ __forceinline__ void finalize_warp(const RateCtx &c, const Best &b, i
 // first is used, so a row costs two round trips (entries, then labels) per
 // 128 neighbours.
 template <bool COMP, class F>
-__device__ __forceinline__ void warp_labels(const RateCtx &c, int64_t u, F &&add) {
+__device__ __forceinline__ void warp_labels(const RateCtx &c, int64_t u, F &&add,
+                                            const ZipNbr *z = nullptr) {
   if constexpr (COMP) {
-    warp_neighbours<true>(c.g, u, -1, [&](bool has, int32_t v, int64_t w, int64_t) {
-      if (has) add(c.label[v], w);
-    });
+    warp_neighbours<true>(
+        c.g, u, -1,
+        [&](bool has, int32_t v, int64_t w, int64_t) {
+          if (has) add(c.label[v], w);
+        },
+        z);
   } else {
     const int64_t e = c.g.xadj[u + 1];
     for (int64_t i = c.g.xadj[u] + lane_id(); i - lane_id() < e; i += 128) {
@@ -375,13 +379,14 @@ __device__ __forceinline__ Best pick_warp(const RateCtx &c, int64_t u, int64_t c
 // Rates vertex u with one warp; the hash table must be empty on entry and is
 // empty again on exit.
 template <bool COMP, int MODE, class V>
-__device__ __forceinline__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys, V *vals, int logcap,
-                                 MoverBuf *mb) {
+__device__ __forceinline__ void rate_vertex_warp(const RateCtx &c, int64_t u, int32_t *keys,
+                                                 V *vals, int logcap, MoverBuf *mb,
+                                                 const ZipNbr *z = nullptr) {
   // every lane adds its neighbour's label to the table (shared-memory
   // atomics are far cheaper than grouping equal labels across lanes first)
   warp_labels<COMP>(c, u, [&](int32_t x, int64_t w) {
     tbl_add<V>(keys, vals, logcap, x, w, c.g.err);
-  });
+  }, z);
   __syncwarp();
   __threadfence_block();
   const int cap = 1 << logcap;
@@ -393,6 +398,14 @@ __device__ __forceinline__ void rate_vertex_warp(const RateCtx &c, int64_t u, in
   for (int i = lane_id(); i < cap; i += 32) keys[i] = -1, vals[i] = 0;
   __syncwarp();
   finalize_warp<MODE>(c, b, u, cu, mb);
+}
+
+// Degree of u, and (compressed) the layout of its record for the decoder.
+template <bool COMP>
+__device__ __forceinline__ int64_t row_degree(const GView &g, int64_t u, ZipNbr &z) {
+  if (!COMP) return g.xadj[u + 1] - g.xadj[u];
+  z = zip_nbr(g, u);
+  return z.deg;
 }
 
 // Warp tiers: the table of a degree-d vertex uses the first 2^lc slots,

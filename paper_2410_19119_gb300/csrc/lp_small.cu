@@ -132,14 +132,15 @@ __global__ void __launch_bounds__(kLpSmallThreads)
       }
       for (int32_t q = boff[2 * s + 1] + w; q < boff[2 * s + 2]; q += kLpSmallWarps) {
         const int32_t u = list[q];
-        const int64_t d = COMP ? zip_nbr(c.g, u).deg : c.g.xadj[u + 1] - c.g.xadj[u];
+        ZipNbr z;
+        const int64_t d = row_degree<COMP>(c.g, u, z);
         const int lc = table_log(c, d, kMidLog);
         int32_t *keys = reinterpret_cast<int32_t *>(&ws.lab[0][0]);
         uint32_t *vals = &ws.aux[0][0];
         __syncwarp();
         for (int i = lane; i < 1 << lc; i += 32) keys[i] = -1, vals[i] = 0;
         __syncwarp();
-        rate_vertex_warp<COMP, M_LP, uint32_t>(c, u, keys, vals, lc, &mb);
+        rate_vertex_warp<COMP, M_LP, uint32_t>(c, u, keys, vals, lc, &mb, &z);
       }
       flush_movers(c, mb);
       sync_all();
