@@ -677,8 +677,7 @@ bool ip_large(int64_t ns, int64_t entries) {
 template <class V>
 Shape ip_shape(int64_t ns, int64_t entries, int64_t attempts, int64_t large_attempts) {
   if (ip_large<V>(ns, entries)) {
-    int64_t cl = 1;
-    while (cl < 16 && 2 * cl * large_attempts <= num_sms()) cl <<= 1;
+    const int64_t cl = std::max<int64_t>(1, std::min<int64_t>(16, num_sms() / large_attempts));
     if (cl > 1 || ns > ip_smem_cap<V>()) return Shape{kIPMaxThreads, (int)cl};
   }
   // smaller CTAs, several per SM, where many attempts are in flight
@@ -706,7 +705,7 @@ void launch_bisect(const IPCtx &c, int64_t attempts, int cluster, cudaStream_t s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // smaller clusters where the device cannot hold all attempts' at once
-  for (; !SM && cluster > 1; cluster >>= 1) {
+  for (; !SM && cluster > 1; --cluster) {
     attr[0].val.clusterDim.x = (unsigned)cluster;
     cfg.gridDim = dim3((unsigned)(attempts * cluster));
     int fit = 0;

@@ -1018,7 +1018,7 @@ __global__ void k_approve_scatter(ApproveCtx a) {
 }
 
 __global__ void k_approve_contested(ApproveCtx a) {
-  approve_targets(a, (int64_t)a.counters[1], (int)blockIdx.x, (int)gridDim.x);
+  approve_targets<2048>(a, (int64_t)a.counters[1], (int)blockIdx.x, (int)gridDim.x);
 }
 
 // D: apply approved moves and reset the per-target counters. The grid covers
@@ -1433,18 +1433,33 @@ __global__ void __launch_bounds__(256) k_bucket(const uint8_t *tier, int64_t n, 
   }
 }
 
-// Tier buckets: count a list's vertices per sub-round (from sub_byte).
-__global__ void k_tier_count(const int32_t *list, int64_t n, const uint8_t *sub_byte, int32_t S,
+// The lists of the warp and block tiers lie side by side (TierCache::lists):
+// start[t] .. start[t + 1] is list t.
+struct TierRanges {
+  int64_t start[LpWork::kTiers + 1];
+  __device__ __forceinline__ int tier(int64_t k) const {
+    int t = 0;
+#pragma unroll
+    for (int i = 1; i < LpWork::kTiers; ++i) t += k >= start[i];
+    return t;
+  }
+};
+
+// Tier buckets: every list's vertices per sub-round (from sub_byte), all lists
+// in one launch.
+__global__ void k_tier_count(const int32_t *lists, TierRanges r, const uint8_t *sub_byte, int32_t S,
                              int64_t *cnt) {
-  __shared__ int32_t sc[32];
-  if (threadIdx.x < 32) sc[threadIdx.x] = 0;
+  __shared__ int32_t sc[LpWork::kTiers * 32];
+  for (int i = threadIdx.x; i < LpWork::kTiers * 32; i += blockDim.x) sc[i] = 0;
   __syncthreads();
+  const int64_t n = r.start[LpWork::kTiers];
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x)
-    atomicAdd(&sc[sub_byte[list[k]] - 1], 1);
+    atomicAdd(&sc[r.tier(k) * 32 + sub_byte[lists[k]] - 1], 1);
   __syncthreads();
-  if (threadIdx.x < S && sc[threadIdx.x])
-    atomicAdd((unsigned long long *)&cnt[threadIdx.x], (unsigned long long)sc[threadIdx.x]);
+  for (int i = threadIdx.x; i < LpWork::kTiers * 32; i += blockDim.x)
+    if (sc[i])
+      atomicAdd((unsigned long long *)&cnt[(i >> 5) * S + (i & 31)], (unsigned long long)sc[i]);
 }
 
 // Offsets of every tier's sub-rounds (one block): off[t * (S + 1) + s].
@@ -1461,31 +1476,33 @@ __global__ void k_tier_offsets(const int64_t *cnt, int32_t S, int tiers, int64_t
   off[t * (S + 1) + S] = run;
 }
 
-// Scatters a list's positions into its sub-round buckets: each block counts
-// its slice per sub-round, reserves the ranges with one atomic each, then
-// places its entries (the order inside a bucket does not matter).
+// Scatters every list's positions into its sub-round buckets: each block counts
+// its slice of the lists per tier and sub-round, reserves the ranges with one
+// atomic each, then places its entries (the order inside a bucket does not
+// matter).
 constexpr int kTierSlice = 4096;
-__global__ void k_tier_scatter(const int32_t *list, int64_t n, const uint8_t *sub_byte, int32_t S,
-                               int64_t *cur, int32_t *pos) {
-  __shared__ int32_t sc[32];
-  __shared__ int64_t base[32];
+__global__ void k_tier_scatter(const int32_t *lists, TierRanges r, const uint8_t *sub_byte,
+                               int32_t S, int64_t *cur, int32_t *pos) {
+  __shared__ int32_t sc[LpWork::kTiers * 32];
+  __shared__ int64_t base[LpWork::kTiers * 32];
+  const int64_t n = r.start[LpWork::kTiers];
   for (int64_t lo = (int64_t)blockIdx.x * kTierSlice; lo < n; lo += (int64_t)gridDim.x * kTierSlice) {
     const int64_t hi = min(lo + kTierSlice, n);
-    if (threadIdx.x < 32) sc[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < LpWork::kTiers * 32; i += blockDim.x) sc[i] = 0;
     __syncthreads();
-    for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) atomicAdd(&sc[sub_byte[list[k]] - 1], 1);
+    for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x)
+      atomicAdd(&sc[r.tier(k) * 32 + sub_byte[lists[k]] - 1], 1);
     __syncthreads();
-    if (threadIdx.x < S) {
-      base[threadIdx.x] = sc[threadIdx.x]
-                              ? (int64_t)atomicAdd((unsigned long long *)&cur[threadIdx.x],
-                                                   (unsigned long long)sc[threadIdx.x])
-                              : 0;
-      sc[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < LpWork::kTiers * 32; i += blockDim.x) {
+      base[i] = sc[i] ? (int64_t)atomicAdd((unsigned long long *)&cur[(i >> 5) * S + (i & 31)],
+                                           (unsigned long long)sc[i])
+                      : 0;
+      sc[i] = 0;
     }
     __syncthreads();
     for (int64_t k = lo + threadIdx.x; k < hi; k += blockDim.x) {
-      const int s = sub_byte[list[k]] - 1;
-      pos[base[s] + atomicAdd(&sc[s], 1)] = (int32_t)k;
+      const int t = r.tier(k), i = t * 32 + sub_byte[lists[k]] - 1;
+      pos[r.start[t] + base[i] + atomicAdd(&sc[i], 1)] = (int32_t)(k - r.start[t]);
     }
     __syncthreads();
   }
@@ -1518,13 +1535,12 @@ __global__ void k_huge_items(const int32_t *bpos, int64_t nh, const int64_t *pre
 // Buckets the warp and block tiers' lists of this round by sub-round.
 static void tier_buckets(tp_graph *g, LpWork &w, int32_t S, cudaStream_t stream) {
   TierCache &T = g->tiers;
-  const int32_t *lists[LpWork::kTiers] = {T.small.get(), T.mid.get(),  T.mid2.get(),
-                                          T.big0.get(),  T.big1.get(), T.big.get(),
-                                          T.big2.get(),  T.huge.get()};
   const int64_t lens[LpWork::kTiers] = {T.n_small, T.n_mid, T.n_mid2, T.n_big0,
                                         T.n_big1,  T.n_big, T.n_big2, T.n_huge};
   int64_t total = 0;
-  for (int t = 0; t < LpWork::kTiers; ++t) w.tb_base[t] = total, total += lens[t];
+  TierRanges r;
+  for (int t = 0; t < LpWork::kTiers; ++t) r.start[t] = w.tb_base[t] = total, total += lens[t];
+  r.start[LpWork::kTiers] = total;
   w.tb_valid = false;
   if (total == 0) return;
   if ((int64_t)w.tb_pos.n < total) w.tb_pos.alloc(total, stream);
@@ -1534,17 +1550,12 @@ static void tier_buckets(tp_graph *g, LpWork &w, int32_t S, cudaStream_t stream)
   }
   TP_CUDA(cudaMemsetAsync(w.tb_cur.get(), 0, sizeof(int64_t) * LpWork::kTiers * S, stream));
   const int sms = num_sms();
-  for (int t = 0; t < LpWork::kTiers; ++t)
-    if (lens[t])
-      launch(k_tier_count, grid_for(lens[t], 256, (int64_t)sms * 4), 256, 0, stream, lists[t],
-             lens[t], w.bucket_sub.get(), S, w.tb_cur.get() + (int64_t)t * S);
+  launch(k_tier_count, grid_for(total, 256, (int64_t)sms * 4), 256, 0, stream, T.lists.get(), r,
+         w.bucket_sub.get(), S, w.tb_cur.get());
   launch(k_tier_offsets, 1, 32, 0, stream, w.tb_cur.get(), S, LpWork::kTiers, w.tb_off.get(),
          w.tb_cur.get());
-  for (int t = 0; t < LpWork::kTiers; ++t)
-    if (lens[t])
-      launch(k_tier_scatter, grid_for(lens[t], kTierSlice, (int64_t)sms * 4), 256, 0, stream,
-             lists[t], lens[t], w.bucket_sub.get(), S, w.tb_cur.get() + (int64_t)t * S,
-             w.tb_pos.get() + w.tb_base[t]);
+  launch(k_tier_scatter, grid_for(total, kTierSlice, (int64_t)sms * 4), 256, 0, stream, T.lists.get(), r,
+         w.bucket_sub.get(), S, w.tb_cur.get(), w.tb_pos.get());
   TP_LAUNCH_CHECK();
   if (T.n_huge) {
     const int64_t nh = T.n_huge;

@@ -890,8 +890,13 @@ __device__ __forceinline__ void approve_small(const ApproveCtx &a, int64_t base,
 // C: the contested targets 0 .. nt - 1, shared out over nblk blocks (this is
 // number blk): each approves the longest fitting prefix of its movers in
 // (gain desc, vertex asc) order. Few movers (the usual case of clustering)
-// take a warp per target, more a block with the radix select.
+// take a warp per target, more a block with the radix select. CACHE: up to
+// that many movers of a target are read once into shared memory: a pass of the
+// select otherwise waits for three dependent loads per mover.
+template <int CACHE>
 __device__ void approve_targets(const ApproveCtx &a, int64_t nt, int blk, int nblk) {
+  __shared__ int64_t ck[CACHE ? CACHE : 1], cwt[CACHE ? CACHE : 1];
+  __shared__ int32_t cu[CACHE ? CACHE : 1];
   const int nwarp = blockDim.x >> 5;
   for (int64_t j = (int64_t)blk * nwarp + (threadIdx.x >> 5); j < nt; j += (int64_t)nblk * nwarp) {
     const int32_t t = a.ctarget[j];
@@ -911,8 +916,24 @@ __device__ void approve_targets(const ApproveCtx &a, int64_t nt, int blk, int nb
     const int64_t base = a.cbase[t], cnt = s_cnt_t;
     if (cnt <= 32) continue;  // a warp's (0: done)
     const int64_t rem = target_cap(a, t) - a.lw[t];
+    const bool cached = cnt <= CACHE;
+    if (cached) {
+      for (int q = threadIdx.x; q < (int)cnt; q += blockDim.x) {
+        const int32_t i = a.cseg[base + q], u = a.mv_u[i];
+        ck[q] = a.mv_g[i];
+        cu[q] = u;
+        cwt[q] = vwt(a, u);
+      }
+      __syncthreads();
+    }
     auto item = [&](int64_t q, uint64_t &hi, uint32_t &lo, int64_t &w) {
-      int32_t i = a.cseg[base + q];
+      if (cached) {
+        hi = ~(uint64_t)ck[q];
+        lo = (uint32_t)cu[q];
+        w = cwt[q];
+        return;
+      }
+      const int32_t i = a.cseg[base + q];
       hi = ~(uint64_t)a.mv_g[i];
       lo = (uint32_t)a.mv_u[i];
       w = vwt(a, a.mv_u[i]);

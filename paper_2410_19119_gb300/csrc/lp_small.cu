@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kLpSmallThreads)
           a.cseg[a.cbase[t] + atomicAdd(&a.cfill[t], 1)] = v0 + i;
         }
         sync_all();
-        approve_targets(a, nt, rank, cs);
+        approve_targets<0>(a, nt, rank, cs);
         sync_all();
         if (rank == 0 && threadIdx.x == 0) s_ctl = LpSmallCtl{0, 0};
       }
