@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(NT, SM && NT <= 512 ? 1024 / NT : 1) k_bisect(
           };
           uint64_t h;
           uint32_t l;
-          block_select(t ? m1 : m0, caps[t] - (t ? lw1 : lw0), item, h, l);
+          block_select(t ? m1 : m0, caps[t] - (t ? lw1 : lw0), W < (int64_t)1 << 31, item, h, l);
           if (threadIdx.x == 0) ctl->khi[t] = h, ctl->klo[t] = l;
         }
         sync_all();

@@ -1001,8 +1001,9 @@ __global__ void k_approve_alloc(ApproveCtx a) {
   int64_t nt = (int64_t)a.counters[1];
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < nt;
        j += (int64_t)gridDim.x * blockDim.x) {
-    int32_t t = a.ctarget[j];
-    a.cbase[t] = (int64_t)atomicAdd(&a.counters[2], (unsigned long long)a.ccnt[t]);
+    const int32_t t = a.ctarget[j], c = a.ccnt[t];
+    a.cbase[t] = (int64_t)atomicAdd(&a.counters[2], (unsigned long long)c);
+    if (c > 32) a.cbig[atomicAdd(&a.counters[3], 1ull)] = t;
   }
 }
 
@@ -1012,13 +1013,16 @@ __global__ void k_approve_scatter(ApproveCtx a) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nm;
        i += (int64_t)gridDim.x * blockDim.x) {
     if (a.mv_ok[i]) continue;
-    int32_t t = a.mv_t[i];
-    a.cseg[a.cbase[t] + atomicAdd(&a.cfill[t], 1)] = (int32_t)i;
+    put_contested(a, i, a.mv_t[i]);
   }
 }
 
-__global__ void k_approve_contested(ApproveCtx a) {
-  approve_targets<2048>(a, (int64_t)a.counters[1], (int)blockIdx.x, (int)gridDim.x);
+// 1024 threads: the movers into a hub's cluster can be 1e5 and more, one
+// block's work (with 256 threads and the gains behind two index loads such a
+// segment took 0.19 ms).
+constexpr int kContestedThreads = 1024;
+__global__ void __launch_bounds__(kContestedThreads) k_approve_contested(ApproveCtx a) {
+  approve_targets(a, (int64_t)a.counters[1], (int64_t)a.counters[3], (int)blockIdx.x, (int)gridDim.x);
 }
 
 // D: apply approved moves and reset the per-target counters. The grid covers
@@ -1659,12 +1663,15 @@ void LpWork::init(int64_t n_vertices, int64_t n_labels, cudaStream_t s) {
   cfill.alloc(L, s);
   cbase.alloc(L, s);
   ctarget.alloc(L, s);
+  cbig.alloc(L, s);
   mv_u.alloc(N, s);
   mv_t.alloc(N, s);
   mv_o.alloc(N, s);
   mv_g.alloc(N, s);
   mv_ok.alloc(N, s);
   cseg.alloc(N, s);
+  cseg_u.alloc(N, s);
+  cseg_g.alloc(N, s);
   counters.alloc(4, s);
   TP_CUDA(cudaMemsetAsync(in_w.get(), 0, L * 8, s));
   TP_CUDA(cudaMemsetAsync(ccnt.get(), 0, L * 4, s));
@@ -1686,7 +1693,7 @@ void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStr
   launch(k_approve_fit, wide, 256, 0, stream, a);
   launch(k_approve_alloc, (unsigned)num_sms(), 256, 0, stream, a);
   launch(k_approve_scatter, blocks, 256, 0, stream, a);
-  launch(k_approve_contested, (unsigned)num_sms() * 2, 256, 0, stream, a);
+  launch(k_approve_contested, (unsigned)num_sms() * 2, kContestedThreads, 0, stream, a);
   launch(k_apply, wide, 256, 0, stream, a);
   if (wake) {
     const int64_t limit = wake->n / (8 * (int64_t)S);
@@ -2049,19 +2056,21 @@ void lp_cluster(tp_graph *g, int64_t U, const tp_params &p, int32_t level, int32
   launch(k_init_singletons, grid_for(n, 256), 256, 0, s, g->unit_vw ? nullptr : g->vw.get(), n,
                                                        d_cluster, Wc.get());
   TP_LAUNCH_CHECK();
-  LpWork w;
-  w.init(n, n, s);
   LpState st{d_cluster, Wc.get(), n, U};
   if (seg) {  // labels are vertices: a label's graph and base are its vertex's
     st.seg = *seg;
     st.seg.lgid = seg->gid;
     st.seg.lb = seg->vb;
   }
-  prof_scope(level == 0 && !seg);
-  if (ev_begin) TP_CUDA(cudaEventRecord(ev_begin, s));
-  lp_rounds(g, st, w, p.seed, kTagCluster, (uint64_t)level, 0, p.cluster_rounds, p.sub_rounds, p, s);
-  if (ev_end) TP_CUDA(cudaEventRecord(ev_end, s));
-  prof_scope(false);
+  {
+    LpWork w;  // gone before the packing's buffers are made
+    w.init(n, n, s);
+    prof_scope(level == 0 && !seg);
+    if (ev_begin) TP_CUDA(cudaEventRecord(ev_begin, s));
+    lp_rounds(g, st, w, p.seed, kTagCluster, (uint64_t)level, 0, p.cluster_rounds, p.sub_rounds, p, s);
+    if (ev_end) TP_CUDA(cudaEventRecord(ev_end, s));
+    prof_scope(false);
+  }
   if (p.two_hop) two_hop(g, d_cluster, Wc.get(), U, p.seed, level, p, s, seg ? &st.seg : nullptr);
   release_hub_tables(g, s);
 }

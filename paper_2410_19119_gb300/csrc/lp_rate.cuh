@@ -851,19 +851,32 @@ struct ApproveCtx {
   const int64_t *mv_g;
   int8_t *mv_ok;
   int64_t *in_w;
-  int32_t *ccnt, *cfill, *cseg, *ctarget;
+  int32_t *ccnt, *cfill, *ctarget, *cbig;
+  // contested movers grouped by target: index, gain and vertex side by side, so
+  // the select reads a segment straight through
+  int32_t *cseg, *cseg_u;
+  int64_t *cseg_g;
   int64_t *cbase;
-  unsigned long long *counters;  // [0] movers [1] contested targets [2] contested pool
+  // [0] movers [1] contested targets [2] contested pool [3] targets of more than 32 movers
+  unsigned long long *counters;
   int32_t *label;
   int64_t *lw;
   int64_t cap;
   const int64_t *vw;
+  bool narrow;  // all vertex weights together fit 31 bits
   // batched graphs: graph of every label and every graph's cap (null: one graph)
   const int32_t *lgid;
   const int64_t *gcap;
 };
 
 __device__ __forceinline__ int64_t vwt(const ApproveCtx &a, int64_t u) { return a.vw ? a.vw[u] : 1; }
+// Mover i's place in its target's segment.
+__device__ __forceinline__ void put_contested(const ApproveCtx &a, int64_t i, int32_t t) {
+  const int64_t at = a.cbase[t] + atomicAdd(&a.cfill[t], 1);
+  a.cseg[at] = (int32_t)i;
+  a.cseg_u[at] = a.mv_u[i];
+  a.cseg_g[at] = a.mv_g[i];
+}
 __device__ __forceinline__ int64_t target_cap(const ApproveCtx &a, int32_t t) {
   return a.lgid ? a.gcap[a.lgid[t]] : a.cap;
 }
@@ -875,8 +888,8 @@ __device__ __forceinline__ void approve_small(const ApproveCtx &a, int64_t base,
   const int lane = lane_id();
   const bool in = lane < cnt;
   const int32_t i = in ? a.cseg[base + lane] : 0;
-  const int64_t g = in ? a.mv_g[i] : 0;
-  const int32_t u = in ? a.mv_u[i] : 0;
+  const int64_t g = in ? a.cseg_g[base + lane] : 0;
+  const int32_t u = in ? a.cseg_u[base + lane] : 0;
   const int64_t w = in ? vwt(a, u) : 0;
   int64_t pre = 0;
   for (int q = 0; q < cnt; ++q) {
@@ -887,16 +900,11 @@ __device__ __forceinline__ void approve_small(const ApproveCtx &a, int64_t base,
   if (in && pre <= rem) a.mv_ok[i] = 1;
 }
 
-// C: the contested targets 0 .. nt - 1, shared out over nblk blocks (this is
-// number blk): each approves the longest fitting prefix of its movers in
+// C: the nt contested targets (and among them the nbig of more than 32 movers,
+// listed apart), shared out over nblk blocks (this is number blk): each approves the longest fitting prefix of its movers in
 // (gain desc, vertex asc) order. Few movers (the usual case of clustering)
-// take a warp per target, more a block with the radix select. CACHE: up to
-// that many movers of a target are read once into shared memory: a pass of the
-// select otherwise waits for three dependent loads per mover.
-template <int CACHE>
-__device__ void approve_targets(const ApproveCtx &a, int64_t nt, int blk, int nblk) {
-  __shared__ int64_t ck[CACHE ? CACHE : 1], cwt[CACHE ? CACHE : 1];
-  __shared__ int32_t cu[CACHE ? CACHE : 1];
+// take a warp per target, more a block with the radix select.
+__device__ void approve_targets(const ApproveCtx &a, int64_t nt, int64_t nbig, int blk, int nblk) {
   const int nwarp = blockDim.x >> 5;
   for (int64_t j = (int64_t)blk * nwarp + (threadIdx.x >> 5); j < nt; j += (int64_t)nblk * nwarp) {
     const int32_t t = a.ctarget[j];
@@ -907,41 +915,21 @@ __device__ void approve_targets(const ApproveCtx &a, int64_t nt, int blk, int nb
     __syncwarp();
     if (lane_id() == 0) a.ccnt[t] = 0, a.cfill[t] = 0;
   }
-  for (int64_t j = blk; j < nt; j += nblk) {
-    __shared__ int32_t s_cnt_t;
-    const int32_t t = a.ctarget[j];
-    __syncthreads();  // the previous target is done with
-    if (threadIdx.x == 0) s_cnt_t = a.ccnt[t];
-    __syncthreads();
-    const int64_t base = a.cbase[t], cnt = s_cnt_t;
-    if (cnt <= 32) continue;  // a warp's (0: done)
+  for (int64_t j = blk; j < nbig; j += nblk) {
+    const int32_t t = a.cbig[j];
+    const int64_t base = a.cbase[t], cnt = a.ccnt[t];
+    __syncthreads();  // every thread has read ccnt, and the previous target is done with
     const int64_t rem = target_cap(a, t) - a.lw[t];
-    const bool cached = cnt <= CACHE;
-    if (cached) {
-      for (int q = threadIdx.x; q < (int)cnt; q += blockDim.x) {
-        const int32_t i = a.cseg[base + q], u = a.mv_u[i];
-        ck[q] = a.mv_g[i];
-        cu[q] = u;
-        cwt[q] = vwt(a, u);
-      }
-      __syncthreads();
-    }
     auto item = [&](int64_t q, uint64_t &hi, uint32_t &lo, int64_t &w) {
-      if (cached) {
-        hi = ~(uint64_t)ck[q];
-        lo = (uint32_t)cu[q];
-        w = cwt[q];
-        return;
-      }
-      const int32_t i = a.cseg[base + q];
-      hi = ~(uint64_t)a.mv_g[i];
-      lo = (uint32_t)a.mv_u[i];
-      w = vwt(a, a.mv_u[i]);
+      const int32_t u = a.cseg_u[base + q];
+      hi = ~(uint64_t)a.cseg_g[base + q];
+      lo = (uint32_t)u;
+      w = vwt(a, u);
     };
     if (rem >= 0) {  // (else nothing can enter: mv_ok is 0 already)
       uint64_t khi;
       uint32_t klo;
-      block_select(cnt, rem, item, khi, klo);
+      block_select(cnt, rem, a.narrow, item, khi, klo);
       for (int64_t q = threadIdx.x; q < cnt; q += blockDim.x) {
         uint64_t hi;
         uint32_t lo;
@@ -965,13 +953,17 @@ ApproveCtx approve_ctx(tp_graph *g, const LpState &st, LpWork &w) {
   a.ccnt = w.ccnt.get();
   a.cfill = w.cfill.get();
   a.cseg = w.cseg.get();
+  a.cseg_u = w.cseg_u.get();
+  a.cseg_g = w.cseg_g.get();
   a.ctarget = w.ctarget.get();
+  a.cbig = w.cbig.get();
   a.cbase = w.cbase.get();
   a.counters = (unsigned long long *)w.counters.get();
   a.label = st.label;
   a.lw = st.lw;
   a.cap = st.cap;
   a.vw = g->unit_vw ? nullptr : g->vw.get();
+  a.narrow = g->total_vw >= 0 && g->total_vw < ((int64_t)1 << 31);
   a.lgid = st.seg.gid ? st.seg.lgid : nullptr;
   a.gcap = st.seg.cap;
   return a;

@@ -44,6 +44,7 @@ static_assert(sizeof(uint32_t) * kLaneMaxDeg * 32 == sizeof(int32_t) << kMidLog,
 struct LpSmallCtl {
   int32_t targets;
   int32_t pool;
+  int32_t big;  // targets of more than 32 movers
 };
 
 template <bool COMP, bool W>
@@ -76,7 +77,7 @@ __global__ void __launch_bounds__(kLpSmallThreads)
   uint32_t *col = &ws.lab[0][lane], *wcol = &ws.aux[0][lane];
   uint8_t *cnt8 = reinterpret_cast<uint8_t *>(&ws.aux[0][0]) + lane;
   MoverBuf mb{ws.mu, ws.mt, ws.mo, ws.mg, 0};
-  if (threadIdx.x == 0) s_ctl = LpSmallCtl{0, 0}, s_cnt = 0;
+  if (threadIdx.x == 0) s_ctl = LpSmallCtl{0, 0, 0}, s_cnt = 0;
   for (int32_t r = 0; r < rounds; ++r) {
     // ---- buckets of this round
     const uint64_t rk = round_key(seed, tag, ra, rb + (uint64_t)r);
@@ -159,19 +160,19 @@ __global__ void __launch_bounds__(kLpSmallThreads)
         // longest fitting prefix in (gain desc, vertex asc) order
         for (int32_t j = rank * kLpSmallThreads + (int32_t)threadIdx.x; j < nt;
              j += cs * kLpSmallThreads) {
-          const int32_t t = a.ctarget[j];
-          a.cbase[t] = atomicAdd(&ctl->pool, a.ccnt[t]);
+          const int32_t t = a.ctarget[j], cnt = a.ccnt[t];
+          a.cbase[t] = atomicAdd(&ctl->pool, cnt);
+          if (cnt > 32) a.cbig[atomicAdd(&ctl->big, 1)] = t;
         }
         sync_all();
         for (int32_t i = threadIdx.x; i < nm; i += kLpSmallThreads) {
           if (a.mv_ok[v0 + i]) continue;
-          const int32_t t = c.mv_t[i];
-          a.cseg[a.cbase[t] + atomicAdd(&a.cfill[t], 1)] = v0 + i;
+          put_contested(a, v0 + i, c.mv_t[i]);
         }
         sync_all();
-        approve_targets<0>(a, nt, rank, cs);
+        approve_targets(a, nt, ctl->big, rank, cs);
         sync_all();
-        if (rank == 0 && threadIdx.x == 0) s_ctl = LpSmallCtl{0, 0};
+        if (rank == 0 && threadIdx.x == 0) s_ctl = LpSmallCtl{0, 0, 0};
       }
       // ---- approved moves
       for (int32_t i = threadIdx.x; i < nm; i += kLpSmallThreads) {

@@ -14,9 +14,12 @@ namespace tp {
 // Bound by its barriers and by the search through the 256 bins, which one
 // warp does with a scan (eight bins a lane): a thread walking the bins took
 // about 4 us a pass at 2 GHz, most of the select for the usual few hundred
-// items.
+// items. narrow: all weights together fit 31 bits, and the bins are summed with
+// native 32-bit shared atomics (the 64-bit ones retry, and most items of a
+// large segment share a few bins).
 template <class Item>
-__device__ void block_select(int64_t cnt, int64_t rem, Item item, uint64_t &khi, uint32_t &klo) {
+__device__ void block_select(int64_t cnt, int64_t rem, bool narrow, Item item, uint64_t &khi,
+                             uint32_t &klo) {
   __shared__ unsigned long long hist[256];
   __shared__ int64_t s_cum;
   __shared__ int s_bin;
@@ -58,8 +61,9 @@ __device__ void block_select(int64_t cnt, int64_t rem, Item item, uint64_t &khi,
         int64_t w;
         item(q, hi, lo, w);
         if ((hi & mhi) != fhi || (lo & mlo) != flo) continue;
-        atomicAdd(&hist[in_hi ? (uint32_t)(hi >> shift) & 255u : (lo >> shift) & 255u],
-                  (unsigned long long)w);
+        const uint32_t d = in_hi ? (uint32_t)(hi >> shift) & 255u : (lo >> shift) & 255u;
+        if (narrow) atomicAdd(reinterpret_cast<unsigned *>(&hist[d]), (unsigned)w);  // (its low half)
+        else atomicAdd(&hist[d], (unsigned long long)w);
       }
       __syncthreads();
       if (threadIdx.x < 32) {  // first bin whose inclusive prefix exceeds rem (else the last)

@@ -442,8 +442,10 @@ struct LpWork {
   Buf<int32_t> mv_o;        // n: the mover's label when it was rated (its source)
   Buf<int64_t> mv_g;        // n
   Buf<int8_t> mv_ok;        // n
-  Buf<int32_t> cseg;        // n (contested mover indices grouped by target)
+  Buf<int32_t> cseg, cseg_u;  // n (contested movers grouped by target: index, vertex)
+  Buf<int64_t> cseg_g;        // n (and gain)
   Buf<int32_t> ctarget;     // nlabels (contested targets)
+  Buf<int32_t> cbig;        // nlabels (those of more than 32 movers)
   Buf<int64_t> counters;    // [0] movers, [1] contested targets, [2] contested pool
   // lane-tier vertices of the current round grouped by sub-round (A3)
   Buf<int32_t> bucket;       // n
