@@ -12,21 +12,25 @@
 //   mid   (deg <= tier_mid):   one warp per vertex, shared table of up to
 //          1024 slots (both warp tiers fill and scan only the least power of
 //          two >= table_slack * degree slots, at least 32);
-//   big   (deg <= 10000):      one block per vertex, shared table of 8192 or
-//          16384 slots;
+//   big   (deg <= 10000):      one block per vertex, shared table of 2048 to
+//          16384 slots by its degree;
 //   huge  (deg > 10000):       one block per chunk of 1000 neighbours (the
 //          compressed format's independently decodable chunks) aggregates in
 //          a shared table and flushes into the vertex's global table with
 //          atomics (the paper's "hash tables as flush buffers" against
 //          contention); blocks then scan that table in segments and one
 //          block per vertex combines the segments' results.
+// Where the labels are at most 1024 blocks (refinement, rebalancing) the tiers
+// above lane count in one counter per block instead of a hash table. Levels of
+// one graph that fit a thread-block cluster run all their rounds in one launch
+// (lp_small.cu).
 // The tier only decides where the sums are formed; integer sums commute and
 // the argmax uses a total order, so the result is tier-independent.
 //
 // Approval: movers add their weight to in_w[target] with atomics. Targets
-// whose weight plus in_w fits approve every mover; for the others one block
-// per target runs a weighted radix select over the key (gain desc, vertex
-// asc) and approves exactly the longest fitting prefix.
+// whose weight plus in_w fits approve every mover; for the others a warp (up
+// to 32 movers) or a block per target runs a weighted radix select over the
+// key (gain desc, vertex asc) and approves exactly the longest fitting prefix.
 #include <algorithm>
 #include <memory>
 #include <mutex>
@@ -172,10 +176,6 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
         lane_batch<COMP, MODE, W, 8, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
       else if (maxdeg <= 16)
         lane_batch<COMP, MODE, W, 16, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
-      else if (!W && !COMP && maxdeg <= 24)
-        // half of the batches of a mesh of average degree 16 (the compressed
-        // kernel, with the decoder beside them, lost a fifth to a third size)
-        lane_batch<COMP, MODE, W, 24, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
       else
         lane_batch<COMP, MODE, W, kLaneMaxDeg, SEG, false, WIDE>(c, has, u, deg, col, wcol, cnt, mb, nmv);
     }
@@ -1900,9 +1900,15 @@ void lp_rounds(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, uint64_
   // quiet vertices: one graph, most entries in the lane tier, and so few
   // sub-rounds that the epoch (one step each at most) fits its byte. In
   // clustering nearly every vertex moves in the first two rounds, which go
-  // without (labels are vertices then: kmax is 0).
+  // without (labels are vertices then: kmax is 0), and the two rounds after
+  // them cost more with the marks than they save: on a mesh of 2^24 vertices 3
+  // rounds took 8.39 ms with and 7.58 without them, 5 rounds 11.27 and 11.20,
+  // 6 rounds 12.30 and 12.98, 12 rounds 16.6 and 23.5 (CSR); where decoding
+  // makes a rating dearer 5 rounds took 11.29 and 12.10.
   const int32_t quiet_from = st.kmax ? 0 : 2;
-  const bool quiet_ok = !st.seg.gid && S <= 32 && (int64_t)rounds * S < 250 && rounds > quiet_from &&
+  // A single round rates every vertex once, so marks are of no use in it.
+  const int32_t quiet_least = st.kmax ? 2 : g->compressed ? 5 : 6;
+  const bool quiet_ok = !st.seg.gid && S <= 32 && (int64_t)rounds * S < 250 && rounds >= quiet_least &&
                         !T.lane_long && !prof_active() && 5 * T.edges[TIER_LANE] >= 4 * g->m2 &&
                         g->n <= kLaneKeyLabels && st.nlabels <= kLaneKeyLabels;
   std::unique_ptr<ApprovalGraph> ag;

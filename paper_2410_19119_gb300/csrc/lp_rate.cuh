@@ -508,35 +508,36 @@ __device__ __forceinline__ void cmp_swap(T &x, T &y) {
   y = hi;
 }
 
-// Merges the two sorted halves of the subsequence a[LO], a[LO + R], ...; only
-// the first LIM elements exist (those beyond would be larger than any, and
-// every comparator leaves the larger of its pair at the higher index).
-template <int LO, int N, int R, int LIM, class T>
+// Merges the two sorted halves of the subsequence a[LO], a[LO + R], ...
+template <int LO, int N, int R, class T>
 __device__ __forceinline__ void oem_merge(T (&a)[kLaneMaxDeg]) {
   constexpr int M = 2 * R;
   if constexpr (M < N) {
-    oem_merge<LO, N, M, LIM>(a);
-    oem_merge<LO + R, N, M, LIM>(a);
+    oem_merge<LO, N, M>(a);
+    oem_merge<LO + R, N, M>(a);
 #pragma unroll
-    for (int i = LO + R; i + R < LO + N && i + R < LIM; i += M) cmp_swap(a[i], a[i + R]);
-  } else if constexpr (LO + R < LIM) {
+    for (int i = LO + R; i + R < LO + N; i += M) cmp_swap(a[i], a[i + R]);
+  } else {
     cmp_swap(a[LO], a[LO + R]);
   }
 }
 
-template <int LO, int N, int LIM, class T>
+// N: 8, 16 or 32. (A network of 24, 32 without its last quarter, fits half of
+// the batches of a mesh of average degree 16, but a further size beside the
+// others cost the compressed kernel 15.0 -> 18.5 ms over 80 launches and the
+// CSR kernel 3.36 -> 3.93 ms for a round of 2^24 vertices.)
+template <int LO, int N, class T>
 __device__ __forceinline__ void oem_sort_range(T (&a)[kLaneMaxDeg]) {
-  if constexpr (N > 1 && LO < LIM) {
-    oem_sort_range<LO, N / 2, LIM>(a);
-    oem_sort_range<LO + N / 2, N / 2, LIM>(a);
-    oem_merge<LO, N, 1, LIM>(a);
+  if constexpr (N > 1) {
+    oem_sort_range<LO, N / 2>(a);
+    oem_sort_range<LO + N / 2, N / 2>(a);
+    oem_merge<LO, N, 1>(a);
   }
 }
 
-// N: 8, 16, 24 (the network of 32 without its last quarter) or 32.
 template <int N, class T>
 __device__ __forceinline__ void oem_sort(T (&a)[kLaneMaxDeg]) {
-  oem_sort_range<0, (N <= 8 ? 8 : N <= 16 ? 16 : 32), N>(a);
+  oem_sort_range<0, N>(a);
 }
 
 // Mover records of one batch.
