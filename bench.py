@@ -112,7 +112,7 @@ def peaks():
 
 
 KERNEL_SOURCES = {  # files that define each profiled kernel family
-    "rate": ("lp.cu", "decode.cuh", "tp_internal.cuh"),
+    "rate": ("lp.cu", "lp_rate.cuh", "decode.cuh", "tp_internal.cuh"),
 }
 
 

@@ -64,7 +64,7 @@ __global__ void k_members(const int32_t *map, const int32_t *place, const int64_
 
 // ---------------------------------------------------------------- table sizes
 // Size 0 and 1: a warp's table of 256 / 1024 slots; 2 and 3: a block's of 4096
-// / 16384; 4: keys and the radix sort. A table takes up to kAggFill distinct
+// / 16384; 4: keys and the radix sort. A table takes up to agg_fill distinct
 // neighbours; a coarse vertex starts with a size whose fill is no less than a
 // fifth of its entries (meshes merge far more than that into one, skewed
 // graphs less and move up).
@@ -841,8 +841,9 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
                    const int64_t *seg_voff, int64_t nseg, int64_t *seg_coff) {
   int64_t n = g->n;
   // a compressed graph with long records is decoded first (each chunk once, by
-  // a warp): in the tables' kernels such a record is one warp's, and R-MAT
-  // 2^22 spent 39 ms in them where decoding and the CSR kernels take 8
+  // a warp): in the tables' kernels such a record is one warp's, and level 0
+  // of R-MAT 2^22 spent 39 ms in them where decoding takes 2 and the CSR
+  // kernels 13.5
   std::unique_ptr<tp_graph> csr;
   if (g->compressed && g->max_deg > kAggDecodeDeg) {
     csr.reset(decompress(g, s));

@@ -973,7 +973,7 @@ __global__ void k_zip_header_check(GView g, const int64_t *xadj, int32_t *bad) {
 // the warp's neighbours lie as they will in the adjacency, and the warp copies
 // the piece out coalesced. (A warp per record used 30 of the 128 bytes of its
 // window and left most lanes idle: 3.15 ms for a mesh of 3 M vertices, where
-// this takes 0.15.) Records of more than kUnzipLane neighbours are listed, a
+// this takes 0.20.) Records of more than kUnzipLane neighbours are listed, a
 // chunk per item, for k_unzip_items. Every rule of the format is checked:
 // VarInts of at most five bytes, gaps of at least one, ids inside the graph,
 // the record's bytes used up exactly.

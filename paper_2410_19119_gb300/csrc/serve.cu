@@ -165,8 +165,8 @@ struct tp_server {
 extern "C" {
 
 // Device bytes of one request, phase by phase from the library's
-// allocations (bytes per vertex n / adjacency entry m / block k), for any graph whose hierarchy stays inside this
-// envelope: the coarse levels together hold at most n vertices and 2 m
+// allocations (bytes per vertex n / adjacency entry m / block k), for any
+// graph whose hierarchy stays inside this envelope: the coarse levels together hold at most n vertices and 2 m
 // adjacency entries (each level has fewer entries than the one below; R-MAT
 // scale 26 coarse levels hold 0.05 n and 1.5 m, random geometric graphs
 // about 0.1 n and 0.3 m), any level may be made of hubs entirely, and the
@@ -176,15 +176,20 @@ extern "C" {
 //   part     4n (the request's result)
 //   levels   coarse CSR 16n + 12m per level; per level a map 4n and a tier
 //            cache 5n + 0.05m  -> within the envelope 30n + 24m
-//   cluster  C, map, cluster weights 16n; LP workspace 62n, 8n more for the
-//            records of a compressed level; two-hop packing 88n; hub rating
-//            tables 14 bytes per slot, fewer than 4 slots per hub neighbour: 56m
-//   contract flags, ranks, offsets 24n + coarse weights 8n; keys and their
-//            radix buffer 16m (weights unpackable into keys: 32m); coarse
-//            CSR 12m while the keys live
-//   initial  T attempts x 53 bytes per coarsest vertex + 40 + its CSR 12m
-//   refine   two partition arrays 8n, LP workspace 50n, hub tables 56m;
-//            block weights and per-block approval state 36k (counted apart)
+//   cluster  C, map, cluster weights 16n; LP workspace 79n, 8n more for the
+//            records of a compressed level, given back before two-hop packing
+//            takes 88n (the sum counted, 174n, is more than either needs); hub
+//            rating tables 14 bytes per slot, fewer than 4 slots per hub
+//            neighbour: 56m
+//   contract flags, ranks, members, offsets 32n; the tables' rows 12m and the
+//            coarse CSR 12m, or, where every coarse vertex is a hub, keys and
+//            weights with their radix buffers 32m; a compressed level decoded
+//            for it 8n + 4m, within what clustering is counted for
+//   initial  T attempts x 53 bytes per coarsest vertex (22 and lists used) + 40
+//            + its CSR 12m
+//   refine   two partition arrays 8n, LP workspace 50n (less than clustering's,
+//            which decides the maximum), hub tables 56m; block weights and
+//            per-block approval state 36k (counted apart)
 // The server admits a request by this figure and caps what its thread may
 // allocate at it; a request that would exceed it fails before allocating
 // and runs again alone with the whole budget.
