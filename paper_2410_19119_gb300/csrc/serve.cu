@@ -166,11 +166,12 @@ extern "C" {
 
 // Device bytes of one request, phase by phase from the library's
 // allocations (bytes per vertex n / adjacency entry m / block k), for any
-// graph whose hierarchy stays inside this envelope: the coarse levels together hold at most n vertices and 2 m
-// adjacency entries (each level has fewer entries than the one below; R-MAT
-// scale 26 coarse levels hold 0.05 n and 1.5 m, random geometric graphs
-// about 0.1 n and 0.3 m), any level may be made of hubs entirely, and the
-// coarsest graph has at most min(n, 4 c_lim k) vertices.
+// graph whose hierarchy stays inside this envelope: the coarse levels
+// together hold at most n vertices and 2 m adjacency entries (each level has
+// fewer entries than the one below; R-MAT scale 26 coarse levels hold 0.05 n
+// and 1.5 m, random geometric graphs about 0.1 n and 0.3 m), any level may be
+// made of hubs entirely, and the coarsest graph has at most min(n, 4 c_lim k)
+// vertices.
 //   upload   CSR 8n + 4m; with compression the stream (<= 10n + 5m + the
 //            chunk tables), its offsets and the encoder's scratch 16n
 //   part     4n (the request's result)
