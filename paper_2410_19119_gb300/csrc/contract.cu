@@ -15,7 +15,8 @@
 // the key a*n' + b, which the library's LSD radix sort and a run-length
 // reduction turn into their rows. (Sorting all entries took five passes over
 // them; a mesh merges about 17 entries into one.) Weights are summed in 32
-// bits where all edge weights together fit.
+// bits where all edge weights together fit or every edge weighs one (a table's
+// coarse vertex has no more than 40 960 entries).
 #include <algorithm>
 #include <memory>
 
@@ -887,7 +888,11 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
     if (!g->unit_vw) TP_CUDA(cudaMemsetAsync(cg->vw.get(), 0, nc * sizeof(int64_t), s));
     const GView v = view(g);
     const bool comp = g->compressed;
-    const bool narrow = ew_sum_bound(g) < ((int64_t)1 << 31);
+    // 32-bit sums in the tables: where all edge weights together fit, or weigh
+    // one each: no coarse vertex of more than agg_start entries enters a table,
+    // however many the graph has (compressed graphs of 2^31 entries and more
+    // among them, whose kernels exist with this type only)
+    const bool narrow = g->unit_ew || ew_sum_bound(g) < ((int64_t)1 << 31);
 
     // members by coarse vertex, and the first table size of each
     Buf<int32_t> members(n, s), lists((kAggSizes + 1) * nc, s);
