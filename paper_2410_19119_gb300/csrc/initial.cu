@@ -662,10 +662,15 @@ constexpr size_t kIPSmem = 220 * 1024;
 // take it over 100 us a pass.
 constexpr int64_t kIPClusterEntries = (int64_t)1 << 19;
 
+// Most vertices whose state fits: a multiple of 16, as a launch rounds its
+// largest node up to one (12 512 vertices, 10 224 with 64-bit differences).
 template <class V>
-int64_t ip_smem_cap() {
-  return (int64_t)((kIPSmem - 16) / (sizeof(V) + 14));
+constexpr int64_t ip_smem_cap() {
+  return (int64_t)((kIPSmem - 16) / (sizeof(V) + 14)) & ~(int64_t)15;
 }
+static_assert(ip_smem_bytes<int32_t>(ip_smem_cap<int32_t>()) <= kIPSmem &&
+                  ip_smem_bytes<int64_t>(ip_smem_cap<int64_t>()) <= kIPSmem,
+              "the largest node's state fits");
 
 template <class V>
 bool ip_large(int64_t ns, int64_t entries) {
