@@ -746,8 +746,11 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
   Buf<int32_t> ord, claimer, cnt, list;  // cluster form only
   Buf<V> dif;
   Buf<uint8_t> sub;
+  Buf<int64_t> cut;
   DepthDev dev, next_dev;
-  TierStreams streams;  // (after the buffers: gone before them)
+  // after every buffer that its kernels use: an error while the classes of a
+  // depth run side by side waits for them before any of it is freed
+  TierStreams streams;
   std::vector<int64_t> host, next_host;
   for (int depth = 0; d.nodes() > 0; ++depth) {
     const int32_t nodes = d.nodes();
@@ -810,7 +813,7 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
       c.ladj = ladj.get();
       c.lew = weighted ? lew.get() : nullptr;
     }
-    Buf<int64_t> cut((int64_t)nodes * T, s);
+    if ((int64_t)cut.n < (int64_t)nodes * T) cut.alloc((int64_t)nodes * T, s);
     c.n = n;
     c.n_nodes = nodes;
     c.vw = g->unit_vw ? nullptr : g->vw.get();
