@@ -22,6 +22,7 @@ struct Error {
   do {                                                                                   \
     cudaError_t e_ = (call);                                                             \
     if (e_ != cudaSuccess) {                                                             \
+      (void)cudaGetLastError(); /* reported here, not by the next launch check */        \
       fprintf(stderr, "terapart: %s failed: %s (%s:%d)\n", #call, cudaGetErrorString(e_), \
               __FILE__, __LINE__);                                                       \
       throw ::tp::Error{e_ == cudaErrorMemoryAllocation ? TP_ERR_OOM : TP_ERR_CUDA};     \
