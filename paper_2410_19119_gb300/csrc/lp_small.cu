@@ -194,18 +194,19 @@ __global__ void __launch_bounds__(kLpSmallThreads)
 }
 
 // Cluster size for a level that k_lp_small can take, 0 for the others: one
-// graph, no vertex above the mid tier, 32-bit ratings, at most 32 sub-rounds,
-// and so few vertices and entries that 16 CTAs rate an eighth of them in about
-// the time that the kernels of a sub-round take to launch. The smallest
-// cluster that gives a CTA at most kLpSmallItems batches or vertices per
-// sub-round: the lanes of a batch read different rows and labels, and an SM's
-// L1 looks up one line a cycle (a batch of degree 16 takes about 700), so 16
-// batches on one SM cost more than four on each of four and their barriers.
+// graph, no vertex above the mid tier, 32-bit ratings, with edge weights labels
+// that fit the lane tier's 32-bit sort keys (block numbers need not), at most 32
+// sub-rounds, and so few vertices and entries that 16 CTAs rate an eighth of
+// them in about the time that the kernels of a sub-round take to launch. The
+// smallest cluster that gives a CTA at most kLpSmallItems batches or vertices
+// per sub-round: the lanes of a batch read different rows and labels, and an
+// SM's L1 looks up one line a cycle (a batch of degree 16 takes about 700), so
+// 16 batches on one SM cost more than four on each of four and their barriers.
 int lp_small_cluster(const tp_graph *g, const LpState &st, int32_t S) {
   const TierCache &T = g->tiers;
   if (st.seg.gid || S > 32 || T.lane_long ||
       T.count[TIER_BIG] + T.count[TIER_HUGE] > 0 ||
-      !(g->unit_ew || ew_sum_bound(g) < ((int64_t)1 << 31)))
+      (!g->unit_ew && (ew_sum_bound(g) >= ((int64_t)1 << 31) || st.nlabels > kLaneKeyLabels)))
     return 0;
   if (g->n > kLpSmallVertices * kLpSmallCluster || g->m2 > kLpSmallEntries * kLpSmallCluster)
     return 0;
