@@ -44,6 +44,14 @@ def test_vertices_without_entries():
     assert _ms(lambda: tp.contract(g, u % 64)) < 10 * usual
 
 
+def test_cut_mesh():
+    n = 1 << 22
+    z = tp.graph_from_csr(*synth.rgg2d(n, 16.0, 3)).compress()
+    u = torch.arange(n, dtype=torch.int64, device="cuda")
+    usual = _ms(lambda: tp.contract(z, (u // 16).to(torch.int32)))
+    assert _ms(lambda: tp.contract(z, (u * 64 // n).to(torch.int32))) < 3 * usual
+
+
 @pytest.mark.parametrize("graph", ["mesh", "skewed", "dense"])
 @pytest.mark.parametrize("weighted", [False, True])
 def test_contraction_equals_oracle(graph, weighted):
