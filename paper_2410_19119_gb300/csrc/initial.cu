@@ -76,7 +76,8 @@ struct IPCtl {
   unsigned long long W, wdeg, acc;
   unsigned long long inw[3][2], dlw[3];
   int32_t ncnt[3][2];
-  int32_t nz, nnew, tail;
+  int32_t nz, nnew;
+  int32_t found[2], fb, fe;  // bfs_alone: vertices of a level and the next, the frontier
   unsigned long long w0;
   unsigned long long khi[2];
   uint32_t klo[2];
@@ -193,6 +194,95 @@ __device__ __forceinline__ void dif_add(int64_t *p, int64_t w) {
   atomicAdd((unsigned long long *)p, (unsigned long long)w);
 }
 
+// Cluster form: a BFS level of up to this many entries (the frontier times the
+// average degree) is the first CTA's alone. A path has a vertex or two a level,
+// and four cluster barriers for each: 20 000 vertices in one node took 116 ms,
+// this way 23; a mesh of 53 953 vertices with 5.8 neighbours each 2.9 -> 2.6
+// (with 8192 a mesh of degree 16 loses 40%). In a kernel of its own, for nodes of
+// up to kIPNarrowDeg neighbours a vertex: denser ones have few levels, and the
+// call alone costs their kernel 9% (36 030 vertices, 63 M entries: 7.3 -> 8.0 ms).
+constexpr int64_t kIPAlone = 2048;
+constexpr int64_t kIPNarrowDeg = 24;
+
+// BFS levels by the first CTA of a cluster, from the frontier ord[fb .. fe) on
+// (fe: the order's length), until one is too wide or nothing is left; the
+// frontier is then in ctl. A level's steps as in k_bisect. Few vertices (a warp)
+// are put in order by (claiming vertex, own number), which is the order of the
+// adjacencies, without counting and emitting them.
+template <int NT>
+__device__ __noinline__ void bfs_alone(const int64_t *lx, const int32_t *ladj, int32_t *ord,
+                                       int32_t *claimer, int32_t *cnt, int32_t *list, IPCtl *ctl,
+                                       int gs, int32_t nz, int32_t width, int32_t fb, int32_t fe) {
+  const int lane = lane_id(), gl = lane & (gs - 1);
+  const unsigned gmask = gs == 32 ? kFull : ((1u << gs) - 1u) << (lane & ~(gs - 1));
+  const int32_t gid = (int32_t)threadIdx.x / gs, ngr = NT / gs;
+  if (threadIdx.x == 0) ctl->found[0] = ctl->found[1] = 0;
+  __syncthreads();
+  for (int32_t lev = 0; fb < fe && fe < nz && fe - fb <= width; ++lev) {
+    int32_t *found = &ctl->found[lev & 1];
+    if (threadIdx.x == 0) ctl->found[~lev & 1] = 0;  // (read before the last level's last barrier)
+    for (int32_t i = fb + gid; i < fe; i += ngr) {
+      const int32_t p = ord[i];
+      if (gl == 0) cnt[i - fb] = 0;
+      const int64_t e = lx[p + 1];
+      for (int64_t q0 = lx[p]; q0 < e; q0 += gs) {
+        const int32_t y = q0 + gl < e ? ladj[q0 + gl] : -1;
+        const bool first = y >= 0 && claimer[y] > i && atomicMin(&claimer[y], i) == INT32_MAX;
+        const unsigned m = __ballot_sync(gmask, first);
+        if (m == 0) continue;
+        int32_t base = 0;
+        const int leader = __ffs(m) - 1;
+        if (lane == leader) base = atomicAdd(found, __popc(m));
+        base = __shfl_sync(gmask, base, leader);
+        if (first) list[base + __popc(m & lanemask_lt())] = y;
+      }
+    }
+    __syncthreads();
+    const int32_t nn = *found;
+    if (nn == 0) {
+      fb = fe;
+      break;
+    }
+    if (nn <= 32) {
+      if (threadIdx.x < 32) {
+        const int32_t y = lane < nn ? list[lane] : 0;
+        const uint64_t k = lane < nn ? (uint64_t)(uint32_t)claimer[y] << 32 | (uint32_t)y : ~0ull;
+        int32_t at = 0;
+        for (int q = 0; q < nn; ++q) at += __shfl_sync(kFull, k, q) < k;
+        if (lane < nn) {
+          ord[fe + at] = y;
+          claimer[y] = -1;
+        }
+      }
+    } else {
+      for (int32_t q = threadIdx.x; q < nn; q += NT) atomicAdd(&cnt[claimer[list[q]] - fb], 1);
+      __syncthreads();
+      block_scan_array<NT>(cnt, fe - fb);
+      for (int32_t i = fb + gid; i < fe; i += ngr) {
+        const int32_t c0 = cnt[i - fb], k = cnt[i - fb + 1] - c0;
+        if (k == 0) continue;
+        const int32_t p = ord[i];
+        const int64_t e = lx[p + 1];
+        int32_t done = 0;
+        for (int64_t q0 = lx[p]; done < k && q0 < e; q0 += gs) {
+          const int32_t y = q0 + gl < e ? ladj[q0 + gl] : -1;
+          const bool mine = y >= 0 && claimer[y] == i;
+          const unsigned m = __ballot_sync(gmask, mine);
+          if (mine) {
+            ord[fe + c0 + done + __popc(m & lanemask_lt())] = y;
+            claimer[y] = -1;
+          }
+          done += __popc(m);
+        }
+      }
+    }
+    __syncthreads();
+    fb = fe;
+    fe += nn;
+  }
+  if (threadIdx.x == 0) ctl->fb = fb, ctl->fe = fe;
+}
+
 // One attempt of one node. SM: one CTA, state in shared memory; otherwise a
 // cluster of any size, state in global memory (L1 lines are dropped by the
 // barriers' acquire). V: type of the connectivity differences (int32_t where
@@ -202,7 +292,8 @@ __device__ __forceinline__ void dif_add(int64_t *p, int64_t w) {
 // Bound by latency: a mesh's BFS has about a hundred levels of four dependent
 // steps with a barrier each, a dense node is read from HBM about four times
 // (BFS claims and emission, D, the movers' rows).
-template <int NT, bool SM, class V>
+// NARROW (clusters): narrow BFS levels are the first CTA's (bfs_alone).
+template <int NT, bool SM, class V, bool NARROW = false>
 __global__ void __launch_bounds__(NT, SM && NT <= 512 ? 1024 / NT : 1) k_bisect(IPCtx c) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ IPCtl s_ctl;
@@ -280,6 +371,17 @@ __global__ void __launch_bounds__(NT, SM && NT <= 512 ? 1024 / NT : 1) k_bisect(
   const int64_t W = (int64_t)ctl->W;
   int32_t tail = 1;
   for (int32_t fb = 0, fe = 1; fb < fe && tail < nz;) {
+    if constexpr (NARROW) {
+      const int32_t width = (int32_t)(kIPAlone / max(avg, (int64_t)gs));
+      if (cs > 1 && fe - fb <= width) {
+        if (rank == 0)
+          bfs_alone<NT>(lx, c.ladj, ord, claimer, cnt, list, &s_ctl, gs, nz, width, fb, fe);
+        sync_all();
+        fb = ctl->fb;
+        fe = tail = ctl->fe;
+        continue;
+      }
+    }
     // every undiscovered neighbour is claimed by its earliest frontier vertex
     // (claimer: INT32_MAX unclaimed, -1 already in the order); the first
     // claim of a vertex lists it
@@ -649,9 +751,13 @@ struct DepthDev {
 
 // How a node's attempts are run: one CTA of `threads` with its state in
 // shared memory (cluster = 0), or a cluster of CTAs.
+// (narrow: narrow BFS levels in the first one alone).
 struct Shape {
   int threads, cluster;
-  bool operator==(const Shape &o) const { return threads == o.threads && cluster == o.cluster; }
+  bool narrow;
+  bool operator==(const Shape &o) const {
+    return threads == o.threads && cluster == o.cluster && narrow == o.narrow;
+  }
 };
 
 // Shared memory of the one-CTA form: what a block may have beside the static
@@ -683,19 +789,20 @@ template <class V>
 Shape ip_shape(int64_t ns, int64_t entries, int64_t attempts, int64_t large_attempts) {
   if (ip_large<V>(ns, entries)) {
     const int64_t cl = std::max<int64_t>(1, std::min<int64_t>(16, num_sms() / large_attempts));
-    if (cl > 1 || ns > ip_smem_cap<V>()) return Shape{kIPMaxThreads, (int)cl};
+    if (cl > 1 || ns > ip_smem_cap<V>())
+      return Shape{kIPMaxThreads, (int)cl, cl > 1 && entries <= kIPNarrowDeg * ns};
   }
   // smaller CTAs, several per SM, where many attempts are in flight
   const bool many = attempts >= 2LL * num_sms();
   const int threads = many ? (ns <= 512 ? 128 : ns <= 2048 ? 256 : ns <= 6144 ? 512 : 1024)
                            : (ns <= 256 ? 256 : ns <= 1024 ? 512 : 1024);
-  return Shape{threads, 0};
+  return Shape{threads, 0, false};
 }
 
-template <int NT, bool SM, class V>
+template <int NT, bool SM, class V, bool NARROW = false>
 void launch_bisect(const IPCtx &c, int64_t attempts, int cluster, cudaStream_t s) {
   const size_t smem = SM ? ip_smem_bytes<V>(c.cap) : 0;
-  auto kern = k_bisect<NT, SM, V>;
+  auto kern = k_bisect<NT, SM, V, NARROW>;
   if (SM)
     TP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kIPSmem));
   else
@@ -778,6 +885,7 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
     }
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
       if (shape[x].cluster != shape[y].cluster) return shape[x].cluster > shape[y].cluster;
+      if (shape[x].narrow != shape[y].narrow) return shape[x].narrow < shape[y].narrow;
       return shape[x].threads > shape[y].threads;
     });
     DepthDev &cur = depth % 2 ? next_dev : dev;
@@ -852,7 +960,8 @@ void bisect_forest(const tp_graph *g, const std::vector<IPRoot> &roots,
       c.nodes = cur.order + b;
       c.cap = (int32_t)((largest + 15) & ~(int64_t)15);
       const int64_t att = (int64_t)(e - b) * T;
-      if (sh.cluster) launch_bisect<kIPMaxThreads, false, V>(c, att, sh.cluster, cls);
+      if (sh.narrow) launch_bisect<kIPMaxThreads, false, V, true>(c, att, sh.cluster, cls);
+      else if (sh.cluster) launch_bisect<kIPMaxThreads, false, V>(c, att, sh.cluster, cls);
       else if (sh.threads == 128) launch_bisect<128, true, V>(c, att, 1, cls);
       else if (sh.threads == 256) launch_bisect<256, true, V>(c, att, 1, cls);
       else if (sh.threads == 512) launch_bisect<512, true, V>(c, att, 1, cls);

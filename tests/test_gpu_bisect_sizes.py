@@ -72,3 +72,59 @@ def test_classes_of_one_depth_side_by_side():
     for (x, a), (part, st) in zip(host, res):
         want, wst = oracle.partition(oracle.Graph(x, a), k, 0.03, oracle.Params(seed=3))
         assert np.array_equal(part.cpu().numpy(), want) and st["cut"] == wst["cut"]
+
+
+def _joined(parts):
+    """The graphs side by side, an edge from each one's last vertex to the next one's first."""
+    u, v, base = [], [], 0
+    for x, a in parts:
+        n = len(x) - 1
+        u.append(np.repeat(np.arange(n), np.diff(x)) + base)
+        v.append(a.astype(np.int64) + base)
+        if base:
+            u.append(np.array([base - 1, base]))
+            v.append(np.array([base, base - 1]))
+        base += n
+    u, v = np.concatenate(u), np.concatenate(v)
+    order = np.lexsort((v, u))
+    x = np.zeros(base + 1, np.int64)
+    np.add.at(x, u + 1, 1)
+    return np.cumsum(x), v[order].astype(np.int32)
+
+
+def _path(n):
+    u = np.arange(n)
+    a = np.stack([u - 1, u + 1], 1).reshape(-1)[1:-1].astype(np.int32)
+    return np.concatenate([[0], 1 + 2 * np.arange(n - 1), [2 * (n - 1)]]).astype(np.int64), a
+
+
+@pytest.mark.parametrize("parts", ["path", "narrow and wide", "star"])
+def test_narrow_and_wide_levels_of_a_cluster(parts):
+    """Nodes of clusters whose BFS has levels of a vertex or two, of hundreds
+    and of thousands, in turn."""
+    graphs = {"path": [_path(14003)],
+              "narrow and wide": [_path(3000), synth.gnm(6001, 60000, 3), _path(2500),
+                                  synth.gnm(3001, 500000, 4), _path(900)],
+              "star": [_path(5000), (np.concatenate([[0], 8000 + np.arange(8001)]).astype(np.int64),
+                                     np.concatenate([1 + np.arange(8000), np.zeros(8000)]).astype(np.int32)),
+                       _path(700)]}[parts]
+    xadj, adj = _joined(graphs)
+    _check(xadj, adj, None, 3)
+
+
+def test_narrow_levels_cost_a_cluster_no_more_than_one_block():
+    """A path just too long for shared memory against one that just fits."""
+    def ms(n):
+        g = tp.graph_from_csr(*_path(n))
+        best = []
+        for _ in range(3):
+            torch.cuda.synchronize()
+            b, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            b.record()
+            tp.initial_partition(g, 2, n)
+            e.record()
+            torch.cuda.synchronize()
+            best.append(b.elapsed_time(e))
+        return min(best)
+
+    assert ms(13000) < 2 * ms(12500)
