@@ -286,30 +286,72 @@ __global__ void __launch_bounds__(lane_warps<W>() * 32, W ? 1 : kLaneBlocksPerSM
 }
 
 // The neighbours of every moved vertex are quiet no longer: low-degree movers
-// by a thread each, the others by a warp. Where a sub-round moved so many that
-// little would stay quiet, the epoch advances instead, which ends all marks.
+// by a thread each, mid ones by a warp, the others by the block. Where a
+// sub-round moved so many that little would stay quiet, or a hub of more than
+// kWakeMost neighbours, the epoch advances instead (once a sub-round: counters[4]),
+// which ends all marks. (A warp for every hub: a mesh of 2^22 vertices with one
+// joined to every eighth refined in 9.4 ms and with one joined to all clustered,
+// compressed, in 32, where rating everything took 4.9 and 7.3.)
+constexpr int64_t kWakeMost = 65536;  // 64 steps of the block, about as many us
 template <bool COMP>
-__global__ void k_wake(GView g, const uint8_t *tier, const unsigned long long *counters,
-                       const int32_t *mv_u, const int8_t *mv_ok, int64_t limit, uint8_t *quiet,
-                       int32_t *epoch) {
+__global__ void __launch_bounds__(256) k_wake(GView g, const uint8_t *tier,
+                                              unsigned long long *counters, const int32_t *mv_u,
+                                              const int8_t *mv_ok, int64_t limit, uint8_t *quiet,
+                                              int32_t *epoch) {
+  __shared__ int32_t big[256], n_big;
   const int64_t nm = (int64_t)counters[0];
   if (nm > limit) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *epoch += 1;
     return;
   }
+  const int w = threadIdx.x >> 5;
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < nm;
        i0 += (int64_t)gridDim.x * blockDim.x) {
+    if (threadIdx.x == 0) n_big = 0;
+    __syncthreads();
     const int64_t i = i0 + threadIdx.x;
     const bool in = i < nm && mv_ok[i];
     const int32_t u = in ? mv_u[i] : 0;
-    const bool low = in && (tier[u] == TIER_LANE || tier[u] == TIER_SMALL);
-    if (low) thread_neighbours<COMP>(g, u, [&](int32_t v, int64_t) { quiet[v] = 0; });
+    const uint8_t t = in ? tier[u] : TIER_LANE;
+    if (in && (t == TIER_LANE || t == TIER_SMALL))
+      thread_neighbours<COMP>(g, u, [&](int32_t v, int64_t) { quiet[v] = 0; });
+    if (t == TIER_BIG || t == TIER_HUGE) {
+      const int64_t d = COMP ? zip_nbr(g, u).deg : g.xadj[u + 1] - g.xadj[u];
+      if (d <= kWakeMost) big[atomicAdd(&n_big, 1)] = u;
+      else if (atomicExch(&counters[4], 1ull) == 0) atomicAdd(epoch, 1);
+    }
     __syncwarp();
-    for (unsigned q = __ballot_sync(kFull, in && !low); q; q &= q - 1)
+    for (unsigned q = __ballot_sync(kFull, t == TIER_MID); q; q &= q - 1)
       warp_neighbours<COMP>(g, __shfl_sync(kFull, u, __ffs(q) - 1), -1,
                             [&](bool has, int32_t v, int64_t, int64_t) {
                               if (has) quiet[v] = 0;
                             });
+    __syncthreads();
+    const int nb = n_big;
+    for (int k = 0; k < nb; ++k) {
+      const int32_t b = big[k];
+      if constexpr (COMP) {  // a chunk is decoded by one warp, a record below the threshold whole
+        const ZipNbr z = zip_nbr(g, b);
+        for (int64_t j = (w + k) & 7; j < z.nchunks; j += 8)
+          warp_neighbours<true>(
+              g, b, z.nchunks > 1 ? j : -1,
+              [&](bool has, int32_t v, int64_t, int64_t) {
+                if (has) quiet[v] = 0;
+              },
+              &z);
+      } else {
+        const int64_t e = g.xadj[b + 1];
+        for (int64_t x = g.xadj[b] + threadIdx.x; x < e; x += 4 * 256) {
+          int32_t v[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) v[r] = x + 256 * r < e ? g.adj[x + 256 * r] : -1;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (v[r] >= 0) quiet[v[r]] = 0;
+        }
+      }
+    }
+    __syncthreads();  // big is listed anew
   }
 }
 
@@ -1672,11 +1714,11 @@ void LpWork::init(int64_t n_vertices, int64_t n_labels, cudaStream_t s) {
   cseg.alloc(N, s);
   cseg_u.alloc(N, s);
   cseg_g.alloc(N, s);
-  counters.alloc(4, s);
+  counters.alloc(5, s);
   TP_CUDA(cudaMemsetAsync(in_w.get(), 0, L * 8, s));
   TP_CUDA(cudaMemsetAsync(ccnt.get(), 0, L * 4, s));
   TP_CUDA(cudaMemsetAsync(cfill.get(), 0, L * 4, s));
-  TP_CUDA(cudaMemsetAsync(counters.get(), 0, 4 * 8, s));
+  TP_CUDA(cudaMemsetAsync(counters.get(), 0, 5 * 8, s));
 }
 
 // The approval of one sub-round: the same five kernels and counter reset on
@@ -1699,7 +1741,7 @@ void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStr
     const int64_t limit = wake->n / (8 * (int64_t)S);
     const unsigned wb = grid_for(std::max<int64_t>(limit, 1), 256);
     const uint8_t *tier = wake->tiers.tier.get();
-    const unsigned long long *cnt = (const unsigned long long *)counters;
+    unsigned long long *cnt = (unsigned long long *)counters;
     if (wake->compressed)
       launch(k_wake<true>, wb, 256, 0, stream, view(wake), tier, cnt, a.mv_u, a.mv_ok, limit,
              w->quiet.get(), w->epoch.get());
@@ -1708,7 +1750,7 @@ void launch_approval(const ApproveCtx &a, int64_t wn, int64_t *counters, cudaStr
              w->quiet.get(), w->epoch.get());
   }
   TP_LAUNCH_CHECK();
-  TP_CUDA(cudaMemsetAsync(counters, 0, 4 * sizeof(int64_t), stream));
+  TP_CUDA(cudaMemsetAsync(counters, 0, 5 * sizeof(int64_t), stream));
 }
 
 // Records the approval of a level's sub-rounds into a CUDA graph on a

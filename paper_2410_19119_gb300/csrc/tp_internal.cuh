@@ -447,7 +447,9 @@ struct LpWork {
   Buf<int64_t> cseg_g;        // n (and gain)
   Buf<int32_t> ctarget;     // nlabels (contested targets)
   Buf<int32_t> cbig;        // nlabels (those of more than 32 movers)
-  Buf<int64_t> counters;    // [0] movers, [1] contested targets, [2] contested pool
+  // [0] movers, [1] contested targets, [2] contested pool, [3] targets of more
+  // than 32 movers, [4] a mover's hub ended the quiet marks
+  Buf<int64_t> counters;
   // lane-tier vertices of the current round grouped by sub-round (A3)
   Buf<int32_t> bucket;       // n
   Buf<uint8_t> bucket_sub;   // n: sub-round + 1 of every vertex this round (0: not listed)
