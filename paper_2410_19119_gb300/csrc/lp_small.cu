@@ -193,22 +193,42 @@ __global__ void __launch_bounds__(kLpSmallThreads)
   }
 }
 
-// Cluster size for a level that k_lp_small can take, 0 for the others: one
-// graph, no vertex above the mid tier, 32-bit ratings, with edge weights labels
-// that fit the lane tier's 32-bit sort keys (block numbers need not), at most 32
-// sub-rounds, and so few vertices and entries that 16 CTAs rate an eighth of
-// them in about the time that the kernels of a sub-round take to launch. The
-// smallest cluster that gives a CTA at most kLpSmallItems batches or vertices
-// per sub-round: the lanes of a batch read different rows and labels, and an
-// SM's L1 looks up one line a cycle (a batch of degree 16 takes about 700), so
-// 16 batches on one SM cost more than four on each of four and their barriers.
-int lp_small_cluster(const tp_graph *g, const LpState &st, int32_t S) {
+// Whether one cluster rates a level's rounds in less time than the kernels of
+// the sub-rounds take, most of it their launches. Both were measured on meshes
+// and uniform random graphs of 2e3 to 2.6e5 vertices and degrees 4 to 450, with
+// 2, 8 and 32 sub-rounds (16 CTAs, random graphs): a round costs a lane-tier
+// vertex 0.4 ns and 0.17 an entry (a fifth more with edge weights, a seventh less
+// compressed), one of the warp tiers 18 and 0.36. A sub-round saves 14 us and a
+// call 0.4 ms, and where the warp tiers are most of the work 48 us a sub-round
+// (they take that long on the other path too). With a limit of 2^21 entries
+// alone, 2.6e5 vertices of degree 8 took 2.24 ms against 1.26, 2e4 of degree 100
+// 5.4 against 2.3; at the line the two are within a tenth on random graphs, and
+// on meshes the cluster is up to a third faster.
+bool lp_small_pays(const tp_graph *g, int32_t rounds, int32_t S) {
+  const TierCache &T = g->tiers;
+  const double lanes = (g->compressed ? 0.85 : g->unit_ew ? 1.0 : 1.2) *
+                       (0.4 * (double)T.count[TIER_LANE] + 0.17 * (double)T.edges[TIER_LANE]);
+  const double warps = 18.0 * (double)(T.count[TIER_SMALL] + T.count[TIER_MID]) +
+                       0.36 * (double)(T.edges[TIER_SMALL] + T.edges[TIER_MID]);
+  return rounds * lanes / (400e3 + 14e3 * rounds * S) + warps / (48e3 * S) <= 1.0;
+}
+
+// Cluster size for a level that k_lp_small can take and that gains by it, 0 for
+// the others: one graph, no vertex above the mid tier, 32-bit ratings, with edge
+// weights labels that fit the lane tier's 32-bit sort keys (block numbers need
+// not), at most 32 sub-rounds. The smallest cluster that gives a CTA at most
+// kLpSmallItems batches or vertices per sub-round: the lanes of a batch read
+// different rows and labels, and an SM's L1 looks up one line a cycle (a batch
+// of degree 16 takes about 700), so 16 batches on one SM cost more than four on
+// each of four and their barriers.
+int lp_small_cluster(const tp_graph *g, const LpState &st, int32_t rounds, int32_t S) {
   const TierCache &T = g->tiers;
   if (st.seg.gid || S > 32 || T.lane_long ||
       T.count[TIER_BIG] + T.count[TIER_HUGE] > 0 ||
       (!g->unit_ew && (ew_sum_bound(g) >= ((int64_t)1 << 31) || st.nlabels > kLaneKeyLabels)))
     return 0;
-  if (g->n > kLpSmallVertices * kLpSmallCluster || g->m2 > kLpSmallEntries * kLpSmallCluster)
+  if (g->n > kLpSmallVertices * kLpSmallCluster || g->m2 > kLpSmallEntries * kLpSmallCluster ||
+      !lp_small_pays(g, rounds, S))
     return 0;
   const int64_t items = (T.count[TIER_LANE] / 32 + T.count[TIER_SMALL] + T.count[TIER_MID]) / S;
   int cs = 1;
@@ -222,7 +242,7 @@ bool lp_rounds_small(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, u
                             uint64_t a, uint64_t b0, int32_t rounds, int32_t S, const tp_params &p,
                             cudaStream_t stream) {
   build_tiers(g, p, stream);
-  int cs = lp_small_cluster(g, st, S);
+  int cs = lp_small_cluster(g, st, rounds, S);
   if (!cs) return false;
   auto kern = g->compressed ? k_lp_small<true, false>
               : g->unit_ew  ? k_lp_small<false, false>
