@@ -96,11 +96,16 @@ __host__ __device__ constexpr int64_t agg_start(int size) {
 }
 
 // Lists every coarse vertex under its first size, its weight where members
-// weigh one each. A member counts for an entry at least: a table's warp or block
-// walks the members, and one cluster of 2^26 vertices without edges was a warp's
-// walk of 2.0 s (now 4.5 ms). lists: kAggSizes + 1 lists of nc entries, cnt: their lengths.
-__global__ void k_agg_classes(const unsigned long long *ent, const int32_t *mcnt, int64_t nc,
-                              int64_t *cvw, int32_t *lists, int32_t *cnt) {
+// weigh one each, and adds up the entries of those that start in a table (rows:
+// no fewer than the tables write). A member counts for an entry at least: a
+// table's warp or block walks the members, and one cluster of 2^26 vertices
+// without edges was a warp's walk of 2.0 s (now 4.5 ms). lists: kAggSizes + 1
+// lists of nc entries, cnt: their lengths.
+__global__ void __launch_bounds__(256)
+    k_agg_classes(const unsigned long long *ent, const int32_t *mcnt, int64_t nc, int64_t *cvw,
+                  int32_t *lists, int32_t *cnt, unsigned long long *rows) {
+  __shared__ int64_t part[8];
+  int64_t mine = 0;
   for (int64_t a0 = (int64_t)blockIdx.x * blockDim.x; a0 < nc;
        a0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t a = a0 + threadIdx.x;
@@ -109,6 +114,7 @@ __global__ void k_agg_classes(const unsigned long long *ent, const int32_t *mcnt
       const int64_t e = max((int64_t)ent[a], (int64_t)mcnt[a]);
       cl = 0;
       while (cl < kAggSizes && e > agg_start(cl)) ++cl;
+      if (cl < kAggSizes) mine += (int64_t)ent[a];
       if (cvw) cvw[a] = mcnt[a];
     }
     const unsigned peers = __match_any_sync(kFull, cl);
@@ -120,6 +126,35 @@ __global__ void k_agg_classes(const unsigned long long *ent, const int32_t *mcnt
       lists[(int64_t)cl * nc + base + __popc(peers & lanemask_lt())] = (int32_t)a;
     }
   }
+  mine = warp_sum(mine);
+  if (lane_id() == 0) part[threadIdx.x >> 5] = mine;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) mine += part[w];
+    if (mine) atomicAdd(rows, (unsigned long long)mine);
+  }
+}
+
+// Inter-cluster entries among those of every (n / kRowSamples)-th vertex's row
+// (its first chunk), a warp each: out[0] of out[1].
+constexpr int64_t kRowSamples = 1024;
+template <bool COMP>
+__global__ void k_row_sample(GView g, const int32_t *map, unsigned long long *out) {
+  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= kRowSamples) return;
+  const int64_t u = g.n / kRowSamples * i;
+  const int32_t a = map[u];
+  int64_t cut = 0, all = 0;
+  warp_neighbours<COMP>(g, u, 0, [&](bool has, int32_t v, int64_t, int64_t) {
+    all += has;
+    cut += has && map[v] != a;
+  });
+  cut = warp_sum(cut);
+  all = warp_sum(all);
+  if (lane_id() == 0 && all) {
+    atomicAdd(&out[1], (unsigned long long)all);
+    if (cut) atomicAdd(&out[0], (unsigned long long)cut);
+  }
 }
 
 struct AggCtx {
@@ -129,6 +164,7 @@ struct AggCtx {
   int64_t nc;
   int32_t *lists, *cnt;        // per size: coarse vertices still to do, how many
   unsigned long long *cursor;  // entries written so far
+  int64_t room;                // entries that fit; the cursor counts on beyond them
   int32_t *out_key;            // neighbours of every coarse vertex, sorted, at toff
   void *out_val;
   int64_t *toff, *deg;
@@ -458,7 +494,7 @@ __global__ void __launch_bounds__(32 * agg_warps(SIZE), SIZE == 0 && !COMP ? 6 :
           x = up ? (x < y ? x : y) : (x < y ? y : x);
         }
       base = __shfl_sync(kFull, base, 0);
-      if (lane < d) {
+      if (lane < d && (int64_t)base + d <= c.room) {
         const V w = s.vals[(uint32_t)x];
         c.out_key[base + lane] = (int32_t)(x >> 32);
         out_val[base + lane] = w;
@@ -471,7 +507,8 @@ __global__ void __launch_bounds__(32 * agg_warps(SIZE), SIZE == 0 && !COMP ? 6 :
       __syncwarp();
       bitonic(s.items, n2, lane, 32, [] { __syncwarp(); });
       base = __shfl_sync(kFull, base, 0);
-      for (int i = lane; i < d; i += 32) {
+      const int fit = (int64_t)base + d <= c.room ? d : 0;
+      for (int i = lane; i < fit; i += 32) {
         const uint64_t x = s.items[i];
         const V w = s.vals[(uint32_t)x];
         c.out_key[base + i] = (int32_t)(x >> 32);
@@ -614,7 +651,8 @@ __global__ void __launch_bounds__(kAggThreads, SIZE == 2 ? 3 : 1) k_agg_block(Ag
     }
     __syncthreads();
     const bool two = n2 > ITEMS;
-    for (int i = tid; i < d; i += kAggThreads) {
+    const int fit = (int64_t)s_base + d <= c.room ? d : 0;
+    for (int i = tid; i < fit; i += kAggThreads) {
       const uint64_t x = items[i];
       int pos = i;
       if (two) {  // rank in the other run
@@ -877,6 +915,9 @@ __global__ void k_add_i64(const int64_t *a, int64_t n, int64_t *b) {
     b[i] += a[i];
 }
 
+// Graphs of at least this many vertices are sampled for the room of the rows.
+constexpr int64_t kSampleFrom = (int64_t)1 << 20;
+
 // The block of k_agg_block / k_agg_warp grids: as many as fit the SMs, no more
 // than the longest the list can become.
 template <bool COMP, class V>
@@ -898,18 +939,12 @@ void launch_agg(const AggCtx &c, const int64_t (&most)[kAggSizes], cudaStream_t 
 
 }  // namespace
 
-tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStream_t s,
-                   const int64_t *seg_voff, int64_t nseg, int64_t *seg_coff) {
-  int64_t n = g->n;
-  // a compressed graph with long records is decoded first (each chunk once, by
-  // a warp): in the tables' kernels such a record is one warp's, and level 0
-  // of R-MAT 2^22 spent 39 ms in them where decoding takes 2 and the CSR
-  // kernels 13.5
-  std::unique_ptr<tp_graph> csr;
-  if (g->compressed && g->max_deg > kAggDecodeDeg) {
-    csr.reset(decompress(g, s));
-    g = csr.get();
-  }
+// The contraction itself. own (nullable): holds g if g is a decoded copy, freed
+// as soon as its rows are summed.
+static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own, const int32_t *C,
+                               int32_t *d_map, cudaStream_t s, const int64_t *seg_voff, int64_t nseg,
+                               int64_t *seg_coff) {
+  const int64_t n = g->n;
   tp_graph *cg = new_graph();
   try {
     cg->err.alloc(1, s);
@@ -957,8 +992,9 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
     // members by coarse vertex, and the first table size of each
     Buf<int32_t> members(n, s), lists((kAggSizes + 1) * nc, s);
     Buf<int64_t> mstart(nc + 1, s);
-    // [0] cursor [1] largest weight [2], [3] items; then the lists' lengths (int32)
-    constexpr int kAcc = 4;
+    // [0] cursor [1] largest weight [2], [3] items [4] rows' bound [5], [6] sample;
+    // then the lists' lengths (int32)
+    constexpr int kAcc = 7;
     Buf<int64_t> acc(kAcc + (kAggSizes + 2) / 2, s);
     TP_CUDA(cudaMemsetAsync(acc.get(), 0, acc.n * sizeof(int64_t), s));
     int32_t *cnt = reinterpret_cast<int32_t *>(acc.get() + kAcc);
@@ -972,23 +1008,34 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
       exclusive_scan_i32_to_i64(mcnt.get(), mstart.get(), nc, s);
       launch(k_members, grid_for(n, 256), 256, 0, s, map, place.get(), mstart.get(), n, members.get());
       launch(k_agg_classes, grid_for(nc, 256), 256, 0, s, ent.get(), mcnt.get(), nc,
-             g->unit_vw ? cg->vw.get() : nullptr, lists.get(), cnt);
+             g->unit_vw ? cg->vw.get() : nullptr, lists.get(), cnt,
+             (unsigned long long *)(acc.get() + 4));
+      if (n >= kSampleFrom)
+        launch(comp ? k_row_sample<true> : k_row_sample<false>, (unsigned)(kRowSamples * 32 / 256), 256,
+               0, s, v, map, (unsigned long long *)(acc.get() + 5));
       TP_LAUNCH_CHECK();
     }
     rank.release();
-    int32_t hc[kAggSizes + 1];
-    TP_CUDA(cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, s));
+    int64_t ha[kAcc + (kAggSizes + 2) / 2];
+    TP_CUDA(cudaMemcpyAsync(ha, acc.get(), sizeof(ha), cudaMemcpyDeviceToHost, s));
     TP_CUDA(cudaStreamSynchronize(s));
+    int32_t hc[kAggSizes + 1];
+    std::copy_n(reinterpret_cast<const int32_t *>(ha + kAcc), kAggSizes + 1, hc);
     // lists can grow by those that move up from the smaller sizes
     int64_t most[kAggSizes], sofar = 0;
     for (int i = 0; i < kAggSizes; ++i) most[i] = sofar += hc[i];
 
-    // the tables' rows: no more entries than the graph has
-    Buf<int32_t> tkey(std::max<int64_t>(g->m2, 1), s);
+    // the tables' rows: no more entries than their coarse vertices' members have,
+    // and in a large graph room for a quarter more than the sampled share of
+    // inter-cluster ones (a third in a mesh, whose rows of all entries were the
+    // peak of a partition); if that falls short the tables are filled again with
+    // the room they turned out to need
+    int64_t room = std::min<int64_t>(ha[4], g->m2);
+    if (n >= kSampleFrom && ha[6] > 0)
+      room = std::min<int64_t>(room, (int64_t)(1.25 * (double)g->m2 * (double)ha[5] / (double)ha[6]) + n / 16);
+    Buf<int32_t> tkey;
     Buf<uint32_t> tval32;
     Buf<unsigned long long> tval64;
-    if (narrow) tval32.alloc(std::max<int64_t>(g->m2, 1), s);
-    else tval64.alloc(std::max<int64_t>(g->m2, 1), s);
     Buf<int64_t> toff(nc, s);
     cg->xadj.alloc(nc + 1, s);
     TP_CUDA(cudaMemsetAsync(cg->xadj.get(), 0, (nc + 1) * sizeof(int64_t), s));
@@ -1002,16 +1049,28 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
     c.cnt = cnt;
     c.cursor = (unsigned long long *)acc.get();
     c.max_w = (unsigned long long *)(acc.get() + 1);
-    c.out_key = tkey.get();
-    c.out_val = narrow ? (void *)tval32.get() : (void *)tval64.get();
     c.toff = toff.get();
     c.deg = cg->xadj.get();
-    if (comp) launch_agg<true, uint32_t>(c, most, s);
-    else if (narrow) launch_agg<false, uint32_t>(c, most, s);
-    else launch_agg<false, unsigned long long>(c, most, s);
-    int64_t ha[kAcc + (kAggSizes + 2) / 2];
-    TP_CUDA(cudaMemcpyAsync(ha, acc.get(), sizeof(ha), cudaMemcpyDeviceToHost, s));
-    TP_CUDA(cudaStreamSynchronize(s));
+    for (;;) {
+      tkey.alloc(std::max<int64_t>(room, 1), s);
+      if (narrow) tval32.alloc(std::max<int64_t>(room, 1), s);
+      else tval64.alloc(std::max<int64_t>(room, 1), s);
+      c.room = room;
+      c.out_key = tkey.get();
+      c.out_val = narrow ? (void *)tval32.get() : (void *)tval64.get();
+      if (comp) launch_agg<true, uint32_t>(c, most, s);
+      else if (narrow) launch_agg<false, uint32_t>(c, most, s);
+      else launch_agg<false, unsigned long long>(c, most, s);
+      TP_CUDA(cudaMemcpyAsync(ha, acc.get(), sizeof(ha), cudaMemcpyDeviceToHost, s));
+      TP_CUDA(cudaStreamSynchronize(s));
+      if (ha[0] <= room) break;
+      room = ha[0];
+      tkey.release();
+      tval32.release();
+      tval64.release();
+      TP_CUDA(cudaMemsetAsync(acc.get(), 0, 2 * sizeof(int64_t), s));
+      TP_CUDA(cudaMemcpyAsync(cnt, hc, sizeof(hc), cudaMemcpyHostToDevice, s));
+    }
     const int64_t n_sorted = reinterpret_cast<const int32_t *>(ha + kAcc)[kAggSizes];
     int64_t max_w = ha[1], m2 = ha[0], runs = 0;
 
@@ -1090,6 +1149,7 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
       max_w = std::max(max_w, max_i64(rval.get(), runs, s));
       m2 += runs;
     }
+    if (own) own->reset();
     exclusive_scan_i64(cg->xadj.get(), cg->xadj.get(), nc, s);
     cg->m2 = m2;
     cg->max_ew = max_w;
@@ -1116,6 +1176,19 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
     throw;
   }
   return cg;
+}
+
+tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStream_t s,
+                   const int64_t *seg_voff, int64_t nseg, int64_t *seg_coff) {
+  // a compressed graph with long records is decoded first (each chunk once, by
+  // a warp): in the tables' kernels such a record is one warp's, and level 0
+  // of R-MAT 2^22 spent 39 ms in them where decoding takes 2 and the CSR
+  // kernels 13.5
+  if (g->compressed && g->max_deg > kAggDecodeDeg) {
+    std::unique_ptr<tp_graph> csr(decompress(g, s));
+    return contract_rows(csr.get(), &csr, C, d_map, s, seg_voff, nseg, seg_coff);
+  }
+  return contract_rows(g, nullptr, C, d_map, s, seg_voff, nseg, seg_coff);
 }
 
 }  // namespace tp

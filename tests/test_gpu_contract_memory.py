@@ -1,0 +1,57 @@
+"""Device memory of the contraction: the rows of its tables take the room that
+they need (and are summed again where a sample of the graph promised too few
+inter-cluster entries)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2410_19119_gb300 as tp  # noqa: E402
+
+
+def _equal(cg, mp, want, want_map):
+    x, a, w, e = (t.cpu().numpy() for t in cg.export_csr())
+    assert np.array_equal(mp.cpu().numpy(), want_map)
+    assert np.array_equal(x, want.xadj) and np.array_equal(a, want.adj)
+    assert np.array_equal(w, want.vw) and np.array_equal(e, want.ew)
+
+
+def test_peak_of_a_mesh():
+    """The labels, weights and mover lists of clustering are the peak, not the
+    entries of the contraction."""
+    n = 1 << 21
+    g = tp.graph_from_csr(*synth.rgg2d(n, 16.0, 5))
+    for q in (g, g.compress()):
+        _, st = tp.partition(q, 64, 0.03)
+        assert st["peak_bytes"] < 125 * n
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+def test_sample_that_falls_short(weighted):
+    """A path in clusters of 64, and, between two sampled vertices, 800 vertices
+    of which each half is joined to all of the other, alone in their clusters."""
+    n, at, half = 1 << 20, (1 << 19) + 100, 400
+    u = np.arange(n - 1, dtype=np.int64)
+    left = at + np.arange(half)
+    heavy = np.stack([np.repeat(left, half), np.tile(left + half, half)], 1)
+    e = np.concatenate([np.stack([u, u + 1], 1), heavy])
+    e = np.concatenate([e, e[:, ::-1]])
+    key = np.unique(e[:, 0] * n + e[:, 1])
+    x = np.zeros(n + 1, np.int64)
+    np.add.at(x, key // n + 1, 1)
+    xadj, adj = np.cumsum(x), (key % n).astype(np.int32)
+    C = (np.arange(n) // 64 * 64).astype(np.int32)
+    C[at - 100 : at + 2 * half + 100] = np.arange(at - 100, at + 2 * half + 100)
+    vw = ew = None
+    if weighted:
+        src = np.repeat(np.arange(n, dtype=np.int64), np.diff(xadj))
+        ew = (np.minimum(src, adj) * 7919 + np.maximum(src, adj) * 104729) % 9 + (1 << 40)
+        vw = np.arange(n, dtype=np.int64) % 5 + 1
+    want, want_map = oracle.contract(oracle.Graph(xadj, adj, vw, ew), C)
+    g = tp.graph_from_csr(xadj, adj, vw, ew)
+    for q in [g] if weighted else [g, g.compress()]:
+        _equal(*tp.contract(q, torch.from_numpy(C).cuda()), want, want_map)
