@@ -1183,10 +1183,15 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
   // a compressed graph with long records is decoded first (each chunk once, by
   // a warp): in the tables' kernels such a record is one warp's, and level 0
   // of R-MAT 2^22 spent 39 ms in them where decoding takes 2 and the CSR
-  // kernels 13.5
+  // kernels 13.5. Where there is no room for the decoded copy the records are
+  // read as they are.
   if (g->compressed && g->max_deg > kAggDecodeDeg) {
-    std::unique_ptr<tp_graph> csr(decompress(g, s));
-    return contract_rows(csr.get(), &csr, C, d_map, s, seg_voff, nseg, seg_coff);
+    try {
+      std::unique_ptr<tp_graph> csr(decompress(g, s));
+      return contract_rows(csr.get(), &csr, C, d_map, s, seg_voff, nseg, seg_coff);
+    } catch (const Error &e) {
+      if (e.code != TP_ERR_OOM && e.code != TP_ERR_BUDGET) throw;
+    }
   }
   return contract_rows(g, nullptr, C, d_map, s, seg_voff, nseg, seg_coff);
 }

@@ -1,6 +1,7 @@
 """Device memory of the contraction: the rows of its tables take the room that
 they need (and are summed again where a sample of the graph promised too few
-inter-cluster entries)."""
+inter-cluster entries), and a compressed graph with long records that there is
+no room to decode is contracted from its records."""
 import numpy as np
 import pytest
 
@@ -55,3 +56,48 @@ def test_sample_that_falls_short(weighted):
     g = tp.graph_from_csr(xadj, adj, vw, ew)
     for q in [g] if weighted else [g, g.compress()]:
         _equal(*tp.contract(q, torch.from_numpy(C).cuda()), want, want_map)
+
+
+def test_no_room_to_decode():
+    """With less memory than the decoded copy and the rows take together the
+    records are contracted, with far less than either the call fails cleanly."""
+    xadj, adj = synth.rmat(16, 16, seed=2)
+    n = len(xadj) - 1
+    assert np.diff(xadj).max() > 1024
+    z = tp.graph_from_csr(xadj, adj).compress()
+    # few coarse entries: the copy lies in the peak (it is gone before they are made)
+    C = torch.arange(n, dtype=torch.int32, device="cuda") // 256
+    want, want_map = oracle.contract(oracle.Graph(xadj, adj), C.cpu().numpy())
+    live, peak, limit = {}, [0], [1 << 60]
+
+    def alloc(nbytes, stream):
+        if sum(live.values()) + nbytes > limit[0]:
+            return 0
+        p = torch.cuda.caching_allocator_alloc(nbytes, stream=stream)
+        live[p] = nbytes
+        peak[0] = max(peak[0], sum(live.values()))
+        return p
+
+    def free(ptr, nbytes, stream):
+        live.pop(ptr)
+        torch.cuda.caching_allocator_delete(ptr)
+
+    tp.set_allocator(alloc, free)
+    try:
+        cg, mp = tp.contract(z, C)
+        _equal(cg, mp, want, want_map)
+        del cg
+        base = sum(live.values())
+        limit[0] = peak[0] - 1  # the copy and its rows do not fit together
+        for _ in range(2):
+            peak[0] = base
+            cg, mp = tp.contract(z, C)
+            _equal(cg, mp, want, want_map)
+            del cg, mp
+        limit[0] = 4 * len(adj)  # not even the copy: refused as before, nothing leaks
+        with pytest.raises(tp.TpError):
+            tp.contract(z, C)
+        torch.cuda.synchronize()
+        assert sum(live.values()) == base
+    finally:
+        tp.set_allocator(None, None)
