@@ -61,7 +61,7 @@ __global__ void k_rate_small(RateCtx c) {
       if (tier_entry<MODE>(c, k, i, u)) {
         ZipNbr z;
         const int64_t d = row_degree<COMP>(c.g, u, z);
-        rate_vertex_warp<COMP, MODE, V>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
+        rate_vertex_warp<COMP, MODE, V, true>(c, u, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
       }
     }
   } else {
@@ -76,7 +76,7 @@ __global__ void k_rate_small(RateCtx c) {
         const int64_t v = base + j;
         ZipNbr z;
         const int64_t d = row_degree<COMP>(c.g, v, z);
-        rate_vertex_warp<COMP, MODE, V>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
+        rate_vertex_warp<COMP, MODE, V, true>(c, v, ws.keys, ws.vals, table_log(c, d, kSmallLog), &mb, &z);
       }
     }
   }
