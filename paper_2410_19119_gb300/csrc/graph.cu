@@ -262,28 +262,25 @@ __device__ __forceinline__ int tpad(int i) { return i + (i >> 5); }
 
 // A tile behind a long run of empty rows has that many rows that start in it,
 // and one block would walk them all. From this many on (512 KB of offsets)
-// every entry of the tile searches its row instead, 16 steps and more of eight
-// independent loads a thread. A graph with a gap of 2^27 rows took 71 ms to
-// validate and 506 ms to compress, with the searches 1.1 and 1.2 ms.
+// every entry of the tile searches its row instead, one after the other in a
+// thread (eight side by side cost every tile registers: validation of a mesh of
+// 4.2 M vertices 0.50 -> 0.53 ms). A graph with a gap of 2^27 rows took 71 ms to
+// validate and 506 ms to compress, with the searches 1.1 and 1.3 ms.
 constexpr int64_t kTileManyRows = 32 * (int64_t)kTile;
 
-// The last of the rows lo .. hi that starts at or before entry e0 + i, for every
-// entry i of the tile: f(i, row).
-template <class F>
-__device__ __forceinline__ void tile_search(const int64_t *xadj, int64_t lo, int64_t hi, int64_t e0,
-                                            F &&f) {
-  int64_t r[kTileItems];
-#pragma unroll
-  for (int j = 0; j < kTileItems; ++j) r[j] = lo;
+// The last of the rows lo .. hi that starts at or before entry e.
+__device__ __forceinline__ int64_t row_of_entry(const int64_t *xadj, int64_t lo, int64_t hi,
+                                                int64_t e) {
   for (int64_t left = hi - lo + 1; left > 1;) {
     const int64_t h = left >> 1;
-#pragma unroll
-    for (int j = 0; j < kTileItems; ++j)
-      if (xadj[r[j] + h] <= e0 + threadIdx.x + j * kTileThreads) r[j] += h;
+    if (xadj[lo + h] <= e) lo += h;
     left -= h;
   }
-#pragma unroll
-  for (int j = 0; j < kTileItems; ++j) f((int)threadIdx.x + j * kTileThreads, r[j]);
+  return lo;
+}
+
+__device__ __forceinline__ bool many_rows(const int32_t *tile_first, int64_t t) {
+  return (int64_t)tile_first[t + 1] - tile_first[t] >= kTileManyRows;
 }
 
 // Row of every entry of tile t, relative to base = tile_first[t] - 1 (the row
@@ -296,15 +293,9 @@ __device__ __forceinline__ void tile_rows(const int64_t *xadj, const int32_t *ti
   __shared__ int32_t wmax[kTileThreads / 32];
   const int64_t e0 = t * kTile;
   const int32_t base = tile_first[t] - 1;
-  const int64_t rend = min((int64_t)tile_first[t + 1], n);
-  if (rend - base > kTileManyRows) {  // uniform over the block
-    tile_search(xadj, max(base, 0), rend - 1, e0,
-                [&](int i, int64_t r) { row[tpad(i)] = (int32_t)(r - base); });
-    __syncthreads();
-    return;
-  }
   for (int i = threadIdx.x; i < kTile; i += kTileThreads) row[tpad(i)] = 0;
   __syncthreads();
+  const int64_t rend = min((int64_t)tile_first[t + 1], n);
   for (int64_t r = (int64_t)base + 1 + threadIdx.x; r < rend; r += kTileThreads)
     atomicMax(&row[tpad((int)(xadj[r] - e0))], (int32_t)(r - base));
   __syncthreads();
@@ -337,6 +328,40 @@ __device__ __forceinline__ void tile_rows(const int64_t *xadj, const int32_t *ti
 // searches run with full warps, kSearch of them in step per thread: bound by
 // the searches' dependent loads.
 constexpr int kSearch = 4;
+
+// The same for a tile of very many rows, an entry at a time and apart from the
+// others (as a branch among them it cost a mesh of 4.2 M vertices 0.50 -> 0.54
+// ms). Returns this thread's upper minus lower entries.
+__device__ __noinline__ int64_t validate_many(const GView &g, const int32_t *tile_first, int64_t t,
+                                              int32_t *bad) {
+  const int64_t lo = max(tile_first[t] - 1, 0), hi = min((int64_t)tile_first[t + 1], g.n) - 1;
+  int64_t diff = 0;
+  for (int64_t e = t * kTile + threadIdx.x; e < min((t + 1) * kTile, g.m2); e += kTileThreads) {
+    const int64_t u = row_of_entry(g.xadj, lo, hi, e);
+    const int32_t v = g.adj[e];
+    int code = 0;
+    if ((uint32_t)v >= (uint32_t)g.n || v == u) {
+      code = 4;
+    } else {
+      if (g.xadj[u] < e && g.adj[e - 1] >= v) code = 6;
+      if (g.ew && g.ew[e] <= 0) code = 7;
+      diff += v > u ? 1 : -1;
+      if (v > u) {  // the mirror: the last entry <= u of row v
+        int64_t b = g.xadj[v], left = g.xadj[v + 1] - b;
+        if (left == 0) {
+          code = 8;
+        } else {
+          for (; left > 1; left -= left >> 1)
+            if (g.adj[b + (left >> 1)] <= u) b += left >> 1;
+          if (g.adj[b] != u || (g.ew && g.ew[b] != g.ew[e])) code = 8;
+        }
+      }
+    }
+    if (code) atomicCAS(bad, 0, code);
+  }
+  return diff;
+}
+
 __global__ void __launch_bounds__(kTileThreads) k_validate(GView g, const int32_t *tile_first,
                                                            int64_t ntiles,
                                                            const int32_t *bad_rows, int32_t *bad,
@@ -347,6 +372,11 @@ __global__ void __launch_bounds__(kTileThreads) k_validate(GView g, const int32_
   if (*bad_rows) return;  // set by k_rows: the rows cannot be followed
   int64_t diff = 0;  // (thread 0)
   for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    if (many_rows(tile_first, t)) {  // uniform over the block
+      const int64_t d = validate_many(g, tile_first, t, bad);
+      if (d) atomicAdd(balance, (unsigned long long)d);
+      continue;
+    }
     if (threadIdx.x == 0) n_upper = 0;
     tile_rows(g.xadj, tile_first, t, g.n, row);  // (with barriers)
     const int64_t e0 = t * kTile;
@@ -800,10 +830,12 @@ __global__ void __launch_bounds__(kTileThreads)
       empty[i] = after ? (int32_t)(r - first_row_at(g.xadj, r, b)) : 0;
       if (after) s_empties = 1;
     };
-    if (rend - base > kTileManyRows) {  // uniform over the block
-      tile_search(g.xadj, max(base, 0), rend - 1, e0, [&](int i, int64_t r) {
-        if (i < len && g.xadj[r] == e0 + i) mark(r, e0 + i);
-      });
+    if (many_rows(tile_first, t)) {  // uniform over the block
+#pragma unroll 1
+      for (int i = threadIdx.x; i < len; i += kTileThreads) {
+        const int64_t r = row_of_entry(g.xadj, max(base, 0), rend - 1, e0 + i);
+        if (g.xadj[r] == e0 + i) mark(r, e0 + i);
+      }
     } else {
       for (int64_t r = (int64_t)base + 1 + threadIdx.x; r < rend; r += kTileThreads) {
         const int64_t b = g.xadj[r];
@@ -924,18 +956,23 @@ __global__ void __launch_bounds__(kTileThreads)
   }
 }
 
-// Headers and offsets of the empty rows, and the offset of the end (row n). An
+// Headers and offsets of the empty rows, and the end: row n's offset, the
+// terminal header (2m) and the zero bytes behind the stream. An
 // empty row's header lies (w - u) headers before that of the next row w with
 // entries, or before the end of the stream, and holds the same number.
-__global__ void k_zip_empty(const int64_t *xadj, int64_t n, int64_t body, bool empties,
+__global__ void k_zip_empty(const int64_t *xadj, int64_t n, int64_t m2, int64_t body, bool empties,
                             uint8_t *out, uint32_t *o32, uint64_t *o64) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (o32) o32[n] = (uint32_t)body;
-    else o64[n] = (uint64_t)body;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) {
+      if (o32) o32[n] = (uint32_t)body;
+      else o64[n] = (uint64_t)body;
+      put_varint64(out + body, (uint64_t)m2);
+    }
+    if (threadIdx.x < kBytePad) out[body + vlen((uint64_t)m2) + threadIdx.x] = 0;
   }
   if (!empties) return;
   const int lane = lane_id();
-  constexpr int64_t kSpan = 1024;  // consecutive rows of a warp, 32 at a time
+  constexpr int64_t kSpan = 256;  // consecutive rows of a warp, 32 at a time
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t s0 = gw * kSpan; s0 < n; s0 += nw * kSpan) {
@@ -999,12 +1036,6 @@ __global__ void k_zip_tables(const int64_t *xadj, int64_t n, const uint32_t *o32
       }
     }
   }
-}
-
-__global__ void k_zip_terminal(uint64_t pos, int64_t m2, uint8_t *out) {
-  uint64_t x = (uint64_t)m2;
-  int l = vlen(x);
-  for (int i = 0; i < l; ++i, x >>= 7) out[pos + i] = (uint8_t)((x & 0x7f) | (i + 1 < l ? 0x80 : 0));
 }
 
 __global__ void k_off_narrow_u64(const uint64_t *off, int64_t cnt, uint32_t *o32) {
@@ -1242,40 +1273,40 @@ tp_graph *compress(const tp_graph *c, cudaStream_t s) {
     GView v = view(c);
     int64_t n = c->n;
     const int64_t ntiles = c->m2 / kTile + 1;
-    Buf<int32_t> tile_first(ntiles + 1, s), flags(2, s);  // [0] (unused) [1] empty rows
-    TP_CUDA(cudaMemsetAsync(flags.get(), 0, 2 * sizeof(int32_t), s));
-    Buf<int64_t> tsize(ntiles + 1, s), cpos;
+    // the tiles' bytes (then their places and the stream's), a flag each of bad
+    // rows and empty rows, and the tiles' first rows: one buffer, one copy back
+    Buf<int64_t> work(ntiles + 2 + (ntiles + 2) / 2, s), cpos;
+    int64_t *tsize = work.get();
+    int32_t *flags = reinterpret_cast<int32_t *>(tsize + ntiles + 1), *tile_first = flags + 2;
+    TP_CUDA(cudaMemsetAsync(flags, 0, 2 * sizeof(int32_t), s));
     const bool hubs = c->max_deg > kChunkThreshold;
     if (hubs) cpos.alloc(c->m2 / kChunkSize + 1, s);
-    launch(k_rows, grid_for(n + 1, 256), 256, 0, s, c->xadj.get(), nullptr, n, c->m2,
-           tile_first.get(), flags.get(), flags.get() + 1);
+    launch(k_rows, grid_for(n + 1, 256), 256, 0, s, c->xadj.get(), nullptr, n, c->m2, tile_first, flags,
+           flags + 1);
     const unsigned tb = grid_for(ntiles, 1, (int64_t)num_sms() * 16);
     launch(hubs ? k_zip_tiles<false, true> : k_zip_tiles<false, false>, tb, kTileThreads, 0, s, v,
-           tile_first.get(), ntiles, tsize.get(), nullptr, nullptr, nullptr, nullptr);
+           tile_first, ntiles, tsize, nullptr, nullptr, nullptr, nullptr);
     TP_LAUNCH_CHECK();
-    exclusive_scan_i64(tsize.get(), tsize.get(), ntiles, s);
-    int64_t body = 0;
-    int32_t empties = 0;
-    TP_CUDA(cudaMemcpyAsync(&empties, flags.get() + 1, 4, cudaMemcpyDeviceToHost, s));
-    TP_CUDA(cudaMemcpyAsync(&body, tsize.get() + ntiles, 8, cudaMemcpyDeviceToHost, s));
+    exclusive_scan_i64(tsize, tsize, ntiles, s);
+    int64_t h[2];  // the body's bytes, the flags
+    TP_CUDA(cudaMemcpyAsync(h, tsize + ntiles, sizeof(h), cudaMemcpyDeviceToHost, s));
     TP_CUDA(cudaStreamSynchronize(s));
+    const int64_t body = h[0];
+    const bool empties = h[1] >> 32 != 0;
     int tl = 1;
     for (uint64_t x = (uint64_t)c->m2; x >= 128; x >>= 7) ++tl;
     z->nbytes = (uint64_t)body + tl;
     z->bytes.alloc(z->nbytes + kBytePad, s);
-    TP_CUDA(cudaMemsetAsync(z->bytes.get() + z->nbytes, 0, kBytePad, s));
     z->off_is64 = wide_offsets(z->nbytes);
     if (z->off_is64) z->off64.alloc(n + 1, s);
     else z->off32.alloc(n + 1, s);
     launch(hubs ? k_zip_tiles<true, true> : k_zip_tiles<true, false>, tb, kTileThreads, 0, s, v,
-           tile_first.get(), ntiles, tsize.get(), z->bytes.get(), z->off32.get(), z->off64.get(),
-           cpos.get());
-    launch(k_zip_empty, empties ? grid_for((n + 31) / 32, 256) : 1, 256, 0, s, c->xadj.get(), n, body,
-           empties != 0, z->bytes.get(), z->off32.get(), z->off64.get());
+           tile_first, ntiles, tsize, z->bytes.get(), z->off32.get(), z->off64.get(), cpos.get());
+    launch(k_zip_empty, empties ? grid_for((n + 7) / 8, 256) : 1, 256, 0, s, c->xadj.get(), n, c->m2,
+           body, empties, z->bytes.get(), z->off32.get(), z->off64.get());
     if (hubs)
       launch(k_zip_tables, grid_for(n, 256), 256, 0, s, c->xadj.get(), n, z->off32.get(),
              z->off64.get(), cpos.get(), z->bytes.get());
-    launch(k_zip_terminal, 1, 1, 0, s, (uint64_t)body, c->m2, z->bytes.get());
     TP_LAUNCH_CHECK();
     z->total_vw = c->total_vw;
     TP_CUDA(cudaStreamSynchronize(s));
