@@ -104,8 +104,8 @@ __host__ __device__ constexpr int64_t agg_start(int size) {
 __global__ void __launch_bounds__(256)
     k_agg_classes(const unsigned long long *ent, const int32_t *mcnt, int64_t nc, int64_t *cvw,
                   int32_t *lists, int32_t *cnt, unsigned long long *rows) {
-  __shared__ int64_t part[8];
-  int64_t mine = 0;
+  __shared__ int64_t part[8], part0[8];
+  int64_t mine = 0, low = 0;
   for (int64_t a0 = (int64_t)blockIdx.x * blockDim.x; a0 < nc;
        a0 += (int64_t)gridDim.x * blockDim.x) {
     const int64_t a = a0 + threadIdx.x;
@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(256)
       cl = 0;
       while (cl < kAggSizes && e > agg_start(cl)) ++cl;
       if (cl < kAggSizes) mine += (int64_t)ent[a];
+      if (cl == 0) low += (int64_t)ent[a];
       if (cvw) cvw[a] = mcnt[a];
     }
     const unsigned peers = __match_any_sync(kFull, cl);
@@ -127,11 +128,13 @@ __global__ void __launch_bounds__(256)
     }
   }
   mine = warp_sum(mine);
-  if (lane_id() == 0) part[threadIdx.x >> 5] = mine;
+  low = warp_sum(low);
+  if (lane_id() == 0) part[threadIdx.x >> 5] = mine, part0[threadIdx.x >> 5] = low;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) mine += part[w];
-    if (mine) atomicAdd(rows, (unsigned long long)mine);
+    for (int w = 1; w < 8; ++w) mine += part[w], low += part0[w];
+    if (mine) atomicAdd(&rows[0], (unsigned long long)mine);
+    if (low) atomicAdd(&rows[1], (unsigned long long)low);
   }
 }
 
@@ -529,6 +532,7 @@ __global__ void __launch_bounds__(32 * agg_warps(SIZE), SIZE == 0 && !COMP ? 6 :
 // Sizes 2 and 3: a block per coarse vertex, its warps taking 32 members each
 // in turn.
 constexpr int64_t kAggDecodeDeg = 1024;  // compressed graphs beyond this degree are decoded first
+constexpr int64_t kSortZip = (int64_t)1 << 23;  // (from this many entries on)
 constexpr int kAggThreads = 256;
 constexpr int kAggWide = 256;
 // The largest table with 64-bit sums has half the slots.
@@ -915,8 +919,27 @@ __global__ void k_add_i64(const int64_t *a, int64_t n, int64_t *b) {
     b[i] += a[i];
 }
 
+// How rows are summed: as it suits the graph, all sorted, or through the tables
+// with no more room than a sample says.
+enum RowMode { ROWS_ANY, ROWS_SORTED, ROWS_TIGHT };
+
 // Graphs of at least this many vertices are sampled for the room of the rows.
 constexpr int64_t kSampleFrom = (int64_t)1 << 20;
+
+// Whether all rows are sorted at once instead of through the tables, which one
+// after the other wait for their longest coarse vertices: skewed graphs of 2^18
+// to 2^25 entries of which some coarse vertices are long (or of which few
+// entries merge: long single rows overflow the table they start in), unless most
+// entries are short rows' or merge strongly. R-MAT of 20 000, 64 752, 2e5, 4e5
+// and 1e6 vertices, k = 2: 0.85, 1.13, 1.46, 1.85, 3.27 ms through the tables,
+// 0.52, 0.63, 0.89, 1.32, 3.35 sorted; meshes of those sizes take twice as long
+// sorted. cnt: coarse vertices by first size, low: entries of those of the
+// smallest.
+bool sort_pays(int64_t m2, int64_t nc, const int32_t (&cnt)[kAggSizes + 1], int64_t low) {
+  if (m2 < ((int64_t)1 << 18) || m2 > ((int64_t)1 << 25) || (m2 > ((int64_t)1 << 21) && 5 * low > 4 * m2))
+    return false;
+  return (cnt[3] + cnt[4] > 0 && m2 <= 1300 * nc) || (cnt[2] > 0 && m2 <= 200 * nc);
+}
 
 // The block of k_agg_block / k_agg_warp grids: as many as fit the SMs, no more
 // than the longest the list can become.
@@ -941,9 +964,9 @@ void launch_agg(const AggCtx &c, const int64_t (&most)[kAggSizes], cudaStream_t 
 
 // The contraction itself. own (nullable): holds g if g is a decoded copy, freed
 // as soon as its rows are summed.
-static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own, const int32_t *C,
-                               int32_t *d_map, cudaStream_t s, const int64_t *seg_voff, int64_t nseg,
-                               int64_t *seg_coff) {
+static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own, RowMode mode,
+                               const int32_t *C, int32_t *d_map, cudaStream_t s,
+                               const int64_t *seg_voff, int64_t nseg, int64_t *seg_coff) {
   const int64_t n = g->n;
   tp_graph *cg = new_graph();
   try {
@@ -992,27 +1015,25 @@ static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own
     // members by coarse vertex, and the first table size of each
     Buf<int32_t> members(n, s), lists((kAggSizes + 1) * nc, s);
     Buf<int64_t> mstart(nc + 1, s);
-    // [0] cursor [1] largest weight [2], [3] items [4] rows' bound [5], [6] sample;
-    // then the lists' lengths (int32)
-    constexpr int kAcc = 7;
+    // [0] cursor [1] largest weight [2], [3] items [4] rows' bound [5] entries of the
+    // smallest table [6], [7] sample; then the lists' lengths (int32)
+    constexpr int kAcc = 8;
     Buf<int64_t> acc(kAcc + (kAggSizes + 2) / 2, s);
     TP_CUDA(cudaMemsetAsync(acc.get(), 0, acc.n * sizeof(int64_t), s));
     int32_t *cnt = reinterpret_cast<int32_t *>(acc.get() + kAcc);
+    Buf<int32_t> place(n, s), mcnt(nc, s);
     {
-      Buf<int32_t> place(n, s), mcnt(nc, s);
       Buf<unsigned long long> ent(nc, s);
       TP_CUDA(cudaMemsetAsync(mcnt.get(), 0, nc * sizeof(int32_t), s));
       TP_CUDA(cudaMemsetAsync(ent.get(), 0, nc * sizeof(unsigned long long), s));
       launch(k_map, grid_for(n, 256), 256, 0, s, v, C, rank.get(), map, cg->vw.get(), place.get(),
              mcnt.get(), ent.get());
-      exclusive_scan_i32_to_i64(mcnt.get(), mstart.get(), nc, s);
-      launch(k_members, grid_for(n, 256), 256, 0, s, map, place.get(), mstart.get(), n, members.get());
       launch(k_agg_classes, grid_for(nc, 256), 256, 0, s, ent.get(), mcnt.get(), nc,
              g->unit_vw ? cg->vw.get() : nullptr, lists.get(), cnt,
              (unsigned long long *)(acc.get() + 4));
-      if (n >= kSampleFrom)
+      if (n >= kSampleFrom || mode == ROWS_TIGHT)
         launch(comp ? k_row_sample<true> : k_row_sample<false>, (unsigned)(kRowSamples * 32 / 256), 256,
-               0, s, v, map, (unsigned long long *)(acc.get() + 5));
+               0, s, v, map, (unsigned long long *)(acc.get() + 6));
       TP_LAUNCH_CHECK();
     }
     rank.release();
@@ -1030,9 +1051,18 @@ static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own
     // inter-cluster ones (a third in a mesh, whose rows of all entries were the
     // peak of a partition); if that falls short the tables are filled again with
     // the room they turned out to need
-    int64_t room = std::min<int64_t>(ha[4], g->m2);
-    if (n >= kSampleFrom && ha[6] > 0)
-      room = std::min<int64_t>(room, (int64_t)(1.25 * (double)g->m2 * (double)ha[5] / (double)ha[6]) + n / 16);
+    const bool keys_only =
+        mode == ROWS_SORTED || (mode == ROWS_ANY && !seg_voff && sort_pays(g->m2, nc, hc, ha[5]));
+    if (!keys_only) {
+      exclusive_scan_i32_to_i64(mcnt.get(), mstart.get(), nc, s);
+      launch(k_members, grid_for(n, 256), 256, 0, s, map, place.get(), mstart.get(), n, members.get());
+      TP_LAUNCH_CHECK();
+    }
+    place.release();
+    mcnt.release();
+    int64_t room = keys_only ? 0 : std::min<int64_t>(ha[4], g->m2);
+    if (!keys_only && ha[7] > 0)
+      room = std::min<int64_t>(room, (int64_t)(1.25 * (double)g->m2 * (double)ha[6] / (double)ha[7]) + n / 16);
     Buf<int32_t> tkey;
     Buf<uint32_t> tval32;
     Buf<unsigned long long> tval64;
@@ -1051,7 +1081,7 @@ static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own
     c.max_w = (unsigned long long *)(acc.get() + 1);
     c.toff = toff.get();
     c.deg = cg->xadj.get();
-    for (;;) {
+    while (!keys_only) {
       tkey.alloc(std::max<int64_t>(room, 1), s);
       if (narrow) tval32.alloc(std::max<int64_t>(room, 1), s);
       else tval64.alloc(std::max<int64_t>(room, 1), s);
@@ -1071,7 +1101,7 @@ static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own
       TP_CUDA(cudaMemsetAsync(acc.get(), 0, 2 * sizeof(int64_t), s));
       TP_CUDA(cudaMemcpyAsync(cnt, hc, sizeof(hc), cudaMemcpyHostToDevice, s));
     }
-    const int64_t n_sorted = reinterpret_cast<const int32_t *>(ha + kAcc)[kAggSizes];
+    const int64_t n_sorted = keys_only ? nc : reinterpret_cast<const int32_t *>(ha + kAcc)[kAggSizes];
     int64_t max_w = ha[1], m2 = ha[0], runs = 0;
 
     // coarse vertices beyond the tables: keys, sort, run lengths
@@ -1080,9 +1110,10 @@ static tp_graph *contract_rows(const tp_graph *g, std::unique_ptr<tp_graph> *own
     Buf<int64_t> rval, rstart;
     if (n_sorted) {
       sorted.alloc(nc, s);
-      TP_CUDA(cudaMemsetAsync(sorted.get(), 0, nc, s));
-      launch(k_mark_sorted, grid_for(n_sorted, 256), 256, 0, s, lists.get() + kAggSizes * nc, n_sorted,
-             sorted.get());
+      TP_CUDA(cudaMemsetAsync(sorted.get(), keys_only ? 1 : 0, nc, s));
+      if (!keys_only)
+        launch(k_mark_sorted, grid_for(n_sorted, 256), 256, 0, s, lists.get() + kAggSizes * nc, n_sorted,
+               sorted.get());
       RowItems ri{};
       ri.room = n + g->m2 / kChunkSize + 1;
       Buf<uint64_t> items((size_t)ri.room, s);
@@ -1184,16 +1215,23 @@ tp_graph *contract(const tp_graph *g, const int32_t *C, int32_t *d_map, cudaStre
   // a warp): in the tables' kernels such a record is one warp's, and level 0
   // of R-MAT 2^22 spent 39 ms in them where decoding takes 2 and the CSR
   // kernels 13.5. Where there is no room for the decoded copy the records are
-  // read as they are.
+  // read as they are (a mesh with a hub needs half as much that way). Small ones
+  // are sorted, which takes a record apart by chunks: R-MAT of 64 752 vertices,
+  // k = 256: 0.97 -> 0.78 ms.
+  RowMode mode = ROWS_ANY;
   if (g->compressed && g->max_deg > kAggDecodeDeg) {
-    try {
-      std::unique_ptr<tp_graph> csr(decompress(g, s));
-      return contract_rows(csr.get(), &csr, C, d_map, s, seg_voff, nseg, seg_coff);
-    } catch (const Error &e) {
-      if (e.code != TP_ERR_OOM && e.code != TP_ERR_BUDGET) throw;
+    mode = ROWS_SORTED;
+    if (g->m2 > kSortZip) {
+      try {
+        std::unique_ptr<tp_graph> csr(decompress(g, s));
+        return contract_rows(csr.get(), &csr, ROWS_ANY, C, d_map, s, seg_voff, nseg, seg_coff);
+      } catch (const Error &e) {
+        if (e.code != TP_ERR_OOM && e.code != TP_ERR_BUDGET) throw;
+      }
+      mode = ROWS_TIGHT;
     }
   }
-  return contract_rows(g, nullptr, C, d_map, s, seg_voff, nseg, seg_coff);
+  return contract_rows(g, nullptr, mode, C, d_map, s, seg_voff, nseg, seg_coff);
 }
 
 }  // namespace tp

@@ -61,12 +61,17 @@ def test_sample_that_falls_short(weighted):
 def test_no_room_to_decode():
     """With less memory than the decoded copy and the rows take together the
     records are contracted, with far less than either the call fails cleanly."""
-    xadj, adj = synth.rmat(16, 16, seed=2)
-    n = len(xadj) - 1
-    assert np.diff(xadj).max() > 1024
+    n, d = 700001, 5000  # a mesh with a hub, more than 2^23 entries (smaller ones are not decoded)
+    mesh = synth.rgg2d(n, 16.0, 3)
+    u = np.repeat(np.arange(n, dtype=np.int64), np.diff(mesh[0]))
+    spokes = np.arange(1, d + 1, dtype=np.int64) * (n // (d + 1))
+    key = np.unique(np.concatenate([u * n + mesh[1], spokes, spokes * n]))
+    xadj = np.zeros(n + 1, np.int64)
+    np.add.at(xadj, key // n + 1, 1)
+    xadj, adj = np.cumsum(xadj), (key % n).astype(np.int32)
+    assert len(adj) > 1 << 23 and np.diff(xadj).max() > 1024
     z = tp.graph_from_csr(xadj, adj).compress()
-    # few coarse entries: the copy lies in the peak (it is gone before they are made)
-    C = torch.arange(n, dtype=torch.int32, device="cuda") // 256
+    C = tp.lp_cluster(z, 300)
     want, want_map = oracle.contract(oracle.Graph(xadj, adj), C.cpu().numpy())
     live, peak, limit = {}, [0], [1 << 60]
 
