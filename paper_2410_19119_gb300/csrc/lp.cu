@@ -1109,7 +1109,9 @@ double tier_round_bytes(const tp_graph *g, int64_t n_t, int64_t e_t) {
 }
 
 // Entries in the tiers above the small one from which their kernels go side by
-// side: a fork and join cost about 10 us of launches per sub-round.
+// side: a fork and join cost about 10 us of launches per sub-round. With against
+// without, clustering: R-MAT with 1.3e6 such entries 0.58, 4e6 0.60, 2.4e7 0.65,
+// a mesh with 1.8e6 0.88, a uniform random graph with 6e6 in one tier 1.05.
 constexpr int64_t kForkEntries = (int64_t)1 << 19;
 
 template <int MODE>
@@ -1942,17 +1944,21 @@ void lp_rounds(tp_graph *g, const LpState &st, LpWork &w, uint64_t seed, uint64_
   // quiet vertices: one graph, most entries in the lane tier, and so few
   // sub-rounds that the epoch (one step each at most) fits its byte. In
   // clustering nearly every vertex moves in the first two rounds, which go
-  // without (labels are vertices then: kmax is 0), and the two rounds after
-  // them cost more with the marks than they save: on a mesh of 2^24 vertices 3
-  // rounds took 8.39 ms with and 7.58 without them, 5 rounds 11.27 and 11.20,
-  // 6 rounds 12.30 and 12.98, 12 rounds 16.6 and 23.5 (CSR); where decoding
-  // makes a rating dearer 5 rounds took 11.29 and 12.10.
+  // without (labels are vertices then: kmax is 0), and the rounds after them
+  // cost more with the marks than they save in small levels and few rounds.
+  // Meshes of degree 16, with marks against without, CSR / compressed: 6e5
+  // vertices, 5 rounds 1.00 (none) / 1.11, 8 rounds 1.12 / 1.14; 2^21, 6 rounds
+  // 0.99 / 0.99, 8 rounds 0.94 / 0.96; 2^23, 5 rounds 1.00 (none) / 0.95, 6
+  // rounds 0.95 / 0.91, 12 rounds 0.74 / 0.75; 2^24 and CSR, 3 rounds 1.11, 5
+  // rounds 1.01. In refinement the marks pay from two rounds on: 6e5 vertices
+  // 0.94 / 0.96, five rounds 0.89 / 0.90; 2^23 0.73 / 0.75 and 0.53 / 0.56.
   const int32_t quiet_from = st.kmax ? 0 : 2;
   // A single round rates every vertex once, so marks are of no use in it.
-  const int32_t quiet_least = st.kmax ? 2 : g->compressed ? 5 : 6;
+  const int32_t quiet_least = st.kmax ? 2 : g->compressed && g->n >= ((int64_t)1 << 22) ? 5 : 6;
   const bool quiet_ok = !st.seg.gid && S <= 32 && (int64_t)rounds * S < 250 && rounds >= quiet_least &&
-                        !T.lane_long && !prof_active() && 5 * T.edges[TIER_LANE] >= 4 * g->m2 &&
-                        g->n <= kLaneKeyLabels && st.nlabels <= kLaneKeyLabels;
+                        (st.kmax || g->n >= ((int64_t)1 << 21)) && !T.lane_long && !prof_active() &&
+                        5 * T.edges[TIER_LANE] >= 4 * g->m2 && g->n <= kLaneKeyLabels &&
+                        st.nlabels <= kLaneKeyLabels;
   std::unique_ptr<ApprovalGraph> ag;
   for (int32_t r = 0; r < rounds; ++r) {
     const bool quiet = quiet_ok && r >= quiet_from;

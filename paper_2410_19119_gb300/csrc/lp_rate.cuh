@@ -585,10 +585,6 @@ __device__ __forceinline__ void emit_lane(const RateCtx &c, bool has, int32_t u,
   }
 }
 
-// Rates one batch: this lane's vertex u with deg neighbours (compressed:
-// already decoded into the column; CSR: adjacency from xadj[u]) and emits
-// the favourite, or queues the move in the warp's window buffer (nmv
-// records so far, warp-uniform). N >= the largest degree of the batch.
 // LIVE: labels change while the kernel runs (k_lp_small), so they are not read
 // through the read-only path.
 template <bool LIVE>
@@ -599,6 +595,10 @@ __device__ __forceinline__ int32_t load_label(const int32_t *p) {
 // Labels below this fit a 32-bit sort key with the slot (weighted lane tier).
 constexpr int64_t kLaneKeyLabels = ((int64_t)1 << 27) - 1;
 
+// Rates one batch: this lane's vertex u with deg neighbours (compressed:
+// already decoded into the column; CSR: adjacency from xadj[u]) and emits
+// the favourite, or queues the move in the warp's window buffer (nmv
+// records so far, warp-uniform). N >= the largest degree of the batch.
 // WIDE (weighted): labels beyond kLaneKeyLabels, sorted with the weights in
 // 64-bit keys.
 // QUIET: vertices without a better label are marked quiet.
