@@ -182,9 +182,10 @@ extern "C" {
 //            takes 88n (the sum counted, 174n, is more than either needs); hub
 //            rating tables 14 bytes per slot, fewer than 4 slots per hub
 //            neighbour: 56m
-//   contract flags, ranks, members, offsets 32n; the tables' rows 12m and the
-//            coarse CSR 12m, or, where every coarse vertex is a hub, keys and
-//            weights with their radix buffers 32m; a compressed level decoded
+//   contract flags, ranks, members, offsets 32n; the tables' rows, 12m at
+//            most, and the coarse CSR 12m, or, where all entries are sorted
+//            (skewed graphs, or all coarse vertices hubs), keys and weights
+//            with their radix buffers 32m; a compressed level decoded
 //            for it 8n + 4m, within what clustering is counted for
 //   initial  T attempts x 53 bytes per coarsest vertex (22 and lists used) + 40
 //            + its CSR 12m
